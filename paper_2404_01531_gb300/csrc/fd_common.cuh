@@ -19,8 +19,17 @@ __device__ __forceinline__ double* ext_at(const Dev& d, int q, int wl) {
     return d.ext + ((int64_t)q * d.chunk + wl) * ext_size(d);
 }
 __device__ __forceinline__ int64_t nface(const Dev& d) { return (int64_t)(d.nc + 1) * d.nc * d.nc; }
-// flux layout: [3][NV][chunk][nface]; curved meshes keep every physical
-// component j: [3 (k)][3 (j)][NV][chunk][nface]
+// A face of direction k is m (0..nc) along k, (ta, tb) across; index
+// ta + nc tb + nc^2 m, so that the threads of neighbouring lines, which reach
+// their faces together, store to neighbouring addresses.
+__device__ __forceinline__ int face_index(int nc, int m, int ta, int tb) { return ta + nc * (tb + nc * m); }
+// face results: boxes the flux [3][NV][chunk][nface]; flat shells the face states
+// [3][NFS][chunk][nface] (k_fd_states); the Kerr-Schild background every
+// physical component j of the flux, [3 (k)][3 (j)][NV][chunk][nface]
+constexpr int NFS = NQ + NV;
+__device__ __forceinline__ double* fstate_at(const Dev& d, int k, int q, int wl) {
+    return d.flux + (((int64_t)k * NFS + q) * d.chunk + wl) * nface(d);
+}
 __device__ __forceinline__ double* flux_at(const Dev& d, int k, int v, int wl) {
     return d.flux + (((int64_t)k * NV + v) * d.chunk + wl) * nface(d);
 }
@@ -52,7 +61,7 @@ __device__ __forceinline__ ShellGeo shell_for(const Dev& d, int e, int& el) {
 // coordinates and radii of its rows (Dev::stab): base indices of the element's
 // angular and radial rows on the half-cell grid, its wedge axes and side.
 struct ShellPts {
-    const double *tx, *tw, *tr, *tir;
+    const double *tx, *tw, *tn, *tr, *tir;
     int gx, gy, gr, pn;
     double s, na, nr, c;
 };
@@ -66,8 +75,9 @@ __device__ __forceinline__ ShellPts shell_pts(const Dev& d, int e, int nc) {
     const int nx = 2 * nc * g.na + 1, nrr = 2 * nc * g.nr + 1;
     p.tx = t;
     p.tw = t + nx;
-    p.tr = t + 2 * nx;
-    p.tir = t + 2 * nx + nrr;
+    p.tn = t + 2 * nx;
+    p.tr = t + 3 * nx;
+    p.tir = t + 3 * nx + nrr;
     p.gx = 2 * nc * ia;
     p.gy = 2 * nc * ib;
     p.gr = 2 * nc * ir;
@@ -92,6 +102,16 @@ __device__ __forceinline__ void shell_face_normal(const ShellPts& p, int k, int 
     shell_normal_closed(k, X, Y, p.pn, p.s, nh);
 }
 
+// grad xi^k at the centre of cell cc (row ijk of its inverse Jacobian) times the unit
+// normal at face m of direction k next to it: for k = 0 with X_c, T the gnomonic
+// coordinates of the centre and the face, na rho/(q (1+X_c^2) r) (1 + X_c T)/sqrt(1 + T^2)
+// (likewise k = 1); for k = 2 both are along x^, and it is |grad xi^2|.
+__device__ __forceinline__ double shell_grad_normal(const ShellPts& p, int k, const int* cc, int m, const double* ijk) {
+    if (k == 2) return p.nr * p.tir[p.gr + 2 * cc[2] + 1] / p.c;
+    const int g = k == 0 ? p.gx : p.gy, pt = (p.pn + 1 + k) % 3;
+    return ijk[pt] * p.tn[g + 2 * m] * fma(p.tx[g + 2 * cc[k] + 1], p.tx[g + 2 * m], 1.0);
+}
+
 __device__ __forceinline__ void axes_of(int dd, int& t1, int& t2) {
     t1 = dd == 0 ? 1 : 0;
     t2 = dd == 2 ? 1 : 2;
@@ -103,90 +123,207 @@ __device__ __forceinline__ int chunk_n(const Dev& d, int ci, int w0) {
     return n < 0 ? 0 : (n > d.chunk ? d.chunk : n);
 }
 
-// WENO5-Z at the face right of v2 from v0..v4 (point-value interpolation
-// candidates, ideal weights (1, 10, 5)/16, Jiang-Shu indicators, Z weights q = 2).
-// The Z weights alpha_k = d_k (1 + tau^2/b_k^2), b_k = beta_k + eps, are scaled
-// by b_0^2 b_1^2 b_2^2 so that the normalised combination needs one division:
-//   A_k = d_k (b_k^2 + tau^2) prod_{j != k} b_j^2,  value = sum A_k p_k / sum A_k.
-// With eps >= 1e-40 every A_k stays above 1e-240, inside the normal range.
-// At the other end the products of six indicators overflow once an indicator
+// WENO5-Z (point-value interpolation candidates, ideal weights (1, 10, 5)/16,
+// Jiang-Shu indicators, Z weights q = 2): the weights
+// alpha_k = d_k (1 + t^2/b_k^2), b_k = beta_k + eps, t = b_0 - b_2, are scaled by
+// X = b_0^2 b_1^2 b_2^2, so that the normalised combination needs one division:
+//   A_k = d_k (X + t^2 prod_{j != k} b_j^2),  value = sum A_k p_k / sum A_k.
+// At the upper end the products of six indicators overflow once an indicator
 // exceeds about 1e51 (stencil differences of about 1e25): the weights then
 // become Inf/NaN and the status word reports it.  Field values that large are
 // far outside any state of this system (the fields are of order one).
-// weno5z_combine: the Z-weighted combination of three candidates from their
-// indicators b_k (eps included); the ideal weights are taken as (1, 10, 5)
-// (scale-free).
-__device__ __forceinline__ double weno5z_combine(double b0, double b1, double b2, double p0, double p1, double p2) {
-    // A_k = d_k (b_k^2 + t^2) P_k with P_k the product of the other two b_j^2
-    // is d_k (X + t^2 P_k), X = b_0^2 b_1^2 b_2^2 shared by the three
-    const double t = b0 - b2;
-    const double t2 = t * t;
-    const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
-    const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1;
-    const double X = q0 * P0;
-    const double A0 = fma(t2, P0, X), A1 = 10.0 * fma(t2, P1, X), A2 = 5.0 * fma(t2, P2, X);
-    return fma(A0, p0, fma(A1, p1, A2 * p2)) * recip_nr(A0 + A1 + A2);
-}
+//
+// Reconstruction along one line of cells (one quantity): cell() takes the cell
+// two ahead of the current centre c and gives both face values of c -- right:
+// the left state of the face to its right, left: the right state of the face to
+// its left -- then moves on to c + 1.  A thread that marches a line so does per
+// cell what a thread per face does twice: the two values of a cell use the same
+// three stencils, hence the same smoothness indicators, and the differences of
+// a stencil are those of the next one shifted.  All offsets are taken from the
+// centre value.
+//
+// WENO5-Z: with a_k the second difference of stencil k (left, centred, right) and
+// e_k / 2 its slope at the centre, the candidate at the face +-1/2 is
+// v_c + a_k / 8 +- e_k / 4, and beta_k = (13/12) a_k^2 + (e_k / 2)^2.  The kept
+// per-stencil values are h = a/8 and k = (13/12) a^2 + eps; ideal weights
+// (1, 10, 5) towards the right face and (5, 10, 1) towards the left one, the Z
+// weights in the form above.  52 FP64 operations per cell and
+// quantity where a thread per face spends 87.  eps is at least 1e-51, so that
+// products of six indicators stay normal.
+struct Weno5zLine {
+    double dA, dB, hA, hB, kA, kB, vc, vn, eps;
+    __device__ __forceinline__ double curv(double h) const { return fma((13.0 / 12.0 * 64.0) * h, h, eps); }
+    __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double weno_eps) {
+        eps = fmax(weno_eps, 1e-51);
+        const double d01 = v1 - v0;
+        dA = v2 - v1;
+        dB = v3 - v2;
+        hA = 0.125 * (dA - d01);
+        hB = 0.125 * (dB - dA);
+        kA = curv(hA);
+        kB = curv(hB);
+        vc = v2;
+        vn = v3;
+    }
+    template <bool LEFT, bool RIGHT>
+    __device__ __forceinline__ void cell(double v4, double& left, double& right) {
+        const double dC = v4 - vn, hC = 0.125 * (dC - dB), kC = curv(hC);
+        const double e0 = fma(4.0, hA, dA), e1 = fma(4.0, hB, dA), e2 = fma(-4.0, hC, dB);   // slopes at the centre
+        const double b0 = fma(e0, e0, kA), b1 = fma(e1, e1, kB), b2 = fma(e2, e2, kC);
+        const double t = b0 - b2, t2 = t * t;
+        const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
+        const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1, X = q0 * P0;
+        const double S0 = fma(t2, P0, X), S1 = 10.0 * fma(t2, P1, X), S2 = fma(t2, P2, X);
+        if (RIGHT) {
+            const double g0 = fma(0.5, e0, hA), g1 = fma(0.5, e1, hB), g2 = fma(0.5, e2, hC), T = 5.0 * S2;
+            right = fma(fma(S0, g0, fma(S1, g1, T * g2)), recip_nr((S0 + S1) + T), vc);
+        }
+        if (LEFT) {
+            const double g0 = fma(-0.5, e0, hA), g1 = fma(-0.5, e1, hB), g2 = fma(-0.5, e2, hC), T = 5.0 * S0;
+            left = fma(fma(T, g0, fma(S1, g1, S2 * g2)), recip_nr((T + S1) + S2), vc);
+        }
+        dA = dB; dB = dC;
+        hA = hB; hB = hC;
+        kA = kB; kB = kC;
+        vc = vn; vn = v4;
+    }
+};
 
-// Both values at the face between v2 and v3 from the six cells v0..v5: uL the
-// WENO5-Z value from v0..v4, uR the one from v5..v1 (mirrored).  Everything is
-// built from the first differences d_i = v_{i+1} - v_i: the candidates (the
-// quadratics through v0..v2, v1..v3, v2..v4 and v3..v5 at the face), the
-// second differences a and the one-sided combinations e of the Jiang-Shu
-// indicators beta = (13/12) a^2 + (1/4) e^2, of which 4 (beta + eps) enter
-// the weights (they are invariant under a common scale of the indicators).
-// The two values share two candidates and two second differences.
-__device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, double v3, double v4, double v5,
-                                            double eps, double& uL, double& uR) {
-    const double d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3, d45 = v5 - v4;
-    const double p123 = fma(0.125, d12, fma(0.375, d23, v2));
-    const double p234 = fma(0.625, d23, fma(-0.125, d34, v2));
-    const double pL0 = fma(-0.375, d01, fma(0.875, d12, v2));
-    const double pR0 = fma(-0.875, d34, fma(0.375, d45, v3));
-    const double a012 = d12 - d01, a123 = d23 - d12, a234 = d34 - d23, a345 = d45 - d34;
-    const double eL0 = fma(2.0, d12, a012), eL1 = d12 + d23, eL2 = fma(-2.0, d23, a234);
-    const double eR0 = fma(-2.0, d34, a345), eR1 = d23 + d34, eR2 = fma(2.0, d23, a123);
-    const double c = 13.0 / 3.0, eps4 = 4.0 * eps;
-    const double c123 = c * a123, c234 = c * a234;
-    const double bL0 = fma(c * a012, a012, fma(eL0, eL0, eps4));
-    const double bL1 = fma(c123, a123, fma(eL1, eL1, eps4));
-    const double bL2 = fma(c234, a234, fma(eL2, eL2, eps4));
-    const double bR0 = fma(c * a345, a345, fma(eR0, eR0, eps4));
-    const double bR1 = fma(c234, a234, fma(eR1, eR1, eps4));
-    const double bR2 = fma(c123, a123, fma(eR2, eR2, eps4));
-    uL = weno5z_combine(bL0, bL1, bL2, pL0, p123, p234);
-    uR = weno5z_combine(bR0, bR1, bR2, pR0, p234, p123);
-}
-
-// MP5 value at the right face of v2 from v0..v4 (point values): Suresh &
-// Huynh's monotonicity-preserving limiter (J. Comput. Phys. 136, 83 (1997))
-// on the 5-point interpolant (3 v0 - 20 v1 + 90 v2 + 60 v3 - 5 v4)/128, alpha = 4:
-// the interpolant when it lies between v2 and v_MP = v2 + minmod(v3 - v2,
-// alpha (v2 - v1)), else its median with the bounds built from v_UL, v_MD,
-// v_LC and the minmod4 curvatures of the second differences.
-__device__ __forceinline__ double minmod2(double a, double b) {
-    return a * b > 0.0 ? (fabs(a) < fabs(b) ? a : b) : 0.0;
-}
+// MP5 (Suresh & Huynh, J. Comput. Phys. 136, 83 (1997)) on the 5-point
+// interpolant (3, -20, 90, 60, -5)/128, alpha = 4: the interpolant where its
+// offset d from v_c lies between 0 and v_MP - v_c = minmod(v_+ - v_c, 4 (v_c -
+// v_-)), else its median with the bounds built from v_UL, v_MD, v_LC and the
+// minmod4 curvatures.  Both bounds contain the centre (lower <= v_c <= upper), so
+// the median is d limited to [-N, P].  Only magnitudes and signs are compared, as
+// integers: an FP64 comparison takes the FP64 pipe, 1/32 of the integer rate.
+__device__ __forceinline__ unsigned long long fbits(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ unsigned long long fmag(double x) { return fbits(x) & 0x7fffffffffffffffULL; }
+__device__ __forceinline__ bool fneg(double x) { return __double_as_longlong(x) < 0; }
+__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
+__device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
 
 __device__ __forceinline__ double minmod4(double a, double b, double c, double d) {
-    if (a > 0.0 && b > 0.0 && c > 0.0 && d > 0.0) return fmin(fmin(a, b), fmin(c, d));
-    if (a < 0.0 && b < 0.0 && c < 0.0 && d < 0.0) return fmax(fmax(a, b), fmax(c, d));
-    return 0.0;
+    const bool s = fneg(a);
+    if (fneg(b) != s || fneg(c) != s || fneg(d) != s) return 0.0;
+    const unsigned long long m = umin(umin(fmag(a), fmag(b)), umin(fmag(c), fmag(d)));
+    return __longlong_as_double((long long)(s ? m | 0x8000000000000000ULL : m));
 }
 
-__device__ __forceinline__ double mp5(double v0, double v1, double v2, double v3, double v4) {
-    const double vL = fma(0.0234375, v0, fma(-0.15625, v1, fma(0.703125, v2, fma(0.46875, v3, -0.0390625 * v4))));
-    const double vMP = v2 + minmod2(v3 - v2, 4.0 * (v2 - v1));
-    if ((vL - v2) * (vL - vMP) <= 0.0) return vL;
-    const double d1 = v0 - 2.0 * v1 + v2, d2 = v1 - 2.0 * v2 + v3, d3 = v2 - 2.0 * v3 + v4;
-    const double dp = minmod4(4.0 * d2 - d3, 4.0 * d3 - d2, d2, d3);
-    const double dm = minmod4(4.0 * d2 - d1, 4.0 * d1 - d2, d2, d1);
-    const double vUL = v2 + 4.0 * (v2 - v1);
-    const double vMD = 0.5 * (v2 + v3) - 0.5 * dp;
-    const double vLC = v2 + 0.5 * (v2 - v1) + (4.0 / 3.0) * dm;
-    const double vmin = fmax(fmin(fmin(v2, v3), vMD), fmin(fmin(v2, vUL), vLC));
-    const double vmax = fmin(fmax(fmax(v2, v3), vMD), fmax(fmax(v2, vUL), vLC));
-    return vL + minmod2(vmin - vL, vmax - vL);
+// d limited to the median bounds of one face: dn the difference towards the
+// face's far cell, du4 four times the upwind one, md and lc the offsets of v_MD
+// and v_LC.  NaN stays NaN.
+__device__ __forceinline__ double mp5_limit(double d, double dn, double du4, double md, double lc) {
+    auto part = [](double x, bool neg) { return fneg(x) == neg ? fmag(x) : 0ULL; };
+    const bool neg = fneg(d);
+    const unsigned long long lim = umin(umax(part(dn, neg), part(md, neg)), umax(part(du4, neg), part(lc, neg)));
+    const unsigned long long m = fmag(d);
+    if (m <= lim || m > 0x7ff0000000000000ULL) return d;
+    return __longlong_as_double((long long)(neg ? lim | 0x8000000000000000ULL : lim));
+}
+
+struct Mp5Line {
+    double d0, dA, dB, aA, aB, vc, vn;
+    __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double) {
+        d0 = v1 - v0;
+        dA = v2 - v1;
+        dB = v3 - v2;
+        aA = dA - d0;
+        aB = dB - dA;
+        vc = v2;
+        vn = v3;
+    }
+    // the interpolant's offset is inside [0, minmod(dn, du4)]
+    static __device__ __forceinline__ bool inside(double d, double dn, double du4) {
+        const unsigned long long m = fmag(d);
+        return m == 0 || (fneg(d) == fneg(dn) && fneg(d) == fneg(du4) && m <= umin(fmag(dn), fmag(du4)));
+    }
+    template <bool LEFT, bool RIGHT>
+    __device__ __forceinline__ void cell(double v4, double& left, double& right) {
+        const double dC = v4 - vn, aC = dC - dB;
+        // (-3 d0 + 17 dA + 55 dB - 5 dC)/128 and its mirror image
+        double r = fma(-0.0234375, d0, fma(0.1328125, dA, fma(0.4296875, dB, -0.0390625 * dC)));
+        double l = fma(0.0234375, dC, fma(-0.1328125, dB, fma(-0.4296875, dA, 0.0390625 * d0)));
+        const double dA4 = 4.0 * dA, dB4 = -4.0 * dB;
+        const bool okr = !RIGHT || inside(r, dB, dA4), okl = !LEFT || inside(l, -dA, dB4);
+        if (!(okr && okl)) {
+            const double mp = minmod4(fma(4.0, aB, -aC), fma(4.0, aC, -aB), aB, aC);   // curvature at the right face
+            const double mm = minmod4(fma(4.0, aB, -aA), fma(4.0, aA, -aB), aB, aA);   // at the left face
+            if (!okr) r = mp5_limit(r, dB, dA4, 0.5 * (dB - mp), fma(4.0 / 3.0, mm, 0.5 * dA));
+            if (!okl) l = mp5_limit(l, -dA, dB4, -0.5 * (dA + mm), fma(4.0 / 3.0, mp, -0.5 * dB));
+        }
+        if (RIGHT) right = vc + r;
+        if (LEFT) left = vc + l;
+        d0 = dA; dA = dB; dB = dC;
+        aA = aB; aB = aC;
+        vc = vn; vn = v4;
+    }
+};
+
+template <int RECON> struct LineOf { using type = Weno5zLine; };
+template <> struct LineOf<FFE_RECON_MP5> { using type = Mp5Line; };
+
+// Reconstructs two quantities along one line of nc cells with 3 ghosts at each
+// end (pa, pb: the line's first ghost; sb: sign bit flipped in every value of
+// the second) and calls emit(m, La, Ra, Sa, Lb, Rb, Sb) at its faces m = 0..nc in
+// order: left and right states and the sum of the two cells at the face.  Two
+// quantities give a thread two independent chains of operations.
+template <int RECON, class Emit>
+__device__ __forceinline__ void recon_lines(const double* pa, const double* pb, int64_t stride, unsigned long long sb,
+                                            int nc, double eps, Emit emit) {
+    auto b_at = [&](const double* p) { return __longlong_as_double((long long)(fbits(*p) ^ sb)); };
+    typename LineOf<RECON>::type A, B;
+    A.init(pa[0], pa[stride], pa[2 * stride], pa[3 * stride], eps);
+    B.init(b_at(pb), b_at(pb + stride), b_at(pb + 2 * stride), b_at(pb + 3 * stride), eps);
+    pa += 4 * stride;
+    pb += 4 * stride;
+    double La, Lb, Ra, Rb, ca = A.vc, cb = B.vc;
+    A.template cell<false, true>(*pa, Ra, La);
+    B.template cell<false, true>(b_at(pb), Rb, Lb);
+#pragma unroll 1
+    for (int m = 0; m < nc; ++m) {
+        pa += stride;
+        pb += stride;
+        double na, nb;
+        const double Sa = ca + A.vc, Sb = cb + B.vc;
+        ca = A.vc;
+        cb = B.vc;
+        A.template cell<true, true>(*pa, Ra, na);
+        B.template cell<true, true>(b_at(pb), Rb, nb);
+        emit(m, La, Ra, Sa, Lb, Rb, Sb);
+        La = na;
+        Lb = nb;
+    }
+    const double Sa = ca + A.vc, Sb = cb + B.vc;
+    A.template cell<true, false>(pa[stride], Ra, La);
+    B.template cell<true, false>(b_at(pb + stride), Rb, Lb);
+    emit(nc, La, Ra, Sa, Lb, Rb, Sb);
+}
+
+// The flat flux along direction k couples the reconstructed quantities in five
+// pairs (a, b) with a sign s: F_a = s b, F_b = s a -- (E_k, psi), (B_k, phi),
+// (E_i, B_j) with s = 1, (E_j, B_i) with s = -1 for (k, i, j) cyclic -- and
+// (q, J_k) with F_q = J_k only; the other two components of J~ do not enter.
+__device__ __forceinline__ void flux_pair(int k, int pr, int& a, int& b, bool& neg) {
+    const int i = k == 2 ? 0 : k + 1, j = k == 0 ? 2 : k - 1;
+    neg = pr == 3;
+    a = pr == 0 ? k : (pr == 1 ? 3 + k : (pr == 2 ? i : (pr == 3 ? j : 8)));
+    b = pr == 0 ? 6 : (pr == 1 ? 7 : (pr == 2 ? 3 + j : (pr == 3 ? 3 + i : NV + k)));
+}
+constexpr int FLUX_PAIRS = 5;
+
+// Rusanov flux (lambda = 1) of a pair from its states, b carrying the sign s:
+// F_a = (b_L + b_R)/2 - (a_R - a_L)/2 and F_b likewise, with the corrector
+// F - (F_m - 2 F + F_p)/6 = (4/3) F - (F_m + F_p)/6 (S: the sum of the two cells).
+__device__ __forceinline__ void rusanov_pair(double La, double Ra, double Sa, double Lb, double Rb, double Sb, bool corr,
+                                             double& Fa, double& Fb) {
+    const double p = La + Lb, m = Rb - Ra;
+    if (corr) {
+        Fa = fma(-1.0 / 6.0, Sb, (2.0 / 3.0) * (p + m));
+        Fb = fma(-1.0 / 6.0, Sa, (2.0 / 3.0) * (p - m));
+    } else {
+        Fa = 0.5 * (p + m);
+        Fb = 0.5 * (p - m);
+    }
 }
 
 // Reverse mode of weno5z_combine for indicators B_k (eps included) and

@@ -117,8 +117,8 @@ struct Dev {
     int shell_na, shell_nr;
     // flat shells, per instance at InstInfo::tab (single context: 0), on the
     // half-cell grid g = 2 nc i + h of each angular / radial element row (h even:
-    // FD faces, h odd: cell centres): X_g = tan(pi/4 e_g), 1/(pi/4 (1 + X_g^2))
-    // [2 nc na + 1 each], then r_g, 1/r_g [2 nc nr + 1 each]
+    // FD faces, h odd: cell centres): X_g = tan(pi/4 e_g), 1/(pi/4 (1 + X_g^2)),
+    // 1/sqrt(1 + X_g^2) [2 nc na + 1 each], then r_g, 1/r_g [2 nc nr + 1 each]
     const double* stab;
     const double* xyz_dg;           // [3][ndg] node coordinates
     const double* xyz_fd;           // [3][xfd_n] subcell-centre coordinates of every element
@@ -144,7 +144,7 @@ struct Dev {
     int* counts;                    // [0] n_dg, [1] n_fd, [2] n_flag, [3] n_near, [4] status bits, [5] free slots
     unsigned long long* units;      // [0] node updates (DG nodes + FD cells per substep), [1] FD and [2] DG element updates
     // FD scratch per chunk of listed FD elements: extended cells [12][chunk][(nc+6)^3],
-    // face fluxes [3 (x3 curved)][9][chunk][(nc+1) nc^2]
+    // face fluxes or states per direction (fd_common.cuh) [3][9, 21 or 27][chunk][(nc+1) nc^2]
     double* ext;
     double* flux;
     // FD->DG face traces of FD elements for their DG neighbours, per FD slot

@@ -1074,8 +1074,8 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
     if ((s = dalloc(c, &d.units, 3))) return s;   // node updates, FD and DG element updates
     if (d.curved) {
         // FD-point tables of the shell map (Dev::stab): gnomonic coordinate
-        // X = tan(pi/4 e) and 1/(pi/4 (1 + X^2)) on the half-cell grid of the
-        // angular rows, r and 1/r on that of the radial rows
+        // X = tan(pi/4 e), 1/(pi/4 (1 + X^2)) and 1/sqrt(1 + X^2) on the half-cell
+        // grid of the angular rows, r and 1/r on that of the radial rows
         std::vector<double> tab;
         auto add = [&](int P, int na, int nr, double r_in, double cc) {
             const int off = (int)tab.size(), nc = 2 * P + 1;
@@ -1085,6 +1085,7 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
             for (size_t g = 0; g < R.size(); ++g) R[g] = (double)(r_in * std::exp((long double)cc * g / (nc * nr)));
             for (double x : X) tab.push_back(x);
             for (double x : X) tab.push_back((double)(1.0L / (q * (1.0L + (long double)x * x))));
+            for (double x : X) tab.push_back((double)(1.0L / sqrtl(1.0L + (long double)x * x)));
             for (double r : R) tab.push_back(r);
             for (double r : R) tab.push_back(1.0 / r);
             return off;
@@ -1130,7 +1131,7 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
     if ((s = alloc_field(c, c->J, NJ))) return s;
     const int64_t ne = d.nc + 2 * GH;
     if ((s = dalloc(c, &d.ext, (size_t)12 * d.chunk * ne * ne * ne))) return s;
-    if ((s = dalloc(c, &d.flux, (size_t)(d.curved ? 9 : 3) * NV * d.chunk * (d.nc + 1) * d.nc * d.nc))) return s;
+    if ((s = dalloc(c, &d.flux, (size_t)(d.ks ? 9 * NV : d.curved ? 3 * (12 + NV) : 3 * NV) * d.chunk * (d.nc + 1) * d.nc * d.nc))) return s;
     if ((s = dalloc(c, &d.ftr, (size_t)fd_cap * 6 * 12 * d.np1 * d.np1))) return s;
     return FFE_OK;
 }

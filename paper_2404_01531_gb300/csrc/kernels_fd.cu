@@ -1,9 +1,10 @@
 // FD-subcell kernels of libffe, Sec. III.C.2:
 //   k_fd_fill_interior / k_fd_fill_ghosts  build, per listed FD element, an
 //       extended block of 12 quantities (U and J~) with 3 ghost layers per face;
-//   k_fd_flux[_curved]  one thread per face: WENO5-Z (point-value interpolation
-//       form, Z weights with q = 2) left/right states of the 12 quantities,
-//       Rusanov flux, optional 4th-order corrector with cell-centred fluxes;
+//   k_fd_flux (boxes), k_fd_states (flat shells)  one thread per line of cells
+//       and pair of quantities: WENO5-Z (point-value interpolation form, Z weights
+//       with q = 2) or MP5 face states, Rusanov flux, optional 4th-order corrector
+//       with cell-centred fluxes; k_fd_flux_ks  one thread per face;
 //   k_fd_update  one thread per cell: flux difference, sources, IMEX stage;
 //   k_rollback_project  DG -> FD projection of a flagged element's substep inputs;
 //   k_fd2dg      end-of-step FD -> DG check with alpha' = alpha + 1 (Sec. III.C.3).
@@ -197,116 +198,111 @@ __global__ void k_fd_fill_ghosts(Dev d, const int* list, int ci, int w0, Field U
     }
 }
 
-// 12 left/right face values (WENO5-Z pair or MP5) and the two cells either side, from the extended block
-template <int RECON>
-__device__ __forceinline__ void reconstruct(const Dev& d, int wl, int k, int m, int ta, int tb, int nc,
-                                            double* UL, double* UR, double* Um, double* Up) {
-    const int ne = nc + 2 * GH;
+// Where the lines of direction k of a chunk's extended blocks start: the first
+// ghost of line (ta, tb), and the step along it.
+__device__ __forceinline__ int64_t line_start(int k, int ta, int tb, int nc, int64_t& stride) {
+    const int64_t ne = nc + 2 * GH;
     int t1, t2;
     axes_of(k, t1, t2);
-    int c[3];
-    c[k] = m;
-    c[t1] = ta + GH;
-    c[t2] = tb + GH;
-    const int64_t base = c[0] + (int64_t)ne * (c[1] + (int64_t)ne * c[2]);
-    const int64_t stride = k == 0 ? 1 : (k == 1 ? ne : (int64_t)ne * ne);
-    if constexpr (RECON == FFE_RECON_MP5) {
-        for (int qq = 0; qq < NQ; ++qq) {
-            const double* src = ext_at(d, qq, wl) + base;
-            const double v0 = src[0], v1 = src[stride], v2 = src[2 * stride];
-            const double v3 = src[3 * stride], v4 = src[4 * stride], v5 = src[5 * stride];
-            UL[qq] = mp5(v0, v1, v2, v3, v4);
-            UR[qq] = mp5(v5, v4, v3, v2, v1);
-            Um[qq] = v2;
-            Up[qq] = v3;
-        }
-    } else {
-        for (int qq = 0; qq < NQ; ++qq) {
-            const double* src = ext_at(d, qq, wl) + base;
-            const double v0 = src[0], v1 = src[stride], v2 = src[2 * stride];
-            const double v3 = src[3 * stride], v4 = src[4 * stride], v5 = src[5 * stride];
-            weno5z_pair(v0, v1, v2, v3, v4, v5, d.weno_eps, UL[qq], UR[qq]);
-            Um[qq] = v2;
-            Up[qq] = v3;
-        }
-    }
+    const int64_t st[3] = {1, ne, ne * ne};
+    stride = st[k];
+    return (ta + GH) * st[t1] + (tb + GH) * st[t2];
 }
 
-// One thread per (chunk position, direction, face): box elements.
+// Box elements: one thread per (chunk position, direction, flux pair, line of
+// cells).  The FP64 pipe (2 lanes a clock and SM) is the limit, everything else
+// is nearly free beside it, so the split is the one with the fewest FP64
+// operations: a thread marches a line and gives both face values of every cell
+// from one set of smoothness indicators (Weno5zLine), for the two quantities
+// that a pair of flux components needs, so that the flux is formed in registers;
+// the two components of J~ across the direction are not reconstructed.  At P = 5
+// that is 610 FP64 operations per face against about 1100 of a thread per face:
+// 384 elements 3.44 -> 1.84 ms (4.8 us an element; 4.2 at the FP64 pipe's full
+// rate), MP5 on 125 elements 1.53 -> 0.41 ms.
 template <int RECON>
 __global__ void __launch_bounds__(128, 4) k_fd_flux(Dev d, const int* list, int ci, int w0) {
     const int n = chunk_n(d, ci, w0);
-    const int64_t nfc = nface(d);
-    const int64_t total = (int64_t)n * 3 * nfc;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-        const int wl = (int)(q / (3 * nfc));
-        const int k = (int)((q / nfc) % 3);
-        const int64_t fi = q % nfc;
-        const int e = list[w0 + wl];
-        const int nc = esz(d, e).nc;
-        int m, ta, tb;
-        if (!face_coords(fi, nc, m, ta, tb)) continue;
-        double UL[NQ], UR[NQ], Um[NQ], Up[NQ];
-        reconstruct<RECON>(d, wl, k, m, ta, tb, nc, UL, UR, Um, Up);
-        // the flat flux is linear in (U, J~): (F(UL) + F(UR))/2 = F((UL + UR)/2)
-        // and the corrector's F(Um) + F(Up) = F(Um + Up)
-        double hS[NQ], Fh[NV], Fs[NV];
-        for (int qq = 0; qq < NQ; ++qq) hS[qq] = 0.5 * (UL[qq] + UR[qq]);
-        flux_dir_flat(hS, hS + NV, k, Fh);
-        for (int v = 0; v < NV; ++v) Fs[v] = fma(-0.5, UR[v] - UL[v], Fh[v]);
-        if (d.fd_corr) {
-            double Sm[NQ], Fm[NV];
-            for (int qq = 0; qq < NQ; ++qq) Sm[qq] = Um[qq] + Up[qq];
-            flux_dir_flat(Sm, Sm + NV, k, Fm);
-            // F - (Fm - 2 F + Fp)/6 = (4/3) F - (Fm + Fp)/6
-            for (int v = 0; v < NV; ++v) Fs[v] = fma(-1.0 / 6.0, Fm[v], (4.0 / 3.0) * Fs[v]);
-        }
-        for (int v = 0; v < NV; ++v) flux_at(d, k, v, wl)[fi] = Fs[v];
+    const int nc = d.nc, nl = nc * nc;
+    const int per = 3 * FLUX_PAIRS * nl;
+    const int64_t total = (int64_t)n * per;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        const int wl = (int)(t / per), r = (int)(t % per), line = r % nl, kp = r / nl;
+        const int k = kp / FLUX_PAIRS, pr = kp % FLUX_PAIRS;
+        int a, b;
+        bool neg;
+        flux_pair(k, pr, a, b, neg);
+        int64_t stride;
+        const int64_t base = line_start(k, line % nc, line / nc, nc, stride);
+        const unsigned long long sb = neg ? 0x8000000000000000ULL : 0ULL;
+        double* fa = flux_at(d, k, a, wl) + line;
+        double* fb = pr < 4 ? flux_at(d, k, b, wl) + line : nullptr;
+        const bool corr = d.fd_corr;
+        recon_lines<RECON>(ext_at(d, a, wl) + base, ext_at(d, b, wl) + base, stride, sb, nc, d.weno_eps,
+                           [&](int m, double La, double Ra, double Sa, double Lb, double Rb, double Sb) {
+                               double Fa, Fb;
+                               rusanov_pair(La, Ra, Sa, Lb, Rb, Sb, corr, Fa, Fb);
+                               fa[m * nl] = Fa;
+                               if (fb) fb[m * nl] = __longlong_as_double((long long)(fbits(Fb) ^ sb));
+                           });
     }
 }
 
-// Curved (flat-metric) variant: all three physical flux components at each
-// face, Rusanov dissipation along the unit face normal n^ (lambda = 1):
-//   F^j = (F^j(L) + F^j(R))/2 - n^_j (U_R - U_L)/2,
-// optional corrector per component.
+// Flat-metric shells: one thread per (chunk position, direction, pair of
+// quantities, line).  All three physical flux components enter a face there,
+//   F^j = (F^j(L) + F^j(R))/2 - n^_j (U_R - U_L)/2  (lambda = 1, n^ the unit normal),
+// optional corrector per component.  They are linear in the face states, so the
+// kernel stores G = (L + R)/2 of the 12 quantities -- with the corrector
+// (2/3)(L + R) - (U_m + U_p)/6 -- and D = (U_R - U_L)/2 -- times 4/3 -- of the 9
+// variables: F^j = F^j(G) - n^_j D, formed once per cell by k_fd_update instead
+// of once per face (21 values a face instead of 27, no normals here): 300 elements
+// 2.74 -> 1.77 ms at P = 5, k_fd_update 0.28 -> 0.31 ms.
 template <int RECON>
-__global__ void __launch_bounds__(128, 4) k_fd_flux_curved(Dev d, const int* list, int ci, int w0) {
+__global__ void __launch_bounds__(128, 4) k_fd_states(Dev d, const int* list, int ci, int w0) {
     const int n = chunk_n(d, ci, w0);
-    const int64_t nfc = nface(d);
-    const int64_t total = (int64_t)n * 3 * nfc;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-        const int wl = (int)(q / (3 * nfc));
-        const int k = (int)((q / nfc) % 3);
-        const int64_t fi = q % nfc;
-        const int e = list[w0 + wl];
-        const int nc = esz(d, e).nc;
-        int m, ta, tb;
-        if (!face_coords(fi, nc, m, ta, tb)) continue;
-        int t1, t2;
-        axes_of(k, t1, t2);
-        double UL[NQ], UR[NQ], Um[NQ], Up[NQ];
-        reconstruct<RECON>(d, wl, k, m, ta, tb, nc, UL, UR, Um, Up);
-        double nh[3];
-        shell_face_normal(shell_pts(d, e, nc), k, m, ta, tb, nh);
-        // the flat flux is linear in (U, J~): (F^j(L) + F^j(R))/2 = F^j((UL + UR)/2),
-        // and the corrector's F(Um) + F(Up) = F(Um + Up)
-        double hS[NQ], dU[NV], Sm[NQ];
-        for (int qq = 0; qq < NQ; ++qq) hS[qq] = 0.5 * (UL[qq] + UR[qq]);
-        for (int v = 0; v < NV; ++v) dU[v] = UR[v] - UL[v];
-        if (d.fd_corr)
-            for (int qq = 0; qq < NQ; ++qq) Sm[qq] = Um[qq] + Up[qq];
-        for (int j = 0; j < 3; ++j) {
-            double Fh[NV], Fs[NV];
-            flux_dir_flat(hS, hS + NV, j, Fh);
-            const double hn = -0.5 * nh[j];
-            for (int v = 0; v < NV; ++v) Fs[v] = fma(hn, dU[v], Fh[v]);
-            if (d.fd_corr) {
-                double Fm[NV];
-                flux_dir_flat(Sm, Sm + NV, j, Fm);
-                for (int v = 0; v < NV; ++v) Fs[v] = fma(-1.0 / 6.0, Fm[v], (4.0 / 3.0) * Fs[v]);
-            }
-            for (int v = 0; v < NV; ++v) flux_at_c(d, k, j, v, wl)[fi] = Fs[v];
-        }
+    const int nlm = d.nc * d.nc;
+    const int per = 3 * (NQ / 2) * nlm;
+    const int64_t total = (int64_t)n * per;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        const int wl = (int)(t / per), r = (int)(t % per), line = r % nlm, kp = r / nlm;
+        const int k = kp / (NQ / 2), a = kp % (NQ / 2), b = a + NQ / 2;
+        const int nc = esz(d, list[w0 + wl]).nc, nl = nc * nc;
+        if (line >= nl) continue;
+        int64_t stride;
+        const int64_t base = line_start(k, line % nc, line / nc, nc, stride);
+        double* ga = fstate_at(d, k, a, wl) + line;
+        double* gb = fstate_at(d, k, b, wl) + line;
+        double* da = fstate_at(d, k, NQ + a, wl) + line;
+        double* db = b < NV ? fstate_at(d, k, NQ + b, wl) + line : nullptr;
+        const bool corr = d.fd_corr;
+        const double c1 = corr ? 2.0 / 3.0 : 0.5;
+        recon_lines<RECON>(ext_at(d, a, wl) + base, ext_at(d, b, wl) + base, stride, 0ULL, nc, d.weno_eps,
+                           [&](int m, double La, double Ra, double Sa, double Lb, double Rb, double Sb) {
+                               double Ga = c1 * (La + Ra), Gb = c1 * (Lb + Rb);
+                               if (corr) {
+                                   Ga = fma(-1.0 / 6.0, Sa, Ga);
+                                   Gb = fma(-1.0 / 6.0, Sb, Gb);
+                               }
+                               ga[m * nl] = Ga;
+                               gb[m * nl] = Gb;
+                               da[m * nl] = c1 * (Ra - La);
+                               if (db) db[m * nl] = c1 * (Rb - Lb);
+                           });
+    }
+}
+
+// 12 left/right values of one face from the extended block
+template <int RECON>
+__device__ __forceinline__ void reconstruct(const Dev& d, int wl, int k, int m, int ta, int tb, int nc,
+                                            double* UL, double* UR) {
+    int64_t stride;
+    const int64_t base = line_start(k, ta, tb, nc, stride) + m * stride;
+    for (int qq = 0; qq < NQ; ++qq) {
+        const double* src = ext_at(d, qq, wl) + base;
+        typename LineOf<RECON>::type A;
+        double none;
+        A.init(src[0], src[stride], src[2 * stride], src[3 * stride], d.weno_eps);
+        A.template cell<false, true>(src[4 * stride], none, UL[qq]);
+        A.template cell<true, false>(src[5 * stride], UR[qq], none);
     }
 }
 
@@ -332,8 +328,8 @@ __global__ void __launch_bounds__(128, 4) k_fd_flux_ks(Dev d, const int* list, i
         const int nc = esz(d, e).nc;
         int m, ta, tb;
         if (!face_coords(fi, nc, m, ta, tb)) continue;
-        double UL[NQ], UR[NQ], Um[NQ], Up[NQ];
-        reconstruct<RECON>(d, wl, k, m, ta, tb, nc, UL, UR, Um, Up);
+        double UL[NQ], UR[NQ];
+        reconstruct<RECON>(d, wl, k, m, ta, tb, nc, UL, UR);
         double nh[3];
         shell_face_normal(shell_pts(d, e, nc), k, m, ta, tb, nh);
         PM pm;
@@ -351,7 +347,7 @@ __global__ void __launch_bounds__(128, 4) k_fd_flux_ks(Dev d, const int* list, i
         flux_gen(hS, hS + NV, pm, F);
         for (int j = 0; j < 3; ++j) {
             const double hn = -0.5 * lam * nu[j] * inrm;
-            for (int v = 0; v < NV; ++v) flux_at_c(d, k, j, v, wl)[fi] = fma(hn, dU[v], F[j][v]);
+            for (int v = 0; v < NV; ++v) flux_at_c(d, k, j, v, wl)[face_index(nc, m, ta, tb)] = fma(hn, dU[v], F[j][v]);
         }
     }
 }
@@ -373,7 +369,11 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
         const int cc[3] = {c % nc, (c / nc) % nc, c / (nc * nc)};
         const int64_t p = fdb(d, e) + c;
         double ij[3][3];
-        if (CURVED) shell_cell(shell_pts(d, e, nc), cc, ij, nullptr);
+        ShellPts sp;
+        if (CURVED) {
+            sp = shell_pts(d, e, nc);
+            shell_cell(sp, cc, ij, nullptr);
+        }
         double du[NV], u0[NV];
         for (int v = 0; v < NV; ++v) u0[v] = a.Uin.fd(v)[p];
         PM m;
@@ -393,20 +393,35 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
         for (int k = 0; k < 3; ++k) {
             int t1, t2;
             axes_of(k, t1, t2);
-            const int64_t f0 = cc[k] + (int64_t)(nc + 1) * (cc[t1] + nc * cc[t2]);
-            if (CURVED) {
+            const int f0 = face_index(nc, cc[k], cc[t1], cc[t2]), f1 = f0 + nc * nc;
+            if (KS) {
                 for (int j = 0; j < 3; ++j) {
                     const double sc = ij[k][j] * (0.5 * nc);
                     for (int v = 0; v < NV; ++v) {
                         const double* fl = flux_at_c(d, k, j, v, wl);
-                        du[v] = fma(-sc, fl[f0 + 1] - fl[f0], du[v]);
+                        du[v] = fma(-sc, fl[f1] - fl[f0], du[v]);
                     }
+                }
+            } else if (CURVED) {
+                // F^j = F^j(G) - n^_j D at each face (k_fd_states)
+                double dG[NQ], sc[3];
+                for (int q = 0; q < NQ; ++q) {
+                    const double* g = fstate_at(d, k, q, wl);
+                    dG[q] = g[f1] - g[f0];
+                }
+                for (int j = 0; j < 3; ++j) sc[j] = ij[k][j] * (0.5 * nc);
+                flux_div_flat(dG, sc, du);
+                const double s0 = (0.5 * nc) * shell_grad_normal(sp, k, cc, cc[k], ij[k]);
+                const double s1 = (0.5 * nc) * shell_grad_normal(sp, k, cc, cc[k] + 1, ij[k]);
+                for (int v = 0; v < NV; ++v) {
+                    const double* g = fstate_at(d, k, NQ + v, wl);
+                    du[v] = fma(s1, g[f1], fma(-s0, g[f0], du[v]));
                 }
             } else {
                 const double sc = d.ijac[3 * e + k] * (0.5 * nc);
                 for (int v = 0; v < NV; ++v) {
                     const double* fl = flux_at(d, k, v, wl);
-                    du[v] = fma(-sc, fl[f0 + 1] - fl[f0], du[v]);
+                    du[v] = fma(-sc, fl[f1] - fl[f0], du[v]);
                 }
             }
         }
@@ -488,11 +503,11 @@ void launch_fd_substep(const Dev& d, int sub, const int* list, int ci, Field Uin
         prof_begin("fd_flux", st);
         if (d.recon == FFE_RECON_MP5) {
             if (d.ks) k_fd_flux_ks<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
-            else if (d.curved) k_fd_flux_curved<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
+            else if (d.curved) k_fd_states<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
             else k_fd_flux<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
         } else {
             if (d.ks) k_fd_flux_ks<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
-            else if (d.curved) k_fd_flux_curved<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
+            else if (d.curved) k_fd_states<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
             else k_fd_flux<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
         }
         prof_end(st);

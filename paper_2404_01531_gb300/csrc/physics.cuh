@@ -77,6 +77,20 @@ __device__ __forceinline__ void flux_dir_flat(const double* U, const double* J, 
     out[8] = J[d];
 }
 
+// du -= sum_j s_j F^j(g), g the 12 quantities (U, J~): curl, gradient and divergence terms.
+__device__ __forceinline__ void flux_div_flat(const double* g, const double* s, double* du) {
+    const double a = s[0], b = s[1], c = s[2];
+    du[0] = fma(b, g[5], fma(-c, g[4], fma(-a, g[6], du[0])));
+    du[1] = fma(c, g[3], fma(-a, g[5], fma(-b, g[6], du[1])));
+    du[2] = fma(a, g[4], fma(-b, g[3], fma(-c, g[6], du[2])));
+    du[3] = fma(c, g[1], fma(-b, g[2], fma(-a, g[7], du[3])));
+    du[4] = fma(a, g[2], fma(-c, g[0], fma(-b, g[7], du[4])));
+    du[5] = fma(b, g[0], fma(-a, g[1], fma(-c, g[7], du[5])));
+    du[6] -= fma(a, g[0], fma(b, g[1], c * g[2]));
+    du[7] -= fma(a, g[3], fma(b, g[4], c * g[5]));
+    du[8] -= fma(a, g[9], fma(b, g[10], c * g[11]));
+}
+
 // Implicit operator G: (-J~_eta, -kpsi psi~, -kphi phi~).
 __device__ __forceinline__ void implicit_G_flat(const double* U, const Dev& d, double* G) {
     double jp[3];
