@@ -24,8 +24,9 @@ __device__ __forceinline__ int64_t nface(const Dev& d) { return (int64_t)(d.nc +
 // their faces together, store to neighbouring addresses.
 __device__ __forceinline__ int face_index(int nc, int m, int ta, int tb) { return ta + nc * (tb + nc * m); }
 // face results: boxes the flux [3][NV][chunk][nface]; flat shells the face states
-// [3][NFS][chunk][nface] (k_fd_states); the Kerr-Schild background every
-// physical component j of the flux, [3 (k)][3 (j)][NV][chunk][nface]
+// [3][NFS][chunk][nface] (k_fd_states); the Kerr-Schild background and the
+// adjoint's forward recomputation every physical component j of the flux,
+// [3 (k)][3 (j)][NV][chunk][nface]
 constexpr int NFS = NQ + NV;
 __device__ __forceinline__ double* fstate_at(const Dev& d, int k, int q, int wl) {
     return d.flux + (((int64_t)k * NFS + q) * d.chunk + wl) * nface(d);
@@ -128,11 +129,60 @@ __device__ __forceinline__ int chunk_n(const Dev& d, int ci, int w0) {
 // alpha_k = d_k (1 + t^2/b_k^2), b_k = beta_k + eps, t = b_0 - b_2, are scaled by
 // X = b_0^2 b_1^2 b_2^2, so that the normalised combination needs one division:
 //   A_k = d_k (X + t^2 prod_{j != k} b_j^2),  value = sum A_k p_k / sum A_k.
-// At the upper end the products of six indicators overflow once an indicator
-// exceeds about 1e51 (stencil differences of about 1e25): the weights then
-// become Inf/NaN and the status word reports it.  Field values that large are
-// far outside any state of this system (the fields are of order one).
-//
+// weno5z_combine: the Z-weighted combination of three candidates from their
+// indicators b_k (eps included); the ideal weights are taken as (1, 10, 5)
+// (scale-free).
+__device__ __forceinline__ double weno5z_combine(double b0, double b1, double b2, double p0, double p1, double p2) {
+    // A_k = d_k (b_k^2 + t^2) P_k with P_k the product of the other two b_j^2
+    // is d_k (X + t^2 P_k), X = b_0^2 b_1^2 b_2^2 shared by the three
+    const double t = b0 - b2;
+    const double t2 = t * t;
+    const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
+    const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1;
+    const double X = q0 * P0;
+    const double A0 = fma(t2, P0, X), A1 = 10.0 * fma(t2, P1, X), A2 = 5.0 * fma(t2, P2, X);
+    return fma(A0, p0, fma(A1, p1, A2 * p2)) * recip_nr(A0 + A1 + A2);
+}
+
+// Both values at the face between v2 and v3 from the six cells v0..v5 (one face
+// at a time: k_fd_flux_faces): uL the
+// WENO5-Z value from v0..v4, uR the one from v5..v1 (mirrored).  Everything is
+// built from the first differences d_i = v_{i+1} - v_i: the candidates (the
+// quadratics through v0..v2, v1..v3, v2..v4 and v3..v5 at the face), the
+// second differences a and the one-sided combinations e of the Jiang-Shu
+// indicators beta = (13/12) a^2 + (1/4) e^2, of which 4 (beta + eps) enter
+// the weights (they are invariant under a common scale of the indicators).
+// The two values share two candidates and two second differences.
+__device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, double v3, double v4, double v5,
+                                            double eps, double& uL, double& uR) {
+    const double d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3, d45 = v5 - v4;
+    const double p123 = fma(0.125, d12, fma(0.375, d23, v2));
+    const double p234 = fma(0.625, d23, fma(-0.125, d34, v2));
+    const double pL0 = fma(-0.375, d01, fma(0.875, d12, v2));
+    const double pR0 = fma(-0.875, d34, fma(0.375, d45, v3));
+    const double a012 = d12 - d01, a123 = d23 - d12, a234 = d34 - d23, a345 = d45 - d34;
+    const double eL0 = fma(2.0, d12, a012), eL1 = d12 + d23, eL2 = fma(-2.0, d23, a234);
+    const double eR0 = fma(-2.0, d34, a345), eR1 = d23 + d34, eR2 = fma(2.0, d23, a123);
+    const double c = 13.0 / 3.0, eps4 = 4.0 * eps;
+    const double c123 = c * a123, c234 = c * a234;
+    const double bL0 = fma(c * a012, a012, fma(eL0, eL0, eps4));
+    const double bL1 = fma(c123, a123, fma(eL1, eL1, eps4));
+    const double bL2 = fma(c234, a234, fma(eL2, eL2, eps4));
+    const double bR0 = fma(c * a345, a345, fma(eR0, eR0, eps4));
+    const double bR1 = fma(c234, a234, fma(eR1, eR1, eps4));
+    const double bR2 = fma(c123, a123, fma(eR2, eR2, eps4));
+    uL = weno5z_combine(bL0, bL1, bL2, pL0, p123, p234);
+    uR = weno5z_combine(bR0, bR1, bR2, pR0, p234, p123);
+}
+
+// Sign and magnitude of a double as integers: a comparison of two doubles takes a
+// slot of the FP64 pipe (2 lanes a clock and SM), one of integers a slot of a pipe
+// that is 32 times wider.
+__device__ __forceinline__ unsigned long long fbits(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ unsigned long long fmag(double x) { return fbits(x) & 0x7fffffffffffffffULL; }
+__device__ __forceinline__ bool fneg(double x) { return __double_as_longlong(x) < 0; }
+__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
+__device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
 // Reconstruction along one line of cells (one quantity): cell() takes the cell
 // two ahead of the current centre c and gives both face values of c -- right:
 // the left state of the face to its right, left: the right state of the face to
@@ -149,7 +199,13 @@ __device__ __forceinline__ int chunk_n(const Dev& d, int ci, int w0) {
 // (1, 10, 5) towards the right face and (5, 10, 1) towards the left one, the Z
 // weights in the form above.  52 FP64 operations per cell and
 // quantity where a thread per face spends 87.  eps is at least 1e-51, so that
-// products of six indicators stay normal.
+// products of six indicators stay normal at the lower end.  At the upper end they
+// overflow once an indicator exceeds about 1e51 (stencil differences of about
+// 1e25): the weights then become Inf/NaN and the status word reports it; field
+// values that large are far outside any state of this system.  WIDE (caller-built
+// blocks): indicators above 2^160 are scaled exactly by the power of two of the
+// largest, under which the weights do not change (6% more FP64 slots).
+template <bool WIDE>
 struct Weno5zLine {
     double dA, dB, hA, hB, kA, kB, vc, vn, eps;
     __device__ __forceinline__ double curv(double h) const { return fma((13.0 / 12.0 * 64.0) * h, h, eps); }
@@ -169,7 +225,17 @@ struct Weno5zLine {
     __device__ __forceinline__ void cell(double v4, double& left, double& right) {
         const double dC = v4 - vn, hC = 0.125 * (dC - dB), kC = curv(hC);
         const double e0 = fma(4.0, hA, dA), e1 = fma(4.0, hB, dA), e2 = fma(-4.0, hC, dB);   // slopes at the centre
-        const double b0 = fma(e0, e0, kA), b1 = fma(e1, e1, kB), b2 = fma(e2, e2, kC);
+        const double c0 = fma(e0, e0, kA), c1 = fma(e1, e1, kB), c2 = fma(e2, e2, kC);
+        double b0 = c0, b1 = c1, b2 = c2;
+        if (WIDE) {
+            const unsigned long long top = umax(fbits(c0), umax(fbits(c1), fbits(c2)));
+            if (top >= (1023ULL + 160) << 52) {
+                const double sc = pow2_inv_scale(__longlong_as_double((long long)top));
+                b0 *= sc;
+                b1 *= sc;
+                b2 *= sc;
+            }
+        }
         const double t = b0 - b2, t2 = t * t;
         const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
         const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1, X = q0 * P0;
@@ -196,12 +262,6 @@ struct Weno5zLine {
 // minmod4 curvatures.  Both bounds contain the centre (lower <= v_c <= upper), so
 // the median is d limited to [-N, P].  Only magnitudes and signs are compared, as
 // integers: an FP64 comparison takes the FP64 pipe, 1/32 of the integer rate.
-__device__ __forceinline__ unsigned long long fbits(double x) { return (unsigned long long)__double_as_longlong(x); }
-__device__ __forceinline__ unsigned long long fmag(double x) { return fbits(x) & 0x7fffffffffffffffULL; }
-__device__ __forceinline__ bool fneg(double x) { return __double_as_longlong(x) < 0; }
-__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
-__device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
-
 __device__ __forceinline__ double minmod4(double a, double b, double c, double d) {
     const bool s = fneg(a);
     if (fneg(b) != s || fneg(c) != s || fneg(d) != s) return 0.0;
@@ -259,19 +319,30 @@ struct Mp5Line {
     }
 };
 
-template <int RECON> struct LineOf { using type = Weno5zLine; };
+template <int RECON> struct LineOf { using type = Weno5zLine<false>; };
 template <> struct LineOf<FFE_RECON_MP5> { using type = Mp5Line; };
+
+// Where line (ta, tb) of direction k starts in an extended block: its first ghost,
+// and the step along it.
+__device__ __forceinline__ int64_t line_start(int k, int ta, int tb, int nc, int64_t& stride) {
+    const int64_t ne = nc + 2 * GH;
+    int t1, t2;
+    axes_of(k, t1, t2);
+    const int64_t st[3] = {1, ne, ne * ne};
+    stride = st[k];
+    return (ta + GH) * st[t1] + (tb + GH) * st[t2];
+}
 
 // Reconstructs two quantities along one line of nc cells with 3 ghosts at each
 // end (pa, pb: the line's first ghost; sb: sign bit flipped in every value of
 // the second) and calls emit(m, La, Ra, Sa, Lb, Rb, Sb) at its faces m = 0..nc in
 // order: left and right states and the sum of the two cells at the face.  Two
 // quantities give a thread two independent chains of operations.
-template <int RECON, class Emit>
+template <class Line, class Emit>
 __device__ __forceinline__ void recon_lines(const double* pa, const double* pb, int64_t stride, unsigned long long sb,
                                             int nc, double eps, Emit emit) {
     auto b_at = [&](const double* p) { return __longlong_as_double((long long)(fbits(*p) ^ sb)); };
-    typename LineOf<RECON>::type A, B;
+    Line A, B;
     A.init(pa[0], pa[stride], pa[2 * stride], pa[3 * stride], eps);
     B.init(b_at(pb), b_at(pb + stride), b_at(pb + 2 * stride), b_at(pb + 3 * stride), eps);
     pa += 4 * stride;

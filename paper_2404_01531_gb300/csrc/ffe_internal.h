@@ -103,16 +103,15 @@ struct Dev {
     const double* metff;
     const double* metgb;
     // faces between cubed-sphere wedges: ghost-table slot of each element face
-    // ([E][6], -1 elsewhere) and per ghost (slot, g, ta, tb) of the slot's face,
-    // [slot][GH nc^2]: the first neighbour cell of its 6-point stencil along each
-    // axis [3] with the stencil weights [3][6], and the Lagrange weights of the
-    // neighbour's LGL nodes along each axis [3][MAXNP]
+    // ([E][6], -1 elsewhere; null: none) and, per slot, the 6-point stencils in the
+    // neighbour's cells (first cell, weights [6]) along its normal axis per layer g
+    // (gsn, gwn [GH]), along the edge per (g, ta) (gst, gwf [GH nc], index g nc_e + ta)
+    // and along the radius per cell (gsr, gwr [nc]); gwl: the Lagrange weights of its
+    // LGL nodes along the edge [GH nc][MAXNP] (k_fd_fill)
     const int* gislot;
-    const int* gst;
-    const double* gwf;
+    const int *gsn, *gst, *gsr;
+    const double *gwn, *gwf, *gwr;
     const double* gwl;
-    const int* gbox;                // [slot][6]: first neighbour cell and extent of the stencils' box per axis
-    int gbox_max;                   // largest box volume (cells)
     double shell_rin, shell_c;
     int shell_na, shell_nr;
     // flat shells, per instance at InstInfo::tab (single context: 0), on the
@@ -129,8 +128,6 @@ struct Dev {
     const int* nbr_face;            // [E][6] the neighbour's face touching mine
     const int* orient;              // [E][6] orientation code of the shared face (shellmap.cuh)
     const int* bc;                  // [E][6] boundary kind when nbr < 0
-    const unsigned char* ginterp;   // [E][6] 1: face between cubed-sphere wedges, FD ghosts
-                                    // interpolated to the extended grid (null: none)
     const int* bface;               // [E][6] boundary-face slot (Dirichlet data) or -1
     const double* bdg;              // [nbf][9][np1*np1] Dirichlet states at face nodes
     const double* bfd;              // [nbf][9][GH][nc*nc] Dirichlet states in ghost cells
@@ -185,21 +182,18 @@ void launch_dg_substep(const Dev& d, int sub, Field Uin, Field J, Field un, Fiel
                        cudaStream_t st);
 void launch_fd_substep(const Dev& d, int sub, const int* list, int count_index, Field Uin, Field J,
                        Field un, Field F2, Field F3, Field G1, Field G2, Field G3, Field G4,
-                       Field Fout, Field Uout, Field Gout, cudaStream_t st);
+                       Field Fout, Field Uout, Field Gout, cudaStream_t st, bool faces = false);
 int fd_chunks(const Dev& d);
 // FD->DG face traces of the listed FD elements for their DG neighbours (Dev::ftr)
 void launch_fd_traces(const Dev& d, Field U, Field J, cudaStream_t st);
 // out += the FD cells' share of the trace adjoints (Dev::ftr_b), reverse of k_fd_traces
 void launch_fd_traces_vjp(const Dev& d, Field U, Field out, cudaStream_t st);
 // extended blocks (U, J~ with ghosts) of the listed FD elements of one chunk
-void launch_fd_fill(const Dev& d, const int* list, int count_index, int w0, Field U, Field J, cudaStream_t st);
+void launch_fd_fill(const Dev& d, const int* list, int count_index, int w0, Field U, Field J, cudaStream_t st,
+                    bool residues = false);
 void launch_eval_recip(const double* x, double* y, int64_t n, cudaStream_t st);
 // register-only DFMA loop: returns its flops, *ms its event-timed duration
 double launch_fma_probe(int nsm, int iters, cudaStream_t st, float* ms);
-// ghosts of the faces between cubed-sphere wedges (kernels_fd_interp.cu)
-void launch_fd_fill_interp(const Dev& d, const int* list, int ci, int w0, Field U, Field J, cudaStream_t st);
-void launch_fdv_ghosts_interp(const Dev& d, const int* list, int ci, int w0, Field U, Field out, const double* extb,
-                              cudaStream_t st);
 void launch_constraints(const Dev& d, Field U, double* part, int blocks, cudaStream_t st);
 void launch_l2_err(const Dev& d, Field U, Field R, int v0, int nv, double* part, int blocks, cudaStream_t st);
 // out += (d RHS_FD/dU)^T L (kernels_adjoint_fd.cu); extb: scratch of the size of d.ext

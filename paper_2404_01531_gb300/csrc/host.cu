@@ -11,6 +11,7 @@
 #include <string>
 #include <tuple>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "ffe_internal.h"
@@ -347,8 +348,6 @@ struct ffe_ctx {
     int graph_kernels = 0;
     int nbf = 0;                     // boundary faces with Dirichlet data
     std::vector<int> h_bface;
-    std::vector<unsigned char> h_ginterp;   // [E][6] faces between cubed-sphere wedges
-    std::vector<int> h_gislot;              // [E][6] their ghost-table slot (-1 elsewhere)
     ShellGeo shell{};
     double lam_max = 1.0;
     // batched contexts
@@ -609,9 +608,9 @@ ffe_status build_ks_fd_tables(ffe_ctx* c, const std::vector<double>& xfd) {
 }
 
 // Faces between cubed-sphere wedges: there the FD ghosts are the neighbour's
-// data interpolated to this element's grid continued past the face
-// (k_fd_fill_ghosts_interp).  nbr: neighbour of every element face.
-ffe_status set_ginterp(ffe_ctx* c, const std::vector<int>& nbr) {
+// data interpolated along the edge to this element's grid continued past the
+// face (k_fd_fill).  nbr: neighbour of every element face.
+ffe_status set_ginterp(ffe_ctx* c, const std::vector<int>& nbr, const std::vector<int>& nbr_face) {
     Dev& d = c->d;
     auto wedge = [&](int e) {
         if (c->batch) {
@@ -620,36 +619,24 @@ ffe_status set_ginterp(ffe_ctx* c, const std::vector<int>& nbr) {
         }
         return e / (c->shell.na * c->shell.na * c->shell.nr);
     };
-    std::vector<unsigned char> gi(6 * (size_t)d.E, 0);
-    bool any = false;
+    std::vector<int> slot(6 * (size_t)d.E, -1);
+    int ns = 0;
     for (int e = 0; e < d.E; ++e)
         for (int f = 0; f < 6; ++f) {
             const int nb = nbr[6 * (size_t)e + f];
-            if (nb >= 0 && wedge(nb) != wedge(e)) {
-                gi[6 * (size_t)e + f] = 1;
-                any = true;
-            }
+            if (nb >= 0 && wedge(nb) != wedge(e)) slot[6 * (size_t)e + f] = ns++;
         }
-    c->h_ginterp = gi;
-    if (!any) return FFE_OK;
-    unsigned char* p;
-    ffe_status s;
-    if ((s = dalloc(c, &p, gi.size()))) return s;
-    CK(cudaMemcpy(p, gi.data(), gi.size(), cudaMemcpyHostToDevice));
-    d.ginterp = p;
-    // per ghost of those faces: its reference coordinates in the neighbour
-    // (closed-form inverse of the neighbour's wedge map) turned into the
-    // interpolation data the kernels use -- the first cell and the 6-point
-    // Lagrange weights of the stencil through the neighbour's subcell centres
-    // along each axis, and the Lagrange weights of its LGL nodes along each
-    // axis -- so that the kernels do no transcendental or division work
-    std::vector<int> slot(gi.size(), -1);
-    int ns = 0;
-    for (size_t i = 0; i < gi.size(); ++i)
-        if (gi[i]) slot[i] = ns++;
-    const int ncm = d.nc, ghn = GH * ncm * ncm;
-    std::vector<int> gst((size_t)ns * ghn * 3, 0);
-    std::vector<double> gwf((size_t)ns * ghn * 18, 0.0), gwl((size_t)ns * ghn * 3 * MAXNP, 0.0);
+    if (ns == 0) return FFE_OK;
+    // the ghosts' reference coordinates in the neighbour (closed-form inverse of its
+    // wedge map) as the first cell and the 6-point Lagrange weights of the stencil
+    // through its subcell centres -- across the face they depend on the layer only,
+    // along the edge on the layer and the position, along the radius on the radial
+    // cell -- and, along the edge, the Lagrange weights of its LGL nodes, so that the
+    // kernels do no transcendental or division work
+    const int ghn = GH * d.nc;
+    std::vector<int> gsn((size_t)ns * GH, 0), gst((size_t)ns * ghn, 0), gsr((size_t)ns * d.nc, 0);
+    std::vector<double> gwn(6 * gsn.size(), 0.0), gwf(6 * gst.size(), 0.0), gwr(6 * gsr.size(), 0.0),
+        gwl(MAXNP * gst.size(), 0.0);
     auto geo_of = [&](int e, int& el) {
         if (c->batch) {
             const InstInfo& in = c->insts[c->h_einst[e]];
@@ -668,58 +655,35 @@ ffe_status set_ginterp(ffe_ctx* c, const std::vector<int>& nbr) {
             const Tables& T = c->tabs_h[P];
             int el, eln;
             const ShellGeo ge = geo_of((int)e, el), gn = geo_of(nb, eln);
-            for (int t = 0; t < GH * nc * nc; ++t) {
-                const int g = t / (nc * nc), ta = t % nc, tb = (t / nc) % nc;
-                double xn[3];
-                shell_ghost_ref(ge, el, gn, eln, f >> 1, f & 1, g, ta, tb, nc, xn);
-                const size_t gi3 = ((size_t)sl * ghn + t) * 3;
-                for (int a = 0; a < 3; ++a) {
-                    gst[gi3 + a] = fd6_stencil(nc, xn[a], &gwf[((size_t)sl * ghn + t) * 18 + 6 * a]);
-                    lagrange_at(T.x, np1, xn[a], &gwl[(gi3 + a) * MAXNP]);
-                }
+            const int f2 = nbr_face[6 * (size_t)e + f], d2 = f2 >> 1, u1 = 1 - d2;   // its normal and edge axes
+            double xn[3];
+            for (int t = 0; t < GH * nc; ++t) {
+                shell_ghost_ref(ge, el, gn, eln, f >> 1, f & 1, t / nc, t % nc, 0, nc, xn);
+                const size_t at = (size_t)sl * ghn + t;
+                gst[at] = fd6_stencil(nc, xn[u1], &gwf[6 * at]);
+                lagrange_at(T.x, np1, xn[u1], &gwl[at * MAXNP]);
+                const size_t an = (size_t)sl * GH + t / nc;
+                if (t % nc == 0) gsn[an] = fd6_stencil(nc, xn[d2], &gwn[6 * an]);
+            }
+            for (int tb = 0; tb < nc; ++tb) {
+                shell_ghost_ref(ge, el, gn, eln, f >> 1, f & 1, 0, 0, tb, nc, xn);
+                const size_t at = (size_t)sl * d.nc + tb;
+                gsr[at] = fd6_stencil(nc, xn[2], &gwr[6 * at]);
             }
         }
     });
-    // per slot the box of neighbour cells its stencils cover (first cell and
-    // extent along each axis): the kernels stage it in shared memory
-    std::vector<int> box((size_t)ns * 6, 0);
-    int vmax = 0;
-    for (int sl = 0; sl < ns; ++sl) {
-        int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-1, -1, -1};
-        for (int t = 0; t < ghn; ++t)
-            for (int a = 0; a < 3; ++a) {
-                const int v = gst[((size_t)sl * ghn + t) * 3 + a];
-                lo[a] = v < lo[a] ? v : lo[a];
-                hi[a] = v > hi[a] ? v : hi[a];
-            }
-        int vol = 1;
-        for (int a = 0; a < 3; ++a) {
-            box[6 * sl + a] = lo[a];
-            box[6 * sl + 3 + a] = hi[a] + 6 - lo[a];
-            vol *= hi[a] + 6 - lo[a];
-        }
-        vmax = vol > vmax ? vol : vmax;
-    }
-    int *d_sl, *d_st, *d_box;
-    double *d_wf, *d_wl;
-    if ((s = dalloc(c, &d_box, box.size()))) return s;
-    CK(cudaMemcpy(d_box, box.data(), box.size() * sizeof(int), cudaMemcpyHostToDevice));
-    d.gbox = d_box;
-    d.gbox_max = vmax;
-    if ((s = dalloc(c, &d_sl, slot.size()))) return s;
-    if ((s = dalloc(c, &d_st, gst.size()))) return s;
-    if ((s = dalloc(c, &d_wf, gwf.size()))) return s;
-    if ((s = dalloc(c, &d_wl, gwl.size()))) return s;
-    CK(cudaMemcpy(d_sl, slot.data(), slot.size() * sizeof(int), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(d_st, gst.data(), gst.size() * sizeof(int), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(d_wf, gwf.data(), gwf.size() * 8, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(d_wl, gwl.data(), gwl.size() * 8, cudaMemcpyHostToDevice));
-    d.gislot = d_sl;
-    d.gst = d_st;
-    d.gwf = d_wf;
-    d.gwl = d_wl;
-    c->h_gislot = slot;
-    return FFE_OK;
+    auto upload = [&](const auto& v, auto** dst) -> ffe_status {
+        std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(*dst)>>>* p;
+        if (ffe_status s = dalloc(c, &p, v.size())) return s;
+        CK(cudaMemcpy(p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice));
+        *dst = p;
+        return FFE_OK;
+    };
+    ffe_status s;
+    if ((s = upload(slot, &d.gislot)) || (s = upload(gsn, &d.gsn)) || (s = upload(gst, &d.gst)) || (s = upload(gsr, &d.gsr)) ||
+        (s = upload(gwn, &d.gwn)) || (s = upload(gwf, &d.gwf)) || (s = upload(gwr, &d.gwr)))
+        return s;
+    return upload(gwl, &d.gwl);
 }
 
 // Six-wedge shell: coordinates, per-node inverse Jacobians, connectivity with
@@ -768,7 +732,7 @@ ffe_status build_shell(ffe_ctx* c) {
         }
     c->nbf = nbfd;
     c->h_bface = bface;
-    if (ffe_status sg = set_ginterp(c, nbr)) return sg;
+    if (ffe_status sg = set_ginterp(c, nbr, nbf)) return sg;
     // (dx)_min along element grid lines
     double dmin = 1e300;
     for (int64_t e = 0; e < E; ++e)
@@ -1131,7 +1095,7 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
     if ((s = alloc_field(c, c->J, NJ))) return s;
     const int64_t ne = d.nc + 2 * GH;
     if ((s = dalloc(c, &d.ext, (size_t)12 * d.chunk * ne * ne * ne))) return s;
-    if ((s = dalloc(c, &d.flux, (size_t)(d.ks ? 9 * NV : d.curved ? 3 * (12 + NV) : 3 * NV) * d.chunk * (d.nc + 1) * d.nc * d.nc))) return s;
+    if ((s = dalloc(c, &d.flux, (size_t)(d.curved ? 9 * NV : 3 * NV) * d.chunk * (d.nc + 1) * d.nc * d.nc))) return s;
     if ((s = dalloc(c, &d.ftr, (size_t)fd_cap * 6 * 12 * d.np1 * d.np1))) return s;
     return FFE_OK;
 }
@@ -2039,7 +2003,7 @@ ffe_status ffe_create_batch(int n_inst, const ffe_domain* doms, const ffe_elemen
     }
     c->nbf = nbfd;
     c->h_bface = bface;
-    if (ffe_status sg = set_ginterp(c, nbr)) return bail(sg);
+    if (ffe_status sg = set_ginterp(c, nbr, nbf)) return bail(sg);
     d.dt = c->insts[0].dt;
     ffe_status s;
     double *d_xdg, *d_geo, *d_bdg, *d_bfd, *d_ijac;
@@ -2390,7 +2354,7 @@ static void rhs_at(ffe_ctx* c, Field U, Field out) {
                              c->st);
     if (c->adj_fd)
         launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out,
-                          c->G1, c->st);
+                          c->G1, c->st, true);
 }
 
 // out = (d RHS/dU)^T L at U for the hybrid operator (fixed mask)

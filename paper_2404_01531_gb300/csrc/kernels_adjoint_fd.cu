@@ -3,7 +3,7 @@
 //   out += (d RHS_FD / d U)^T lambda  over every listed FD element.
 // The forward operator of an FD element is: extended block of the 12
 // quantities (U and J~ = J~(U)) with 3 ghost layers from FD neighbours
-// (copies; interpolated across faces between wedges, k_fdv_ghosts_interp), DG neighbours (their polynomials of U and of the nodal J~ at the
+// (copies; interpolated along the edge across faces between wedges), DG neighbours (their polynomials of U and of the nodal J~ at the
 // ghost subcell centres) or the boundary states; WENO5-Z left/right values at every face; Rusanov flux
 // of every physical component with the unit face normal; optional 4th-order
 // corrector with the cell-centred fluxes; flux difference with the inverse
@@ -184,8 +184,9 @@ __global__ void k_fdv_cells(Dev d, const int* list, int ci, int w0, Field U, Fie
     }
 }
 
-// shared doubles for the DG-neighbour ghosts (U and J~): t1 [12][GH][np1][np1] |
-// t2 [12][GH][np1][nc] | ub [12][GH][nc][nc]
+// shared doubles of one face's ghosts (U and J~): DG neighbour t1 [12][GH][np1][np1]
+// | t2 [12][GH][np1][nc] | ub [12][GH][nc][nc]; FD neighbour across wedges
+// W [GH][nc (its cell)][nc (ghost)] | ub [12][GH][nc][nc] (fits in the same)
 size_t fdv_ghost_smem(const Dev& d) {
     return (size_t)(NQ * GH * d.np1 * d.np1 + NQ * GH * d.np1 * d.nc + NQ * GH * d.nc * d.nc) * sizeof(double);
 }
@@ -199,7 +200,7 @@ __global__ void k_fdv_ghosts(Dev d, const int* list, int ci, int w0, Field U, Fi
     for (int item = blockIdx.x; item < n * 6; item += gridDim.x) {
         const int wl = item / 6, f = item % 6;
         const int e = list[w0 + wl];
-        if (d.ginterp && d.ginterp[e * 6 + f]) continue;   // k_fdv_ghosts_interp
+        const int gsl = d.gislot ? d.gislot[e * 6 + f] : -1;   // a face between wedges: its weights (k_fd_fill)
         const ES es = esz(d, e);
         const Tables& T = d.tabs[es.P];
         const int nc = es.nc, ne = nc + 2 * GH, np1 = es.np1, nn = es.nn;
@@ -228,6 +229,48 @@ __global__ void k_fdv_ghosts(Dev d, const int* list, int ci, int w0, Field U, Fi
             axes_of(d2, u1, u2);
             const int o = d.orient[e * 6 + f];
             const int64_t nbase = fdb(d, nb);
+            if (gsl >= 0) {
+                // Each cell (g, a2, radial tb) of the neighbour gathers its share of the
+                // ghosts of its layer and radius through the transposed 6-point weights
+                // along the edge (a small dense matrix in shared memory), then takes the
+                // current's chain rule: one addition per cell and variable into out
+                double* W = sm;
+                double* ubo = W + GH * nc * nc;   // [12][GH][nc (tb)][nc (ta)]
+                for (int t = threadIdx.x; t < GH * nc * nc; t += blockDim.x) {
+                    const int g = t / (nc * nc), cell = (t / nc) % nc, ta = t % nc;
+                    const int gi = gsl * GH * d.nc + g * nc + ta, m = cell - d.gst[gi];
+                    W[t] = m >= 0 && m < 6 ? d.gwf[6 * (int64_t)gi + m] : 0.0;
+                }
+                for (int t = threadIdx.x; t < nper; t += blockDim.x) {
+                    const int64_t og = ghost_offset(t / (nc * nc), t % nc, (t / nc) % nc);
+                    for (int v = 0; v < NQ; ++v) ubo[v * nper + t] = extb_at(d, (double*)extb, v, wl)[og];
+                }
+                __syncthreads();
+                for (int t = threadIdx.x; t < nper; t += blockDim.x) {
+                    const int g = t / (nc * nc), cell = t % nc, tb = (t / nc) % nc;
+                    int a2, b2;
+                    orient_map(o, nc, 0, tb, a2, b2);
+                    int c[3];
+                    c[d2] = s2 ? nc - 1 - g : g;
+                    c[u1] = cell;
+                    c[u2] = b2;
+                    const int64_t p = nbase + c[0] + nc * (c[1] + nc * c[2]);
+                    double w[NQ];
+                    for (int v = 0; v < NQ; ++v) w[v] = 0.0;
+                    for (int ta = 0; ta < nc; ++ta) {
+                        const double wt = W[(g * nc + cell) * nc + ta];
+                        if (wt == 0.0) continue;
+                        for (int v = 0; v < NQ; ++v) w[v] = fma(wt, ubo[v * nper + (g * nc + tb) * nc + ta], w[v]);
+                    }
+                    double u[NV];
+                    for (int v = 0; v < NV; ++v) u[v] = U.fd(v)[p];
+                    current_vjp(u, d.eta, w + NV, w + NV, w);
+                    for (int v = 0; v < NV; ++v)
+                        if (w[v] != 0.0) atomicAdd(out.fd(v) + p, w[v]);
+                }
+                __syncthreads();
+                continue;
+            }
             for (int t = threadIdx.x; t < nper; t += blockDim.x) {
                 const int g = t / (nc * nc), ta = t % nc, tb = (t / nc) % nc;
                 int a2, b2;
@@ -259,6 +302,7 @@ __global__ void k_fdv_ghosts(Dev d, const int* list, int ci, int w0, Field U, Fi
                 const int g = t / (nc * nc), ta = t % nc, tb = (t / nc) % nc;
                 int a2, b2;   // the neighbour's subcell (along u1, u2) under this ghost cell
                 orient_map(o, nc, ta, tb, a2, b2);
+                if (gsl >= 0) a2 = ta;
                 const int64_t og = ghost_offset(g, ta, tb);
                 for (int v = 0; v < NQ; ++v)
                     ubo[((v * GH + g) * nc + b2) * nc + a2] = extb_at(d, (double*)extb, v, wl)[og];
@@ -277,8 +321,9 @@ __global__ void k_fdv_ghosts(Dev d, const int* list, int ci, int w0, Field U, Fi
             for (int t = threadIdx.x; t < NQ * GH * np1 * np1; t += blockDim.x) {
                 const int v = t / (GH * np1 * np1), r = t % (GH * np1 * np1);
                 const int g = r / (np1 * np1), a2 = (r / np1) % np1, mm = r % np1;
+                const double* w = gsl >= 0 ? d.gwl + ((int64_t)gsl * GH * d.nc + g * nc) * MAXNP + mm : &T.P2F[0][mm];
                 double acc = 0.0;
-                for (int ta = 0; ta < nc; ++ta) acc = fma(T.P2F[ta][mm], t2b[((v * GH + g) * np1 + a2) * nc + ta], acc);
+                for (int ta = 0; ta < nc; ++ta) acc = fma(w[ta * MAXNP], t2b[((v * GH + g) * np1 + a2) * nc + ta], acc);
                 t1b[((v * GH + g) * np1 + a2) * np1 + mm] = acc;
             }
             __syncthreads();
@@ -458,7 +503,6 @@ void launch_fd_rhs_vjp(const Dev& dc, Field U, Field J, Field L, Field out, doub
         prof_end(st);
         prof_begin("fdv_ghosts", st);
         k_fdv_ghosts<<<d.nsm * 2, 256, smem, st>>>(d, d.fd_list, 1, w0, U, J, out, extb, omega_bar);
-        launch_fdv_ghosts_interp(d, d.fd_list, 1, w0, U, out, extb, st);
         prof_end(st);
         g_launch_counter += 4;
     }

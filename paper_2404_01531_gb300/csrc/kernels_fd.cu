@@ -1,6 +1,6 @@
 // FD-subcell kernels of libffe, Sec. III.C.2:
-//   k_fd_fill_interior / k_fd_fill_ghosts  build, per listed FD element, an
-//       extended block of 12 quantities (U and J~) with 3 ghost layers per face;
+//   k_fd_fill  builds, per listed FD element, an extended block of 12 quantities
+//       (U and J~) with 3 ghost layers per face;
 //   k_fd_flux (boxes), k_fd_states (flat shells)  one thread per line of cells
 //       and pair of quantities: WENO5-Z (point-value interpolation form, Z weights
 //       with q = 2) or MP5 face states, Rusanov flux, optional 4th-order corrector
@@ -8,8 +8,6 @@
 //   k_fd_update  one thread per cell: flux difference, sources, IMEX stage;
 //   k_rollback_project  DG -> FD projection of a flagged element's substep inputs;
 //   k_fd2dg      end-of-step FD -> DG check with alpha' = alpha + 1 (Sec. III.C.3).
-// Ghosts across faces between cubed-sphere wedges are filled by
-// k_fd_fill_ghosts_interp (kernels_fd_interp.cu).
 // Listed FD elements are processed in chunks of d.chunk so that the scratch
 // (extended blocks, face fluxes) is bounded whatever the number of FD elements.
 // Elements may have different orders (batched contexts): every size below is
@@ -25,31 +23,56 @@
 namespace ffe {
 
 // ---------------------------------------------------------------------------
-__global__ void k_fd_fill_interior(Dev d, const int* list, int ci, int w0, Field U, Field J) {
-    const int n = chunk_n(d, ci, w0);
-    const int64_t total = (int64_t)n * d.ncell;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-        const int wl = (int)(q / d.ncell), c = (int)(q % d.ncell);
-        const int e = list[w0 + wl];
-        const ES s = esz(d, e);
-        if (c >= s.ncell) continue;
-        const int nc = s.nc, ne = nc + 2 * GH;
+// The element's own cells, to the middle of its extended block.
+__device__ __forceinline__ void fill_interior(const Dev& d, int wl, int e, const Field& U, const Field& J) {
+    const ES s = esz(d, e);
+    const int nc = s.nc, ne = nc + 2 * GH;
+    const int64_t fb = fdb(d, e);
+    for (int c = threadIdx.x; c < s.ncell; c += blockDim.x) {
         const int x = c % nc, y = (c / nc) % nc, z = c / (nc * nc);
-        const int64_t p = fdb(d, e) + c;
-        const int64_t o = (x + GH) + ne * ((y + GH) + ne * (z + GH));
-        for (int v = 0; v < NV; ++v) ext_at(d, v, wl)[o] = U.fd(v)[p];
-        for (int k = 0; k < 3; ++k) ext_at(d, NV + k, wl)[o] = J.fd(3 + k)[p];
+        const int o = (x + GH) + ne * ((y + GH) + ne * (z + GH));
+        for (int v = 0; v < NV; ++v) ext_at(d, v, wl)[o] = U.fd(v)[fb + c];
+        for (int k = 0; k < 3; ++k) ext_at(d, NV + k, wl)[o] = J.fd(3 + k)[fb + c];
     }
 }
 
-// One CTA per (chunk position, face): fill the 3 ghost layers of that face.
-__global__ void k_fd_fill_ghosts(Dev d, const int* list, int ci, int w0, Field U, Field J) {
+// 6 stencil weights of entry i of a per-slot table
+__device__ __forceinline__ const double* gi_w(const double* table, const Dev& d, int slot, int i) {
+    const int per = table == d.gwn ? GH : (table == d.gwr ? d.nc : GH * d.nc);
+    return table + 6 * ((int64_t)slot * per + i);
+}
+
+// One CTA per (chunk position, face or interior): fill the extended block.
+//
+// Ghosts inside a wedge and on boxes are the neighbour's cells, or a DG
+// neighbour's polynomial at its own subcell centres: the neighbour's grid lines
+// continue this element's.  Across a face between two cubed-sphere wedges they
+// bend, and a ghost is the neighbour's data at the ghost centre of this element's
+// grid continued past the face (Sec. III.C.1): 6-point Lagrange interpolation of
+// its cells and of their current J~, or its polynomial.  The map is equiangular
+// and the radius is shared, so layer g of ghosts lies on the neighbour's own
+// layer g and on its own radial cell centres: only the coordinate along the edge
+// differs, and by an amount that depends on (g, ta) alone.  So of the 6 x 6 x 6
+// weights of the tensor stencil only 6 are not zero, up to residues of 1e-15 where
+// the two centres' coordinates differ in the last bit (one layer in six): the host
+// tabulates the three axes' weights (Dev::gwn, gwf, gwr), zero ones and residues are
+// skipped -- the residues are kept (36 or 216 products) for the adjoint's
+// recomputation, which keeps its bits, see k_fd_flux_faces -- and a DG neighbour's
+// polynomial takes three sum-factorised contractions.  With the interior's copy in
+// the same launch, two launches fewer; 300 elements of a shell 1.99 -> 0.20 ms
+// (0.53 with the residues).
+__global__ void k_fd_fill(Dev d, const int* list, int ci, int w0, Field U, Field J, bool residues) {
     const int n = chunk_n(d, ci, w0);
+    const unsigned long long skip = residues ? 0ULL : fbits(1e-10);   // weights up to this are skipped
     extern __shared__ double sm[];
-    for (int item = blockIdx.x; item < n * 6; item += gridDim.x) {
-        const int wl = item / 6, f = item % 6;
+    for (int item = blockIdx.x; item < n * 7; item += gridDim.x) {
+        const int wl = item / 7, f = item % 7;
         const int e = list[w0 + wl];
-        if (d.ginterp && d.ginterp[e * 6 + f]) continue;   // k_fd_fill_ghosts_interp
+        if (f == 6) {
+            fill_interior(d, wl, e, U, J);
+            continue;
+        }
+        const int gsl = d.gislot ? d.gislot[e * 6 + f] : -1;   // a face between wedges: its weights
         const ES es = esz(d, e);
         const Tables& T = d.tabs[es.P];
         const int nc = es.nc, ne = nc + 2 * GH, np1 = es.np1, nn = es.nn;
@@ -80,6 +103,37 @@ __global__ void k_fd_fill_ghosts(Dev d, const int* list, int ci, int w0, Field U
                 int a2, b2;
                 orient_map(o, nc, ta, tb, a2, b2);
                 int c[3];
+                if (gsl >= 0) {
+                    // stencil weights along the neighbour's axes: all but one of those
+                    // across the edge are zero, or a rounding residue for some layers
+                    const double *w[3] = {nullptr, nullptr, gi_w(d.gwr, d, gsl, b2)};
+                    int st[3];
+                    w[d2] = gi_w(d.gwn, d, gsl, g);
+                    w[u1] = gi_w(d.gwf, d, gsl, g * nc + ta);
+                    st[d2] = d.gsn[gsl * GH + g];
+                    st[u1] = d.gst[gsl * GH * d.nc + g * nc + ta];
+                    st[2] = d.gsr[gsl * d.nc + b2];
+                    const int64_t og = ghost_offset(g, ta, tb);
+                    const int64_t p = nbase + st[0] + nc * (st[1] + nc * st[2]);
+                    double acc[NQ];
+                    for (int v = 0; v < NQ; ++v) acc[v] = 0.0;
+                    for (int cz = 0; cz < 6; ++cz) {
+                        if (fmag(w[2][cz]) <= skip) continue;
+                        for (int cy = 0; cy < 6; ++cy) {
+                            const double wzy = w[2][cz] * w[1][cy];
+                            if (fmag(w[1][cy]) <= skip) continue;
+                            for (int cx = 0; cx < 6; ++cx) {
+                                if (fmag(w[0][cx]) <= skip) continue;
+                                const double wt = wzy * w[0][cx];
+                                const int64_t q = p + cx + nc * (cy + nc * cz);
+                                for (int v = 0; v < NV; ++v) acc[v] = fma(wt, U.fd(v)[q], acc[v]);
+                                for (int k = 0; k < 3; ++k) acc[NV + k] = fma(wt, J.fd(3 + k)[q], acc[NV + k]);
+                            }
+                        }
+                    }
+                    for (int v = 0; v < NQ; ++v) ext_at(d, v, wl)[og] = acc[v];
+                    continue;
+                }
                 c[d2] = s2 ? nc - 1 - g : g;
                 c[u1] = a2;
                 c[u2] = b2;
@@ -122,8 +176,10 @@ __global__ void k_fd_fill_ghosts(Dev d, const int* list, int ci, int w0, Field U
             for (int t = threadIdx.x; t < NQ * GH * nc * np1; t += blockDim.x) {
                 const int v = t / (GH * nc * np1), r = t % (GH * nc * np1);
                 const int g = r / (nc * np1), ta = r % nc, a2 = (r / nc) % np1;
+                // along u1: at the neighbour's cell ta, or at ghost ta's own point
+                const double* w = gsl >= 0 ? d.gwl + ((int64_t)gsl * GH * d.nc + g * nc + ta) * MAXNP : T.P2F[ta];
                 double acc = 0.0;
-                for (int m = 0; m < np1; ++m) acc = fma(T.P2F[ta][m], t1b[((v * GH + g) * np1 + a2) * np1 + m], acc);
+                for (int m = 0; m < np1; ++m) acc = fma(w[m], t1b[((v * GH + g) * np1 + a2) * np1 + m], acc);
                 t2b[t] = acc;
             }
             __syncthreads();
@@ -131,6 +187,7 @@ __global__ void k_fd_fill_ghosts(Dev d, const int* list, int ci, int w0, Field U
                 const int g = t / (nc * nc), ta = t % nc, tb = (t / nc) % nc;
                 int a2, b2;   // the neighbour's subcell (along u1, u2) under this ghost cell
                 orient_map(o, nc, ta, tb, a2, b2);
+                if (gsl >= 0) a2 = ta;
                 const int64_t og = ghost_offset(g, ta, tb);
                 for (int v = 0; v < NQ; ++v) {
                     double acc = 0.0;
@@ -198,17 +255,6 @@ __global__ void k_fd_fill_ghosts(Dev d, const int* list, int ci, int w0, Field U
     }
 }
 
-// Where the lines of direction k of a chunk's extended blocks start: the first
-// ghost of line (ta, tb), and the step along it.
-__device__ __forceinline__ int64_t line_start(int k, int ta, int tb, int nc, int64_t& stride) {
-    const int64_t ne = nc + 2 * GH;
-    int t1, t2;
-    axes_of(k, t1, t2);
-    const int64_t st[3] = {1, ne, ne * ne};
-    stride = st[k];
-    return (ta + GH) * st[t1] + (tb + GH) * st[t2];
-}
-
 // Box elements: one thread per (chunk position, direction, flux pair, line of
 // cells).  The FP64 pipe (2 lanes a clock and SM) is the limit, everything else
 // is nearly free beside it, so the split is the one with the fewest FP64
@@ -220,7 +266,7 @@ __device__ __forceinline__ int64_t line_start(int k, int ta, int tb, int nc, int
 // 384 elements 3.44 -> 1.84 ms (4.8 us an element; 4.2 at the FP64 pipe's full
 // rate), MP5 on 125 elements 1.53 -> 0.41 ms.
 template <int RECON>
-__global__ void __launch_bounds__(128, 4) k_fd_flux(Dev d, const int* list, int ci, int w0) {
+__global__ void __launch_bounds__(64, 8) k_fd_flux(Dev d, const int* list, int ci, int w0) {
     const int n = chunk_n(d, ci, w0);
     const int nc = d.nc, nl = nc * nc;
     const int per = 3 * FLUX_PAIRS * nl;
@@ -237,7 +283,7 @@ __global__ void __launch_bounds__(128, 4) k_fd_flux(Dev d, const int* list, int 
         double* fa = flux_at(d, k, a, wl) + line;
         double* fb = pr < 4 ? flux_at(d, k, b, wl) + line : nullptr;
         const bool corr = d.fd_corr;
-        recon_lines<RECON>(ext_at(d, a, wl) + base, ext_at(d, b, wl) + base, stride, sb, nc, d.weno_eps,
+        recon_lines<typename LineOf<RECON>::type>(ext_at(d, a, wl) + base, ext_at(d, b, wl) + base, stride, sb, nc, d.weno_eps,
                            [&](int m, double La, double Ra, double Sa, double Lb, double Rb, double Sb) {
                                double Fa, Fb;
                                rusanov_pair(La, Ra, Sa, Lb, Rb, Sb, corr, Fa, Fb);
@@ -257,7 +303,7 @@ __global__ void __launch_bounds__(128, 4) k_fd_flux(Dev d, const int* list, int 
 // of once per face (21 values a face instead of 27, no normals here): 300 elements
 // 2.74 -> 1.77 ms at P = 5, k_fd_update 0.28 -> 0.31 ms.
 template <int RECON>
-__global__ void __launch_bounds__(128, 4) k_fd_states(Dev d, const int* list, int ci, int w0) {
+__global__ void __launch_bounds__(64, 8) k_fd_states(Dev d, const int* list, int ci, int w0) {
     const int n = chunk_n(d, ci, w0);
     const int nlm = d.nc * d.nc;
     const int per = 3 * (NQ / 2) * nlm;
@@ -275,7 +321,7 @@ __global__ void __launch_bounds__(128, 4) k_fd_states(Dev d, const int* list, in
         double* db = b < NV ? fstate_at(d, k, NQ + b, wl) + line : nullptr;
         const bool corr = d.fd_corr;
         const double c1 = corr ? 2.0 / 3.0 : 0.5;
-        recon_lines<RECON>(ext_at(d, a, wl) + base, ext_at(d, b, wl) + base, stride, 0ULL, nc, d.weno_eps,
+        recon_lines<typename LineOf<RECON>::type>(ext_at(d, a, wl) + base, ext_at(d, b, wl) + base, stride, 0ULL, nc, d.weno_eps,
                            [&](int m, double La, double Ra, double Sa, double Lb, double Rb, double Sb) {
                                double Ga = c1 * (La + Ra), Gb = c1 * (Lb + Rb);
                                if (corr) {
@@ -287,6 +333,61 @@ __global__ void __launch_bounds__(128, 4) k_fd_states(Dev d, const int* list, in
                                da[m * nl] = c1 * (Ra - La);
                                if (db) db[m * nl] = c1 * (Rb - Lb);
                            });
+    }
+}
+
+// Flat shells, forward recomputation of the adjoint: one thread per face, all
+// three flux components there.  A reverse step amplifies the rounding of the
+// stages it is linearised at by up to 1e9 (J~ carries eta times the rounding of
+// E~.B~, and the WENO5-Z weights' derivatives carry J~'s differences): inputs
+// moved by one rounding move single entries of lambda_n by 7e-7 of their size.  So
+// gradients stay comparable from one version to the next only if the
+// recomputed stages keep their bits, and this kernel keeps the order of operations
+// of a thread per face (k_fd_states: 1.5 times faster, different last bits).
+__global__ void __launch_bounds__(128, 4) k_fd_flux_faces(Dev d, const int* list, int ci, int w0) {
+    const int n = chunk_n(d, ci, w0);
+    const int64_t nfc = nface(d);
+    const int64_t total = (int64_t)n * 3 * nfc;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+        const int wl = (int)(q / (3 * nfc));
+        const int k = (int)((q / nfc) % 3);
+        const int64_t fi = q % nfc;
+        const int e = list[w0 + wl];
+        const int nc = esz(d, e).nc;
+        int m, ta, tb;
+        if (!face_coords(fi, nc, m, ta, tb)) continue;
+        double UL[NQ], UR[NQ], Um[NQ], Up[NQ];
+        int64_t stride;
+        const int64_t base = line_start(k, ta, tb, nc, stride) + m * stride;
+        for (int qq = 0; qq < NQ; ++qq) {
+            const double* src = ext_at(d, qq, wl) + base;
+            const double v0 = src[0], v1 = src[stride], v2 = src[2 * stride];
+            const double v3 = src[3 * stride], v4 = src[4 * stride], v5 = src[5 * stride];
+            weno5z_pair(v0, v1, v2, v3, v4, v5, d.weno_eps, UL[qq], UR[qq]);
+            Um[qq] = v2;
+            Up[qq] = v3;
+        }
+        double nh[3];
+        shell_face_normal(shell_pts(d, e, nc), k, m, ta, tb, nh);
+        // the flat flux is linear in (U, J~): (F^j(L) + F^j(R))/2 = F^j((UL + UR)/2),
+        // and the corrector's F(Um) + F(Up) = F(Um + Up)
+        double hS[NQ], dU[NV], Sm[NQ];
+        for (int qq = 0; qq < NQ; ++qq) hS[qq] = 0.5 * (UL[qq] + UR[qq]);
+        for (int v = 0; v < NV; ++v) dU[v] = UR[v] - UL[v];
+        if (d.fd_corr)
+            for (int qq = 0; qq < NQ; ++qq) Sm[qq] = Um[qq] + Up[qq];
+        for (int j = 0; j < 3; ++j) {
+            double Fh[NV], Fs[NV];
+            flux_dir_flat(hS, hS + NV, j, Fh);
+            const double hn = -0.5 * nh[j];
+            for (int v = 0; v < NV; ++v) Fs[v] = fma(hn, dU[v], Fh[v]);
+            if (d.fd_corr) {
+                double Fm[NV];
+                flux_dir_flat(Sm, Sm + NV, j, Fm);
+                for (int v = 0; v < NV; ++v) Fs[v] = fma(-1.0 / 6.0, Fm[v], (4.0 / 3.0) * Fs[v]);
+            }
+            for (int v = 0; v < NV; ++v) flux_at_c(d, k, j, v, wl)[face_index(nc, m, ta, tb)] = Fs[v];
+        }
     }
 }
 
@@ -355,8 +456,9 @@ __global__ void __launch_bounds__(128, 4) k_fd_flux_ks(Dev d, const int* list, i
 // One thread per (chunk position, cell): flux difference + sources + stage.
 // KS: the Kerr-Schild background (metric and its derivative terms at the
 // subcell centre from Dev::metfd; sources, stiff solve, clamp and implicit
-// operator in their metric-general forms).
-template <int SUB, bool CURVED, bool KS = false>
+// operator in their metric-general forms).  FACES: the flux components of every
+// face instead of its states.
+template <int SUB, bool CURVED, bool KS = false, bool FACES = KS>
 __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
     const int n = chunk_n(d, ci, w0);
     const int64_t total = (int64_t)n * d.ncell;
@@ -394,7 +496,7 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
             int t1, t2;
             axes_of(k, t1, t2);
             const int f0 = face_index(nc, cc[k], cc[t1], cc[t2]), f1 = f0 + nc * nc;
-            if (KS) {
+            if (FACES) {
                 for (int j = 0; j < 3; ++j) {
                     const double sc = ij[k][j] * (0.5 * nc);
                     for (int v = 0; v < NV; ++v) {
@@ -464,13 +566,11 @@ static size_t ghost_smem(const Dev& d) {
     return (size_t)(NQ * d.nn + NQ * GH * d.np1 * d.np1 + NQ * GH * d.nc * d.np1) * sizeof(double);
 }
 
-void launch_fd_fill(const Dev& d, const int* list, int ci, int w0, Field U, Field J, cudaStream_t st) {
+void launch_fd_fill(const Dev& d, const int* list, int ci, int w0, Field U, Field J, cudaStream_t st, bool residues) {
     const size_t smem = ghost_smem(d);
-    cudaFuncSetAttribute(k_fd_fill_ghosts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_fd_fill_interior<<<d.nsm * 8, 256, 0, st>>>(d, list, ci, w0, U, J);
-    k_fd_fill_ghosts<<<d.nsm * 2, 256, smem, st>>>(d, list, ci, w0, U, J);
-    g_launch_counter += 2;
-    launch_fd_fill_interp(d, list, ci, w0, U, J, st);
+    cudaFuncSetAttribute(k_fd_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_fd_fill<<<d.nsm * 4, 256, smem, st>>>(d, list, ci, w0, U, J, residues);
+    g_launch_counter += 1;
 }
 
 template <int SUB>
@@ -482,33 +582,25 @@ static void launch_update(const Dev& d, const int* list, int ci, int w0, const S
 
 void launch_fd_substep(const Dev& d, int sub, const int* list, int ci, Field Uin, Field J, Field un, Field F2,
                        Field F3, Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool faces) {
     SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout};
     const int grid = d.nsm * 8;
-    const size_t smem = ghost_smem(d);
-    cudaFuncSetAttribute(k_fd_fill_ghosts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     for (int k = 0, nch = fd_chunks(d); k < nch; ++k) {
         const int w0 = k * d.chunk;
-        prof_begin("fd_fill_interior", st);
-        k_fd_fill_interior<<<grid, 256, 0, st>>>(d, list, ci, w0, Uin, J);
+        prof_begin("fd_fill", st);
+        launch_fd_fill(d, list, ci, w0, Uin, J, st, faces);
         prof_end(st);
-        prof_begin("fd_fill_ghosts", st);
-        k_fd_fill_ghosts<<<d.nsm * 2, 256, smem, st>>>(d, list, ci, w0, Uin, J);
-        prof_end(st);
-        if (d.ginterp) {
-            prof_begin("fd_fill_ghosts_interp", st);
-            launch_fd_fill_interp(d, list, ci, w0, Uin, J, st);
-            prof_end(st);
-        }
         prof_begin("fd_flux", st);
-        if (d.recon == FFE_RECON_MP5) {
+        if (faces) {
+            k_fd_flux_faces<<<grid, 128, 0, st>>>(d, list, ci, w0);
+        } else if (d.recon == FFE_RECON_MP5) {
             if (d.ks) k_fd_flux_ks<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
-            else if (d.curved) k_fd_states<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
-            else k_fd_flux<FFE_RECON_MP5><<<grid, 128, 0, st>>>(d, list, ci, w0);
+            else if (d.curved) k_fd_states<FFE_RECON_MP5><<<grid, 64, 0, st>>>(d, list, ci, w0);
+            else k_fd_flux<FFE_RECON_MP5><<<grid, 64, 0, st>>>(d, list, ci, w0);
         } else {
             if (d.ks) k_fd_flux_ks<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
-            else if (d.curved) k_fd_states<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
-            else k_fd_flux<FFE_RECON_WENO5Z><<<grid, 128, 0, st>>>(d, list, ci, w0);
+            else if (d.curved) k_fd_states<FFE_RECON_WENO5Z><<<grid, 64, 0, st>>>(d, list, ci, w0);
+            else k_fd_flux<FFE_RECON_WENO5Z><<<grid, 64, 0, st>>>(d, list, ci, w0);
         }
         prof_end(st);
         prof_begin("fd_update", st);
@@ -516,10 +608,12 @@ void launch_fd_substep(const Dev& d, int sub, const int* list, int ci, Field Uin
             case SUB_A: launch_update<SUB_A>(d, list, ci, w0, a, st); break;
             case SUB_B: launch_update<SUB_B>(d, list, ci, w0, a, st); break;
             case SUB_C: launch_update<SUB_C>(d, list, ci, w0, a, st); break;
-            default: launch_update<SUB_RHS>(d, list, ci, w0, a, st); break;
+            default:
+                if (faces) k_fd_update<SUB_RHS, true, false, true><<<d.nsm * 8, 256, 0, st>>>(d, list, ci, w0, a);
+                else launch_update<SUB_RHS>(d, list, ci, w0, a, st);
         }
         prof_end(st);
-        g_launch_counter += 4;
+        g_launch_counter += 2;
     }
 }
 

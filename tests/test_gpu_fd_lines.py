@@ -25,7 +25,7 @@ def _random_state(pr, P, seed):
 @pytest.mark.parametrize("corr", [0, 1])
 def test_box_lines(ffe, P, recon, corr):  # noqa: F811
     cfg = W.breakdown(nx=3, ny=2, nz=1, P=P, x_half=0.1)
-    cfg.update(lo=(-0.1, -0.05, -0.2), hi=(0.1, 0.07, 0.1))
+    cfg.update(lo=(-0.16, -0.05, -0.2), hi=(0.14, 0.07, 0.1))
     cfg["params"].update(eta=7.0, recon=recon, fd_corrector=corr)
     pr = Problem(cfg)
     assert _rhs_parity(ffe, cfg, _random_state(pr, P, 10 * P + 2 * recon + corr), pr) <= 1e-11
