@@ -175,14 +175,6 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
     uR = weno5z_combine(bR0, bR1, bR2, pR0, p234, p123);
 }
 
-// Sign and magnitude of a double as integers: a comparison of two doubles takes a
-// slot of the FP64 pipe (2 lanes a clock and SM), one of integers a slot of a pipe
-// that is 32 times wider.
-__device__ __forceinline__ unsigned long long fbits(double x) { return (unsigned long long)__double_as_longlong(x); }
-__device__ __forceinline__ unsigned long long fmag(double x) { return fbits(x) & 0x7fffffffffffffffULL; }
-__device__ __forceinline__ bool fneg(double x) { return __double_as_longlong(x) < 0; }
-__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
-__device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
 // Reconstruction along one line of cells (one quantity): cell() takes the cell
 // two ahead of the current centre c and gives both face values of c -- right:
 // the left state of the face to its right, left: the right state of the face to

@@ -46,11 +46,28 @@ struct Tables {
     int f2d_lo[MAXNP];             // first subcell of the 6-point stencil of node i
 };
 
+// Constants of the pointwise stiff solve with dta = dt a: c = eta dta, 1/(1 + kappa dta)
+// of the two cleaning fields, -c/(1+c) and eta/(1+c).
+struct SolveK {
+    double dta, c, ipsi, iphi, cm, eta1;
+};
+inline SolveK solve_consts(double eta, double kpsi, double kphi, double dt) {
+    SolveK k;
+    k.dta = dt * IM_A;
+    k.c = eta * k.dta;
+    k.ipsi = 1.0 / (1.0 + kpsi * k.dta);
+    k.iphi = 1.0 / (1.0 + kphi * k.dta);
+    k.cm = -k.c / (1.0 + k.c);
+    k.eta1 = eta / (1.0 + k.c);
+    return k;
+}
+
 // Per-instance data of a batched context (one magnetosphere per instance).
 struct InstInfo {
     double r_in, c, dt, omega;   // shell map r = r_in exp(c (er + 1)), time step, star rotation
     int na, nr, e0, P;           // elements per wedge side / radially, first element, order
     int tab;                     // offset of the instance's FD-point tables in Dev::stab
+    SolveK sk;
 };
 
 // A field buffer in state-vector layout: [nv][n_dg] then [nv][n_fd].
@@ -88,6 +105,7 @@ struct Dev {
     double eta, kpsi, kphi, dt, weno_eps, omega;
     int mode, filter_on, tci_on, fd_corr, recon;
     double thr_dg, thr_fd;          // (P+1-M)^-alpha and (P+1-M)^-(alpha+1)
+    SolveK sk;                      // of dt (batches: per instance, InstInfo)
     // geometry of the affine box: d xi / d x per element and axis
     const double* ijac;             // [E][3]
     // curved meshes: d xi^k / d x^i per DG node [9][ndg] (index 3 k + i), the
@@ -171,18 +189,20 @@ __device__ __forceinline__ int64_t fdb(const Dev& d, int e) {
 }
 __device__ __forceinline__ int fd_slot_of(const Dev& d, int e) { return d.fd_slot ? d.fd_slot[e] : e; }
 __device__ __forceinline__ double dt_of(const Dev& d, int e) { return d.einst ? d.inst[d.einst[e]].dt : d.dt; }
+__device__ __forceinline__ SolveK solve_k(const Dev& d, int e) { return d.einst ? d.inst[d.einst[e]].sk : d.sk; }
 __device__ __forceinline__ double omega_of(const Dev& d, int e) { return d.einst ? d.inst[d.einst[e]].omega : d.omega; }
 
 // kernel launchers (kernels_*.cu); all enqueue on `st`
 void launch_build_lists(const Dev& d, cudaStream_t st);
 void launch_current(const Dev& d, Field U, Field J, const int* list_or_null, int which_count, cudaStream_t st);
-void launch_stage12(const Dev& d, Field un, Field Ua, Field G1, Field G2, cudaStream_t st);
+void launch_stage12(const Dev& d, Field un, Field Ua, Field G1, Field G2, Field J, cudaStream_t st);
+// Jout: J~ of the substep's result (flat metric; unused on the Kerr-Schild background)
 void launch_dg_substep(const Dev& d, int sub, Field Uin, Field J, Field un, Field F2, Field F3,
-                       Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout,
+                       Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
                        cudaStream_t st);
 void launch_fd_substep(const Dev& d, int sub, const int* list, int count_index, Field Uin, Field J,
                        Field un, Field F2, Field F3, Field G1, Field G2, Field G3, Field G4,
-                       Field Fout, Field Uout, Field Gout, cudaStream_t st, bool faces = false);
+                       Field Fout, Field Uout, Field Gout, Field Jout, cudaStream_t st, bool faces = false);
 int fd_chunks(const Dev& d);
 // FD->DG face traces of the listed FD elements for their DG neighbours (Dev::ftr)
 void launch_fd_traces(const Dev& d, Field U, Field J, cudaStream_t st);
@@ -207,7 +227,8 @@ void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field F
 void launch_fd2dg(const Dev& d, Field un, cudaStream_t st);
 void launch_tci_ratio(const Dev& d, const double* Udg, double* ratio, cudaStream_t st);
 void launch_dg_substep_curved(const Dev& d, int sub, Field Uin, Field J, Field un, Field F2, Field F3, Field G1,
-                              Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, cudaStream_t st);
+                              Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
+                              cudaStream_t st);
 void launch_stage12_ks(const Dev& d, Field un, Field Ua, Field G1, Field G2, cudaStream_t st);
 
 // adjoint (kernels_adjoint.cu)

@@ -3,7 +3,20 @@
 
 namespace ffe {
 
-// 1/d for a positive normal d whose reciprocal is normal: the hardware
+// Sign and magnitude of a double as integers: a comparison of two doubles takes a
+// slot of the FP64 pipe (2 lanes a clock and SM), one of integers a slot of a pipe
+// that is 32 times wider.
+__device__ __forceinline__ unsigned long long fbits(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ unsigned long long fmag(double x) { return fbits(x) & 0x7fffffffffffffffULL; }
+__device__ __forceinline__ bool fneg(double x) { return __double_as_longlong(x) < 0; }
+__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
+__device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
+__device__ __forceinline__ double flip(double x, unsigned long long sign) {
+    return __longlong_as_double((long long)(fbits(x) ^ sign));
+}
+__device__ __forceinline__ bool is_zero(double x) { return fmag(x) == 0; }
+
+// 1/d for a normal d whose reciprocal is normal: the hardware
 // approximation rcp.approx.ftz.f64 refined by two Newton-Raphson steps for
 // f(y) = 1/y - d, y <- y + y (1 - d y) (each squares the relative error; the
 // residual 1 - d y is exact in one FMA when y is close to 1/d).  Within about
@@ -29,11 +42,10 @@ __device__ __forceinline__ double pow2_inv_scale(double x) {
 }
 
 // 1/x for any finite nonzero x: recip_nr inside the range where it is
-// defined (2^-1000 < |x| < 2^1000), the IEEE quotient outside it.
+// defined (2^-1000 <= |x| < 2^1000), the IEEE quotient outside it.
 __device__ __forceinline__ double recip_any(double x) {
-    const double ax = fabs(x);
-    if (ax > 9.33e-302 && ax < 1.07e301) return x > 0.0 ? recip_nr(x) : -recip_nr(-x);
-    return 1.0 / x;
+    const unsigned e = (unsigned)(fmag(x) >> 52) - (1023u - 1000u);
+    return e < 2000u ? recip_nr(x) : 1.0 / x;
 }
 
 }  // namespace ffe

@@ -341,7 +341,7 @@ struct ffe_ctx {
     int id_kind = -1;
     std::vector<double> id_prm;
     std::vector<void*> allocs;
-    Field un{}, Ua{}, Ub{}, F2{}, F3{}, G1{}, G2{}, G3{}, G4{}, J{}, Fs{};
+    Field un{}, Ua{}, Ub{}, F2{}, F3{}, G1{}, G2{}, G3{}, G4{}, J{}, J2{}, Fs{};
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     bool graph_ok = true;
@@ -873,26 +873,29 @@ void enqueue_step(ffe_ctx* c) {
     cudaMemsetAsync(d.switched, 0, d.E, st);
     launch_build_lists(d, st);
     if (d.ks) launch_stage12_ks(d, c->un, c->Ua, c->G1, c->G2, st);
-    else launch_stage12(d, c->un, c->Ua, c->G1, c->G2, st);
-    struct S { int sub; Field Uin, Fout, Uout, Gout; };
-    const S subs[3] = {{SUB_A, c->Ua, c->F2, c->Ub, c->G3},
-                       {SUB_B, c->Ub, c->F3, c->Ua, c->G4},
-                       {SUB_C, c->Ua, c->Fs, c->un, c->G4}};
+    else launch_stage12(d, c->un, c->Ua, c->G1, c->G2, c->J, st);
+    // J~ of each substep's input: left by the stage before it (flat metric) in one
+    // of two buffers, since a substep's neighbours still read the other one
+    struct S { int sub; Field Uin, J, Fout, Uout, Gout, Jout; };
+    const S subs[3] = {{SUB_A, c->Ua, c->J, c->F2, c->Ub, c->G3, c->J2},
+                       {SUB_B, c->Ub, c->J2, c->F3, c->Ua, c->G4, c->J},
+                       {SUB_C, c->Ua, c->J, c->Fs, c->un, c->G4, c->J2}};
     for (const S& s : subs) {
-        if (!d.ks || d.metfd) launch_current(d, s.Uin, c->J, nullptr, 0, st);
+        const Field J = d.ks ? c->J : s.J;
+        if (d.ks && d.metfd) launch_current(d, s.Uin, J, nullptr, 0, st);
         if (d.curved)
-            launch_dg_substep_curved(d, s.sub, s.Uin, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
-                                     s.Uout, s.Gout, st);
+            launch_dg_substep_curved(d, s.sub, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
+                                     s.Uout, s.Gout, s.Jout, st);
         else
-            launch_dg_substep(d, s.sub, s.Uin, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
-                              s.Uout, s.Gout, st);
-        launch_fd_substep(d, s.sub, d.fd_list, 1, s.Uin, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4,
-                          s.Fout, s.Uout, s.Gout, st);
+            launch_dg_substep(d, s.sub, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout, s.Uout,
+                              s.Gout, s.Jout, st);
+        launch_fd_substep(d, s.sub, d.fd_list, 1, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
+                          s.Uout, s.Gout, s.Jout, st);
         if (d.tci_on) {
             launch_rollback_project(d, s.sub, c->un, s.Uin, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, st);
-            launch_current(d, s.Uin, c->J, d.flag_list, 2, st);
-            launch_fd_substep(d, s.sub, d.flag_list, 2, s.Uin, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3,
-                              c->G4, s.Fout, s.Uout, s.Gout, st);
+            launch_current(d, s.Uin, J, d.flag_list, 2, st);
+            launch_fd_substep(d, s.sub, d.flag_list, 2, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4,
+                              s.Fout, s.Uout, s.Gout, s.Jout, st);
             cudaMemsetAsync(d.counts + 2, 0, sizeof(int), st);
             launch_build_lists(d, st);
         }
@@ -928,10 +931,10 @@ ffe_status autotune(ffe_ctx* c) {
                 CK(cudaEventRecord(a, c->st));
                 if (d.curved)
                     launch_dg_substep_curved(d, SUB_RHS, c->un, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4,
-                                             c->Fs, c->Fs, c->G1, c->st);
+                                             c->Fs, c->Fs, c->G1, c->J2, c->st);
                 else
                     launch_dg_substep(d, SUB_RHS, c->un, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, c->Fs,
-                                      c->Fs, c->G1, c->st);
+                                      c->Fs, c->G1, c->J2, c->st);
                 CK(cudaEventRecord(b, c->st));
                 CK(cudaEventSynchronize(b));
                 float ms = 0.0f;
@@ -1067,6 +1070,7 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
         int *eP8, *ein;
         InstInfo* dinst;
         std::vector<unsigned char> ep(c->h_eP.begin(), c->h_eP.end());
+        for (auto& in : c->insts) in.sk = solve_consts(d.eta, d.kpsi, d.kphi, in.dt);
         unsigned char* dep;
         if ((s = dalloc(c, &dep, d.E))) return s;
         if ((s = dalloc(c, &ein, d.E))) return s;
@@ -1093,6 +1097,8 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
     for (Field* f : {&c->G1, &c->G2, &c->G3, &c->G4})
         if ((s = alloc_field(c, *f, NG))) return s;
     if ((s = alloc_field(c, c->J, NJ))) return s;
+    if (!d.ks && (s = alloc_field(c, c->J2, NJ))) return s;
+    d.sk = solve_consts(d.eta, d.kpsi, d.kphi, d.dt);
     const int64_t ne = d.nc + 2 * GH;
     if ((s = dalloc(c, &d.ext, (size_t)12 * d.chunk * ne * ne * ne))) return s;
     if ((s = dalloc(c, &d.flux, (size_t)(d.curved ? 9 * NV : 3 * NV) * d.chunk * (d.nc + 1) * d.nc * d.nc))) return s;
@@ -2117,11 +2123,11 @@ ffe_status ffe_rhs(ffe_ctx* c, const double* U_dev, double* dUdt_dev) try {
     launch_current(d, U, c->J, nullptr, 0, c->st);
     if (d.curved)
         launch_dg_substep_curved(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1,
-                                 c->st);
+                                 c->J2, c->st);
     else
-        launch_dg_substep(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1, c->st);
+        launch_dg_substep(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1, c->J2, c->st);
     launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R,
-                      c->G1, c->st);
+                      c->G1, c->J2, c->st);
     CK(cudaGetLastError());
     return FFE_OK;
 } catch (...) {
@@ -2351,10 +2357,10 @@ static void rhs_at(ffe_ctx* c, Field U, Field out) {
     const Dev& d = c->d;
     if (c->adj_fd) launch_current(d, U, c->J, nullptr, 0, c->st);
     launch_dg_substep_curved(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out, c->G1,
-                             c->st);
+                             c->J2, c->st);
     if (c->adj_fd)
         launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out,
-                          c->G1, c->st, true);
+                          c->G1, c->J2, c->st, true);
 }
 
 // out = (d RHS/dU)^T L at U for the hybrid operator (fixed mask)

@@ -342,14 +342,13 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
             if (KS) {
                 if (SUB != SUB_C && !stiff_solve_gen(u, m, d, dt * IM_A)) atomic_status(d, 2);
                 if (d.mode != FFE_RELAX) hard_clamp_gen(u, m);
+                if (SUB != SUB_C) {
+                    double g[NG];
+                    implicit_G_gen(u, m, d, g);
+                    for (int c = 0; c < NG; ++c) a.Gout.dg(c)[eb + tid] = g[c];
+                }
             } else {
-                substep_implicit(d, SUB, dt, u);
-            }
-            if (SUB != SUB_C) {
-                double g[NG];
-                if (KS) implicit_G_gen(u, m, d, g);
-                else implicit_G_flat(u, d, g);
-                for (int c = 0; c < NG; ++c) a.Gout.dg(c)[eb + tid] = g[c];
+                substep_implicit<SUB>(d, solve_k(d, e), a, eb + tid, false, u);
             }
         }
         bool flagged = false;
@@ -458,8 +457,9 @@ static void curved_dispatch(const Dev& d, int sub, const SubArgs& a, cudaStream_
 }
 
 void launch_dg_substep_curved(const Dev& d, int sub, Field Uin, Field J, Field un, Field F2, Field F3, Field G1,
-                              Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, cudaStream_t st) {
-    SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout};
+                              Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
+                              cudaStream_t st) {
+    SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout, Jout};
     if (!d.ks || d.metfd) launch_fd_traces(d, Uin, J, st);
     prof_begin(sub == SUB_RHS ? "dg_rhs_curved" : "dg_substep_curved", st);
     if (d.ks) {

@@ -13,6 +13,7 @@
 #include <cstdio>
 
 #include "dgfilter.cuh"
+#include "fd_common.cuh"
 #include "ffe_internal.h"
 #include "physics.cuh"
 #include "physics_gen.cuh"
@@ -29,10 +30,12 @@ struct DGK {
     static constexpr int nf = np1 * np1;
     static constexpr int NT = ((nn + 31) / 32) * 32;
     static constexpr int NW = NT / 32;
-    // shared doubles: U[9][nn] | J[6][nn] + C[6][9][nf] (aliased by the filter buffer [9][nn]) | red[2][NW]
-    // | D scaled by the element's d xi/d x, per axis [3][np1][np1]
-    static constexpr int AUX = (6 * nn + 54 * nf) > 9 * nn ? (6 * nn + 54 * nf) : 9 * nn;
-    static constexpr int SMEM = (9 * nn + AUX + 2 * NW + 3 * nf) * 8;
+    static constexpr int FR = (6 * nf + NT - 1) / NT;   // face nodes per thread
+    // CTAs per SM the registers are bounded for
+    static constexpr int CTAS = P == 6 ? 2 : 3;
+    // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn] | dU/dt[9][nn] |
+    // red[2][NW] | D scaled by the element's d xi/d x, per axis [3][np1][np1]
+    static constexpr int SMEM = (21 * nn + 2 * NW + 3 * nf) * 8;
 };
 
 // ---------------------------------------------------------------------------
@@ -108,36 +111,37 @@ void launch_current(const Dev& d, Field U, Field J, const int* list, int count_i
 }
 
 // ---------------------------------------------------------------------------
-// Stages 1 and 2 are pointwise: U1 = solve(u_n), G1 = G(U1); U2 = solve(u_n - dt a G1), G2 = G(U2).
+// Stages 1 and 2 are pointwise: U1 = solve(u_n), G1 = G(U1); U2 = solve(u_n - dt a G1), G2 = G(U2);
+// J~(U2), which the first right-hand side reads, comes with the second solve.
 // Over the DG nodes of DG elements and the cells of the FD list (built first).
-__device__ __forceinline__ void stage12_point(const Dev& d, double dt, double* u, double* g1, double* g2) {
-    const double dta = dt * IM_A;
-    double U1[NV];
-    for (int v = 0; v < NV; ++v) U1[v] = u[v];
-    if (!stiff_solve_flat(U1, d, dta)) atomic_status(d, 2);
-    if (d.mode != FFE_RELAX) hard_clamp_flat(U1);
-    implicit_G_flat(U1, d, g1);
-    u[0] = fma(-dta, g1[0], u[0]);
-    u[1] = fma(-dta, g1[1], u[1]);
-    u[2] = fma(-dta, g1[2], u[2]);
-    u[6] = fma(-dta, g1[3], u[6]);
-    u[7] = fma(-dta, g1[4], u[7]);
-    if (!stiff_solve_flat(u, d, dta)) atomic_status(d, 2);
-    if (d.mode != FFE_RELAX) hard_clamp_flat(u);
-    implicit_G_flat(u, d, g2);
+__device__ __forceinline__ void stage12_point(const Dev& d, const SolveK& k, bool isfd, int64_t p, const Field& un,
+                                              const Field& Ua, const Field& G1, const Field& G2, const Field& J) {
+    auto at = [&](const Field& f, int v) { return (isfd ? f.fd(v) : f.dg(v)) + p; };
+    double u[NV], U1[NV], jp[3], ib2, g1[NG], g2[NG], jd[3], jf[3];
+    for (int v = 0; v < NV; ++v) U1[v] = u[v] = *at(un, v);
+    bool ok = implicit_stage_flat(U1, d, k, jp, ib2);
+    stage_G_flat(U1, d, jp, g1);
+    u[0] = fma(-k.dta, g1[0], u[0]);
+    u[1] = fma(-k.dta, g1[1], u[1]);
+    u[2] = fma(-k.dta, g1[2], u[2]);
+    u[6] = fma(-k.dta, g1[3], u[6]);
+    u[7] = fma(-k.dta, g1[4], u[7]);
+    ok &= implicit_stage_flat(u, d, k, jp, ib2);
+    if (!ok) atomic_status(d, 2);
+    stage_G_flat(u, d, jp, g2);
+    stage_current_flat(u, jp, ib2, jd, jf);
+    for (int v = 0; v < NV; ++v) *at(Ua, v) = u[v];
+    for (int c = 0; c < NG; ++c) { *at(G1, c) = g1[c]; *at(G2, c) = g2[c]; }
+    for (int c = 0; c < 3; ++c) { *at(J, c) = jd[c]; *at(J, 3 + c) = jf[c]; }
 }
 
-__global__ void k_stage12(Dev d, Field un, Field Ua, Field G1, Field G2) {
+__global__ void k_stage12(Dev d, Field un, Field Ua, Field G1, Field G2, Field J) {
     int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t p = tid; p < d.ndg; p += stride) {
         const int e = (int)(p / d.nn);
         if (d.mask[e] != 0 || (int)(p % d.nn) >= esz(d, e).nn) continue;
-        double u[NV], g1[NG], g2[NG];
-        for (int v = 0; v < NV; ++v) u[v] = un.dg(v)[p];
-        stage12_point(d, dt_of(d, e), u, g1, g2);
-        for (int v = 0; v < NV; ++v) Ua.dg(v)[p] = u[v];
-        for (int c = 0; c < NG; ++c) { G1.dg(c)[p] = g1[c]; G2.dg(c)[p] = g2[c]; }
+        stage12_point(d, solve_k(d, e), false, p, un, Ua, G1, G2, J);
     }
     // FD cells: the elements of the FD list only (an FD slot pool may be mostly empty)
     const int64_t nfdq = (int64_t)d.counts[1] * d.ncell;
@@ -145,18 +149,13 @@ __global__ void k_stage12(Dev d, Field un, Field Ua, Field G1, Field G2) {
         const int e = d.fd_list[q / d.ncell];
         const int c = (int)(q % d.ncell);
         if (c >= esz(d, e).ncell) continue;
-        const int64_t p = fdb(d, e) + c;
-        double u[NV], g1[NG], g2[NG];
-        for (int v = 0; v < NV; ++v) u[v] = un.fd(v)[p];
-        stage12_point(d, dt_of(d, e), u, g1, g2);
-        for (int v = 0; v < NV; ++v) Ua.fd(v)[p] = u[v];
-        for (int c = 0; c < NG; ++c) { G1.fd(c)[p] = g1[c]; G2.fd(c)[p] = g2[c]; }
+        stage12_point(d, solve_k(d, e), true, fdb(d, e) + c, un, Ua, G1, G2, J);
     }
 }
 
-void launch_stage12(const Dev& d, Field un, Field Ua, Field G1, Field G2, cudaStream_t st) {
+void launch_stage12(const Dev& d, Field un, Field Ua, Field G1, Field G2, Field J, cudaStream_t st) {
     prof_begin("stage12", st);
-    k_stage12<<<d.nsm * 8, 256, 0, st>>>(d, un, Ua, G1, G2);
+    k_stage12<<<d.nsm * 8, 256, 0, st>>>(d, un, Ua, G1, G2, J);
     prof_end(st);
     g_launch_counter += 1;
 }
@@ -245,15 +244,23 @@ __device__ void dg_external_state(const Dev& d, const SubArgs& a, int e, int f, 
     current_flat(Ue, d.eta, jd, Je);
 }
 
+// What bounds it: the FP64 pipe (2 lanes a clock and SM; a warp instruction takes
+// 16 clocks of an SM), at 7 warps an element about 430 FP64 slots a thread in
+// substep A, of which 162 are the line contractions.  So the work per node is what
+// counts: five lift values per face node instead of nine, their sum into dU/dt axis
+// by axis instead of node by node under divergence, no FP64 comparisons, and the
+// stage's G and currents from its solve (substep_implicit).  Three CTAs an SM: their
+// barriers hide each other's.  4096 elements at P = 5, average of the substeps:
+// 0.870 -> 0.757 ms, and the separate current launches (0.075 ms each) are gone.
 template <int P, int SUB>
-__global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) {
+__global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, SubArgs a) {
     using K = DGK<P>;
     constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NT = K::NT, NW = K::NW;
     extern __shared__ double sm[];
     double* sU = sm;                 // [9][nn]
-    double* sJ = sU + 9 * nn;        // [6][nn]
-    double* sC = sJ + 6 * nn;        // [6][9][nf]
-    double* red = sU + 9 * nn + K::AUX;
+    double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
+    double* sR = sJ + 3 * nn;        // [9][nn] dU/dt
+    double* red = sR + 9 * nn;
     double* sD = red + 2 * NW;       // [3][np1][np1]: (d xi^a/d x^a) D
     __shared__ int s_flag;
     const Tables& T = *d.tab;
@@ -267,11 +274,16 @@ __global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) 
         const int64_t eb = (int64_t)e * nn;
         const double sx = d.ijac[3 * e], sy = d.ijac[3 * e + 1], sz = d.ijac[3 * e + 2];
         for (int t = tid; t < NV * nn; t += NT) sU[t] = a.Uin.dg(t / nn)[eb + t % nn];
-        for (int t = tid; t < NJ * nn; t += NT) sJ[t] = a.J.dg(t / nn)[eb + t % nn];
-        if (tid < 3 * nf) sD[tid] = (tid < nf ? sx : (tid < 2 * nf ? sy : sz)) * T.D[(tid % nf) / np1][tid % np1];
+        for (int t = tid; t < 3 * nn; t += NT) sJ[t] = a.J.dg(3 + t / nn)[eb + t % nn];
+        for (int t = tid; t < 3 * nf; t += NT)
+            sD[t] = (t < nf ? sx : (t < 2 * nf ? sy : sz)) * T.D[(t % nf) / np1][t % np1];
+        double eX = 0.0, eY = 0.0, eZ = 0.0;
+        if (act) {
+            eX = -a.J.dg(0)[eb + tid];
+            eY = -a.J.dg(1)[eb + tid];
+            eZ = -a.J.dg(2)[eb + tid];
+        }
         __syncthreads();
-
-        double du[NV];
         if (act) {
             const double* Dx = sD + np1 * i;
             const double* Dy = sD + nf + np1 * j;
@@ -280,7 +292,6 @@ __global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) 
             const int oy = i + np1 * np1 * k;     // y-line start, stride np1
             const int oz = i + np1 * j;           // z-line start, stride np1^2
             auto U = [&](int v, int idx) { return sU[v * nn + idx]; };
-            double eX = -sJ[0 * nn + tid], eY = -sJ[1 * nn + tid], eZ = -sJ[2 * nn + tid];
             double bX = 0.0, bY = 0.0, bZ = 0.0;
             double ps = U(8, tid), ph = 0.0, qq = 0.0;
 #pragma unroll
@@ -297,14 +308,23 @@ __global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) 
                 // psi: -div E + q ; phi: -div B ; q: -div J
                 ps = fma(-Dx[m], U(0, ix), ps); ps = fma(-Dy[m], U(1, iy), ps); ps = fma(-Dz[m], U(2, iz), ps);
                 ph = fma(-Dx[m], U(3, ix), ph); ph = fma(-Dy[m], U(4, iy), ph); ph = fma(-Dz[m], U(5, iz), ph);
-                qq = fma(-Dx[m], sJ[3 * nn + ix], qq); qq = fma(-Dy[m], sJ[4 * nn + iy], qq);
-                qq = fma(-Dz[m], sJ[5 * nn + iz], qq);
+                qq = fma(-Dx[m], sJ[ix], qq); qq = fma(-Dy[m], sJ[nn + iy], qq);
+                qq = fma(-Dz[m], sJ[2 * nn + iz], qq);
             }
-            du[0] = eX; du[1] = eY; du[2] = eZ; du[3] = bX; du[4] = bY; du[5] = bZ;
-            du[6] = ps; du[7] = ph; du[8] = qq;
+            double* r = sR + tid;
+            r[0] = eX; r[nn] = eY; r[2 * nn] = eZ; r[3 * nn] = bX; r[4 * nn] = bY; r[5 * nn] = bZ;
+            r[6 * nn] = ps; r[7 * nn] = ph; r[8 * nn] = qq;
         }
-        // lift: one thread per face node
-        for (int t = tid; t < 6 * nf; t += NT) {
+        // Lift, one thread per face node.  The jump (dU, dJ) to the exterior state
+        // enters through the pairs (a, b, s) of flux_pair: with t = s (outward sign)
+        // the correction of a is c = (t db - da) |grad xi|/(2 w0), that of b is -t c:
+        // five values per face node.
+        double cor[K::FR][5];
+        int me[K::FR];
+#pragma unroll
+        for (int r = 0; r < K::FR; ++r) {
+            const int t = tid + r * NT;
+            if (t >= 6 * nf) break;
             const int f = t / nf, ab = t % nf, ta = ab % np1, tb = ab / np1;
             const int dd = f >> 1, s = f & 1;
             int t1, t2;
@@ -313,33 +333,47 @@ __global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) 
             c[dd] = s ? P : 0;
             c[t1] = ta;
             c[t2] = tb;
-            const int me = node_index<P>(c[0], c[1], c[2]);
+            me[r] = node_index<P>(c[0], c[1], c[2]);
             double Ui[NV], Ue[NV], Je[3], xn[3];
-            for (int v = 0; v < NV; ++v) Ui[v] = sU[v * nn + me];
+            for (int v = 0; v < NV; ++v) Ui[v] = sU[v * nn + me[r]];
             if (d.nbr[e * 6 + f] < 0 && d.bc[e * 6 + f] == FFE_BC_STAR)
-                for (int q = 0; q < 3; ++q) xn[q] = d.xyz_dg[(int64_t)q * d.ndg + eb + me];
+                for (int q = 0; q < 3; ++q) xn[q] = d.xyz_dg[(int64_t)q * d.ndg + eb + me[r]];
             dg_external_state<P>(d, a, e, f, ta, tb, Ui, xn, Ue, Je);
-            double dU[NV], dJ[3], dF[NV];
-            for (int v = 0; v < NV; ++v) dU[v] = Ue[v] - Ui[v];
-            for (int q = 0; q < 3; ++q) dJ[q] = Je[q] - sJ[(3 + q) * nn + me];
-            flux_dir_flat(dU, dJ, dd, dF);
-            const double sg = s ? 1.0 : -1.0;
-            const double scale = 0.5 * d.ijac[3 * e + dd] * w0inv;   // |grad xi^d| / (2 w0)
-            for (int v = 0; v < NV; ++v) sC[(f * NV + v) * nf + ab] = scale * fma(sg, dF[v], -dU[v]);
+            const double jump = (dd == 0 ? Je[0] : (dd == 1 ? Je[1] : Je[2])) - sJ[dd * nn + me[r]];
+            const unsigned long long sg = s ? 0ULL : 0x8000000000000000ULL;
+            const double scale = 0.5 * (dd == 0 ? sx : (dd == 1 ? sy : sz)) * w0inv;   // |grad xi^d| / (2 w0)
+            for (int v = 0; v < NV; ++v) Ue[v] -= Ui[v];
+            auto pair = [&](double da, double db, bool neg) { return scale * (flip(db, neg ? sg ^ 0x8000000000000000ULL : sg) - da); };
+            auto pick = [&](double x, double y, double z) { return dd == 0 ? x : (dd == 1 ? y : z); };
+            cor[r][0] = pair(pick(Ue[0], Ue[1], Ue[2]), Ue[6], false);
+            cor[r][1] = pair(pick(Ue[3], Ue[4], Ue[5]), Ue[7], false);
+            cor[r][2] = pair(pick(Ue[1], Ue[2], Ue[0]), pick(Ue[5], Ue[3], Ue[4]), false);
+            cor[r][3] = pair(pick(Ue[2], Ue[0], Ue[1]), pick(Ue[4], Ue[5], Ue[3]), true);
+            cor[r][4] = pair(Ue[8], jump, false);
         }
-        __syncthreads();
-        if (act) {
-            const int cc[3] = {i, j, k};
-            for (int dd = 0; dd < 3; ++dd) {
-                int t1, t2;
-                face_axes(dd, t1, t2);
-                const int ab = cc[t1] + np1 * cc[t2];
-                if (cc[dd] == 0)
-                    for (int v = 0; v < NV; ++v) du[v] -= sC[((2 * dd) * NV + v) * nf + ab];
-                if (cc[dd] == P)
-                    for (int v = 0; v < NV; ++v) du[v] -= sC[((2 * dd + 1) * NV + v) * nf + ab];
+        // added axis by axis: edge and corner nodes lie on faces of several axes, so a
+        // node-wise sum would diverge in every warp (54 FP64 slots a warp where 12 do)
+        for (int dd = 0; dd < 3; ++dd) {
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < K::FR; ++r) {
+                const int t = tid + r * NT;
+                if (t < 2 * dd * nf || t >= 2 * (dd + 1) * nf) continue;
+                const unsigned long long sg = (t / nf) & 1 ? 0ULL : 0x8000000000000000ULL;
+#pragma unroll
+                for (int pr = 0; pr < 5; ++pr) {
+                    int va, vb;
+                    bool neg;
+                    flux_pair(dd, pr, va, vb, neg);
+                    sR[va * nn + me[r]] -= cor[r][pr];
+                    if (pr < 4) sR[vb * nn + me[r]] += flip(cor[r][pr], neg ? sg ^ 0x8000000000000000ULL : sg);
+                }
             }
         }
+        __syncthreads();
+        double du[NV];
+        if (act)
+            for (int v = 0; v < NV; ++v) du[v] = sR[v * nn + tid];
         if (SUB == SUB_RHS) {
             if (act)
                 for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
@@ -352,7 +386,6 @@ __global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) 
                 for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
             substep_explicit(d, SUB, du, eb + tid, false, a, d.dt, u);
         }
-        __syncthreads();   // sU, sJ, sC are free from here on
         if (d.filter_on) {
             if (act)
                 for (int v = 0; v < NV; ++v) sU[v * nn + tid] = u[v];
@@ -362,14 +395,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, 3) k_dg_substep(Dev d, SubArgs a) 
                 for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
         }
         // implicit part after the filter; G at the stage value: G_s = (U_s - R~_s)/(dt a)
-        if (act) {
-            substep_implicit(d, SUB, d.dt, u);
-            if (SUB != SUB_C) {
-                double g[NG];
-                implicit_G_flat(u, d, g);
-                for (int c = 0; c < NG; ++c) a.Gout.dg(c)[eb + tid] = g[c];
-            }
-        }
+        if (act) substep_implicit<SUB>(d, d.sk, a, eb + tid, false, u);
         bool flagged = false;
         if (d.tci_on) {
             // u = |B~| ; u^ = u - (Pi x Pi x Pi) u ; ratio = sqrt(sum u^2 / sum u^)
@@ -456,9 +482,9 @@ static void dg_sub_dispatch(const Dev& d, int sub, const SubArgs& a, cudaStream_
 }
 
 void launch_dg_substep(const Dev& d, int sub, Field Uin, Field J, Field un, Field F2, Field F3,
-                       Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout,
+                       Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
                        cudaStream_t st) {
-    SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout};
+    SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout, Jout};
     launch_fd_traces(d, Uin, J, st);
     prof_begin(sub == SUB_RHS ? "dg_rhs" : "dg_substep", st);
     switch (d.P) {

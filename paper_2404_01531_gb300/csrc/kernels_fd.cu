@@ -538,12 +538,17 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
         if (SUB != SUB_C)
             for (int v = 0; v < NV; ++v) a.Fout.fd(v)[p] = du[v];
         double u[NV];
+        substep_explicit(d, SUB, du, p, true, a, dt_of(d, e), u);
         if (KS) {
-            substep_explicit(d, SUB, du, p, true, a, dt_of(d, e), u);
             if (SUB != SUB_C && !stiff_solve_gen(u, m, d, dt_of(d, e) * IM_A)) atomic_status(d, 2);
             if (d.mode != FFE_RELAX) hard_clamp_gen(u, m);
+            if (SUB != SUB_C) {
+                double g[NG];
+                implicit_G_gen(u, m, d, g);
+                for (int cg = 0; cg < NG; ++cg) a.Gout.fd(cg)[p] = g[cg];
+            }
         } else {
-            substep_combine(d, SUB, du, p, true, a, dt_of(d, e), u);
+            substep_implicit<SUB>(d, solve_k(d, e), a, p, true, u);
         }
         bool bad = false;
         for (int v = 0; v < NV; ++v) {
@@ -551,12 +556,6 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
             bad |= !isfinite(u[v]);
         }
         if (bad) atomic_status(d, 1);
-        if (SUB != SUB_C) {
-            double g[NG];
-            if (KS) implicit_G_gen(u, m, d, g);
-            else implicit_G_flat(u, d, g);
-            for (int cg = 0; cg < NG; ++cg) a.Gout.fd(cg)[p] = g[cg];
-        }
     }
 }
 
@@ -582,8 +581,8 @@ static void launch_update(const Dev& d, const int* list, int ci, int w0, const S
 
 void launch_fd_substep(const Dev& d, int sub, const int* list, int ci, Field Uin, Field J, Field un, Field F2,
                        Field F3, Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout,
-                       cudaStream_t st, bool faces) {
-    SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout};
+                       Field Jout, cudaStream_t st, bool faces) {
+    SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout, Jout};
     const int grid = d.nsm * 8;
     for (int k = 0, nch = fd_chunks(d); k < nch; ++k) {
         const int w0 = k * d.chunk;

@@ -6,7 +6,7 @@
 namespace ffe {
 
 struct SubArgs {
-    Field Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout;
+    Field Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout, Jout;
 };
 
 __device__ __forceinline__ void atomic_status(const Dev& d, int bits) { atomicOr(&d.counts[4], bits); }
@@ -39,18 +39,23 @@ __device__ __forceinline__ void substep_explicit(const Dev& d, int sub, const do
     }
 }
 
-// Implicit part: stiff solve (stages 3, 4) and the algebraic clamp when asked for.
-__device__ __forceinline__ void substep_implicit(const Dev& d, int sub, double dt, double* u) {
-    if (sub != SUB_C) {
-        if (!stiff_solve_flat(u, d, dt * IM_A)) atomic_status(d, 2);
+// Implicit part at point p and what is stored of it: stages 3 and 4 (substeps A, B)
+// solve, clamp, and leave G and J~ (the next substep's input); substep C clamps.
+template <int SUB>
+__device__ __forceinline__ void substep_implicit(const Dev& d, const SolveK& k, const SubArgs& a, int64_t p, bool isfd, double* u) {
+    if (SUB == SUB_C) {
+        if (d.mode != FFE_RELAX) hard_clamp_flat(u);
+        return;
     }
-    if (d.mode != FFE_RELAX) hard_clamp_flat(u);
-}
-
-__device__ __forceinline__ void substep_combine(const Dev& d, int sub, const double* f, int64_t p, bool isfd,
-                                                const SubArgs& a, double dt, double* u) {
-    substep_explicit(d, sub, f, p, isfd, a, dt, u);
-    substep_implicit(d, sub, dt, u);
+    double jp[3], ib2, g[NG], jd[3], jf[3];
+    if (!implicit_stage_flat(u, d, k, jp, ib2)) atomic_status(d, 2);
+    stage_G_flat(u, d, jp, g);
+    for (int c = 0; c < NG; ++c) (isfd ? a.Gout.fd(c) : a.Gout.dg(c))[p] = g[c];
+    stage_current_flat(u, jp, ib2, jd, jf);
+    for (int c = 0; c < 3; ++c) {
+        (isfd ? a.Jout.fd(c) : a.Jout.dg(c))[p] = jd[c];
+        (isfd ? a.Jout.fd(3 + c) : a.Jout.dg(3 + c))[p] = jf[c];
+    }
 }
 
 // A DG element the indicator flags needs an FD slot.  Contexts with a slot
