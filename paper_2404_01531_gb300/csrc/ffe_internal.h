@@ -20,6 +20,7 @@ constexpr int GH = 3;          // FD ghost layers
 // d_j alpha, d_j beta^i (index 3 j + i), gamma^jk Gamma^i_jk, K.
 enum MetIdx : int { M_ALPHA = 0, M_BETA = 1, M_GL = 4, M_GU = 10, M_SQRTG = 16, M_DALPHA = 17,
                     M_DBETA = 20, M_GTRACE = 29, M_K = 32, NMET = 33 };
+constexpr int NFG = 5;         // stored geometry values per DG face node (Dev::fgeo)
 constexpr int NPM = 17;        // the pointwise part (alpha .. sqrt(gamma)), without derivatives
 
 // IMEX-SSP3(4,3,3) coefficients (Pareschi & Russo 2005).
@@ -114,6 +115,9 @@ struct Dev {
     int curved, ks;
     const double* geo;
     const double* met;
+    // per DG face node of curved elements [E][6][NFG][np1^2]: outward unit normal (3),
+    // |grad xi|_gamma / (2 w0), lambda (k_face_geo)
+    const double* fgeo;
     // Kerr-Schild metric at FD points (null in flat space): subcell centres
     // [NMET][E ncell]; face points [3][NPM][E (nc+1) nc^2]; ghost centres across
     // Dirichlet faces [nbf][NPM][GH nc^2]
@@ -229,6 +233,7 @@ void launch_tci_ratio(const Dev& d, const double* Udg, double* ratio, cudaStream
 void launch_dg_substep_curved(const Dev& d, int sub, Field Uin, Field J, Field un, Field F2, Field F3, Field G1,
                               Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
                               cudaStream_t st);
+void launch_face_geo(const Dev& d, double* out, cudaStream_t st);
 void launch_stage12_ks(const Dev& d, Field un, Field Ua, Field G1, Field G2, cudaStream_t st);
 
 // adjoint (kernels_adjoint.cu)

@@ -1103,6 +1103,15 @@ ffe_status finish_create(ffe_ctx* c, int fd_cap, const std::vector<int>& orders)
     if ((s = dalloc(c, &d.ext, (size_t)12 * d.chunk * ne * ne * ne))) return s;
     if ((s = dalloc(c, &d.flux, (size_t)(d.curved ? 9 * NV : 3 * NV) * d.chunk * (d.nc + 1) * d.nc * d.nc))) return s;
     if ((s = dalloc(c, &d.ftr, (size_t)fd_cap * 6 * 12 * d.np1 * d.np1))) return s;
+    if (d.curved) {
+        double* fg;
+        if ((s = dalloc(c, &fg, (size_t)d.E * 6 * NFG * d.np1 * d.np1))) return s;
+        // on the stream of the allocation's clearing, done before the context is used
+        launch_face_geo(d, fg, nullptr);
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(nullptr));
+        d.fgeo = fg;
+    }
     return FFE_OK;
 }
 
@@ -2355,7 +2364,7 @@ static ffe_status filter_or_copy(ffe_ctx* c, Field in, Field out, int transpose)
 // right-hand side of the hybrid operator at U (fixed mask)
 static void rhs_at(ffe_ctx* c, Field U, Field out) {
     const Dev& d = c->d;
-    if (c->adj_fd) launch_current(d, U, c->J, nullptr, 0, c->st);
+    launch_current(d, U, c->J, nullptr, 0, c->st);
     launch_dg_substep_curved(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out, c->G1,
                              c->J2, c->st);
     if (c->adj_fd)

@@ -17,36 +17,21 @@
 
 namespace ffe {
 
-template <int P>
+template <int P, bool KS>
 struct DGC {
     static constexpr int np1 = P + 1;
     static constexpr int nn = np1 * np1 * np1;
     static constexpr int nf = np1 * np1;
     static constexpr int NT = ((nn + 31) / 32) * 32;
     static constexpr int NW = NT / 32;
-    // shared doubles: U[9][nn] | F[27][nn] (the filter buffer [9][nn] aliases it) | C[6][9][nf] | red[2][NW]
-    static constexpr int SMEM = (9 * nn + 27 * nn + 54 * nf + 2 * NW + 1) * 8;
+    static constexpr int FR = (6 * nf + NT - 1) / NT;   // face nodes per thread
+    // CTAs per SM the registers are bounded for (see k_dg_curved)
+    static constexpr int CTAS = NT <= 128 ? (KS ? 3 : 4) : 2;
+    // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn], Kerr-Schild:
+    // J[3][nn], F[27][nn] | dU/dt[9][nn] | red[2][NW] and the flag
+    static constexpr int NS = KS ? 30 : 3;
+    static constexpr int SMEM = ((18 + NS) * nn + 2 * NW + 1) * 8;
 };
-
-template <bool KS>
-__device__ __forceinline__ void node_metric(const Dev& d, int64_t p, PM& m) {
-    if (KS) {
-        load_pm(d.met, d.ndg, p, m);
-    } else {
-        m.a = 1.0;
-        m.b[0] = m.b[1] = m.b[2] = 0.0;
-        for (int i = 0; i < 6; ++i) m.gl[i] = m.gu[i] = (i == 0 || i == 3 || i == 5) ? 1.0 : 0.0;
-        m.sg = 1.0;
-    }
-}
-
-template <bool KS>
-__device__ __forceinline__ void fluxes_at(const double* U, const PM& m, double eta, double F[3][NV], double* jd) {
-    double jf[3];
-    if (KS) current_gen(U, m, eta, jd, jf);
-    else current_flat(U, eta, jd, jf);
-    flux_gen(U, jf, m, F);
-}
 
 template <int NW>
 __device__ __forceinline__ void block_sum2c(double& x, double& y, double* red) {
@@ -80,68 +65,197 @@ __device__ __forceinline__ void nbr_node(const Dev& d, int e, int f, int ta, int
     c[u2] = b2;
 }
 
+// Outward unit normal (lower index) at face node ab of face f, |grad xi|_gamma / (2 w0)
+// and lambda = alpha + |beta.n| (Dev::fgeo, k_face_geo)
+__device__ __forceinline__ const double* face_geo(const Dev& d, int e, int f, int ab) {
+    return d.fgeo + (((int64_t)e * 6 + f) * NFG) * d.np1 * d.np1 + ab;
+}
+
+__global__ void k_face_geo(Dev d, double* out) {
+    const int nfm = d.np1 * d.np1;
+    const int64_t total = (int64_t)d.E * 6 * nfm;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        const int ab = (int)(t % nfm), f = (int)((t / nfm) % 6), e = (int)(t / (6 * nfm));
+        const ES es = esz(d, e);
+        const int np1 = es.np1;
+        if (ab >= np1 * np1) continue;
+        const int dd = f >> 1, s = f & 1;
+        int c[3];
+        c[dd] = s ? es.P : 0;
+        c[dd == 0 ? 1 : 0] = ab % np1;
+        c[dd == 2 ? 1 : 2] = ab / np1;
+        const int64_t p = (int64_t)e * d.nn + c[0] + np1 * (c[1] + np1 * c[2]);
+        const double w0inv = 1.0 / d.tabs[es.P].w0;
+        double nl[3], nu[3], lam = 1.0;
+        for (int i = 0; i < 3; ++i) nu[i] = nl[i] = (s ? 1.0 : -1.0) * d.geo[(int64_t)(3 * dd + i) * d.ndg + p];
+        PM m;
+        if (d.ks) {
+            load_pm(d.met, d.ndg, p, m);
+            for (int i = 0; i < 3; ++i)
+                nu[i] = fma(m.gu[sym3(i, 0)], nl[0], fma(m.gu[sym3(i, 1)], nl[1], m.gu[sym3(i, 2)] * nl[2]));
+        }
+        const double norm = sqrt(d3(nu, nl)), inrm = 1.0 / norm;
+        for (int i = 0; i < 3; ++i) nl[i] *= inrm;
+        if (d.ks) lam = m.a + fabs(d3(m.b, nl));
+        double* o = out + (((int64_t)e * 6 + f) * NFG) * nfm + ab;
+        for (int i = 0; i < 3; ++i) o[i * nfm] = nl[i];
+        o[3 * nfm] = 0.5 * norm * w0inv;
+        o[4 * nfm] = lam;
+    }
+}
+
+void launch_face_geo(const Dev& d, double* out, cudaStream_t st) {
+    k_face_geo<<<d.nsm * 8, 256, 0, st>>>(d, out);
+    g_launch_counter += 1;
+}
+
+// Exterior state at face node (face f, tangential ta, tb; node p, interior state Ui,
+// outward unit normal nl) and its current J~; false where the current is J~(Ue)
+template <int P, bool KS>
+__device__ __forceinline__ bool curved_external(const Dev& d, const SubArgs& a, int e, int f, int ta, int tb, int64_t p,
+                                                const double* Ui, const double* nl, double* Ue, double* Je) {
+    constexpr int np1 = P + 1, nf = np1 * np1;
+    const int nb = d.nbr[e * 6 + f];
+    if (nb >= 0) {
+        int cn[3];
+        nbr_node<P>(d, e, f, ta, tb, cn);
+        if (d.mask[nb] == 0) {
+            const int64_t q = (int64_t)nb * d.nn + cn[0] + np1 * (cn[1] + np1 * cn[2]);
+            for (int v = 0; v < NV; ++v) Ue[v] = a.Uin.dg(v)[q];
+            if (!KS)
+                for (int k = 0; k < 3; ++k) Je[k] = a.J.dg(3 + k)[q];
+            return !KS;
+        }
+        // FD->DG projection (6-point stencils) of the neighbour's cells and of
+        // their current J~ (the current of a projected state would carry its
+        // projection error in E~.B~ amplified by eta into the q~ flux), from the face
+        // traces k_fd_traces left for it, indexed along the neighbour's own face axes
+        const int f2 = d.nbr_face[e * 6 + f], d2 = f2 >> 1;
+        const int u1 = d2 == 0 ? 1 : 0, u2 = d2 == 2 ? 1 : 2;
+        const int nfm = d.np1 * d.np1;
+        const double* tr = d.ftr + ((int64_t)fd_slot_of(d, nb) * 6 + f2) * 12 * nfm + cn[u1] + np1 * cn[u2];
+        for (int v = 0; v < NV; ++v) Ue[v] = tr[v * nfm];
+        for (int q = 0; q < 3; ++q) Je[q] = tr[(NV + q) * nfm];
+        return true;
+    }
+    const int kind = d.bc[e * 6 + f];
+    if (kind == FFE_BC_DIRICHLET) {
+        const double* src = d.bdg + (int64_t)d.bface[e * 6 + f] * NV * nf;
+        for (int v = 0; v < NV; ++v) Ue[v] = src[v * nf + ta + np1 * tb];
+    } else if (kind == FFE_BC_NO_INCOMING) {
+        if (KS) {
+            PM mf;
+            load_pm(d.met, d.ndg, p, mf);
+            bc_no_incoming_gen(Ui, mf, nl, Ue);
+        } else {
+            bc_no_incoming_flat(Ui, nl, Ue);
+        }
+    } else if (kind == FFE_BC_OUTFLOW) {
+        for (int v = 0; v < NV; ++v) Ue[v] = Ui[v];
+    } else {
+        double xn[3];
+        for (int q = 0; q < 3; ++q) xn[q] = d.xyz_dg[(int64_t)q * d.ndg + p];
+        bc_star_flat(Ui, xn, omega_of(d, e), Ue);
+    }
+    return false;
+}
+
+// n_j F^j of the flat flux at a jump (dU, dJ)
+__device__ __forceinline__ void flux_normal_flat(const double* n, const double* U, const double* J, double* o) {
+    const double *E = U, *B = U + 3;
+    o[0] = fma(n[2], B[1], fma(n[1], -B[2], n[0] * U[6]));
+    o[1] = fma(n[2], -B[0], fma(n[1], U[6], n[0] * B[2]));
+    o[2] = fma(n[2], U[6], fma(n[1], B[0], n[0] * -B[1]));
+    o[3] = fma(n[2], -E[1], fma(n[1], E[2], n[0] * U[7]));
+    o[4] = fma(n[2], E[0], fma(n[1], U[7], n[0] * -E[2]));
+    o[5] = fma(n[2], U[7], fma(n[1], -E[0], n[0] * E[1]));
+    o[6] = fma(n[2], E[2], fma(n[1], E[1], n[0] * E[0]));
+    o[7] = fma(n[2], B[2], fma(n[1], B[1], n[0] * B[0]));
+    o[8] = fma(n[2], J[2], fma(n[1], J[1], n[0] * J[0]));
+}
+
+// n_j F^j with the metric (flux_gen contracted with n)
+__device__ __forceinline__ void flux_normal_gen(const double* n, const PM& m, const double* U, const double* J, double* o) {
+    double El[3], Bl[3], nu[3];
+    lowr(m, U, El);
+    lowr(m, U + 3, Bl);
+    const double bn = d3(m.b, n), ia = m.a / m.sg;
+    for (int i = 0; i < 3; ++i)
+        nu[i] = m.a * fma(m.gu[sym3(i, 0)], n[0], fma(m.gu[sym3(i, 1)], n[1], m.gu[sym3(i, 2)] * n[2]));
+    for (int i = 0; i < 3; ++i) {
+        const int j = i == 2 ? 0 : i + 1, k = i == 0 ? 2 : i - 1;   // [ijk] n_j B_k = n_j B_k - n_k B_j, (i, j, k) cyclic
+        o[i] = fma(-bn, U[i], fma(nu[i], U[6], -ia * fma(n[j], Bl[k], -n[k] * Bl[j])));
+        o[3 + i] = fma(-bn, U[3 + i], fma(nu[i], U[7], ia * fma(n[j], El[k], -n[k] * El[j])));
+    }
+    o[6] = fma(-bn, U[6], m.a * d3(n, U));
+    o[7] = fma(-bn, U[7], m.a * d3(n, U + 3));
+    o[8] = fma(-bn, U[8], d3(n, J));
+}
+
 // One element of order P processed by a block of NT threads (NT >= (P+1)^3).
 template <int P, int NT, int SUB, bool KS>
 __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, int e, double* sm) {
-    using K = DGC<P>;
+    using K = DGC<P, KS>;
     constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NW = NT / 32;
     double* sU = sm;                 // [9][nn]
-    double* sF = sU + 9 * nn;        // [3][9][nn]
-    double* sC = sF + 27 * nn;       // [6][9][nf]
-    double* red = sC + 54 * nf;
+    double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
+    double* sF = sJ + 3 * nn;        // Kerr-Schild: [3][9][nn] F^j
+    double* sR = sJ + K::NS * nn;    // [9][nn] dU/dt
+    double* red = sR + 9 * nn;
     const Tables& T = d.tabs[P];
     const int tid = threadIdx.x;
     const bool act = tid < nn;
     const int ci[3] = {tid % np1, (tid / np1) % np1, tid / (np1 * np1)};
-    const double w0inv = 1.0 / T.w0;
-    {
-        const int64_t eb = (int64_t)e * d.nn;
-        const double dt = dt_of(d, e);
-        for (int t = tid; t < NV * nn; t += NT) sU[t] = a.Uin.dg(t / nn)[eb + t % nn];
-        __syncthreads();
-        PM m;
-        double jd[3] = {0.0, 0.0, 0.0}, ij[3][3];
+    const int64_t eb = (int64_t)e * d.nn;
+    const double dt = dt_of(d, e);
+    for (int t = tid; t < NV * nn; t += NT) sU[t] = a.Uin.dg(t / nn)[eb + t % nn];
+    if (!KS)
+        for (int t = tid; t < 3 * nn; t += NT) sJ[t] = a.J.dg(3 + t / nn)[eb + t % nn];
+    __syncthreads();
+    if (KS) {
         if (act) {
-            node_metric<KS>(d, eb + tid, m);
-            for (int k = 0; k < 3; ++k)
-                for (int i = 0; i < 3; ++i) ij[k][i] = d.geo[(int64_t)(3 * k + i) * d.ndg + eb + tid];
-            double u[NV];
+            PM m;
+            load_pm(d.met, d.ndg, eb + tid, m);
+            double u[NV], jd[3], jf[3], F[3][NV], S[NV];
             for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
-            if (KS) {
-                double F[3][NV];
-                fluxes_at<KS>(u, m, d.eta, F, jd);
-                for (int j = 0; j < 3; ++j)
-                    for (int v = 0; v < NV; ++v) sF[(j * NV + v) * nn + tid] = F[j][v];
-            } else {
-                // flat metric: the fluxes are fixed linear combinations of E~, B~,
-                // psi~, phi~ and J~, so only J~ (full) is stored beside U
-                double jf[3];
-                current_flat(u, d.eta, jd, jf);
-                for (int i = 0; i < 3; ++i) sF[i * nn + tid] = jf[i];
-            }
+            current_gen(u, m, d.eta, jd, jf);
+            flux_gen(u, jf, m, F);
+            for (int i = 0; i < 3; ++i) sJ[i * nn + tid] = jf[i];
+            for (int j = 0; j < 3; ++j)
+                for (int v = 0; v < NV; ++v) sF[(j * NV + v) * nn + tid] = F[j][v];
+            sources_gen(u, jd, m, d.met, d.ndg, eb + tid, S);
+            for (int v = 0; v < NV; ++v) sR[v * nn + tid] = S[v];
         }
         __syncthreads();
+    }
+    if (act) {
         double du[NV];
-        if (act && !KS) {
-            // flat metric: D_k F^j = +-D_k of one field (D_k is linear), so the
-            // volume term is built from the reference derivatives R = D_k X of the
-            // 11 fields X = E~, B~, psi~, phi~, J~ and the node's d xi^k/d x^j:
-            //   E~: curl B~ - grad psi~,  B~: -curl E~ - grad phi~,
-            //   psi~: -div E~,  phi~: -div B~,  q~: -div J~
-            for (int v = 0; v < NV; ++v) du[v] = 0.0;
+        for (int v = 0; v < NV; ++v) du[v] = KS ? sR[v * nn + tid] : 0.0;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
-                const int base = tid - ci[k] * stride;
-                double Dk[np1];
-                for (int mm = 0; mm < np1; ++mm) Dk[mm] = T.D[ci[k]][mm];
-                auto R = [&](const double* f) {
-                    double acc = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
+            const int base = tid - ci[k] * stride;
+            double Dk[np1];
+            for (int mm = 0; mm < np1; ++mm) Dk[mm] = T.D[ci[k]][mm];
+            auto R = [&](const double* f) {
+                double acc = 0.0;
 #pragma unroll
-                    for (int mm = 0; mm < np1; ++mm) acc = fma(Dk[mm], f[base + mm * stride], acc);
-                    return acc;
-                };
-                const double ka = ij[k][0], kb = ij[k][1], kc = ij[k][2];
+                for (int mm = 0; mm < np1; ++mm) acc = fma(Dk[mm], f[base + mm * stride], acc);
+                return acc;
+            };
+            double g[3];
+            for (int i = 0; i < 3; ++i) g[i] = d.geo[(int64_t)(3 * k + i) * d.ndg + eb + tid];
+            if (KS) {
+                for (int j = 0; j < 3; ++j)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) du[v] = fma(-g[j], R(sF + (j * NV + v) * nn), du[v]);
+            } else {
+                // flat metric: D_k F^j = +-D_k of one field (D_k is linear), so the
+                // volume term is built from the reference derivatives R = D_k X of the
+                // 11 fields X = E~, B~, psi~, phi~, J~ and the node's d xi^k/d x^j:
+                //   E~: curl B~ - grad psi~,  B~: -curl E~ - grad phi~,
+                //   psi~: -div E~,  phi~: -div B~,  q~: -div J~
+                const double ka = g[0], kb = g[1], kc = g[2];
                 double r;
                 r = R(sU + 0 * nn);   // E0
                 du[4] = fma(-kc, r, du[4]); du[5] = fma(kb, r, du[5]); du[6] = fma(-ka, r, du[6]);
@@ -159,273 +273,193 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
                 du[0] = fma(-ka, r, du[0]); du[1] = fma(-kb, r, du[1]); du[2] = fma(-kc, r, du[2]);
                 r = R(sU + 7 * nn);   // phi
                 du[3] = fma(-ka, r, du[3]); du[4] = fma(-kb, r, du[4]); du[5] = fma(-kc, r, du[5]);
-                r = R(sF + 0 * nn);   // J0
+                r = R(sJ + 0 * nn);   // J0
                 du[8] = fma(-ka, r, du[8]);
-                r = R(sF + 1 * nn);   // J1
+                r = R(sJ + 1 * nn);   // J1
                 du[8] = fma(-kb, r, du[8]);
-                r = R(sF + 2 * nn);   // J2
+                r = R(sJ + 2 * nn);   // J2
                 du[8] = fma(-kc, r, du[8]);
             }
         }
-        if (act && KS) {
-            for (int v = 0; v < NV; ++v) du[v] = 0.0;
-            for (int k = 0; k < 3; ++k) {
-                const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
-                const int base = tid - ci[k] * stride;
-                double Dk[np1];
-                for (int mm = 0; mm < np1; ++mm) Dk[mm] = T.D[ci[k]][mm];
-                for (int j = 0; j < 3; ++j) {
-                    const double s = -ij[k][j];
-                    for (int v = 0; v < NV; ++v) {
-                        const double* src = sF + (j * NV + v) * nn + base;
-                        double acc = 0.0;
-#pragma unroll
-                        for (int mm = 0; mm < np1; ++mm) acc = fma(Dk[mm], src[mm * stride], acc);
-                        du[v] = fma(s, acc, du[v]);
-                    }
-                }
-            }
+        if (!KS) {
+            for (int i = 0; i < 3; ++i) du[i] -= a.J.dg(i)[eb + tid];
+            du[6] += sU[8 * nn + tid];
         }
-        if (act) {
-            double u[NV], S[NV];
-            for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
-            if (KS) {
-                sources_gen(u, jd, m, d.met, d.ndg, eb + tid, S);
-                for (int v = 0; v < NV; ++v) du[v] += S[v];
-            } else {
-                du[0] -= jd[0]; du[1] -= jd[1]; du[2] -= jd[2];
-                du[6] += u[8];
-            }
-        }
-        // lift: one thread per face node
-        for (int t = tid; t < 6 * nf; t += NT) {
-            const int f = t / nf, ab = t % nf, ta = ab % np1, tb = ab / np1;
-            const int dd = f >> 1, s = f & 1;
-            const int t1 = dd == 0 ? 1 : 0, t2 = dd == 2 ? 1 : 2;
-            int c[3];
-            c[dd] = s ? P : 0;
-            c[t1] = ta;
-            c[t2] = tb;
-            const int me = c[0] + np1 * (c[1] + np1 * c[2]);
-            const int64_t p = eb + me;
-            PM mf;
-            node_metric<KS>(d, p, mf);
-            double nl[3];
-            for (int i = 0; i < 3; ++i) nl[i] = (s ? 1.0 : -1.0) * d.geo[(int64_t)(3 * dd + i) * d.ndg + p];
-            double nu[3];
-            for (int i = 0; i < 3; ++i) nu[i] = fma(mf.gu[sym3(i, 0)], nl[0], fma(mf.gu[sym3(i, 1)], nl[1], mf.gu[sym3(i, 2)] * nl[2]));
-            const double norm = sqrt(d3(nu, nl));
-            const double inrm = 1.0 / norm;
-            for (int i = 0; i < 3; ++i) nl[i] *= inrm;
-            double Ui[NV], Ue[NV], Je[3];
-            bool jx = false;   // exterior current given (FD neighbour), not J~(Ue)
-            for (int v = 0; v < NV; ++v) Ui[v] = sU[v * nn + me];
-            const int nb = d.nbr[e * 6 + f];
-            if (nb >= 0) {
-                int cn[3];
-                nbr_node<P>(d, e, f, ta, tb, cn);
-                if (d.mask[nb] == 0) {
-                    const int64_t q = (int64_t)nb * d.nn + cn[0] + np1 * (cn[1] + np1 * cn[2]);
-                    for (int v = 0; v < NV; ++v) Ue[v] = a.Uin.dg(v)[q];
-                } else {
-                    // FD->DG projection (6-point stencils) of the neighbour's cells and of
-                    // their current J~ (the current of a projected state would carry its
-                    // projection error in E~.B~ amplified by eta into the q~ flux)
-                    // (from the face traces k_fd_traces left for it, indexed along
-                    // the neighbour's own face axes)
-                    jx = true;
-                    const int f2 = d.nbr_face[e * 6 + f], d2 = f2 >> 1;
-                    const int u1 = d2 == 0 ? 1 : 0, u2 = d2 == 2 ? 1 : 2;
-                    const int nfm = d.np1 * d.np1;
-                    const double* tr = d.ftr + ((int64_t)fd_slot_of(d, nb) * 6 + f2) * 12 * nfm + cn[u1] + np1 * cn[u2];
-                    for (int v = 0; v < NV; ++v) Ue[v] = tr[v * nfm];
-                    for (int q = 0; q < 3; ++q) Je[q] = tr[(NV + q) * nfm];
-                }
-            } else {
-                const int kind = d.bc[e * 6 + f];
-                if (kind == FFE_BC_DIRICHLET) {
-                    const double* src = d.bdg + (int64_t)d.bface[e * 6 + f] * NV * nf;
-                    for (int v = 0; v < NV; ++v) Ue[v] = src[v * nf + ta + np1 * tb];
-                } else if (kind == FFE_BC_NO_INCOMING) {
-                    if (KS) bc_no_incoming_gen(Ui, mf, nl, Ue);
-                    else bc_no_incoming_flat(Ui, nl, Ue);
-                } else if (kind == FFE_BC_OUTFLOW) {
-                    for (int v = 0; v < NV; ++v) Ue[v] = Ui[v];
-                } else {
-                    double xn[3];
-                    for (int q = 0; q < 3; ++q) xn[q] = d.xyz_dg[(int64_t)q * d.ndg + p];
-                    bc_star_flat(Ui, xn, omega_of(d, e), Ue);
-                }
-            }
-            const double lam = mf.a + fabs(d3(mf.b, nl));
-            const double sc = 0.5 * norm * w0inv;
-            if (KS) {
-                double Fe[3][NV], jde[3];
-                if (jx) flux_gen(Ue, Je, mf, Fe);
-                else fluxes_at<KS>(Ue, mf, d.eta, Fe, jde);
-                for (int v = 0; v < NV; ++v) {
-                    double dfn = 0.0;
-                    for (int j = 0; j < 3; ++j) dfn = fma(nl[j], Fe[j][v] - sF[(j * NV + v) * nn + me], dfn);
-                    sC[(f * NV + v) * nf + ab] = sc * fma(-lam, Ue[v] - Ui[v], dfn);
-                }
-            } else {
-                // the flat flux is linear in (U, J~): F(Ue) - F(Ui) = F(Ue - Ui, Je - Ji),
-                // Ji the node's stored current, Je the exterior one
-                if (!jx) {
-                    double jde[3];
-                    current_flat(Ue, d.eta, jde, Je);
-                }
-                double dUv[NV], dJv[3], Fd[3][NV];
-                for (int v = 0; v < NV; ++v) dUv[v] = Ue[v] - Ui[v];
-                for (int i = 0; i < 3; ++i) dJv[i] = Je[i] - sF[i * nn + me];
-                flux_gen(dUv, dJv, mf, Fd);
-                for (int v = 0; v < NV; ++v) {
-                    const double dfn = fma(nl[2], Fd[2][v], fma(nl[1], Fd[1][v], nl[0] * Fd[0][v]));
-                    sC[(f * NV + v) * nf + ab] = sc * fma(-lam, dUv[v], dfn);
-                }
-            }
-        }
-        __syncthreads();
-        if (act) {
-            for (int dd = 0; dd < 3; ++dd) {
-                const int t1 = dd == 0 ? 1 : 0, t2 = dd == 2 ? 1 : 2;
-                const int ab = ci[t1] + np1 * ci[t2];
-                if (ci[dd] == 0)
-                    for (int v = 0; v < NV; ++v) du[v] -= sC[((2 * dd) * NV + v) * nf + ab];
-                if (ci[dd] == P)
-                    for (int v = 0; v < NV; ++v) du[v] -= sC[((2 * dd + 1) * NV + v) * nf + ab];
-            }
-        }
-        if (SUB == SUB_RHS) {
-            if (act)
-                for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
-            __syncthreads();
-            return;
-        }
-        double u[NV];
-        if (act) {
-            if (SUB != SUB_C)
-                for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
-            if (KS) {
-                // explicit part of the stage (the metric-aware solve and clamp follow the filter)
-                const int gv[NG] = {0, 1, 2, 6, 7};
-                for (int v = 0; v < NV; ++v) u[v] = a.un.dg(v)[eb + tid];
-                if (SUB == SUB_A) {
-                    for (int v = 0; v < NV; ++v) u[v] = fma(dt, du[v], u[v]);
-                    for (int c = 0; c < NG; ++c) u[gv[c]] = fma(dt * (1.0 - IM_A), a.G2.dg(c)[eb + tid], u[gv[c]]);
-                } else if (SUB == SUB_B) {
-                    for (int v = 0; v < NV; ++v) u[v] = fma(0.25 * dt, a.F2.dg(v)[eb + tid] + du[v], u[v]);
-                    const double z = 0.5 - IM_B - IM_H - IM_A;
-                    for (int c = 0; c < NG; ++c)
-                        u[gv[c]] = fma(dt, IM_B * a.G1.dg(c)[eb + tid] + IM_H * a.G2.dg(c)[eb + tid] + z * a.G3.dg(c)[eb + tid], u[gv[c]]);
-                } else {
-                    for (int v = 0; v < NV; ++v)
-                        u[v] = fma(dt, (a.F2.dg(v)[eb + tid] + a.F3.dg(v)[eb + tid]) * (1.0 / 6.0) + du[v] * (2.0 / 3.0), u[v]);
-                    for (int c = 0; c < NG; ++c)
-                        u[gv[c]] = fma(dt, (a.G2.dg(c)[eb + tid] + a.G3.dg(c)[eb + tid]) * (1.0 / 6.0) + a.G4.dg(c)[eb + tid] * (2.0 / 3.0), u[gv[c]]);
-                }
-            } else {
-                substep_explicit(d, SUB, du, eb + tid, false, a, dt, u);
-            }
-        }
-        __syncthreads();
-        if (d.filter_on) {
-            if (act)
-                for (int v = 0; v < NV; ++v) sU[v * nn + tid] = u[v];
-            __syncthreads();
-            filter_lowrank<P, NT>(T, sU);
-            if (act)
-                for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
-        }
-        // implicit part after the filter; G at the stage value: G_s = (U_s - R~_s)/(dt a)
-        if (act) {
-            if (KS) {
-                if (SUB != SUB_C && !stiff_solve_gen(u, m, d, dt * IM_A)) atomic_status(d, 2);
-                if (d.mode != FFE_RELAX) hard_clamp_gen(u, m);
-                if (SUB != SUB_C) {
-                    double g[NG];
-                    implicit_G_gen(u, m, d, g);
-                    for (int c = 0; c < NG; ++c) a.Gout.dg(c)[eb + tid] = g[c];
-                }
-            } else {
-                substep_implicit<SUB>(d, solve_k(d, e), a, eb + tid, false, u);
-            }
-        }
-        bool flagged = false;
-        if (d.tci_on) {
-            double mag = 0.0;
-            if (act) mag = KS ? bnorm_gen(u, m) : sqrt(fma(u[5], u[5], fma(u[4], u[4], u[3] * u[3])));
-            if (act) sU[tid] = mag;
-            __syncthreads();
-            double low = 0.0;
-            for (int k = 0; k < 3; ++k) {
-                const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
-                if (act) {
-                    const int base = tid - ci[k] * stride;
-                    double acc = 0.0;
-                    for (int mm = 0; mm < np1; ++mm) acc = fma(T.Pi[ci[k]][mm], sU[k * nn + base + mm * stride], acc);
-                    if (k < 2) sU[(k + 1) * nn + tid] = acc;
-                    else low = acc;
-                }
-                __syncthreads();
-            }
-            double num = 0.0, den = 0.0;
-            if (act) {
-                const double uh = mag - low;
-                num = uh * uh;
-                den = mag * mag;
-            }
-            block_sum2c<NW>(num, den, red);
-            const double ratio = den > 0.0 ? sqrt(num / den) : 0.0;
-            const double thr = d.thr_dgP[P];
-            if (tid == 0) {
-                int fl = ratio > thr;
-                if (fabs(ratio - thr) <= 1e-12 * thr) d.near_list[atomicAdd(&d.counts[3], 1) & 4095] = e;
-                if (fl && take_fd_slot(d, e)) {
-                    d.flag_list[atomicAdd(&d.counts[2], 1)] = e;
-                    d.switched[e] = 1;
-                } else {
-                    fl = 0;
-                }
-                red[2 * NW] = fl;
-            }
-            __syncthreads();
-            flagged = red[2 * NW] != 0.0;
-        }
-        if (!flagged && tid == 0) {
-            atomicAdd(d.units, (unsigned long long)nn);
-            atomicAdd(d.units + 2, 1ull);
-        }
-        if (!flagged && act) {
-            bool bad = false;
-            for (int v = 0; v < NV; ++v) {
-                a.Uout.dg(v)[eb + tid] = u[v];
-                bad |= !isfinite(u[v]);
-            }
-            if (bad) atomic_status(d, 1);
-        }
-        __syncthreads();
+        for (int v = 0; v < NV; ++v) sR[v * nn + tid] = du[v];
     }
+    // lift: one thread per face node.  The flux at a fixed point is linear in
+    // (U, J~): F(Ue) - F(Ui) = F(Ue - Ui, Je - Ji), contracted with the normal at once
+    double cor[K::FR][NV];
+    int me[K::FR];
+#pragma unroll
+    for (int r = 0; r < K::FR; ++r) {
+        const int t = tid + r * NT;
+        if (t >= 6 * nf) break;
+        const int f = t / nf, ab = t % nf, ta = ab % np1, tb = ab / np1;
+        const int dd = f >> 1;
+        int c[3];
+        c[dd] = (f & 1) ? P : 0;
+        c[dd == 0 ? 1 : 0] = ta;
+        c[dd == 2 ? 1 : 2] = tb;
+        me[r] = c[0] + np1 * (c[1] + np1 * c[2]);
+        const int64_t p = eb + me[r];
+        const double* fg = face_geo(d, e, f, ab);
+        const int nfm = d.np1 * d.np1;
+        const double nl[3] = {fg[0], fg[nfm], fg[2 * nfm]}, sc = fg[3 * nfm];
+        double Ui[NV], Ue[NV], Je[3];
+        for (int v = 0; v < NV; ++v) Ui[v] = sU[v * nn + me[r]];
+        const bool given = curved_external<P, KS>(d, a, e, f, ta, tb, p, Ui, nl, Ue, Je);
+        if (KS) {
+            PM mf;
+            load_pm(d.met, d.ndg, p, mf);
+            if (!given) {
+                double jde[3];
+                current_gen(Ue, mf, d.eta, jde, Je);
+            }
+            for (int v = 0; v < NV; ++v) Ue[v] -= Ui[v];
+            for (int i = 0; i < 3; ++i) Je[i] -= sJ[i * nn + me[r]];
+            flux_normal_gen(nl, mf, Ue, Je, cor[r]);
+            const double lam = fg[4 * nfm];
+            for (int v = 0; v < NV; ++v) cor[r][v] = sc * fma(-lam, Ue[v], cor[r][v]);
+        } else {
+            if (!given) {
+                double jde[3];
+                current_flat(Ue, d.eta, jde, Je);
+            }
+            for (int v = 0; v < NV; ++v) Ue[v] -= Ui[v];
+            for (int i = 0; i < 3; ++i) Je[i] -= sJ[i * nn + me[r]];
+            flux_normal_flat(nl, Ue, Je, cor[r]);
+            for (int v = 0; v < NV; ++v) cor[r][v] = sc * (cor[r][v] - Ue[v]);
+        }
+    }
+    // added axis by axis (edge and corner nodes lie on faces of several axes; see k_dg_substep)
+    for (int dd = 0; dd < 3; ++dd) {
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < K::FR; ++r) {
+            const int t = tid + r * NT;
+            if (t < 2 * dd * nf || t >= 2 * (dd + 1) * nf) continue;
+            for (int v = 0; v < NV; ++v) sR[v * nn + me[r]] -= cor[r][v];
+        }
+    }
+    __syncthreads();
+    double du[NV], u[NV];
+    if (act)
+        for (int v = 0; v < NV; ++v) du[v] = sR[v * nn + tid];
+    if (SUB == SUB_RHS) {
+        if (act)
+            for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
+        __syncthreads();
+        return;
+    }
+    if (act) {
+        if (SUB != SUB_C)
+            for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
+        substep_explicit(d, SUB, du, eb + tid, false, a, dt, u);
+    }
+    if (d.filter_on) {
+        if (act)
+            for (int v = 0; v < NV; ++v) sU[v * nn + tid] = u[v];
+        __syncthreads();
+        filter_lowrank<P, NT>(T, sU);
+        if (act)
+            for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
+    }
+    // implicit part after the filter; G at the stage value: G_s = (U_s - R~_s)/(dt a)
+    double mag = 0.0;
+    if (act) {
+        if (KS) {
+            PM m;
+            load_pm(d.met, d.ndg, eb + tid, m);
+            if (SUB != SUB_C && !stiff_solve_gen(u, m, d, dt * IM_A)) atomic_status(d, 2);
+            if (d.mode != FFE_RELAX) hard_clamp_gen(u, m);
+            if (SUB != SUB_C) {
+                double g[NG];
+                implicit_G_gen(u, m, d, g);
+                for (int c = 0; c < NG; ++c) a.Gout.dg(c)[eb + tid] = g[c];
+            }
+            if (d.tci_on) mag = bnorm_gen(u, m);
+        } else {
+            substep_implicit<SUB>(d, solve_k(d, e), a, eb + tid, false, u);
+            if (d.tci_on) mag = sqrt(fma(u[5], u[5], fma(u[4], u[4], u[3] * u[3])));
+        }
+    }
+    bool flagged = false;
+    if (d.tci_on) {
+        if (act) sU[tid] = mag;
+        __syncthreads();
+        double low = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
+            if (act) {
+                const int base = tid - ci[k] * stride;
+                double acc = 0.0;
+                for (int mm = 0; mm < np1; ++mm) acc = fma(T.Pi[ci[k]][mm], sU[k * nn + base + mm * stride], acc);
+                if (k < 2) sU[(k + 1) * nn + tid] = acc;
+                else low = acc;
+            }
+            __syncthreads();
+        }
+        double num = 0.0, den = 0.0;
+        if (act) {
+            const double uh = mag - low;
+            num = uh * uh;
+            den = mag * mag;
+        }
+        block_sum2c<NW>(num, den, red);
+        const double ratio = den > 0.0 ? sqrt(num / den) : 0.0;
+        const double thr = d.thr_dgP[P];
+        if (tid == 0) {
+            int fl = ratio > thr;
+            if (fabs(ratio - thr) <= 1e-12 * thr) d.near_list[atomicAdd(&d.counts[3], 1) & 4095] = e;
+            if (fl && take_fd_slot(d, e)) {
+                d.flag_list[atomicAdd(&d.counts[2], 1)] = e;
+                d.switched[e] = 1;
+            } else {
+                fl = 0;
+            }
+            red[2 * NW] = fl;
+        }
+        __syncthreads();
+        flagged = red[2 * NW] != 0.0;
+    }
+    if (!flagged && tid == 0) {
+        atomicAdd(d.units, (unsigned long long)nn);
+        atomicAdd(d.units + 2, 1ull);
+    }
+    if (!flagged && act) {
+        bool bad = false;
+        for (int v = 0; v < NV; ++v) {
+            a.Uout.dg(v)[eb + tid] = u[v];
+            bad |= !isfinite(u[v]);
+        }
+        if (bad) atomic_status(d, 1);
+    }
+    __syncthreads();
 }
 
 
 // Persistent kernel over a DG work list of order-P elements (list, count in
-// d.counts[ci]); flat metric: two CTAs per SM (four for the 128-thread CTAs of
-// orders <= 4; registers bounded accordingly), the metric-aware variant one.
-// Batched contexts launch each order's elements separately, in CTAs sized for
-// that order (one kernel dispatching on the order would keep every order's
-// registers live and spill).
+// d.counts[ci]).  Bound by the FP64 pipe, as the box kernel (k_dg_substep): J~ is read
+// instead of formed again at the nodes and at every face node, the normals and
+// |grad xi| are tabulated, the jump's flux is contracted with the normal at once
+// (27 FMAs; with the general metric's flux and a constant flat metric it was 170
+// slots), and the face sums go axis by axis.  Two CTAs an SM at P = 5 (P <= 4: three
+// or four), also with the metric, which had one and idled at its barriers.
+// 7146 elements of orders 4 and 5: substep 1.42 -> 0.97 ms; Kerr-Schild, 1536
+// elements: 0.89 -> 0.77 ms.  Batched contexts launch each order's elements separately, in
+// CTAs sized for that order (one kernel dispatching on the order would keep every
+// order's registers live and spill).
 template <int P, int SUB, bool KS>
-__global__ void __launch_bounds__(DGC<P>::NT, KS ? 1 : (DGC<P>::NT <= 128 ? 4 : 2))
-    k_dg_curved(Dev d, SubArgs a, const int* list, int ci) {
+__global__ void __launch_bounds__(DGC<P, KS>::NT, DGC<P, KS>::CTAS) k_dg_curved(Dev d, SubArgs a, const int* list, int ci) {
     extern __shared__ double sm[];
     const int nwork = d.counts[ci];
-    for (int w = blockIdx.x; w < nwork; w += gridDim.x) dg_curved_elem<P, DGC<P>::NT, SUB, KS>(d, a, list[w], sm);
+    for (int w = blockIdx.x; w < nwork; w += gridDim.x) dg_curved_elem<P, DGC<P, KS>::NT, SUB, KS>(d, a, list[w], sm);
 }
 
 template <int P, bool KS, int SUB>
 static void curved_launch(const Dev& d, const SubArgs& a, const int* list, int ci, int grid, cudaStream_t st) {
-    using K = DGC<P>;
+    using K = DGC<P, KS>;
     cudaFuncSetAttribute(k_dg_curved<P, SUB, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM);
     k_dg_curved<P, SUB, KS><<<grid, K::NT, K::SMEM, st>>>(d, a, list, ci);
     g_launch_counter += 1;
