@@ -389,89 +389,81 @@ __device__ __forceinline__ void rusanov_pair(double La, double Ra, double Sa, do
     }
 }
 
-// Reverse mode of weno5z_combine for indicators B_k (eps included) and
-// candidates p_k: from the value's adjoint yb, the candidates' adjoints pb_k
-// and the indicators' adjoints Bb_k.  With A_k = d_k s_k P_k, s_k = b_k^2 +
-// t^2, t = b_0 - b_2, P_k the product of the other two b_j^2, d = (1, 10, 5)
-// and W_k = d_k dL/dA_k = d_k yb (p_k - value) / sum A:
+// Reverse mode of the two face values of a cell (Weno5zLine, WENO5-Z): from the
+// adjoints yl, yr of its left and right value, the adjoints of the window's
+// differences and scaled second differences (h = a/8), added to them:
+// hb0..hb2 (of h at c-1, c, c+1), dAb, dBb (of the differences left and right
+// of c); the centre value's adjoint is yl + yr.  With S_k = (b_k^2 + t^2) P_k,
+// t = b_0 - b_2, P_k the product of the other two b_j^2, and W_k = dL/dS_k summed
+// over both values (y d_k (g_k - value) / sum A):
 //   dL/db_0 = 2 (t T + b_0 (W_0 P_0 + W_1 s_1 b_2^2 + W_2 s_2 b_1^2)),
 //   dL/db_1 = 2 b_1 (W_0 s_0 b_2^2 + W_1 P_1 + W_2 s_2 b_0^2),
 //   dL/db_2 = 2 (-t T + b_2 (W_0 s_0 b_1^2 + W_1 s_1 b_0^2 + W_2 P_2)),
-// T = sum_k W_k P_k.  The weights are homogeneous of degree 0 in the b_k, so
-// the B_k are first scaled exactly by the power of two of their maximum; the
-// A_k are then O(1) and their derivatives stay in range.
-__device__ __forceinline__ void weno5z_combine_vjp(double B0, double B1, double B2, double p0, double p1, double p2,
-                                                   double yb, double& pb0, double& pb1, double& pb2, double& Bb0,
-                                                   double& Bb1, double& Bb2) {
-    const double sc = pow2_inv_scale(fmax(B0, fmax(B1, B2)));
-    const double b0 = B0 * sc, b1 = B1 * sc, b2 = B2 * sc;
-    const double t = b0 - b2, t2 = t * t;
-    const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
-    const double s0 = q0 + t2, s1 = q1 + t2, s2 = q2 + t2;
-    const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1;
-    const double A0 = s0 * P0, A1 = 10.0 * (s1 * P1), A2 = 5.0 * (s2 * P2);
-    const double iS = recip_nr(A0 + A1 + A2);
-    const double val = fma(A0, p0, fma(A1, p1, A2 * p2)) * iS;
-    const double y = yb * iS;
-    pb0 = y * A0;
-    pb1 = y * A1;
-    pb2 = y * A2;
-    const double W0 = y * (p0 - val), W1 = (10.0 * y) * (p1 - val), W2 = (5.0 * y) * (p2 - val);
-    const double W0P0 = W0 * P0, W0s0 = W0 * s0, W1s1 = W1 * s1, W2s2 = W2 * s2;
-    const double T = fma(W1, P1, fma(W2, P2, W0P0));
-    const double X0 = fma(W1s1, q2, fma(W2s2, q1, W0P0));
-    const double X1 = fma(W0s0, q2, fma(W2s2, q0, W1 * P1));
-    const double X2 = fma(W0s0, q1, fma(W1s1, q0, W2 * P2));
-    const double sc2 = 2.0 * sc;
-    Bb0 = sc2 * fma(t, T, b0 * X0);
-    Bb1 = sc2 * (b1 * X1);
-    Bb2 = sc2 * fma(-t, T, b2 * X2);
-}
-
-// Reverse mode of weno5z_pair: g[i] += ybL d uL/d v_i + ybR d uR/d v_i,
-// i = 0..5, through the shared candidates and second differences (same
-// first-difference form and 4x-scaled indicators as the forward pair).
-__device__ __forceinline__ void weno5z_pair_vjp(double v0, double v1, double v2, double v3, double v4, double v5,
-                                                double eps, double ybL, double ybR, double* g) {
-    const double d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3, d45 = v5 - v4;
-    const double p123 = fma(0.125, d12, fma(0.375, d23, v2));
-    const double p234 = fma(0.625, d23, fma(-0.125, d34, v2));
-    const double pL0 = fma(-0.375, d01, fma(0.875, d12, v2));
-    const double pR0 = fma(-0.875, d34, fma(0.375, d45, v3));
-    const double a012 = d12 - d01, a123 = d23 - d12, a234 = d34 - d23, a345 = d45 - d34;
-    const double eL0 = fma(2.0, d12, a012), eL1 = d12 + d23, eL2 = fma(-2.0, d23, a234);
-    const double eR0 = fma(-2.0, d34, a345), eR1 = d23 + d34, eR2 = fma(2.0, d23, a123);
-    const double c = 13.0 / 3.0, eps4 = 4.0 * eps;
-    const double k123 = (c * a123) * a123, k234 = (c * a234) * a234;
-    const double BL0 = fma(c * a012, a012, fma(eL0, eL0, eps4));
-    const double BL1 = k123 + fma(eL1, eL1, eps4);
-    const double BL2 = k234 + fma(eL2, eL2, eps4);
-    const double BR0 = fma(c * a345, a345, fma(eR0, eR0, eps4));
-    const double BR1 = k234 + fma(eR1, eR1, eps4);
-    const double BR2 = k123 + fma(eR2, eR2, eps4);
-    double pbL0, pbL1, pbL2, BbL0, BbL1, BbL2, pbR0, pbR1, pbR2, BbR0, BbR1, BbR2;
-    weno5z_combine_vjp(BL0, BL1, BL2, pL0, p123, p234, ybL, pbL0, pbL1, pbL2, BbL0, BbL1, BbL2);
-    weno5z_combine_vjp(BR0, BR1, BR2, pR0, p234, p123, ybR, pbR0, pbR1, pbR2, BbR0, BbR1, BbR2);
-    // adjoints of the shared and one-sided intermediates (B = c a^2 + e^2 + 4 eps)
-    const double p123b = pbL1 + pbR2, p234b = pbL2 + pbR1;
-    const double c2 = 2.0 * c;
-    const double a012b = c2 * a012 * BbL0, a345b = c2 * a345 * BbR0;
-    const double a123b = c2 * a123 * (BbL1 + BbR2), a234b = c2 * a234 * (BbL2 + BbR1);
-    const double eL0b = 2.0 * eL0 * BbL0, eL1b = 2.0 * eL1 * BbL1, eL2b = 2.0 * eL2 * BbL2;
-    const double eR0b = 2.0 * eR0 * BbR0, eR1b = 2.0 * eR1 * BbR1, eR2b = 2.0 * eR2 * BbR2;
-    // to the cells: p123 = (-v1 + 6 v2 + 3 v3)/8, p234 = (3 v2 + 6 v3 - v4)/8,
-    // pL0 = (3 v0 - 10 v1 + 15 v2)/8, pR0 = (15 v3 - 10 v4 + 3 v5)/8,
-    // eL0 = v0 - 4 v1 + 3 v2, eL1 = v3 - v1, eL2 = 3 v2 - 4 v3 + v4,
-    // eR0 = 3 v3 - 4 v4 + v5, eR1 = v4 - v2, eR2 = v1 - 4 v2 + 3 v3
-    g[0] += fma(0.375, pbL0, a012b + eL0b);
-    g[1] += fma(-1.25, pbL0, fma(-0.125, p123b, fma(-2.0, a012b, fma(-4.0, eL0b, a123b - eL1b + eR2b))));
-    g[2] += fma(1.875, pbL0, fma(0.75, p123b, fma(0.375, p234b, fma(-2.0, a123b, fma(3.0, eL0b + eL2b,
-               fma(-4.0, eR2b, a012b + a234b - eR1b))))));
-    g[3] += fma(0.375, p123b, fma(0.75, p234b, fma(1.875, pbR0, fma(-2.0, a234b, fma(3.0, eR0b + eR2b,
-               fma(-4.0, eL2b, a123b + a345b + eL1b))))));
-    g[4] += fma(-0.125, p234b, fma(-1.25, pbR0, fma(-2.0, a345b, fma(-4.0, eR0b, a234b + eL2b + eR1b))));
-    g[5] += fma(0.375, pbR0, a345b + eR0b);
-}
+// T = sum_k W_k P_k, s_k = b_k^2 + t^2.  The weights are homogeneous of degree 0 in
+// the b_k, so these are first scaled exactly by the power of two of their maximum;
+// the S_k are then O(1) and their derivatives stay in range.
+struct Weno5zLineVjp {
+    double dA, dB, hA, hB, kA, kB, vn, eps;
+    __device__ __forceinline__ double curv(double h) const { return fma((13.0 / 12.0 * 64.0) * h, h, eps); }
+    __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double weno_eps) {
+        eps = fmax(weno_eps, 1e-51);
+        const double d01 = v1 - v0;
+        dA = v2 - v1;
+        dB = v3 - v2;
+        hA = 0.125 * (dA - d01);
+        hB = 0.125 * (dB - dA);
+        kA = curv(hA);
+        kB = curv(hB);
+        vn = v3;
+    }
+    __device__ __forceinline__ void cell(double v4, double yl, double yr, double& hb0, double& hb1, double& hb2, double& dAb,
+                                         double& dBb) {
+        const double dC = v4 - vn, hC = 0.125 * (dC - dB), kC = curv(hC);
+        const double e0 = fma(4.0, hA, dA), e1 = fma(4.0, hB, dA), e2 = fma(-4.0, hC, dB);
+        const double c0 = fma(e0, e0, kA), c1 = fma(e1, e1, kB), c2 = fma(e2, e2, kC);
+        // positive: ordered as integers
+        const double sc = pow2_inv_scale(__longlong_as_double((long long)umax(fbits(c0), umax(fbits(c1), fbits(c2)))));
+        const double b0 = c0 * sc, b1 = c1 * sc, b2 = c2 * sc;
+        const double t = b0 - b2, t2 = t * t;
+        const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
+        const double s0 = q0 + t2, s1 = q1 + t2, s2 = q2 + t2;
+        const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1;
+        const double S0 = s0 * P0, S1 = 10.0 * (s1 * P1), S2 = s2 * P2;
+        // right value: weights (1, 10, 5), g = h + e/2; left value: (5, 10, 1), h - e/2
+        const double T2 = 5.0 * S2, T0 = 5.0 * S0;
+        const double iR = recip_nr((S0 + S1) + T2), iL = recip_nr((T0 + S1) + S2);
+        const double r0 = fma(0.5, e0, hA), r1 = fma(0.5, e1, hB), r2 = fma(0.5, e2, hC);
+        const double l0 = fma(-0.5, e0, hA), l1 = fma(-0.5, e1, hB), l2 = fma(-0.5, e2, hC);
+        const double vr = fma(S0, r0, fma(S1, r1, T2 * r2)) * iR, vl = fma(T0, l0, fma(S1, l1, S2 * l2)) * iL;
+        const double y = yr * iR, z = yl * iL;
+        const double R0 = y * S0, R1 = y * S1, R2 = y * T2, L0 = z * T0, L1 = z * S1, L2 = z * S2;   // of r_k, l_k
+        const double y5 = 5.0 * y, z5 = 5.0 * z;
+        const double W0 = fma(y, r0 - vr, z5 * (l0 - vl));
+        const double W1 = 2.0 * fma(y5, r1 - vr, z5 * (l1 - vl));
+        const double W2 = fma(y5, r2 - vr, z * (l2 - vl));
+        const double W0P0 = W0 * P0, W0s0 = W0 * s0, W1s1 = W1 * s1, W2s2 = W2 * s2;
+        const double T = fma(W1, P1, fma(W2, P2, W0P0));
+        const double X0 = fma(W1s1, q2, fma(W2s2, q1, W0P0));
+        const double X1 = fma(W0s0, q2, fma(W2s2, q0, W1 * P1));
+        const double X2 = fma(W0s0, q1, fma(W1s1, q0, W2 * P2));
+        const double sc2 = 2.0 * sc;
+        const double B0 = sc2 * fma(t, T, b0 * X0), B1 = sc2 * (b1 * X1), B2 = sc2 * fma(-t, T, b2 * X2);
+        // b = e^2 + K h^2 + eps: to e (slopes) and h
+        const double E0 = fma(2.0 * e0, B0, 0.5 * (R0 - L0));
+        const double E1 = fma(2.0 * e1, B1, 0.5 * (R1 - L1));
+        const double E2 = fma(2.0 * e2, B2, 0.5 * (R2 - L2));
+        constexpr double K2 = 13.0 / 12.0 * 128.0;
+        hb0 += fma(K2 * hA, B0, fma(4.0, E0, R0 + L0));
+        hb1 += fma(K2 * hB, B1, fma(4.0, E1, R1 + L1));
+        hb2 += fma(K2 * hC, B2, fma(-4.0, E2, R2 + L2));
+        dAb += E0 + E1;
+        dBb += E2;
+        dA = dB; dB = dC;
+        hA = hB; hB = hC;
+        kA = kB; kB = kC;
+        vn = v4;
+    }
+};
 
 // face fi of direction k: position m along k, tangential (ta, tb); false past the element's faces
 __device__ __forceinline__ bool face_coords(int64_t fi, int nc, int& m, int& ta, int& tb) {

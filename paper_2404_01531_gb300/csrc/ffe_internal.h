@@ -221,9 +221,10 @@ double launch_fma_probe(int nsm, int iters, cudaStream_t st, float* ms);
 void launch_constraints(const Dev& d, Field U, double* part, int blocks, cudaStream_t st);
 void launch_l2_err(const Dev& d, Field U, Field R, int v0, int nv, double* part, int blocks, cudaStream_t st);
 // out += (d RHS_FD/dU)^T L (kernels_adjoint_fd.cu); extb: scratch of the size of d.ext
-// FD elements per chunk of the FD reverse mode (its per-face buffer gb holds
-// [3][12][FDV_CHUNK][(nc+1) nc^2][6] doubles)
+// FD elements per chunk of the FD reverse mode, and the doubles of its scratch gb
+// for a chunk
 constexpr int FDV_CHUNK = 1024;
+size_t fdv_scratch(const Dev& d, int chunk);
 void launch_fd_rhs_vjp(const Dev& d, Field U, Field J, Field L, Field out, double* extb, double* gb,
                        double* omega_bar, cudaStream_t st);
 void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field F2, Field F3,

@@ -367,7 +367,7 @@ struct ffe_ctx {
     AdjArgs adj{};
     bool adj_fd = false;             // the current mask has FD elements
     double* d_extb = nullptr;        // extended-block adjoint of one FD chunk
-    double* d_gbuf = nullptr;        // per-face contributions to it (FD reverse mode)
+    double* d_gbuf = nullptr;        // scratch of the FD reverse mode (fdv_scratch)
     double* d_omega_bar = nullptr;
     double* d_cons = nullptr;        // per-block partials of ffe_constraints
     double* d_ref = nullptr;         // analytic initial data (reference of the L2 error), state layout
@@ -2342,7 +2342,7 @@ static ffe_status adjoint_ready(ffe_ctx* c) {
     if ((s = dalloc(c, &c->d_extb, (size_t)12 * d.chunk * ne * ne * ne))) return s;
     if ((s = dalloc(c, &c->d.ftr_b, (size_t)d.fd_cap * 6 * 12 * d.np1 * d.np1))) return s;
     const size_t fch = (size_t)(d.chunk < FDV_CHUNK ? d.chunk : FDV_CHUNK);
-    if ((s = dalloc(c, &c->d_gbuf, (size_t)3 * 12 * fch * (d.nc + 1) * d.nc * d.nc * 6))) return s;
+    if ((s = dalloc(c, &c->d_gbuf, fdv_scratch(d, (int)fch)))) return s;
     c->adj_ready = true;
     return FFE_OK;
 }
