@@ -4,6 +4,8 @@
 #pragma once
 #include "ffe_internal.h"
 #include "fp64util.cuh"
+#include "physics.cuh"
+#include "physics_gen.cuh"
 #include "shellmap.cuh"
 
 namespace ffe {
@@ -464,6 +466,22 @@ struct Weno5zLineVjp {
         vn = v4;
     }
 };
+
+// J~ (drift, full) at cell c of FD element e
+__device__ __forceinline__ void current_fd_cell(const Dev& d, int e, int c, const Field& U, const Field& J) {
+    if (d.mask[e] != 1 || c >= esz(d, e).ncell) return;
+    const int64_t p = fdb(d, e) + c;
+    double u[NV], jd[3], jf[3];
+    for (int v = 0; v < NV; ++v) u[v] = U.fd(v)[p];
+    if (d.ks) {
+        PM m;
+        load_pm(d.metfd, (int64_t)d.E * d.ncell, (int64_t)e * d.ncell + c, m);
+        current_gen(u, m, d.eta, jd, jf);
+    } else {
+        current_flat(u, d.eta, jd, jf);
+    }
+    for (int k = 0; k < 3; ++k) { J.fd(k)[p] = jd[k]; J.fd(3 + k)[p] = jf[k]; }
+}
 
 // face fi of direction k: position m along k, tangential (ta, tb); false past the element's faces
 __device__ __forceinline__ bool face_coords(int64_t fi, int nc, int& m, int& ta, int& tb) {

@@ -167,7 +167,7 @@ struct Dev {
     double* ext;
     double* flux;
     // FD->DG face traces of FD elements for their DG neighbours, per FD slot
-    // [6][12][np1^2] (k_fd_traces; null: none), and their adjoints in the
+    // [6][12][np1^2] (face_trace), and their adjoints in the
     // reverse mode (written by the DG reverse kernel, allocated with the adjoint)
     double* ftr;
     double* ftr_b;
@@ -197,8 +197,10 @@ __device__ __forceinline__ SolveK solve_k(const Dev& d, int e) { return d.einst 
 __device__ __forceinline__ double omega_of(const Dev& d, int e) { return d.einst ? d.inst[d.einst[e]].omega : d.omega; }
 
 // kernel launchers (kernels_*.cu); all enqueue on `st`
-void launch_build_lists(const Dev& d, cudaStream_t st);
-void launch_current(const Dev& d, Field U, Field J, const int* list_or_null, int which_count, cudaStream_t st);
+// clear: also the flag count, or what a step starts from (flag and near counts, switched)
+enum ListsClear : int { LISTS_ONLY = 0, LISTS_FLAGS = 1, LISTS_STEP = 2 };
+void launch_build_lists(const Dev& d, cudaStream_t st, int clear = LISTS_ONLY);
+void launch_current(const Dev& d, Field U, Field J, cudaStream_t st);
 void launch_stage12(const Dev& d, Field un, Field Ua, Field G1, Field G2, Field J, cudaStream_t st);
 // Jout: J~ of the substep's result (flat metric; unused on the Kerr-Schild background)
 void launch_dg_substep(const Dev& d, int sub, Field Uin, Field J, Field un, Field F2, Field F3,
@@ -208,13 +210,12 @@ void launch_fd_substep(const Dev& d, int sub, const int* list, int count_index, 
                        Field un, Field F2, Field F3, Field G1, Field G2, Field G3, Field G4,
                        Field Fout, Field Uout, Field Gout, Field Jout, cudaStream_t st, bool faces = false);
 int fd_chunks(const Dev& d);
-// FD->DG face traces of the listed FD elements for their DG neighbours (Dev::ftr)
-void launch_fd_traces(const Dev& d, Field U, Field J, cudaStream_t st);
-// out += the FD cells' share of the trace adjoints (Dev::ftr_b), reverse of k_fd_traces
+// out += the FD cells' share of the trace adjoints (Dev::ftr_b), reverse of face_trace
 void launch_fd_traces_vjp(const Dev& d, Field U, Field out, cudaStream_t st);
-// extended blocks (U, J~ with ghosts) of the listed FD elements of one chunk
+// extended blocks (U, J~ with ghosts) of the listed FD elements of one chunk and,
+// with traces, their FD->DG face traces for their DG neighbours (Dev::ftr)
 void launch_fd_fill(const Dev& d, const int* list, int count_index, int w0, Field U, Field J, cudaStream_t st,
-                    bool residues = false);
+                    bool residues = false, bool traces = false);
 void launch_eval_recip(const double* x, double* y, int64_t n, cudaStream_t st);
 // register-only DFMA loop: returns its flops, *ms its event-timed duration
 double launch_fma_probe(int nsm, int iters, cudaStream_t st, float* ms);
@@ -227,7 +228,7 @@ constexpr int FDV_CHUNK = 1024;
 size_t fdv_scratch(const Dev& d, int chunk);
 void launch_fd_rhs_vjp(const Dev& d, Field U, Field J, Field L, Field out, double* extb, double* gb,
                        double* omega_bar, cudaStream_t st);
-void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field F2, Field F3,
+void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field J, Field F2, Field F3,
                              Field G1, Field G2, Field G3, Field G4, cudaStream_t st);
 void launch_fd2dg(const Dev& d, Field un, cudaStream_t st);
 void launch_tci_ratio(const Dev& d, const double* Udg, double* ratio, cudaStream_t st);

@@ -868,9 +868,7 @@ ffe_status fill_dirichlet(ffe_ctx* c) {
 // One IMEX-SSP3(4,3,3) step with the hybrid control loop, enqueued on st.
 void enqueue_step(ffe_ctx* c, cudaStream_t st) {
     const Dev& d = c->d;
-    cudaMemsetAsync(d.counts + 2, 0, 2 * sizeof(int), st);
-    cudaMemsetAsync(d.switched, 0, d.E, st);
-    launch_build_lists(d, st);
+    launch_build_lists(d, st, LISTS_STEP);
     if (d.ks) launch_stage12_ks(d, c->un, c->Ua, c->G1, c->G2, st);
     else launch_stage12(d, c->un, c->Ua, c->G1, c->G2, c->J, st);
     // J~ of each substep's input: left by the stage before it (flat metric) in one
@@ -881,22 +879,24 @@ void enqueue_step(ffe_ctx* c, cudaStream_t st) {
                        {SUB_C, c->Ua, c->J, c->Fs, c->un, c->G4, c->J2}};
     for (const S& s : subs) {
         const Field J = d.ks ? c->J : s.J;
-        if (d.ks && d.metfd) launch_current(d, s.Uin, J, nullptr, 0, st);
+        // FD elements first: their face traces are the exterior states of DG neighbours.
+        // (No FD elements on a Kerr-Schild background without its FD metric tables.)
+        const bool fd = !d.ks || d.metfd;
+        if (d.ks && fd) launch_current(d, s.Uin, J, st);
+        if (fd)
+            launch_fd_substep(d, s.sub, d.fd_list, 1, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
+                              s.Uout, s.Gout, s.Jout, st);
         if (d.curved)
             launch_dg_substep_curved(d, s.sub, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
                                      s.Uout, s.Gout, s.Jout, st);
         else
             launch_dg_substep(d, s.sub, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout, s.Uout,
                               s.Gout, s.Jout, st);
-        launch_fd_substep(d, s.sub, d.fd_list, 1, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, s.Fout,
-                          s.Uout, s.Gout, s.Jout, st);
         if (d.tci_on) {
-            launch_rollback_project(d, s.sub, c->un, s.Uin, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, st);
-            launch_current(d, s.Uin, J, d.flag_list, 2, st);
+            launch_rollback_project(d, s.sub, c->un, s.Uin, J, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, st);
             launch_fd_substep(d, s.sub, d.flag_list, 2, s.Uin, J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4,
                               s.Fout, s.Uout, s.Gout, s.Jout, st);
-            cudaMemsetAsync(d.counts + 2, 0, sizeof(int), st);
-            launch_build_lists(d, st);
+            launch_build_lists(d, st, LISTS_FLAGS);
         }
     }
     if (d.tci_on) launch_fd2dg(d, c->un, st);
@@ -915,7 +915,7 @@ ffe_status autotune(ffe_ctx* c) {
     CK(cudaEventCreate(&a));
     CK(cudaEventCreate(&b));
     launch_build_lists(d, c->st);
-    if (!d.ks || d.metfd) launch_current(d, c->un, c->J, nullptr, 0, c->st);
+    if (!d.ks || d.metfd) launch_current(d, c->un, c->J, c->st);
     int* slots[3] = {&d.dg_grid, &d.dg_grid_lo, &d.dg_grid_lo2};
     const int nord = c->batch ? 3 : 1;
     for (int o = 0; o < nord; ++o) {
@@ -2146,14 +2146,16 @@ ffe_status ffe_rhs(ffe_ctx* c, const double* U_dev, double* dUdt_dev) try {
     const Dev& d = c->d;
     Field U{(double*)U_dev, NV, d.ndg, d.nfd}, R{dUdt_dev, NV, d.ndg, d.nfd};
     launch_build_lists(d, c->st);
-    launch_current(d, U, c->J, nullptr, 0, c->st);
+    launch_current(d, U, c->J, c->st);
+    if (!d.ks || d.metfd)
+        launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1,
+                          c->J2, c->st);
     if (d.curved)
         launch_dg_substep_curved(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1,
                                  c->J2, c->st);
     else
-        launch_dg_substep(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1, c->J2, c->st);
-    launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R,
-                      c->G1, c->J2, c->st);
+        launch_dg_substep(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, R, R, c->G1, c->J2,
+                          c->st);
     CK(cudaGetLastError());
     return FFE_OK;
 } catch (...) {
@@ -2381,12 +2383,12 @@ static ffe_status filter_or_copy(ffe_ctx* c, Field in, Field out, int transpose)
 // right-hand side of the hybrid operator at U (fixed mask)
 static void rhs_at(ffe_ctx* c, Field U, Field out) {
     const Dev& d = c->d;
-    launch_current(d, U, c->J, nullptr, 0, c->st);
-    launch_dg_substep_curved(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out, c->G1,
-                             c->J2, c->st);
+    launch_current(d, U, c->J, c->st);
     if (c->adj_fd)
         launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out,
                           c->G1, c->J2, c->st, true);
+    launch_dg_substep_curved(d, SUB_RHS, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out, c->G1,
+                             c->J2, c->st);
 }
 
 // out = (d RHS/dU)^T L at U for the hybrid operator (fixed mask)
@@ -2396,7 +2398,7 @@ static void rhs_vjp_at(ffe_ctx* c, Field U, Field L, Field out) {
     launch_rhs_vjp(d, U, L, out, c->d_omega_bar, c->st);
     if (c->adj_fd) {
         launch_fd_traces_vjp(d, U, out, c->st);
-        launch_current(d, U, c->J, nullptr, 0, c->st);
+        launch_current(d, U, c->J, c->st);
         launch_fd_rhs_vjp(d, U, c->J, L, out, c->d_extb, c->d_gbuf, c->d_omega_bar, c->st);
     }
 }

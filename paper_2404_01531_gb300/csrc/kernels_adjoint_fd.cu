@@ -460,7 +460,7 @@ __global__ void k_fdv_ghosts(Dev d, const int* list, int ci, int w0, Field U, Fi
     }
 }
 
-// Reverse of k_fd_traces: the adjoints the DG reverse mode left at the trace
+// Reverse of face_trace: the adjoints the DG reverse mode left at the trace
 // nodes of FD faces with a DG neighbour (Dev::ftr_b, [slot][6][12][np1^2]) go
 // back through the transposed sum-factorised FD->DG projection -- the two
 // tangential directions, then the normal one -- to the 6 cell layers next to

@@ -129,7 +129,7 @@ __device__ __forceinline__ bool curved_external(const Dev& d, const SubArgs& a, 
         // FD->DG projection (6-point stencils) of the neighbour's cells and of
         // their current J~ (the current of a projected state would carry its
         // projection error in E~.B~ amplified by eta into the q~ flux), from the face
-        // traces k_fd_traces left for it, indexed along the neighbour's own face axes
+        // traces face_trace left for it, indexed along the neighbour's own face axes
         const int f2 = d.nbr_face[e * 6 + f], d2 = f2 >> 1;
         const int u1 = d2 == 0 ? 1 : 0, u2 = d2 == 2 ? 1 : 2;
         const int nfm = d.np1 * d.np1;
@@ -494,7 +494,6 @@ void launch_dg_substep_curved(const Dev& d, int sub, Field Uin, Field J, Field u
                               Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
                               cudaStream_t st) {
     SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout, Jout};
-    if (!d.ks || d.metfd) launch_fd_traces(d, Uin, J, st);
     prof_begin(sub == SUB_RHS ? "dg_rhs_curved" : "dg_substep_curved", st);
     if (d.ks) {
         switch (d.P) {

@@ -39,73 +39,96 @@ struct DGK {
 };
 
 // ---------------------------------------------------------------------------
+// Work lists of the mask: FD elements and, per order, DG elements.
+__device__ __forceinline__ int list_of(const Dev& d, int e, int** list) {
+    if (d.mask[e] != 0) { *list = d.fd_list; return 1; }
+    if (!d.dg_list_lo || elem_P(d, e) == d.P) { *list = d.dg_list; return 0; }
+    if (elem_P(d, e) == d.P - 1) { *list = d.dg_list_lo; return 6; }
+    *list = d.dg_list_lo2;
+    return 7;
+}
+
 __global__ void k_build_lists(Dev d) {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= d.E) return;
-    if (d.mask[e] != 0) d.fd_list[atomicAdd(&d.counts[1], 1)] = e;
-    else if (!d.dg_list_lo || elem_P(d, e) == d.P) d.dg_list[atomicAdd(&d.counts[0], 1)] = e;
-    else if (elem_P(d, e) == d.P - 1) d.dg_list_lo[atomicAdd(&d.counts[6], 1)] = e;
-    else d.dg_list_lo2[atomicAdd(&d.counts[7], 1)] = e;
+    int* list;
+    const int c = list_of(d, e, &list);
+    list[atomicAdd(&d.counts[c], 1)] = e;
 }
 
-void launch_build_lists(const Dev& d, cudaStream_t st) {
-    cudaMemsetAsync(d.counts, 0, 2 * sizeof(int), st);
-    if (d.dg_list_lo) cudaMemsetAsync(d.counts + 6, 0, 2 * sizeof(int), st);
+// The same in one CTA, which clears the counters itself.
+__global__ void __launch_bounds__(1024) k_build_lists_small(Dev d, int clear) {
+    __shared__ int n[8];
+    if (threadIdx.x < 8) n[threadIdx.x] = 0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < d.E; e += blockDim.x) {
+        int* list;
+        const int c = list_of(d, e, &list);
+        list[atomicAdd(&n[c], 1)] = e;
+        if (clear & LISTS_STEP) d.switched[e] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        d.counts[0] = n[0];
+        d.counts[1] = n[1];
+        if (d.dg_list_lo) {
+            d.counts[6] = n[6];
+            d.counts[7] = n[7];
+        }
+        if (clear & (LISTS_FLAGS | LISTS_STEP)) d.counts[2] = 0;
+        if (clear & LISTS_STEP) d.counts[3] = 0;
+    }
+}
+
+// One CTA up to 8192 elements: 8 loads in a row per thread cost less than the two
+// to five clears that the grid version needs before it (each a node of its own in
+// a step's graph).
+void launch_build_lists(const Dev& d, cudaStream_t st, int clear) {
+    const bool small = d.E <= 8192;
+    if (!small) {
+        cudaMemsetAsync(d.counts, 0, 2 * sizeof(int), st);
+        if (d.dg_list_lo) cudaMemsetAsync(d.counts + 6, 0, 2 * sizeof(int), st);
+        if (clear & LISTS_STEP) {
+            cudaMemsetAsync(d.counts + 2, 0, 2 * sizeof(int), st);
+            cudaMemsetAsync(d.switched, 0, d.E, st);
+        } else if (clear & LISTS_FLAGS) {
+            cudaMemsetAsync(d.counts + 2, 0, sizeof(int), st);
+        }
+    }
     prof_begin("build_lists", st);
-    k_build_lists<<<(d.E + 255) / 256, 256, 0, st>>>(d);
+    if (small) k_build_lists_small<<<1, 1024, 0, st>>>(d, clear);
+    else k_build_lists<<<(d.E + 255) / 256, 256, 0, st>>>(d);
     prof_end(st);
     g_launch_counter += 1;
 }
 
 // ---------------------------------------------------------------------------
 // J~ (drift, full) at every DG node of DG elements and at the cells of the FD
-// list (counts[1], as built by k_build_lists); with a list, only the FD cells
-// of the listed elements.
-__global__ void k_current(Dev d, Field U, Field J, const int* list, int count_index) {
+// list (counts[1], as built by k_build_lists).
+__global__ void k_current(Dev d, Field U, Field J) {
     int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    if (list == nullptr) {
-        for (int64_t p = tid; p < d.ndg; p += stride) {
-            const int e = (int)(p / d.nn);
-            if (d.mask[e] != 0 || (int)(p % d.nn) >= esz(d, e).nn) continue;
-            double u[NV], jd[3], jf[3];
-            for (int v = 0; v < NV; ++v) u[v] = U.dg(v)[p];
-            if (d.ks) {
-                PM m;
-                load_pm(d.met, d.ndg, p, m);
-                current_gen(u, m, d.eta, jd, jf);
-            } else {
-                current_flat(u, d.eta, jd, jf);
-            }
-            for (int c = 0; c < 3; ++c) { J.dg(c)[p] = jd[c]; J.dg(3 + c)[p] = jf[c]; }
+    for (int64_t p = tid; p < d.ndg; p += stride) {
+        const int e = (int)(p / d.nn);
+        if (d.mask[e] != 0 || (int)(p % d.nn) >= esz(d, e).nn) continue;
+        double u[NV], jd[3], jf[3];
+        for (int v = 0; v < NV; ++v) u[v] = U.dg(v)[p];
+        if (d.ks) {
+            PM m;
+            load_pm(d.met, d.ndg, p, m);
+            current_gen(u, m, d.eta, jd, jf);
+        } else {
+            current_flat(u, d.eta, jd, jf);
         }
-        list = d.fd_list;
-        count_index = 1;
+        for (int c = 0; c < 3; ++c) { J.dg(c)[p] = jd[c]; J.dg(3 + c)[p] = jf[c]; }
     }
-    {
-        const int n = d.counts[count_index];
-        for (int64_t q = tid; q < (int64_t)n * d.ncell; q += stride) {
-            const int e = list[q / d.ncell];
-            const int c = (int)(q % d.ncell);
-            if (d.mask[e] != 1 || c >= esz(d, e).ncell) continue;
-            const int64_t p = fdb(d, e) + c;
-            double u[NV], jd[3], jf[3];
-            for (int v = 0; v < NV; ++v) u[v] = U.fd(v)[p];
-            if (d.ks) {
-                PM m;
-                load_pm(d.metfd, (int64_t)d.E * d.ncell, (int64_t)e * d.ncell + c, m);
-                current_gen(u, m, d.eta, jd, jf);
-            } else {
-                current_flat(u, d.eta, jd, jf);
-            }
-            for (int c2 = 0; c2 < 3; ++c2) { J.fd(c2)[p] = jd[c2]; J.fd(3 + c2)[p] = jf[c2]; }
-        }
-    }
+    const int64_t n = (int64_t)d.counts[1] * d.ncell;
+    for (int64_t q = tid; q < n; q += stride) current_fd_cell(d, d.fd_list[q / d.ncell], (int)(q % d.ncell), U, J);
 }
 
-void launch_current(const Dev& d, Field U, Field J, const int* list, int count_index, cudaStream_t st) {
+void launch_current(const Dev& d, Field U, Field J, cudaStream_t st) {
     prof_begin("current", st);
-    k_current<<<d.nsm * 8, 256, 0, st>>>(d, U, J, list, count_index);
+    k_current<<<d.nsm * 8, 256, 0, st>>>(d, U, J);
     prof_end(st);
     g_launch_counter += 1;
 }
@@ -219,7 +242,7 @@ __device__ void dg_external_state(const Dev& d, const SubArgs& a, int e, int f, 
         // FD neighbour: its FD->DG projection evaluated at this node (6-point
         // stencils), for the state and for its current J~ (the current of the
         // projected state would carry the projection error of E~.B~ times eta),
-        // from the face traces k_fd_traces left for it (same face axes: boxes)
+        // from the face traces face_trace left for it (same face axes: boxes)
         (void)T;
         const int nfm = d.np1 * d.np1;
         const double* tr = d.ftr + ((int64_t)fd_slot_of(d, nb) * 6 + f2) * 12 * nfm + ta + np1 * tb;
@@ -485,7 +508,6 @@ void launch_dg_substep(const Dev& d, int sub, Field Uin, Field J, Field un, Fiel
                        Field G1, Field G2, Field G3, Field G4, Field Fout, Field Uout, Field Gout, Field Jout,
                        cudaStream_t st) {
     SubArgs a{Uin, J, un, F2, F3, G1, G2, G3, G4, Fout, Uout, Gout, Jout};
-    launch_fd_traces(d, Uin, J, st);
     prof_begin(sub == SUB_RHS ? "dg_rhs" : "dg_substep", st);
     switch (d.P) {
         case 2: dg_sub_dispatch<2>(d, sub, a, st); break;

@@ -36,13 +36,69 @@ __device__ __forceinline__ void fill_interior(const Dev& d, int wl, int e, const
     }
 }
 
+// Face trace of an FD element for a DG neighbour (Sec. III.C.2 interface): at
+// every LGL node of face f, if its neighbour is on DG, the FD->DG projection
+// (6-point stencils along each axis) of the element's cells, for U and for its
+// current J~.  A DG element facing an FD neighbour reads its exterior state here
+// instead of projecting 6 x 6 x 6 cells per face node itself (which left most of
+// its block idle).  Layout: per FD slot [6 faces][12 quantities][np1max^2], face
+// node index a + np1 b along the face's axes (axes_of of its normal).  One CTA per
+// (element, face): the projection is sum-factorised -- normal direction straight
+// from the 6 cell layers next to the face, then the two tangential ones through
+// shared memory -- 6 (nc^2 + nc np1 + np1^2) FMAs per quantity instead of 216 per
+// face node.  Ends with a barrier.
+__device__ __forceinline__ void face_trace(const Dev& d, int e, int f, const Field& U, const Field& J, double* sm) {
+    const int nb = d.nbr[e * 6 + f];
+    if (nb < 0 || d.mask[nb] != 0) return;
+    const ES es = esz(d, e);
+    const int np1 = es.np1, nc = es.nc, nc2 = nc * nc, nfm = d.np1 * d.np1;
+    const Tables& T = d.tabs[es.P];
+    const int dd = f >> 1;
+    int t1, t2;
+    axes_of(dd, t1, t2);
+    const int cn = (f & 1) ? es.P : 0;       // the face's LGL index along the normal
+    const int lo = T.f2d_lo[cn];
+    double* A = sm;                            // [12][nc (t2)][nc (t1)]
+    double* B = A + NQ * nc2;                  // [12][nc (t2)][np1 (t1)]
+    const int64_t base = fdb(d, e);
+    const int cs[3] = {1, nc, nc2};
+    for (int t = threadIdx.x; t < NQ * nc2; t += blockDim.x) {
+        const int q = t / nc2, ab = t % nc2;
+        const double* src = (q < NV ? U.fd(q) : J.fd(3 + q - NV)) + base + lo * cs[dd] + (ab % nc) * cs[t1] + (ab / nc) * cs[t2];
+        double acc = 0.0;
+        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[cn][lo + m], src[m * cs[dd]], acc);
+        A[t] = acc;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < NQ * nc * np1; t += blockDim.x) {
+        const int q = t / (nc * np1), r = t % (nc * np1);
+        const int b = r / np1, i = r % np1;
+        const int li = T.f2d_lo[i];
+        double acc = 0.0;
+        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[i][li + m], A[(q * nc + b) * nc + li + m], acc);
+        B[t] = acc;
+    }
+    __syncthreads();
+    double* dst = d.ftr + ((int64_t)fd_slot_of(d, e) * 6 + f) * NQ * nfm;
+    for (int t = threadIdx.x; t < NQ * np1 * np1; t += blockDim.x) {
+        const int q = t / (np1 * np1), r = t % (np1 * np1);
+        const int j = r / np1, i = r % np1;
+        const int lj = T.f2d_lo[j];
+        double acc = 0.0;
+        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[j][lj + m], B[(q * nc + lj + m) * np1 + i], acc);
+        dst[q * nfm + i + np1 * j] = acc;
+    }
+    __syncthreads();
+}
+
 // 6 stencil weights of entry i of a per-slot table
 __device__ __forceinline__ const double* gi_w(const double* table, const Dev& d, int slot, int i) {
     const int per = table == d.gwn ? GH : (table == d.gwr ? d.nc : GH * d.nc);
     return table + 6 * ((int64_t)slot * per + i);
 }
 
-// One CTA per (chunk position, face or interior): fill the extended block.
+// One CTA per (chunk position, face or interior): fill the extended block; with
+// traces, also the element's face traces (both only read U and J~).
 //
 // Ghosts inside a wedge and on boxes are the neighbour's cells, or a DG
 // neighbour's polynomial at its own subcell centres: the neighbour's grid lines
@@ -61,15 +117,20 @@ __device__ __forceinline__ const double* gi_w(const double* table, const Dev& d,
 // polynomial takes three sum-factorised contractions.  With the interior's copy in
 // the same launch, two launches fewer; 300 elements of a shell 1.99 -> 0.20 ms
 // (0.53 with the residues).
-__global__ void k_fd_fill(Dev d, const int* list, int ci, int w0, Field U, Field J, bool residues) {
+__global__ void k_fd_fill(Dev d, const int* list, int ci, int w0, Field U, Field J, bool residues, bool traces) {
     const int n = chunk_n(d, ci, w0);
     const unsigned long long skip = residues ? 0ULL : fbits(1e-10);   // weights up to this are skipped
     extern __shared__ double sm[];
-    for (int item = blockIdx.x; item < n * 7; item += gridDim.x) {
-        const int wl = item / 7, f = item % 7;
+    const int items = traces ? 13 : 7;
+    for (int item = blockIdx.x; item < n * items; item += gridDim.x) {
+        const int wl = item / items, f = item % items;
         const int e = list[w0 + wl];
         if (f == 6) {
             fill_interior(d, wl, e, U, J);
+            continue;
+        }
+        if (f > 6) {
+            face_trace(d, e, f - 7, U, J, sm);
             continue;
         }
         const int gsl = d.gislot ? d.gislot[e * 6 + f] : -1;   // a face between wedges: its weights
@@ -565,10 +626,11 @@ static size_t ghost_smem(const Dev& d) {
     return (size_t)(NQ * d.nn + NQ * GH * d.np1 * d.np1 + NQ * GH * d.nc * d.np1) * sizeof(double);
 }
 
-void launch_fd_fill(const Dev& d, const int* list, int ci, int w0, Field U, Field J, cudaStream_t st, bool residues) {
+void launch_fd_fill(const Dev& d, const int* list, int ci, int w0, Field U, Field J, cudaStream_t st, bool residues,
+                    bool traces) {
     const size_t smem = ghost_smem(d);
     cudaFuncSetAttribute(k_fd_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_fd_fill<<<d.nsm * 4, 256, smem, st>>>(d, list, ci, w0, U, J, residues);
+    k_fd_fill<<<d.nsm * 4, 256, smem, st>>>(d, list, ci, w0, U, J, residues, traces);
     g_launch_counter += 1;
 }
 
@@ -587,7 +649,7 @@ void launch_fd_substep(const Dev& d, int sub, const int* list, int ci, Field Uin
     for (int k = 0, nch = fd_chunks(d); k < nch; ++k) {
         const int w0 = k * d.chunk;
         prof_begin("fd_fill", st);
-        launch_fd_fill(d, list, ci, w0, Uin, J, st, faces);
+        launch_fd_fill(d, list, ci, w0, Uin, J, st, faces, ci == 1);
         prof_end(st);
         prof_begin("fd_flux", st);
         if (faces) {
@@ -617,166 +679,67 @@ void launch_fd_substep(const Dev& d, int sub, const int* list, int ci, Field Uin
 }
 
 // ---------------------------------------------------------------------------
-// Face traces of FD elements for their DG neighbours (Sec. III.C.2 interface):
-// at every LGL node of each face whose neighbour is on DG, the FD->DG
-// projection (6-point stencils along each axis) of the element's cells, for U
-// and for its current J~.  A DG element facing an FD neighbour reads its
-// exterior state here instead of projecting 6 x 6 x 6 cells per face node
-// itself (which left most of its block idle).  Layout: per FD slot [6 faces]
-// [12 quantities][np1max^2], face node index a + np1 b along the face's axes
-// (axes_of of its normal).  One CTA per (element, face): the 6 cell layers
-// next to the face (the normal stencil of a face node) go to shared memory and
-// the projection is sum-factorised -- normal direction, then the two
-// tangential ones -- 6 (nc^2 + nc np1 + np1^2) FMAs per quantity instead of
-// 216 per face node.
-__global__ void k_fd_traces(Dev d, Field U, Field J) {
-    extern __shared__ double sm[];
-    const int n = d.counts[1];
-    const int nfm = d.np1 * d.np1;
-    for (int item = blockIdx.x; item < n * 6; item += gridDim.x) {
-        const int w = item / 6, f = item % 6;
-        const int e = d.fd_list[w];
-        const int nb = d.nbr[e * 6 + f];
-        if (nb < 0 || d.mask[nb] != 0) continue;
-        const ES es = esz(d, e);
-        const int np1 = es.np1, nc = es.nc, nc2 = nc * nc;
-        const Tables& T = d.tabs[es.P];
-        const int dd = f >> 1;
-        int t1, t2;
-        axes_of(dd, t1, t2);
-        const int cn = (f & 1) ? es.P : 0;       // the face's LGL index along the normal
-        const int lo = T.f2d_lo[cn];
-        double* L = sm;                            // [12][6][nc (t2)][nc (t1)]
-        double* A = L + NQ * 6 * nc2;              // [12][nc (t2)][nc (t1)]
-        double* B = A + NQ * nc2;                  // [12][nc (t2)][np1 (t1)]
-        const int64_t base = fdb(d, e);
-        for (int t = threadIdx.x; t < NQ * 6 * nc2; t += blockDim.x) {
-            const int q = t / (6 * nc2), r = t % (6 * nc2);
-            const int nn = r / nc2, ab = r % nc2;
-            int c[3];
-            c[dd] = lo + nn;
-            c[t1] = ab % nc;
-            c[t2] = ab / nc;
-            const double* src = q < NV ? U.fd(q) : J.fd(3 + q - NV);
-            L[t] = src[base + c[0] + nc * (c[1] + nc * c[2])];
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < NQ * nc2; t += blockDim.x) {
-            const int q = t / nc2, ab = t % nc2;
-            double acc = 0.0;
-            for (int m = 0; m < 6; ++m) acc = fma(T.F2D[cn][lo + m], L[(q * 6 + m) * nc2 + ab], acc);
-            A[t] = acc;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < NQ * nc * np1; t += blockDim.x) {
-            const int q = t / (nc * np1), r = t % (nc * np1);
-            const int b = r / np1, i = r % np1;
-            const int li = T.f2d_lo[i];
-            double acc = 0.0;
-            for (int m = 0; m < 6; ++m) acc = fma(T.F2D[i][li + m], A[(q * nc + b) * nc + li + m], acc);
-            B[t] = acc;
-        }
-        __syncthreads();
-        double* dst = d.ftr + ((int64_t)fd_slot_of(d, e) * 6 + f) * NQ * nfm;
-        for (int t = threadIdx.x; t < NQ * np1 * np1; t += blockDim.x) {
-            const int q = t / (np1 * np1), r = t % (np1 * np1);
-            const int j = r / np1, i = r % np1;
-            const int lj = T.f2d_lo[j];
-            double acc = 0.0;
-            for (int m = 0; m < 6; ++m) acc = fma(T.F2D[j][lj + m], B[(q * nc + lj + m) * np1 + i], acc);
-            dst[q * nfm + i + np1 * j] = acc;
-        }
-        __syncthreads();
-    }
-}
-
-void launch_fd_traces(const Dev& d, Field U, Field J, cudaStream_t st) {
-    if (!d.ftr) return;
-    const size_t smem = (size_t)(NQ * 6 * d.nc * d.nc + NQ * d.nc * d.nc + NQ * d.nc * d.np1) * sizeof(double);
-    cudaFuncSetAttribute(k_fd_traces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    prof_begin("fd_traces", st);
-    k_fd_traces<<<d.nsm * 2, 256, smem, st>>>(d, U, J);
-    prof_end(st);
-    g_launch_counter += 1;
-}
-
-// ---------------------------------------------------------------------------
 // DG -> FD projection (tensor Lagrange evaluation at subcell centres) of `nv`
-// variables of element e, from its DG slot to its FD slot.
+// variables of element e, from its DG slot to its FD slot, all at once.
 __device__ void project_dg2fd_element(const Dev& d, const Field& F, int nv, int e, double* sm) {
     const ES es = esz(d, e);
     const Tables& T = d.tabs[es.P];
-    const int np1 = es.np1, nn = es.nn, nc = es.nc;
+    const int np1 = es.np1, nc = es.nc, nb = nc * np1 * np1, ncc = nc * nc * np1;
     const int64_t fb = fdb(d, e);
-    double* a = sm;                     // [np1^3]
-    double* b = a + nn;                 // [np1][np1][nc]
-    double* c = b + nc * np1 * np1;     // [np1][nc][nc]
-    for (int v = 0; v < nv; ++v) {
-        for (int t = threadIdx.x; t < nn; t += blockDim.x) a[t] = F.dg(v)[(int64_t)e * d.nn + t];
-        __syncthreads();
-        for (int t = threadIdx.x; t < nc * np1 * np1; t += blockDim.x) {
-            const int x = t % nc, jk = t / nc;
-            double acc = 0.0;
-            for (int m = 0; m < np1; ++m) acc = fma(T.P2F[x][m], a[m + np1 * jk], acc);
-            b[t] = acc;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < nc * nc * np1; t += blockDim.x) {
-            const int x = t % nc, y = (t / nc) % nc, k = t / (nc * nc);
-            double acc = 0.0;
-            for (int m = 0; m < np1; ++m) acc = fma(T.P2F[y][m], b[x + nc * (m + np1 * k)], acc);
-            c[t] = acc;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < nc * nc * nc; t += blockDim.x) {
-            const int xy = t % (nc * nc), z = t / (nc * nc);
-            double acc = 0.0;
-            for (int m = 0; m < np1; ++m) acc = fma(T.P2F[z][m], c[xy + nc * nc * m], acc);
-            F.fd(v)[fb + t] = acc;
-        }
-        __syncthreads();
+    double* b = sm;                 // [nv][np1][np1][nc]
+    double* c = b + nv * nb;        // [nv][np1][nc][nc]
+    for (int t = threadIdx.x; t < nv * nb; t += blockDim.x) {
+        const int v = t / nb, x = t % nc, jk = (t % nb) / nc;
+        const double* src = F.dg(v) + (int64_t)e * d.nn + np1 * jk;
+        double acc = 0.0;
+        for (int m = 0; m < np1; ++m) acc = fma(T.P2F[x][m], src[m], acc);
+        b[t] = acc;
     }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nv * ncc; t += blockDim.x) {
+        const int v = t / ncc, r = t % ncc, x = r % nc, y = (r / nc) % nc, k = r / (nc * nc);
+        double acc = 0.0;
+        for (int m = 0; m < np1; ++m) acc = fma(T.P2F[y][m], b[v * nb + x + nc * (m + np1 * k)], acc);
+        c[t] = acc;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nv * es.ncell; t += blockDim.x) {
+        const int v = t / es.ncell, r = t % es.ncell, xy = r % (nc * nc), z = r / (nc * nc);
+        double acc = 0.0;
+        for (int m = 0; m < np1; ++m) acc = fma(T.P2F[z][m], c[v * ncc + xy + nc * nc * m], acc);
+        F.fd(v)[fb + r] = acc;
+    }
+    __syncthreads();
 }
 
 struct RollArgs {
     Field f[8];
     int nv[8];
     int nf;
+    Field J;   // J~ of the stage state (f[1])
 };
 
-// Flagged elements: take an FD slot (slot pool), project the substep inputs, mark FD.
+// Flagged elements (the indicator gave each an FD slot): one CTA per (element,
+// field) projects a substep input to the subcells; the one of the stage state also
+// forms J~ there and marks the element FD.
 __global__ void k_rollback_project(Dev d, RollArgs r) {
     extern __shared__ double sm[];
-    __shared__ int s_ok;
     const int n = d.counts[2];
-    for (int w = blockIdx.x; w < n; w += gridDim.x) {
-        const int e = d.flag_list[w];
-        if (threadIdx.x == 0) {
-            s_ok = 1;
-            if (d.fd_slot && d.fd_slot[e] < 0) {
-                const int top = atomicSub(&d.counts[5], 1) - 1;
-                if (top < 0) {
-                    s_ok = 0;   // pool exhausted: reported through the status word
-                    atomicOr(&d.counts[4], 4);
-                } else {
-                    const int sl = d.free_slots[top];
-                    d.fd_slot[e] = sl;
-                    d.slot_elem[sl] = e;
-                }
-            }
-        }
-        __syncthreads();
-        if (s_ok) {
-            for (int i = 0; i < r.nf; ++i) project_dg2fd_element(d, r.f[i], r.nv[i], e, sm);
+    for (int w = blockIdx.x; w < n * r.nf; w += gridDim.x) {
+        const int e = d.flag_list[w / r.nf], i = w % r.nf;
+        project_dg2fd_element(d, r.f[i], r.nv[i], e, sm);
+        if (i == 1) {
             if (threadIdx.x == 0) d.mask[e] = 1;
+            __syncthreads();
+            for (int c = threadIdx.x; c < d.ncell; c += blockDim.x) current_fd_cell(d, e, c, r.f[1], r.J);
         }
-        __syncthreads();
     }
 }
 
-void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field F2, Field F3, Field G1, Field G2,
+void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field J, Field F2, Field F3, Field G1, Field G2,
                              Field G3, Field G4, cudaStream_t st) {
     RollArgs r{};
+    r.J = J;
     int k = 0;
     auto add = [&](Field f, int nv) {
         r.f[k] = f;
@@ -789,56 +752,62 @@ void launch_rollback_project(const Dev& d, int sub, Field un, Field Uin, Field F
     if (sub == SUB_B) { add(F2, NV); add(G1, NG); add(G2, NG); add(G3, NG); }
     if (sub == SUB_C) { add(F2, NV); add(F3, NV); add(G2, NG); add(G3, NG); add(G4, NG); }
     r.nf = k;
-    const int np1 = d.np1, nn = d.nn, nc = d.nc;
-    const size_t smem = (size_t)(nn + nc * np1 * np1 + nc * nc * np1) * sizeof(double);
+    const int np1 = d.np1, nc = d.nc;
+    const size_t smem = (size_t)NV * (nc * np1 * np1 + nc * nc * np1) * sizeof(double);
+    cudaFuncSetAttribute(k_rollback_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     prof_begin("rollback_project", st);
-    k_rollback_project<<<d.nsm, 256, smem, st>>>(d, r);
+    k_rollback_project<<<d.nsm * 2, 256, smem, st>>>(d, r);
     prof_end(st);
     g_launch_counter += 1;
 }
 
 // ---------------------------------------------------------------------------
-// FD -> DG (6-point Lagrange per direction) of one variable block src
-// ([nc^3]) into dst ([np1^3]), sum-factorised through shared memory.
-__device__ void project_fd2dg_var(const ES& es, const Tables& T, const double* src, double* dst, double* sm) {
-    const int np1 = es.np1, nc = es.nc, ncell = es.ncell;
-    double* a = sm;                    // [nc^3]
-    double* b = a + ncell;             // [nc][nc][np1]
-    double* c = b + nc * nc * np1;     // [nc][np1][np1]
-    for (int t = threadIdx.x; t < ncell; t += blockDim.x) a[t] = src[t];
-    __syncthreads();
-    for (int t = threadIdx.x; t < nc * nc * np1; t += blockDim.x) {
-        const int i = t % np1, yz = t / np1;
+// FD -> DG (6-point Lagrange per direction) of nv variable blocks ([nc^3], one
+// every `stride` doubles from src) into dst ([nv][np1^3]), sum-factorised through
+// shared memory, all variables at once.
+__device__ void project_fd2dg_vars(const ES& es, const Tables& T, const double* src, int64_t stride, int nv, double* dst,
+                                   double* sm) {
+    const int np1 = es.np1, nc = es.nc, nb = nc * nc * np1, ncc = nc * np1 * np1, nn = es.nn;
+    double* b = sm;                // [nv][nc][nc][np1]
+    double* c = b + nv * nb;       // [nv][nc][np1][np1]
+    for (int t = threadIdx.x; t < nv * nb; t += blockDim.x) {
+        const int v = t / nb, i = t % np1, yz = (t % nb) / np1;
         const int lo = T.f2d_lo[i];
+        const double* a = src + v * stride + lo + nc * yz;
         double acc = 0.0;
-        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[i][lo + m], a[lo + m + nc * yz], acc);
+        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[i][lo + m], a[m], acc);
         b[t] = acc;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < nc * np1 * np1; t += blockDim.x) {
-        const int i = t % np1, j = (t / np1) % np1, z = t / (np1 * np1);
+    for (int t = threadIdx.x; t < nv * ncc; t += blockDim.x) {
+        const int v = t / ncc, r = t % ncc, i = r % np1, j = (r / np1) % np1, z = r / (np1 * np1);
         const int lo = T.f2d_lo[j];
         double acc = 0.0;
-        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[j][lo + m], b[i + np1 * ((lo + m) + nc * z)], acc);
+        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[j][lo + m], b[v * nb + i + np1 * ((lo + m) + nc * z)], acc);
         c[t] = acc;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < np1 * np1 * np1; t += blockDim.x) {
-        const int ij = t % (np1 * np1), k = t / (np1 * np1);
+    for (int t = threadIdx.x; t < nv * nn; t += blockDim.x) {
+        const int v = t / nn, r = t % nn, ij = r % (np1 * np1), k = r / (np1 * np1);
         const int lo = T.f2d_lo[k];
         double acc = 0.0;
-        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[k][lo + m], c[ij + np1 * np1 * (lo + m)], acc);
+        for (int m = 0; m < 6; ++m) acc = fma(T.F2D[k][lo + m], c[v * ncc + ij + np1 * np1 * (lo + m)], acc);
         dst[t] = acc;
     }
     __syncthreads();
 }
 
+// shared doubles of k_fd2dg: projection scratch of 6 variables | B~ [3][nn] or 6 variables
+// [6][nn] | tmp [3][nn] | red [2][8]
+static size_t fd2dg_smem(const Dev& d) {
+    return (size_t)(6 * (d.nc * d.nc * d.np1 + d.nc * d.np1 * d.np1) + 9 * d.nn + 16) * sizeof(double);
+}
+
 // End of step: FD elements that did not switch during the step return to DG
 // when the indicator with alpha' = alpha + 1 finds their FD->DG projection
 // admissible; their FD slot returns to the pool.
-__global__ void k_fd2dg(Dev d, Field un) {
+__global__ void __launch_bounds__(256) k_fd2dg(Dev d, Field un) {
     extern __shared__ double sm[];
-    __shared__ double red[2];
     const int n = d.counts[1];
     for (int w = blockIdx.x; w < n; w += gridDim.x) {
         const int e = d.fd_list[w];
@@ -846,17 +815,18 @@ __global__ void k_fd2dg(Dev d, Field un) {
         const ES es = esz(d, e);
         const Tables& T = d.tabs[es.P];
         const int np1 = es.np1, nn = es.nn;
-        double* work = sm;                                                            // projection scratch
-        double* proj = work + d.ncell + d.nc * d.nc * d.np1 + d.nc * d.np1 * d.np1;   // [9][nn]
-        double* tmp = proj + NV * d.nn;                                               // [3][nn]
-        const int64_t fb = fdb(d, e);
-        for (int v = 3; v < 6; ++v) project_fd2dg_var(es, T, un.fd(v) + fb, proj + v * nn, work);
+        double* work = sm;                                                     // projection scratch
+        double* proj = work + 6 * (d.nc * d.nc * d.np1 + d.nc * d.np1 * d.np1);   // [6][nn]
+        double* tmp = proj + 6 * d.nn;                                         // [3][nn]
+        double* red = tmp + 3 * d.nn;                                          // [2][8]
+        const int64_t fb = fdb(d, e), db = (int64_t)e * d.nn;
+        project_fd2dg_vars(es, T, un.fd(3) + fb, un.nfd, 3, proj, work);
         for (int t = threadIdx.x; t < nn; t += blockDim.x) {
-            const double bx = proj[3 * nn + t], by = proj[4 * nn + t], bz = proj[5 * nn + t];
+            const double bx = proj[t], by = proj[nn + t], bz = proj[2 * nn + t];
             if (d.ks) {
                 // |B~| with the spatial metric at the node
                 PM m;
-                load_pm(d.met, d.ndg, (int64_t)e * d.nn + t, m);
+                load_pm(d.met, d.ndg, db + t, m);
                 const double u[NV] = {0.0, 0.0, 0.0, bx, by, bz, 0.0, 0.0, 0.0};
                 tmp[t] = bnorm_gen(u, m);
             } else {
@@ -878,8 +848,8 @@ __global__ void k_fd2dg(Dev d, Field un) {
             tmp[2 * nn + t] = acc;
         }
         __syncthreads();
-        // third low-pass direction and the two sums: per-thread partial sums in a
-        // fixed order, combined by thread 0 in thread order (deterministic)
+        // third low-pass direction and the two sums: per-thread partial sums in a fixed
+        // order, then a fixed tree over the lanes and the warps (deterministic)
         double pn = 0.0, pd = 0.0;
         for (int t = threadIdx.x; t < nn; t += blockDim.x) {
             const int i = t % np1, j = (t / np1) % np1;
@@ -889,32 +859,37 @@ __global__ void k_fd2dg(Dev d, Field un) {
             pn = fma(uh, uh, pn);
             pd = fma(tmp[t], tmp[t], pd);
         }
-        double* part = tmp + 3 * nn;   // [2][blockDim]
-        part[threadIdx.x] = pn;
-        part[blockDim.x + threadIdx.x] = pd;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double num = 0.0, den = 0.0;
-            for (int t = 0; t < (int)blockDim.x; ++t) { num += part[t]; den += part[blockDim.x + t]; }
-            const double thr = d.thr_fdP[es.P];
-            const double ratio = den > 0.0 ? sqrt(num / den) : 0.0;
-            if (fabs(ratio - thr) <= 1e-12 * thr) d.near_list[atomicAdd(&d.counts[3], 1) & 4095] = e;
-            red[0] = ratio > thr ? 1.0 : 0.0;
+        for (int o = 16; o > 0; o >>= 1) {
+            pn += __shfl_down_sync(0xffffffffu, pn, o);
+            pd += __shfl_down_sync(0xffffffffu, pd, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            red[threadIdx.x >> 5] = pn;
+            red[8 + (threadIdx.x >> 5)] = pd;
         }
         __syncthreads();
-        const bool stay = red[0] != 0.0;
-        __syncthreads();
-        if (stay) continue;
-        for (int v = 0; v < NV; ++v)
-            if (v < 3 || v > 5) project_fd2dg_var(es, T, un.fd(v) + fb, proj + v * nn, work);
-        for (int t = threadIdx.x; t < NV * nn; t += blockDim.x) un.dg(t / nn)[(int64_t)e * d.nn + t % nn] = proj[t];
-        if (threadIdx.x == 0) {
-            d.mask[e] = 0;
-            if (d.fd_slot) {
-                const int sl = d.fd_slot[e];
-                d.fd_slot[e] = -1;
-                d.slot_elem[sl] = -1;
-                d.free_slots[atomicAdd(&d.counts[5], 1)] = sl;
+        double num = 0.0, den = 0.0;
+        for (int i = 0; i < (int)blockDim.x / 32; ++i) { num += red[i]; den += red[8 + i]; }
+        const double thr = d.thr_fdP[es.P];
+        const double ratio = den > 0.0 ? sqrt(num / den) : 0.0;
+        if (threadIdx.x == 0 && fabs(ratio - thr) <= 1e-12 * thr) d.near_list[atomicAdd(&d.counts[3], 1) & 4095] = e;
+        if (!(ratio > thr)) {
+            for (int t = threadIdx.x; t < 3 * nn; t += blockDim.x) un.dg(3 + t / nn)[db + t % nn] = proj[t];
+            __syncthreads();
+            project_fd2dg_vars(es, T, un.fd(0) + fb, un.nfd, 3, proj, work);
+            project_fd2dg_vars(es, T, un.fd(6) + fb, un.nfd, 3, proj + 3 * nn, work);
+            for (int t = threadIdx.x; t < 6 * nn; t += blockDim.x) {
+                const int v = t / nn;
+                un.dg(v < 3 ? v : v + 3)[db + t % nn] = proj[t];
+            }
+            if (threadIdx.x == 0) {
+                d.mask[e] = 0;
+                if (d.fd_slot) {
+                    const int sl = d.fd_slot[e];
+                    d.fd_slot[e] = -1;
+                    d.slot_elem[sl] = -1;
+                    d.free_slots[atomicAdd(&d.counts[5], 1)] = sl;
+                }
             }
         }
         __syncthreads();
@@ -922,11 +897,10 @@ __global__ void k_fd2dg(Dev d, Field un) {
 }
 
 void launch_fd2dg(const Dev& d, Field un, cudaStream_t st) {
-    const int np1 = d.np1, nn = d.nn, nc = d.nc;
-    const size_t smem = (size_t)(d.ncell + nc * nc * np1 + nc * np1 * np1 + NV * nn + 3 * nn + 2 * 256) * sizeof(double);
+    const size_t smem = fd2dg_smem(d);
     cudaFuncSetAttribute(k_fd2dg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     prof_begin("fd2dg", st);
-    k_fd2dg<<<d.nsm, 256, smem, st>>>(d, un);
+    k_fd2dg<<<d.nsm * 2, 256, smem, st>>>(d, un);
     prof_end(st);
     g_launch_counter += 1;
 }
