@@ -13,6 +13,7 @@
 // 1e-20) leaves the fields unchanged.
 #pragma once
 #include "ffe_internal.h"
+#include "fixed.cuh"
 
 namespace ffe {
 
@@ -50,6 +51,86 @@ __device__ __forceinline__ void filter_lowrank(const Tables& T, double* sU) {
         }
         __syncthreads();
     }
+}
+
+// The same on fields in fixed point (z: [NV][nn], each below 2^fx_bits in its own
+// units): one rounding per mode and axis at the fields' quantum, no FP64 work.
+// nfr = 0 as above; barriers as above.
+template <int P, int NT>
+__device__ __forceinline__ void filter_fixed(const Tables& T, long long* z) {
+    constexpr int np1 = P + 1, nl = np1 * np1, nn = nl * np1;
+    const int nfr = T.nfr, k = T.fx_k;
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd) {
+        const int stride = dd == 0 ? 1 : (dd == 1 ? np1 : nl);
+        for (int q = threadIdx.x; q < NV * nl; q += NT) {
+            const int v = q / nl, line = q - v * nl;
+            const int base = dd == 0 ? np1 * line : (dd == 1 ? line % np1 + nl * (line / np1) : line);
+            long long* p = z + v * nn + base;
+            long long y[np1];
+            Fx x[np1];
+#pragma unroll
+            for (int m = 0; m < np1; ++m) {
+                y[m] = p[stride * m];
+                x[m] = fx_limbs(y[m]);
+            }
+#pragma unroll 1
+            for (int r = 0; r < nfr; ++r) {
+                FxSum s;
+#pragma unroll
+                for (int m = 0; m < np1; ++m) s.add(x[m], T.FxW[r][m]);
+                const Fx c = fx_limbs((s.a << k) + (s.b >> (28 - k)));
+#pragma unroll
+                for (int m = 0; m < np1; ++m) {
+                    FxSum t;
+                    t.add(c, T.FxV[r][m]);
+                    y[m] -= t.top();
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < np1; ++m) p[stride * m] = y[m];
+        }
+        __syncthreads();
+    }
+}
+
+// Filters an element's fields, u[NV] of the thread's node (act: it has one).  The
+// fixed-point form gives the filter's correction, exact in integers, which is added
+// in FP64: one FP64 operation a value instead of 12.  sU [NV][nn] and z [NV][nn] are
+// scratch; word [NV] is zero on entry.
+template <int P, int NT>
+__device__ __forceinline__ void filter_element(const Tables& T, bool act, double* sU, long long* z, unsigned* word, double* u) {
+    constexpr int nn = (P + 1) * (P + 1) * (P + 1);
+    const int tid = threadIdx.x, bits = T.fx_bits;
+    if (T.nfr == 0) return;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        if (act) sU[v * nn + tid] = u[v];
+        const unsigned w = __reduce_max_sync(0xffffffffu, act ? fx_word(u[v]) : 0u);
+        if ((tid & 31) == 0) atomicMax(word + v, w);
+    }
+    __syncthreads();
+    unsigned top = 0;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) top = max(top, word[v]);
+    if (bits == 0 || top >= (unsigned)FX_EMAX << 20) {
+        filter_lowrank<P, NT>(T, sU);
+        if (act)
+            for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
+        return;
+    }
+    if (act)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) z[v * nn + tid] = fx_from(sU[v * nn + tid], fx_exp(word[v]), bits);
+    __syncthreads();
+    filter_fixed<P, NT>(T, z);
+    if (act)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const double x = sU[v * nn + tid];
+            const int e = fx_exp(word[v]);
+            u[v] = x + fx_double(z[v * nn + tid] - fx_from(x, e, bits), e - 1022 - bits);
+        }
 }
 
 }  // namespace ffe

@@ -31,6 +31,11 @@ constexpr double IM_H = 0.12915286960590;
 // substep kinds of the device stage kernels
 enum Sub : int { SUB_A = 0, SUB_B = 1, SUB_C = 2, SUB_RHS = 3 };
 
+// two limbs of a fixed-point number, hi 2^28 + lo (fixed.cuh)
+struct Fx {
+    int hi, lo;
+};
+
 // 1-D operator tables of one order P (built on the host in long double).
 struct Tables {
     int P, np1, nc;
@@ -41,6 +46,13 @@ struct Tables {
     // more than 1e-20 (FrV[r][i] = P_m(x_i), FrW[r][j] = (1 - sigma_m) (V^-1)[m][j])
     int nfr;
     double FrV[MAXNP][MAXNP], FrW[MAXNP][MAXNP];
+    // the same in units of 2^-56 and 2^(fx_k - 56) (filter_fixed), for fields of
+    // fx_bits bits; fx_bits = 0: this filter takes the FP64 form
+    int fx_bits, fx_k;
+    Fx FxV[MAXNP][MAXNP], FxW[MAXNP][MAXNP];
+    double Dabs;                   // largest row sum of |D|
+    int fx_d;                      // D in units of 2^-fx_d (its rows sum to less than 2^59)
+    Fx FxD[MAXNP][MAXNP];
     double Pi[MAXNP][MAXNP];       // projection on Legendre modes p <= P - M
     double P2F[MAXNC][MAXNP];      // DG -> FD (Lagrange evaluation at subcell centres)
     double F2D[MAXNP][MAXNC];      // FD -> DG (6-point Lagrange, shifted inside)
@@ -105,6 +117,7 @@ struct Dev {
     // physics and scheme parameters
     double eta, kpsi, kphi, dt, weno_eps, omega;
     int mode, filter_on, tci_on, fd_corr, recon;
+    int fp64_lines;                 // curved DG: the volume term's line contractions in FP64 (rhs_at)
     double thr_dg, thr_fd;          // (P+1-M)^-alpha and (P+1-M)^-(alpha+1)
     SolveK sk;                      // of dt (batches: per instance, InstInfo)
     // geometry of the affine box: d xi / d x per element and axis

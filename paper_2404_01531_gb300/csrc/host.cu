@@ -129,6 +129,38 @@ ld lagrange(const std::vector<ld>& xs, int j, ld y) {
     return r;
 }
 
+Fx fx_limbs_host(ld v) {
+    const long long z = llrintl(v), lo = ((z + (1LL << 27)) & ((1LL << 28) - 1)) - (1LL << 27);
+    return {(int)((z - lo) / (1LL << 28)), (int)lo};
+}
+
+// The filter's vectors in fixed point.  Along the three axes a field grows by at most
+// the filter's row sum each, and a mode's coefficient is at most its row of W times
+// the field: both have to stay below 2^58.  Filters that would leave the fields fewer
+// than 55 bits keep the FP64 form (three more than FP64's 53 cover the cuts).
+void fixed_filter(Tables& T) {
+    const int np1 = T.np1;
+    double row = 1.0, w = 0.0;
+    for (int i = 0; i < np1; ++i) {
+        double s = 0.0;
+        for (int j = 0; j < np1; ++j) s += fabs(T.Filt[i][j]);
+        row = std::max(row, s);
+    }
+    for (int r = 0; r < T.nfr; ++r) {
+        double s = 0.0;
+        for (int j = 0; j < np1; ++j) s += fabs(T.FrW[r][j]);
+        w = std::max(w, s);
+    }
+    T.fx_bits = 58 - (int)ceil(log2(std::max(row * row * row, row * row * w)));
+    T.fx_k = w > 4.0 ? (int)ceil(log2(w)) - 2 : 0;
+    if (T.fx_bits < 55) T.fx_bits = 0;
+    for (int r = 0; r < T.nfr; ++r)
+        for (int i = 0; i < np1; ++i) {
+            T.FxV[r][i] = fx_limbs_host(ldexpl((ld)T.FrV[r][i], 56));
+            T.FxW[r][i] = fx_limbs_host(ldexpl((ld)T.FrW[r][i], 56 - T.fx_k));
+        }
+}
+
 void build_tables(int P, double fa, double fb, int M, Tables& T) {
     memset(&T, 0, sizeof T);
     const int np1 = P + 1, nc = 2 * P + 1;
@@ -177,6 +209,15 @@ void build_tables(int P, double fa, double fb, int M, Tables& T) {
             T.FrW[r][i] = (double)(dm * Vi[m * np1 + i]);
         }
     }
+    for (int i = 0; i < np1; ++i) {
+        double s = 0.0;
+        for (int j = 0; j < np1; ++j) s += fabs(T.D[i][j]);
+        T.Dabs = std::max(T.Dabs, s);
+    }
+    T.fx_d = 59 - (int)ceil(log2(T.Dabs));
+    for (int i = 0; i < np1; ++i)
+        for (int j = 0; j < np1; ++j) T.FxD[i][j] = fx_limbs_host(ldexpl((ld)T.D[i][j], T.fx_d));
+    fixed_filter(T);
     std::vector<ld> xc(nc);
     const ld dxi = 2.0L / nc;
     for (int c = 0; c < nc; ++c) xc[c] = -1.0L + (c + 0.5L) * dxi;
@@ -2380,9 +2421,12 @@ static ffe_status filter_or_copy(ffe_ctx* c, Field in, Field out, int transpose)
     return FFE_OK;
 }
 
-// right-hand side of the hybrid operator at U (fixed mask)
+// right-hand side of the hybrid operator at U (fixed mask).  It keeps its bits (faces,
+// fp64_lines): the reverse mode amplifies the rounding of the stages it is linearised
+// at by up to 1e9 (k_fd_flux_faces).
 static void rhs_at(ffe_ctx* c, Field U, Field out) {
-    const Dev& d = c->d;
+    Dev d = c->d;
+    d.fp64_lines = 1;
     launch_current(d, U, c->J, c->st);
     if (c->adj_fd)
         launch_fd_substep(d, SUB_RHS, d.fd_list, 1, U, c->J, c->un, c->F2, c->F3, c->G1, c->G2, c->G3, c->G4, out, out,

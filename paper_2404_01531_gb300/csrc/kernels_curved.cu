@@ -27,9 +27,10 @@ struct DGC {
     static constexpr int FR = (6 * nf + NT - 1) / NT;   // face nodes per thread
     // CTAs per SM the registers are bounded for (see k_dg_curved)
     static constexpr int CTAS = NT <= 128 ? (KS ? 3 : 4) : 2;
-    // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn], Kerr-Schild:
-    // J[3][nn], F[27][nn] | dU/dt[9][nn] | red[2][NW] and the flag
-    static constexpr int NS = KS ? 30 : 3;
+    // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn] | fixed point:
+    // U and J [12][nn], Kerr-Schild: F[27][nn] as doubles, then in fixed point (later the
+    // filter's fields) | dU/dt[9][nn] | red[2][NW] and the flag
+    static constexpr int NS = KS ? 30 : 15;
     static constexpr int SMEM = ((18 + NS) * nn + 2 * NW + 1) * 8;
 };
 
@@ -193,13 +194,17 @@ __device__ __forceinline__ void flux_normal_gen(const double* n, const PM& m, co
 }
 
 // One element of order P processed by a block of NT threads (NT >= (P+1)^3).
+// s_word, s_wordf [NV]: the largest words (fx_word) of the volume term's blocks, zero
+// on entry and on return, and of the filter's.
 template <int P, int NT, int SUB, bool KS>
-__device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, int e, double* sm) {
+__device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, int e, double* sm, unsigned* s_word,
+                                               unsigned* s_wordf) {
     using K = DGC<P, KS>;
     constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NW = NT / 32;
     double* sU = sm;                 // [9][nn]
     double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
-    double* sF = sJ + 3 * nn;        // Kerr-Schild: [3][9][nn] F^j
+    double* sF = sJ + 3 * nn;        // fixed point [12][nn]; Kerr-Schild: [3][9][nn] F^j
+    Fx* fF = (Fx*)sF;
     double* sR = sJ + K::NS * nn;    // [9][nn] dU/dt
     double* red = sR + 9 * nn;
     const Tables& T = d.tabs[P];
@@ -208,12 +213,21 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
     const int ci[3] = {tid % np1, (tid / np1) % np1, tid / (np1 * np1)};
     const int64_t eb = (int64_t)e * d.nn;
     const double dt = dt_of(d, e);
-    for (int t = tid; t < NV * nn; t += NT) sU[t] = a.Uin.dg(t / nn)[eb + t % nn];
-    if (!KS)
-        for (int t = tid; t < 3 * nn; t += NT) sJ[t] = a.J.dg(3 + t / nn)[eb + t % nn];
-    __syncthreads();
-    if (KS) {
-        if (act) {
+    // Values of the volume term's contractions (fixed.cuh): 12 fields in three blocks --
+    // E~ and phi~ meet in the B~ equations, B~ and psi~ in those of E~, J~ alone --
+    // or on the Kerr-Schild background 27 fluxes in a block per variable.
+    constexpr int NB = KS ? NV : 3;
+    auto block = [](int v) { return KS ? v % NV : (v < 3 || v == 7 ? 0 : (v < NV ? 1 : 2)); };
+    unsigned word[NB];
+    for (int b = 0; b < NB; ++b) word[b] = 0;
+    if (act) {
+#pragma unroll
+        for (int v = 0; v < (KS ? NV : 12); ++v) {
+            const double x = v < NV ? a.Uin.dg(v)[eb + tid] : a.J.dg(3 + v - NV)[eb + tid];
+            sU[v * nn + tid] = x;
+            if (!KS) word[block(v)] = max(word[block(v)], fx_word(x));
+        }
+        if (KS) {
             PM m;
             load_pm(d.met, d.ndg, eb + tid, m);
             double u[NV], jd[3], jf[3], F[3][NV], S[NV];
@@ -222,33 +236,41 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
             flux_gen(u, jf, m, F);
             for (int i = 0; i < 3; ++i) sJ[i * nn + tid] = jf[i];
             for (int j = 0; j < 3; ++j)
-                for (int v = 0; v < NV; ++v) sF[(j * NV + v) * nn + tid] = F[j][v];
+                for (int v = 0; v < NV; ++v) {
+                    sF[(j * NV + v) * nn + tid] = F[j][v];
+                    word[v % NB] = max(word[v % NB], fx_word(F[j][v]));
+                }
             sources_gen(u, jd, m, d.met, d.ndg, eb + tid, S);
             for (int v = 0; v < NV; ++v) sR[v * nn + tid] = S[v];
         }
-        __syncthreads();
     }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        word[b] = __reduce_max_sync(0xffffffffu, word[b]);
+        if ((tid & 31) == 0) atomicMax(s_word + b, word[b]);
+    }
+    __syncthreads();
+    if (tid < NV) s_wordf[tid] = 0;
+    unsigned top = 0;
+    for (int b = 0; b < NB; ++b) top = max(top, s_word[b]);
+    const bool fixed = !d.fp64_lines && top < (unsigned)FX_EMAX << 20;
+    if (act && fixed) {
+#pragma unroll
+        for (int v = 0; v < (KS ? 27 : 12); ++v)
+            fF[v * nn + tid] = fx_limbs(fx_from((KS ? sF : sU)[v * nn + tid], fx_exp(s_word[block(v)]), FX_BITS));
+    }
+    __syncthreads();
     if (act) {
         double du[NV];
         for (int v = 0; v < NV; ++v) du[v] = KS ? sR[v * nn + tid] : 0.0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
-            const int base = tid - ci[k] * stride;
-            double Dk[np1];
-            for (int mm = 0; mm < np1; ++mm) Dk[mm] = T.D[ci[k]][mm];
-            auto R = [&](const double* f) {
-                double acc = 0.0;
-#pragma unroll
-                for (int mm = 0; mm < np1; ++mm) acc = fma(Dk[mm], f[base + mm * stride], acc);
-                return acc;
-            };
+        // derivatives along axis k with R(v) = D_k of value v
+        auto volume = [&](int k, auto R) {
             double g[3];
             for (int i = 0; i < 3; ++i) g[i] = d.geo[(int64_t)(3 * k + i) * d.ndg + eb + tid];
             if (KS) {
                 for (int j = 0; j < 3; ++j)
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) du[v] = fma(-g[j], R(sF + (j * NV + v) * nn), du[v]);
+                    for (int v = 0; v < NV; ++v) du[v] = fma(-g[j], R(j * NV + v), du[v]);
             } else {
                 // flat metric: D_k F^j = +-D_k of one field (D_k is linear), so the
                 // volume term is built from the reference derivatives R = D_k X of the
@@ -257,28 +279,57 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
                 //   psi~: -div E~,  phi~: -div B~,  q~: -div J~
                 const double ka = g[0], kb = g[1], kc = g[2];
                 double r;
-                r = R(sU + 0 * nn);   // E0
+                r = R(0);   // E0
                 du[4] = fma(-kc, r, du[4]); du[5] = fma(kb, r, du[5]); du[6] = fma(-ka, r, du[6]);
-                r = R(sU + 1 * nn);   // E1
+                r = R(1);   // E1
                 du[3] = fma(kc, r, du[3]); du[5] = fma(-ka, r, du[5]); du[6] = fma(-kb, r, du[6]);
-                r = R(sU + 2 * nn);   // E2
+                r = R(2);   // E2
                 du[3] = fma(-kb, r, du[3]); du[4] = fma(ka, r, du[4]); du[6] = fma(-kc, r, du[6]);
-                r = R(sU + 3 * nn);   // B0
+                r = R(3);   // B0
                 du[1] = fma(kc, r, du[1]); du[2] = fma(-kb, r, du[2]); du[7] = fma(-ka, r, du[7]);
-                r = R(sU + 4 * nn);   // B1
+                r = R(4);   // B1
                 du[0] = fma(-kc, r, du[0]); du[2] = fma(ka, r, du[2]); du[7] = fma(-kb, r, du[7]);
-                r = R(sU + 5 * nn);   // B2
+                r = R(5);   // B2
                 du[0] = fma(kb, r, du[0]); du[1] = fma(-ka, r, du[1]); du[7] = fma(-kc, r, du[7]);
-                r = R(sU + 6 * nn);   // psi
+                r = R(6);   // psi
                 du[0] = fma(-ka, r, du[0]); du[1] = fma(-kb, r, du[1]); du[2] = fma(-kc, r, du[2]);
-                r = R(sU + 7 * nn);   // phi
+                r = R(7);   // phi
                 du[3] = fma(-ka, r, du[3]); du[4] = fma(-kb, r, du[4]); du[5] = fma(-kc, r, du[5]);
-                r = R(sJ + 0 * nn);   // J0
+                r = R(9);   // J0
                 du[8] = fma(-ka, r, du[8]);
-                r = R(sJ + 1 * nn);   // J1
+                r = R(10);  // J1
                 du[8] = fma(-kb, r, du[8]);
-                r = R(sJ + 2 * nn);   // J2
+                r = R(11);  // J2
                 du[8] = fma(-kc, r, du[8]);
+            }
+        };
+        if (fixed) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
+                const int base = tid - ci[k] * stride;
+                Fx Dk[np1];
+                for (int mm = 0; mm < np1; ++mm) Dk[mm] = T.FxD[ci[k]][mm];
+                volume(k, [&](int v) {
+                    FxSum s;
+#pragma unroll
+                    for (int mm = 0; mm < np1; ++mm) s.add(Dk[mm], fF[v * nn + base + mm * stride]);
+                    // units: 2^56 2^-fx_d 2^(e - 1022 - 58)
+                    return fx_double(s.top(), fx_exp(s_word[block(v)]) - 1024 - T.fx_d);
+                });
+            }
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < 3; ++k) {
+                const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
+                const int base = tid - ci[k] * stride;
+                volume(k, [&](int v) {
+                    double acc = 0.0;
+#pragma unroll (KS ? 1 : np1)
+                    for (int mm = 0; mm < np1; ++mm)
+                        acc = fma(T.D[ci[k]][mm], (KS ? sF : sU)[v * nn + base + mm * stride], acc);
+                    return acc;
+                });
             }
         }
         if (!KS) {
@@ -335,6 +386,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
     // added axis by axis (edge and corner nodes lie on faces of several axes; see k_dg_substep)
     for (int dd = 0; dd < 3; ++dd) {
         __syncthreads();
+        if (dd == 0 && tid < NB) s_word[tid] = 0;
 #pragma unroll
         for (int r = 0; r < K::FR; ++r) {
             const int t = tid + r * NT;
@@ -358,12 +410,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
         substep_explicit(d, SUB, du, eb + tid, false, a, dt, u);
     }
     if (d.filter_on) {
-        if (act)
-            for (int v = 0; v < NV; ++v) sU[v * nn + tid] = u[v];
-        __syncthreads();
-        filter_lowrank<P, NT>(T, sU);
-        if (act)
-            for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
+        filter_element<P, NT>(T, act, sU, (long long*)sF, s_wordf, u);
     }
     // implicit part after the filter; G at the stage value: G_s = (U_s - R~_s)/(dt a)
     double mag = 0.0;
@@ -440,21 +487,27 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
 
 
 // Persistent kernel over a DG work list of order-P elements (list, count in
-// d.counts[ci]).  Bound by the FP64 pipe, as the box kernel (k_dg_substep): J~ is read
-// instead of formed again at the nodes and at every face node, the normals and
-// |grad xi| are tabulated, the jump's flux is contracted with the normal at once
-// (27 FMAs; with the general metric's flux and a constant flat metric it was 170
-// slots), and the face sums go axis by axis.  Two CTAs an SM at P = 5 (P <= 4: three
-// or four), also with the metric, which had one and idled at its barriers.
-// 7146 elements of orders 4 and 5: substep 1.42 -> 0.97 ms; Kerr-Schild, 1536
-// elements: 0.89 -> 0.77 ms.  Batched contexts launch each order's elements separately, in
+// d.counts[ci]).  Bound by the FP64 pipe, as the box kernel (k_dg_substep): the
+// contractions of the volume term (198 FP64 slots a node, 486 with the metric) and of
+// the filter run on the integer pipes, J~ is read instead of formed again at the nodes
+// and at every face node, the normals and |grad xi| are tabulated, the jump's flux is
+// contracted with the normal at once (27 FMAs; with the general metric's flux and a
+// constant flat metric it was 170 slots), and the face sums go axis by axis.  Two CTAs
+// an SM at P = 5 (P <= 4: three or four), also with the metric, which had one and idled
+// at its barriers.  7146 elements of orders 4 and 5: substep 0.97 -> 0.71 ms (1.42 before
+// the work outside the contractions went down); Kerr-Schild, 1536 elements: 0.77 ->
+// 0.50 ms.  Batched contexts launch each order's elements separately, in
 // CTAs sized for that order (one kernel dispatching on the order would keep every
 // order's registers live and spill).
 template <int P, int SUB, bool KS>
 __global__ void __launch_bounds__(DGC<P, KS>::NT, DGC<P, KS>::CTAS) k_dg_curved(Dev d, SubArgs a, const int* list, int ci) {
     extern __shared__ double sm[];
+    __shared__ unsigned s_word[NV], s_wordf[NV];
+    if (threadIdx.x < NV) s_word[threadIdx.x] = 0;
+    __syncthreads();
     const int nwork = d.counts[ci];
-    for (int w = blockIdx.x; w < nwork; w += gridDim.x) dg_curved_elem<P, DGC<P, KS>::NT, SUB, KS>(d, a, list[w], sm);
+    for (int w = blockIdx.x; w < nwork; w += gridDim.x)
+        dg_curved_elem<P, DGC<P, KS>::NT, SUB, KS>(d, a, list[w], sm, s_word, s_wordf);
 }
 
 template <int P, bool KS, int SUB>

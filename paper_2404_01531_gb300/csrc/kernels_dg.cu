@@ -34,8 +34,9 @@ struct DGK {
     // CTAs per SM the registers are bounded for
     static constexpr int CTAS = P == 6 ? 2 : 3;
     // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn] | dU/dt[9][nn] |
-    // red[2][NW] | D scaled by the element's d xi/d x, per axis [3][np1][np1]
-    static constexpr int SMEM = (21 * nn + 2 * NW + 3 * nf) * 8;
+    // fixed point: U and J [12][nn] (later the filter's fields) | red[2][NW] | D scaled by the
+    // element's d xi/d x, per axis [3][np1][np1]
+    static constexpr int SMEM = (33 * nn + 2 * NW + 3 * nf) * 8;
 };
 
 // ---------------------------------------------------------------------------
@@ -267,14 +268,43 @@ __device__ void dg_external_state(const Dev& d, const SubArgs& a, int e, int f, 
     current_flat(Ue, d.eta, jd, Je);
 }
 
+// The volume term in FP64, for elements whose values fixed point does not hold.
+template <int P>
+__device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* sU, const double* sJ, const double* sD, double* r) {
+    constexpr int np1 = P + 1, nf = np1 * np1, nn = nf * np1;
+    const int tid = threadIdx.x, i = tid % np1, j = (tid / np1) % np1, k = tid / nf;
+    const double *Dx = sD + np1 * i, *Dy = sD + nf + np1 * j, *Dz = sD + 2 * nf + np1 * k;
+    const int ox = np1 * (j + np1 * k), oy = i + nf * k, oz = i + np1 * j;
+    auto U = [&](int v, int idx) { return sU[v * nn + idx]; };
+    double eX = -J.dg(0)[eb + tid], eY = -J.dg(1)[eb + tid], eZ = -J.dg(2)[eb + tid];
+    double bX = 0.0, bY = 0.0, bZ = 0.0, ps = U(8, tid), ph = 0.0, qq = 0.0;
+#pragma unroll 1
+    for (int m = 0; m < np1; ++m) {
+        const int ix = ox + m, iy = oy + np1 * m, iz = oz + nf * m;
+        eX += Dy[m] * U(5, iy) - Dz[m] * U(4, iz) - Dx[m] * U(6, ix);
+        eY += Dz[m] * U(3, iz) - Dx[m] * U(5, ix) - Dy[m] * U(6, iy);
+        eZ += Dx[m] * U(4, ix) - Dy[m] * U(3, iy) - Dz[m] * U(6, iz);
+        bX += Dz[m] * U(1, iz) - Dy[m] * U(2, iy) - Dx[m] * U(7, ix);
+        bY += Dx[m] * U(2, ix) - Dz[m] * U(0, iz) - Dy[m] * U(7, iy);
+        bZ += Dy[m] * U(0, iy) - Dx[m] * U(1, ix) - Dz[m] * U(7, iz);
+        ps -= Dx[m] * U(0, ix) + Dy[m] * U(1, iy) + Dz[m] * U(2, iz);
+        ph -= Dx[m] * U(3, ix) + Dy[m] * U(4, iy) + Dz[m] * U(5, iz);
+        qq -= Dx[m] * sJ[ix] + Dy[m] * sJ[nn + iy] + Dz[m] * sJ[2 * nn + iz];
+    }
+    r[0] = eX; r[nn] = eY; r[2 * nn] = eZ; r[3 * nn] = bX; r[4 * nn] = bY; r[5 * nn] = bZ;
+    r[6 * nn] = ps; r[7 * nn] = ph; r[8 * nn] = qq;
+}
+
 // What bounds it: the FP64 pipe (2 lanes a clock and SM; a warp instruction takes
-// 16 clocks of an SM), at 7 warps an element about 430 FP64 slots a thread in
-// substep A, of which 162 are the line contractions.  So the work per node is what
-// counts: five lift values per face node instead of nine, their sum into dU/dt axis
-// by axis instead of node by node under divergence, no FP64 comparisons, and the
-// stage's G and currents from its solve (substep_implicit).  Three CTAs an SM: their
-// barriers hide each other's.  4096 elements at P = 5, average of the substeps:
-// 0.870 -> 0.757 ms, and the separate current launches (0.075 ms each) are gone.
+// 16 clocks of an SM).  So the line contractions of the volume term and of the filter,
+// 270 of 430 FP64 slots a thread, run on the integer pipes (fixed.cuh: a 32 x 32 -> 64
+// bit multiply-add takes one clock a warp, three of them replace an FMA); in the rest
+// the work per node is what counts: five lift values per face node instead of nine,
+// their sum into dU/dt axis by axis instead of node by node under divergence, no FP64
+// comparisons, and the stage's G and currents from its solve (substep_implicit).
+// Three CTAs an SM: their barriers hide each other's (two without spills: 3% slower).
+// 4096 elements at P = 5, average of the substeps: 0.757 -> 0.551 ms (0.870 with the
+// work per node as it was).
 template <int P, int SUB>
 __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, SubArgs a) {
     using K = DGK<P>;
@@ -283,60 +313,112 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
     double* sU = sm;                 // [9][nn]
     double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
     double* sR = sJ + 3 * nn;        // [9][nn] dU/dt
-    double* red = sR + 9 * nn;
+    Fx* fU = (Fx*)(sR + 9 * nn);     // [12][nn] U and J~ in fixed point
+    double* red = sR + 21 * nn;
     double* sD = red + 2 * NW;       // [3][np1][np1]: (d xi^a/d x^a) D
+    Fx* fD = (Fx*)sD;
     __shared__ int s_flag;
+    __shared__ unsigned s_word[3], s_wordf[NV];  // largest words (fx_word) of the volume term's blocks, of the filter's
     const Tables& T = *d.tab;
     const int tid = threadIdx.x;
     const bool act = tid < nn;
     const int i = tid % np1, j = (tid / np1) % np1, k = tid / (np1 * np1);
     const double w0inv = 1.0 / T.w0;
     const int nwork = d.counts[0];
+    if (tid < 3) s_word[tid] = 0;
+    __syncthreads();
     for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
         const int e = d.dg_list[w];
         const int64_t eb = (int64_t)e * nn;
         const double sx = d.ijac[3 * e], sy = d.ijac[3 * e + 1], sz = d.ijac[3 * e + 2];
-        for (int t = tid; t < NV * nn; t += NT) sU[t] = a.Uin.dg(t / nn)[eb + t % nn];
-        for (int t = tid; t < 3 * nn; t += NT) sJ[t] = a.J.dg(3 + t / nn)[eb + t % nn];
-        for (int t = tid; t < 3 * nf; t += NT)
-            sD[t] = (t < nf ? sx : (t < 2 * nf ? sy : sz)) * T.D[(t % nf) / np1][t % np1];
-        double eX = 0.0, eY = 0.0, eZ = 0.0;
+        double* r = sR + tid;
+        unsigned wE = 0, wB = 0, wJ = 0;
         if (act) {
-            eX = -a.J.dg(0)[eb + tid];
-            eY = -a.J.dg(1)[eb + tid];
-            eZ = -a.J.dg(2)[eb + tid];
+#pragma unroll
+            for (int v = 0; v < 12; ++v) {
+                const double x = v < NV ? a.Uin.dg(v)[eb + tid] : a.J.dg(3 + v - NV)[eb + tid];
+                sU[v * nn + tid] = x;
+                const unsigned w = fx_word(x);
+                if (v < 3 || v == 7) wE = max(wE, w);
+                else if (v < 7) wB = max(wB, w);
+                else if (v >= NV) wJ = max(wJ, w);
+            }
+        }
+        // blocks: E~ and phi~ meet in the B~ equations, B~ and psi~ in those of E~, J~ alone
+        wE = __reduce_max_sync(0xffffffffu, wE);
+        wB = __reduce_max_sync(0xffffffffu, wB);
+        wJ = __reduce_max_sync(0xffffffffu, wJ);
+        if ((tid & 31) == 0) {
+            atomicMax(&s_word[0], wE);
+            atomicMax(&s_word[1], wB);
+            atomicMax(&s_word[2], wJ);
+        }
+        const double rows = T.Dabs * (fabs(sx) + fabs(sy) + fabs(sz));   // bounds the sums' |D| entries
+        const int eD = (int)(fx_word(rows) >> 20);
+        __syncthreads();
+        if (tid < NV) s_wordf[tid] = 0;
+        const int eE = fx_exp(s_word[0]), eB = fx_exp(s_word[1]), eJ = fx_exp(s_word[2]);
+        const bool fixed = max(eE, max(eB, eJ)) < FX_EMAX && eD > 1023 - 60 && eD < 1023 + 60;
+        for (int t = tid; t < 3 * nf; t += NT) {
+            const double D = (t < nf ? sx : (t < 2 * nf ? sy : sz)) * T.D[(t % nf) / np1][t % np1];
+            if (fixed) fD[t] = fx_limbs(fx_from(D, eD, FX_BITS + 1));
+            else sD[t] = D;
+        }
+        if (act && fixed) {
+#pragma unroll
+            for (int v = 0; v < 12; ++v)
+                fU[v * nn + tid] = fx_limbs(fx_from(sU[v * nn + tid], v < 3 || v == 7 ? eE : (v < 7 ? eB : eJ), FX_BITS));
         }
         __syncthreads();
-        if (act) {
-            const double* Dx = sD + np1 * i;
-            const double* Dy = sD + nf + np1 * j;
-            const double* Dz = sD + 2 * nf + np1 * k;
-            const int ox = np1 * (j + np1 * k);   // x-line start
-            const int oy = i + np1 * np1 * k;     // y-line start, stride np1
-            const int oz = i + np1 * j;           // z-line start, stride np1^2
-            auto U = [&](int v, int idx) { return sU[v * nn + idx]; };
-            double bX = 0.0, bY = 0.0, bZ = 0.0;
-            double ps = U(8, tid), ph = 0.0, qq = 0.0;
+        if (tid < 3) s_word[tid] = 0;
+        if (act && fixed) {
+            const int ox = np1 * (j + np1 * k), oy = i + np1 * np1 * k, oz = i + np1 * j;
+            const Fx *Dx = fD + np1 * i, *Dy = fD + nf + np1 * j, *Dz = fD + 2 * nf + np1 * k;
+            auto ux = [&](int v, int m) { return fU[v * nn + ox + m]; };
+            auto uy = [&](int v, int m) { return fU[v * nn + oy + np1 * m]; };
+            auto uz = [&](int v, int m) { return fU[v * nn + oz + np1 * np1 * m]; };
+            // units: 2^56 2^(e - 1022 - 58) 2^(eD - 1022 - 59)
+            auto out = [&](const FxSum& X, int e) { return fx_double(X.top(), e + eD - 2105); };
+            {   // E: curl B - grad psi, phi: -div B
+                FxSum X, Y, Z, W;
 #pragma unroll
-            for (int m = 0; m < np1; ++m) {
-                const int ix = ox + m, iy = oy + np1 * m, iz = oz + np1 * np1 * m;
-                // E: curl B - grad psi
-                eX = fma(Dy[m], U(5, iy), eX); eX = fma(-Dz[m], U(4, iz), eX); eX = fma(-Dx[m], U(6, ix), eX);
-                eY = fma(Dz[m], U(3, iz), eY); eY = fma(-Dx[m], U(5, ix), eY); eY = fma(-Dy[m], U(6, iy), eY);
-                eZ = fma(Dx[m], U(4, ix), eZ); eZ = fma(-Dy[m], U(3, iy), eZ); eZ = fma(-Dz[m], U(6, iz), eZ);
-                // B: -curl E - grad phi
-                bX = fma(-Dy[m], U(2, iy), bX); bX = fma(Dz[m], U(1, iz), bX); bX = fma(-Dx[m], U(7, ix), bX);
-                bY = fma(-Dz[m], U(0, iz), bY); bY = fma(Dx[m], U(2, ix), bY); bY = fma(-Dy[m], U(7, iy), bY);
-                bZ = fma(-Dx[m], U(1, ix), bZ); bZ = fma(Dy[m], U(0, iy), bZ); bZ = fma(-Dz[m], U(7, iz), bZ);
-                // psi: -div E + q ; phi: -div B ; q: -div J
-                ps = fma(-Dx[m], U(0, ix), ps); ps = fma(-Dy[m], U(1, iy), ps); ps = fma(-Dz[m], U(2, iz), ps);
-                ph = fma(-Dx[m], U(3, ix), ph); ph = fma(-Dy[m], U(4, iy), ph); ph = fma(-Dz[m], U(5, iz), ph);
-                qq = fma(-Dx[m], sJ[ix], qq); qq = fma(-Dy[m], sJ[nn + iy], qq);
-                qq = fma(-Dz[m], sJ[2 * nn + iz], qq);
+                for (int m = 0; m < np1; ++m) {
+                    const Fx p = Dx[m], q = Dy[m], t = Dz[m], np = fx_neg(p), nq = fx_neg(q), nt = fx_neg(t);
+                    X.add(uy(5, m), q); X.add(uz(4, m), nt); X.add(ux(6, m), np);
+                    Y.add(uz(3, m), t); Y.add(ux(5, m), np); Y.add(uy(6, m), nq);
+                    Z.add(ux(4, m), p); Z.add(uy(3, m), nq); Z.add(uz(6, m), nt);
+                    W.add(ux(3, m), np); W.add(uy(4, m), nq); W.add(uz(5, m), nt);
+                }
+                r[0] = out(X, eB) - a.J.dg(0)[eb + tid];
+                r[nn] = out(Y, eB) - a.J.dg(1)[eb + tid];
+                r[2 * nn] = out(Z, eB) - a.J.dg(2)[eb + tid];
+                r[7 * nn] = out(W, eB);
             }
-            double* r = sR + tid;
-            r[0] = eX; r[nn] = eY; r[2 * nn] = eZ; r[3 * nn] = bX; r[4 * nn] = bY; r[5 * nn] = bZ;
-            r[6 * nn] = ps; r[7 * nn] = ph; r[8 * nn] = qq;
+            {   // B: -curl E - grad phi, psi: -div E + q
+                FxSum X, Y, Z, W;
+#pragma unroll
+                for (int m = 0; m < np1; ++m) {
+                    const Fx p = Dx[m], q = Dy[m], t = Dz[m], np = fx_neg(p), nq = fx_neg(q), nt = fx_neg(t);
+                    X.add(uy(2, m), nq); X.add(uz(1, m), t); X.add(ux(7, m), np);
+                    Y.add(uz(0, m), nt); Y.add(ux(2, m), p); Y.add(uy(7, m), nq);
+                    Z.add(ux(1, m), np); Z.add(uy(0, m), q); Z.add(uz(7, m), nt);
+                    W.add(ux(0, m), np); W.add(uy(1, m), nq); W.add(uz(2, m), nt);
+                }
+                r[3 * nn] = out(X, eE);
+                r[4 * nn] = out(Y, eE);
+                r[5 * nn] = out(Z, eE);
+                r[6 * nn] = out(W, eE) + sU[8 * nn + tid];
+            }
+            {   // q: -div J
+                FxSum X;
+#pragma unroll
+                for (int m = 0; m < np1; ++m) {
+                    X.add(ux(9, m), fx_neg(Dx[m])); X.add(uy(10, m), fx_neg(Dy[m])); X.add(uz(11, m), fx_neg(Dz[m]));
+                }
+                r[8 * nn] = out(X, eJ);
+            }
+        } else if (act) {
+            volume_fp64<P>(a.J, eb, sU, sJ, sD, r);
         }
         // Lift, one thread per face node.  The jump (dU, dJ) to the exterior state
         // enters through the pairs (a, b, s) of flux_pair: with t = s (outward sign)
@@ -410,12 +492,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
             substep_explicit(d, SUB, du, eb + tid, false, a, d.dt, u);
         }
         if (d.filter_on) {
-            if (act)
-                for (int v = 0; v < NV; ++v) sU[v * nn + tid] = u[v];
-            __syncthreads();
-            filter_lowrank<P, NT>(T, sU);
-            if (act)
-                for (int v = 0; v < NV; ++v) u[v] = sU[v * nn + tid];
+            filter_element<P, NT>(T, act, sU, (long long*)fU, s_wordf, u);
         }
         // implicit part after the filter; G at the stage value: G_s = (U_s - R~_s)/(dt a)
         if (act) substep_implicit<SUB>(d, d.sk, a, eb + tid, false, u);
