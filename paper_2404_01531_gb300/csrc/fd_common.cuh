@@ -187,38 +187,44 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
 // centre value.
 //
 // WENO5-Z: with a_k the second difference of stencil k (left, centred, right) and
-// e_k / 2 its slope at the centre, the candidate at the face +-1/2 is
-// v_c + a_k / 8 +- e_k / 4, and beta_k = (13/12) a_k^2 + (e_k / 2)^2.  The kept
-// per-stencil values are h = a/8 and k = (13/12) a^2 + eps; ideal weights
-// (1, 10, 5) towards the right face and (5, 10, 1) towards the left one, the Z
-// weights in the form above.  52 FP64 operations per cell and
-// quantity where a thread per face spends 87.  eps is at least 1e-51, so that
-// products of six indicators stay normal at the lower end.  At the upper end they
-// overflow once an indicator exceeds about 1e51 (stencil differences of about
-// 1e25): the weights then become Inf/NaN and the status word reports it; field
-// values that large are far outside any state of this system.  WIDE (caller-built
-// blocks): indicators above 2^160 are scaled exactly by the power of two of the
-// largest, under which the weights do not change (6% more FP64 slots).
+// e_k its slope at the centre, the candidate at the face +-1/2 is
+// v_c + a_k / 8 +- e_k / 2, and beta_k = (13/12) a_k^2 + e_k^2 (the kept per-stencil
+// values are a and k = (13/12) a^2 + eps); ideal weights (1, 10, 5) towards the
+// right face and (5, 10, 1) towards the left one.  Neighbouring candidates differ by
+// third differences t_0 = a_1 - a_0, t_1 = a_2 - a_1 only, so that
+//   right = v_c + a_1/8 + e_1/2 - (3/8 S_0 t_0 + 5/8 S_2 t_1) / (S_0 + 10 S_1 + 5 S_2),
+//   left  = v_c + a_1/8 - e_1/2 + (5/8 S_0 t_0 + 3/8 S_2 t_1) / (5 S_0 + 10 S_1 + S_2),
+// and with T = b_0 - b_2 the scaled Z weights S_k = (1 + T^2/b_k^2) (b_0 b_1 b_2)^2 are
+// sums of two squares: (b_0 b_1 b_2)^2 + (T b_1 b_2)^2 and its permutations.  44 FP64
+// operations per cell and quantity (52 with the candidates and the squares formed
+// one by one, 87 in a thread per face); the kernels are bound by their number.  eps is
+// at least 1e-51, so that products of six indicators stay normal at the lower end.
+// At the upper end they overflow once an indicator exceeds about 1e51 (stencil
+// differences of about 1e25): the weights then become Inf/NaN and the status word
+// reports it; field values that large are far outside any state of this system.
+// WIDE (caller-built blocks): indicators above 2^160 are scaled exactly by the power
+// of two of the largest, under which the weights do not change.
 template <bool WIDE>
 struct Weno5zLine {
-    double dA, dB, hA, hB, kA, kB, vc, vn, eps;
-    __device__ __forceinline__ double curv(double h) const { return fma((13.0 / 12.0 * 64.0) * h, h, eps); }
+    double dA, dB, aA, aB, kA, kB, tA, vc, vn, eps;
+    __device__ __forceinline__ double curv(double a) const { return fma((13.0 / 12.0) * a, a, eps); }
     __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double weno_eps) {
         eps = fmax(weno_eps, 1e-51);
         const double d01 = v1 - v0;
         dA = v2 - v1;
         dB = v3 - v2;
-        hA = 0.125 * (dA - d01);
-        hB = 0.125 * (dB - dA);
-        kA = curv(hA);
-        kB = curv(hB);
+        aA = dA - d01;
+        aB = dB - dA;
+        tA = aB - aA;
+        kA = curv(aA);
+        kB = curv(aB);
         vc = v2;
         vn = v3;
     }
     template <bool LEFT, bool RIGHT>
     __device__ __forceinline__ void cell(double v4, double& left, double& right) {
-        const double dC = v4 - vn, hC = 0.125 * (dC - dB), kC = curv(hC);
-        const double e0 = fma(4.0, hA, dA), e1 = fma(4.0, hB, dA), e2 = fma(-4.0, hC, dB);   // slopes at the centre
+        const double dC = v4 - vn, aC = dC - dB, tB = aC - aB, kC = curv(aC);
+        const double e0 = fma(0.5, aA, dA), e1 = fma(0.5, aB, dA), e2 = fma(-0.5, aC, dB);   // slopes at the centre
         const double c0 = fma(e0, e0, kA), c1 = fma(e1, e1, kB), c2 = fma(e2, e2, kC);
         double b0 = c0, b1 = c1, b2 = c2;
         if (WIDE) {
@@ -230,21 +236,16 @@ struct Weno5zLine {
                 b2 *= sc;
             }
         }
-        const double t = b0 - b2, t2 = t * t;
-        const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
-        const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1, X = q0 * P0;
-        const double S0 = fma(t2, P0, X), S1 = 10.0 * fma(t2, P1, X), S2 = fma(t2, P2, X);
-        if (RIGHT) {
-            const double g0 = fma(0.5, e0, hA), g1 = fma(0.5, e1, hB), g2 = fma(0.5, e2, hC), T = 5.0 * S2;
-            right = fma(fma(S0, g0, fma(S1, g1, T * g2)), recip_nr((S0 + S1) + T), vc);
-        }
-        if (LEFT) {
-            const double g0 = fma(-0.5, e0, hA), g1 = fma(-0.5, e1, hB), g2 = fma(-0.5, e2, hC), T = 5.0 * S0;
-            left = fma(fma(T, g0, fma(S1, g1, S2 * g2)), recip_nr((T + S1) + S2), vc);
-        }
+        const double t = b0 - b2, w = t * b1, v = b0 * b2, r0 = w * b2, r1 = t * v, r2 = w * b0;
+        const double Y = b1 * v, X = Y * Y;
+        const double S0 = fma(r0, r0, X), S1 = fma(r1, r1, X), S2 = fma(r2, r2, X);
+        const double x = S0 * tA, y = S2 * tB, z = fma(0.125, aB, vc);
+        if (RIGHT) right = fma(fma(-0.375, x, -0.625 * y), recip_nr3(fma(5.0, fma(2.0, S1, S2), S0)), fma(0.5, e1, z));
+        if (LEFT) left = fma(fma(0.625, x, 0.375 * y), recip_nr3(fma(5.0, fma(2.0, S1, S0), S2)), fma(-0.5, e1, z));
         dA = dB; dB = dC;
-        hA = hB; hB = hC;
+        aA = aB; aB = aC;
         kA = kB; kB = kC;
+        tA = tB;
         vc = vn; vn = v4;
     }
 };

@@ -34,6 +34,16 @@ __device__ __forceinline__ double recip_nr(double d) {
     return fma(y, r, y);
 }
 
+// The same in one step of third order, y + y (e + e^2) with e = 1 - d y: the
+// approximation is good to 2^-20 or better, so that e^3 is below 2^-60, in one FP64
+// operation less (the adjoint's recomputation keeps recip_nr and its last bits).
+__device__ __forceinline__ double recip_nr3(double d) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 // 2^-floor(log2 x) for a positive normal x below 2^1022: x times it lies in
 // [1, 2) and the product is exact (integer operations on the exponent field).
 __device__ __forceinline__ double pow2_inv_scale(double x) {
