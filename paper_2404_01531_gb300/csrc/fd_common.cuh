@@ -186,6 +186,45 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
 // a stencil are those of the next one shifted.  All offsets are taken from the
 // centre value.
 //
+// The Z weights S_k = (1 + T^2/b_k^2) (b_0 b_1 b_2)^2, T = b_0 - b_2, in integers:
+// sums of two squares, (b_0 b_1 b_2)^2 + (T b_1 b_2)^2 and its permutations.  Products
+// of the 64-bit fractions f in [1/2, 1) of b and |T| keep the upper half (11
+// multiplications of 4 clocks an SM where an FP64 one takes 16), their powers of two
+// are known, and the sums are formed at the scale of the largest term: cut at 2^-58
+// of the largest, where FP64 rounds each of 10 operations at 2^-53.  No range of
+// indicators overflows.  right and left: S_0 + 10 S_1 + 5 S_2 and 5 S_0 + 10 S_1 + S_2.
+// b_k > 0; where one is not finite the weights mean nothing but are finite.
+struct ZWeights {
+    double s0, s2, right, left;
+};
+__device__ __forceinline__ unsigned long long frac64(unsigned long long bits) { return (bits << 11) | 0x8000000000000000ULL; }
+// a positive integer (as 1 where it is 0), rounded to nearest
+__device__ __forceinline__ double u64_double(unsigned long long a) {
+    a |= 1ULL;
+    const int lz = __clzll((long long)a);
+    const unsigned long long m = a << lz;
+    return __longlong_as_double((long long)((m >> 11) + ((m >> 10) & 1ULL) + ((unsigned long long)(1085 - lz) << 52)));
+}
+__device__ __forceinline__ ZWeights z_weights(double b0, double b1, double b2) {
+    const unsigned long long i0 = fbits(b0), i1 = fbits(b1), i2 = fbits(b2), it = fmag(b0 - b2);
+    const int et = (int)(it >> 52);
+    // half the right shifts of T's terms against the first square, none of them below the least
+    int s0 = (int)(i0 >> 52) - et, s1 = (int)(i1 >> 52) - et, s2 = (int)(i2 >> 52) - et;
+    const int least = min(0, min(s0, min(s1, s2)));
+    const int n0 = 2 * (s0 - least), n1 = 2 * (s1 - least), n2 = 2 * (s2 - least), nX = -2 * least;
+    const unsigned long long f0 = frac64(i0), f1 = frac64(i1), f2 = frac64(i2), ft = it ? frac64(it) : 0ULL;
+    const unsigned long long c0 = __umul64hi(f1, f2), c1 = __umul64hi(f0, f2), c2 = __umul64hi(f0, f1);
+    const unsigned long long r0 = __umul64hi(ft, c0), r1 = __umul64hi(ft, c1), r2 = __umul64hi(ft, c2);
+    const unsigned long long Y = __umul64hi(f1, c1);
+    const unsigned long long q0 = __umul64hi(r0, r0), q1 = __umul64hi(r1, r1), q2 = __umul64hi(r2, r2), qX = __umul64hi(Y, Y);
+    // the largest term is 2^58 or more; five bits of room for the weighted sums
+    auto top = [](unsigned long long q, int n) { return (unsigned)(q >> 32) >> min(n, 31); };
+    const int room = 5 - min(5, __clz((int)(top(q0, n0) | top(q1, n1) | top(q2, n2) | top(qX, nX))));
+    auto down = [&](unsigned long long q, int n) { return q >> min(n + room, 63); };
+    const unsigned long long X = down(qX, nX), S0 = X + down(q0, n0), S1 = X + down(q1, n1), S2 = X + down(q2, n2);
+    return {u64_double(S0), u64_double(S2), u64_double(S0 + 5 * (2 * S1 + S2)), u64_double(S2 + 5 * (2 * S1 + S0))};
+}
+
 // WENO5-Z: with a_k the second difference of stencil k (left, centred, right) and
 // e_k its slope at the centre, the candidate at the face +-1/2 is
 // v_c + a_k / 8 +- e_k / 2, and beta_k = (13/12) a_k^2 + e_k^2 (the kept per-stencil
@@ -193,18 +232,10 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
 // right face and (5, 10, 1) towards the left one.  Neighbouring candidates differ by
 // third differences t_0 = a_1 - a_0, t_1 = a_2 - a_1 only, so that
 //   right = v_c + a_1/8 + e_1/2 - (3/8 S_0 t_0 + 5/8 S_2 t_1) / (S_0 + 10 S_1 + 5 S_2),
-//   left  = v_c + a_1/8 - e_1/2 + (5/8 S_0 t_0 + 3/8 S_2 t_1) / (5 S_0 + 10 S_1 + S_2),
-// and with T = b_0 - b_2 the scaled Z weights S_k = (1 + T^2/b_k^2) (b_0 b_1 b_2)^2 are
-// sums of two squares: (b_0 b_1 b_2)^2 + (T b_1 b_2)^2 and its permutations.  44 FP64
-// operations per cell and quantity (52 with the candidates and the squares formed
-// one by one, 87 in a thread per face); the kernels are bound by their number.  eps is
-// at least 1e-51, so that products of six indicators stay normal at the lower end.
-// At the upper end they overflow once an indicator exceeds about 1e51 (stencil
-// differences of about 1e25): the weights then become Inf/NaN and the status word
-// reports it; field values that large are far outside any state of this system.
-// WIDE (caller-built blocks): indicators above 2^160 are scaled exactly by the power
-// of two of the largest, under which the weights do not change.
-template <bool WIDE>
+//   left  = v_c + a_1/8 - e_1/2 + (5/8 S_0 t_0 + 3/8 S_2 t_1) / (5 S_0 + 10 S_1 + S_2).
+// 29 FP64 operations per cell and quantity, the pipe that bounds these kernels
+// (52 with the candidates formed one by one and the weights in FP64, 87 in a thread
+// per face).  eps is at least 1e-51.
 struct Weno5zLine {
     double dA, dB, aA, aB, kA, kB, tA, vc, vn, eps;
     __device__ __forceinline__ double curv(double a) const { return fma((13.0 / 12.0) * a, a, eps); }
@@ -225,23 +256,10 @@ struct Weno5zLine {
     __device__ __forceinline__ void cell(double v4, double& left, double& right) {
         const double dC = v4 - vn, aC = dC - dB, tB = aC - aB, kC = curv(aC);
         const double e0 = fma(0.5, aA, dA), e1 = fma(0.5, aB, dA), e2 = fma(-0.5, aC, dB);   // slopes at the centre
-        const double c0 = fma(e0, e0, kA), c1 = fma(e1, e1, kB), c2 = fma(e2, e2, kC);
-        double b0 = c0, b1 = c1, b2 = c2;
-        if (WIDE) {
-            const unsigned long long top = umax(fbits(c0), umax(fbits(c1), fbits(c2)));
-            if (top >= (1023ULL + 160) << 52) {
-                const double sc = pow2_inv_scale(__longlong_as_double((long long)top));
-                b0 *= sc;
-                b1 *= sc;
-                b2 *= sc;
-            }
-        }
-        const double t = b0 - b2, w = t * b1, v = b0 * b2, r0 = w * b2, r1 = t * v, r2 = w * b0;
-        const double Y = b1 * v, X = Y * Y;
-        const double S0 = fma(r0, r0, X), S1 = fma(r1, r1, X), S2 = fma(r2, r2, X);
-        const double x = S0 * tA, y = S2 * tB, z = fma(0.125, aB, vc);
-        if (RIGHT) right = fma(fma(-0.375, x, -0.625 * y), recip_nr3(fma(5.0, fma(2.0, S1, S2), S0)), fma(0.5, e1, z));
-        if (LEFT) left = fma(fma(0.625, x, 0.375 * y), recip_nr3(fma(5.0, fma(2.0, S1, S0), S2)), fma(-0.5, e1, z));
+        const ZWeights S = z_weights(fma(e0, e0, kA), fma(e1, e1, kB), fma(e2, e2, kC));
+        const double x = S.s0 * tA, y = S.s2 * tB, z = fma(0.125, aB, vc);
+        if (RIGHT) right = fma(fma(-0.375, x, -0.625 * y), recip_nr3(S.right), fma(0.5, e1, z));
+        if (LEFT) left = fma(fma(0.625, x, 0.375 * y), recip_nr3(S.left), fma(-0.5, e1, z));
         dA = dB; dB = dC;
         aA = aB; aB = aC;
         kA = kB; kB = kC;
@@ -314,7 +332,7 @@ struct Mp5Line {
     }
 };
 
-template <int RECON> struct LineOf { using type = Weno5zLine<false>; };
+template <int RECON> struct LineOf { using type = Weno5zLine; };
 template <> struct LineOf<FFE_RECON_MP5> { using type = Mp5Line; };
 
 // Where line (ta, tb) of direction k starts in an extended block: its first ghost,

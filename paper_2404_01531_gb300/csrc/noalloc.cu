@@ -77,13 +77,13 @@ __global__ void __launch_bounds__(32) k_na_flux(NA a) {
         const unsigned long long sb = neg ? 0x8000000000000000ULL : 0ULL;
         double* fa = a.F + (((int64_t)k * NV + qa) * a.n + w) * a.nface + line;
         double* fb = pr < 4 ? a.F + (((int64_t)k * NV + qb) * a.n + w) * a.nface + line : nullptr;
-        recon_lines<Weno5zLine<true>>(pa, pb, stride, sb, nc, a.eps,
-                                      [&](int m, double La, double Ra, double Sa, double Lb, double Rb, double Sb) {
-                                          double Fa, Fb;
-                                          rusanov_pair(La, Ra, Sa, Lb, Rb, Sb, a.corr, Fa, Fb);
-                                          fa[m * nl] = Fa;
-                                          if (fb) fb[m * nl] = __longlong_as_double((long long)(fbits(Fb) ^ sb));
-                                      });
+        recon_lines<Weno5zLine>(pa, pb, stride, sb, nc, a.eps,
+                                [&](int m, double La, double Ra, double Sa, double Lb, double Rb, double Sb) {
+                                    double Fa, Fb;
+                                    rusanov_pair(La, Ra, Sa, Lb, Rb, Sb, a.corr, Fa, Fb);
+                                    fa[m * nl] = Fa;
+                                    if (fb) fb[m * nl] = __longlong_as_double((long long)(fbits(Fb) ^ sb));
+                                });
     }
 }
 

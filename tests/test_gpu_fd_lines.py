@@ -37,3 +37,27 @@ def test_shell_lines(ffe, P, recon, corr):  # noqa: F811
     cfg["params"].update(eta=7.0, recon=recon, fd_corrector=corr)
     pr = Problem(cfg)
     assert _rhs_parity(ffe, cfg, _random_state(pr, P, 77 + P), pr) <= 1e-11
+
+
+@pytest.mark.parametrize("kind", ["constant", "spread", "steps", "large"])
+def test_box_lines_indicators(ffe, kind):  # noqa: F811
+    """Smoothness indicators that are equal, 1e-50 apart, zero next to order one, or of order 1e30."""
+    cfg = W.breakdown(nx=3, ny=2, nz=1, P=4, x_half=0.1)
+    cfg["params"].update(eta=0.0, recon=0, fd_corrector=0)
+    pr = Problem(cfg)
+    st = _random_state(pr, 4, 5)
+    rng = np.random.default_rng(6)
+    st["mask"][:] = 1
+    u = st["ufd"]
+    if kind == "constant":
+        u[:] = np.arange(1.0, 10.0)[:, None, None, None, None]
+    elif kind == "spread":
+        u *= 10.0 ** rng.uniform(-25.0, 0.0, size=u.shape)
+    elif kind == "steps":
+        # heights at random, q~ = 0: between two heights, and in rounded values such as J~,
+        # b_0 - b_2 cancels and the last bit of the values decides the weights
+        u[:] = np.where(rng.random(u.shape) < 0.4, 1.0 + rng.random(u.shape), 1.0)
+        u[8] = 0.0
+    else:
+        u *= 1e15
+    assert _rhs_parity(ffe, cfg, st, pr) <= 1e-11
