@@ -186,18 +186,38 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
 // a stencil are those of the next one shifted.  All offsets are taken from the
 // centre value.
 //
-// The Z weights S_k = (1 + T^2/b_k^2) (b_0 b_1 b_2)^2, T = b_0 - b_2, in integers:
-// sums of two squares, (b_0 b_1 b_2)^2 + (T b_1 b_2)^2 and its permutations.  Products
-// of the 64-bit fractions f in [1/2, 1) of b and |T| keep the upper half (11
-// multiplications of 4 clocks an SM where an FP64 one takes 16), their powers of two
-// are known, and the sums are formed at the scale of the largest term: cut at 2^-58
-// of the largest, where FP64 rounds each of 10 operations at 2^-53.  No range of
-// indicators overflows.  right and left: S_0 + 10 S_1 + 5 S_2 and 5 S_0 + 10 S_1 + S_2.
-// b_k > 0; where one is not finite the weights mean nothing but are finite.
-struct ZWeights {
-    double s0, s2, right, left;
+// The smoothness indicators b_k = (13/12) a_k^2 + eps + e_k^2 and the Z weights
+// S_k = (1 + T^2/b_k^2) (b_0 b_1 b_2)^2, T = b_0 - b_2, in integers: every term is a
+// square, and the weights are sums of two of them, (b_0 b_1 b_2)^2 + (T b_1 b_2)^2 and
+// its permutations.  A positive number is m 2^(e - 1022 - 64); products of 64-bit
+// fractions m keep the upper half (4 clocks of an SM where an FP64 product takes 16),
+// sums the bits that both terms have at the larger one's scale.  Cut at 2^-58 of the
+// largest term, where FP64 rounds each of 16 operations at 2^-53.  No range of
+// indicators overflows; arguments that are not finite give finite weights without
+// meaning (the third differences they multiply are not finite either).
+struct Pos {
+    unsigned long long m;
+    int e;
 };
-__device__ __forceinline__ unsigned long long frac64(unsigned long long bits) { return (bits << 11) | 0x8000000000000000ULL; }
+struct ZWeights {
+    double s0, s2, right, left;   // S_0, S_2, S_0 + 10 S_1 + 5 S_2 and 5 S_0 + 10 S_1 + S_2
+};
+__device__ __forceinline__ Pos pos_of(double x) {
+    return {(fbits(x) << 11) | 0x8000000000000000ULL, (int)(fmag(x) >> 52)};
+}
+__device__ __forceinline__ Pos pos_square(double x) {   // 2^62 <= m; a zero counts as 2^-2044
+    const Pos p = pos_of(x);
+    return {__umul64hi(p.m, p.m), 2 * p.e - 1022};
+}
+__device__ __forceinline__ Pos pos_add(Pos x, Pos y) {
+    const int e = max(x.e, y.e) + 1;
+    return {(x.m >> min(e - x.e, 63)) + (y.m >> min(e - y.e, 63)), e};
+}
+// m >= 2^32 to 2^63 <= m
+__device__ __forceinline__ Pos pos_norm(Pos x) {
+    const int lz = __clz((int)(x.m >> 32));
+    return {x.m << lz, x.e - lz};
+}
 // a positive integer (as 1 where it is 0), rounded to nearest
 __device__ __forceinline__ double u64_double(unsigned long long a) {
     a |= 1ULL;
@@ -205,17 +225,18 @@ __device__ __forceinline__ double u64_double(unsigned long long a) {
     const unsigned long long m = a << lz;
     return __longlong_as_double((long long)((m >> 11) + ((m >> 10) & 1ULL) + ((unsigned long long)(1085 - lz) << 52)));
 }
-__device__ __forceinline__ ZWeights z_weights(double b0, double b1, double b2) {
-    const unsigned long long i0 = fbits(b0), i1 = fbits(b1), i2 = fbits(b2), it = fmag(b0 - b2);
-    const int et = (int)(it >> 52);
+// b_k of magnitude 2^63 <= m
+__device__ __forceinline__ ZWeights z_weights(Pos b0, Pos b1, Pos b2) {
+    const int eM = max(b0.e, b2.e);
+    const unsigned long long u = b0.m >> min(eM - b0.e, 63), v = b2.m >> min(eM - b2.e, 63), tt = u > v ? u - v : v - u;
+    const int lzt = __clzll((long long)(tt | 1ULL)), et = eM - lzt;
+    const unsigned long long ft = tt << lzt;
     // half the right shifts of T's terms against the first square, none of them below the least
-    int s0 = (int)(i0 >> 52) - et, s1 = (int)(i1 >> 52) - et, s2 = (int)(i2 >> 52) - et;
-    const int least = min(0, min(s0, min(s1, s2)));
+    const int s0 = b0.e - et, s1 = b1.e - et, s2 = b2.e - et, least = min(0, min(s0, min(s1, s2)));
     const int n0 = 2 * (s0 - least), n1 = 2 * (s1 - least), n2 = 2 * (s2 - least), nX = -2 * least;
-    const unsigned long long f0 = frac64(i0), f1 = frac64(i1), f2 = frac64(i2), ft = it ? frac64(it) : 0ULL;
-    const unsigned long long c0 = __umul64hi(f1, f2), c1 = __umul64hi(f0, f2), c2 = __umul64hi(f0, f1);
+    const unsigned long long c0 = __umul64hi(b1.m, b2.m), c1 = __umul64hi(b0.m, b2.m), c2 = __umul64hi(b0.m, b1.m);
     const unsigned long long r0 = __umul64hi(ft, c0), r1 = __umul64hi(ft, c1), r2 = __umul64hi(ft, c2);
-    const unsigned long long Y = __umul64hi(f1, c1);
+    const unsigned long long Y = __umul64hi(b1.m, c1);
     const unsigned long long q0 = __umul64hi(r0, r0), q1 = __umul64hi(r1, r1), q2 = __umul64hi(r2, r2), qX = __umul64hi(Y, Y);
     // the largest term is 2^58 or more; five bits of room for the weighted sums
     auto top = [](unsigned long long q, int n) { return (unsigned)(q >> 32) >> min(n, 31); };
@@ -233,14 +254,18 @@ __device__ __forceinline__ ZWeights z_weights(double b0, double b1, double b2) {
 // third differences t_0 = a_1 - a_0, t_1 = a_2 - a_1 only, so that
 //   right = v_c + a_1/8 + e_1/2 - (3/8 S_0 t_0 + 5/8 S_2 t_1) / (S_0 + 10 S_1 + 5 S_2),
 //   left  = v_c + a_1/8 - e_1/2 + (5/8 S_0 t_0 + 3/8 S_2 t_1) / (5 S_0 + 10 S_1 + S_2).
-// 29 FP64 operations per cell and quantity, the pipe that bounds these kernels
+// 23 FP64 operations per cell and quantity, the pipe that bounds these kernels
 // (52 with the candidates formed one by one and the weights in FP64, 87 in a thread
 // per face).  eps is at least 1e-51.
 struct Weno5zLine {
-    double dA, dB, aA, aB, kA, kB, tA, vc, vn, eps;
-    __device__ __forceinline__ double curv(double a) const { return fma((13.0 / 12.0) * a, a, eps); }
+    double dA, dB, aA, aB, tA, vc, vn;
+    Pos kA, kB, eps;
+    __device__ __forceinline__ Pos curv(double a) const {
+        const Pos q = pos_square(a);
+        return pos_add({__umul64hi(q.m, 0x8aaaaaaaaaaaaaabULL), q.e + 1}, eps);   // 13/24 2^64
+    }
     __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double weno_eps) {
-        eps = fmax(weno_eps, 1e-51);
+        eps = pos_of(fmax(weno_eps, 1e-51));
         const double d01 = v1 - v0;
         dA = v2 - v1;
         dB = v3 - v2;
@@ -254,9 +279,11 @@ struct Weno5zLine {
     }
     template <bool LEFT, bool RIGHT>
     __device__ __forceinline__ void cell(double v4, double& left, double& right) {
-        const double dC = v4 - vn, aC = dC - dB, tB = aC - aB, kC = curv(aC);
+        const double dC = v4 - vn, aC = dC - dB, tB = aC - aB;
+        const Pos kC = curv(aC);
         const double e0 = fma(0.5, aA, dA), e1 = fma(0.5, aB, dA), e2 = fma(-0.5, aC, dB);   // slopes at the centre
-        const ZWeights S = z_weights(fma(e0, e0, kA), fma(e1, e1, kB), fma(e2, e2, kC));
+        const ZWeights S = z_weights(pos_norm(pos_add(pos_square(e0), kA)), pos_norm(pos_add(pos_square(e1), kB)),
+                                     pos_norm(pos_add(pos_square(e2), kC)));
         const double x = S.s0 * tA, y = S.s2 * tB, z = fma(0.125, aB, vc);
         if (RIGHT) right = fma(fma(-0.375, x, -0.625 * y), recip_nr3(S.right), fma(0.5, e1, z));
         if (LEFT) left = fma(fma(0.625, x, 0.375 * y), recip_nr3(S.left), fma(-0.5, e1, z));

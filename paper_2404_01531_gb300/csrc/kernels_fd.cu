@@ -323,11 +323,11 @@ __global__ void k_fd_fill(Dev d, const int* list, int ci, int w0, Field U, Field
 // from one set of smoothness indicators (Weno5zLine), for the two quantities
 // that a pair of flux components needs, so that the flux is formed in registers;
 // the two components of J~ across the direction are not reconstructed.  At P = 5
-// that is 380 FP64 operations per face, and as much time again hidden on the integer
-// pipes for the weights (z_weights), against about 1100 of a thread per face: 384
-// elements 3.44 -> 1.84 ms with 610 of them; two steps of the 64x8x8 current sheet
-// 14.8 -> 13.7 ms from 610 to 530 and 13.7 -> 11.6 ms with the weights in integers; MP5
-// on 125 elements 1.53 -> 0.41 ms.
+// that is 320 FP64 operations per face, the indicators and weights hidden on the
+// integer pipes (z_weights), against about 1100 of a thread per face: 384 elements
+// 3.44 -> 1.84 ms with 610 of them; two steps of the 64x8x8 current sheet 14.8 -> 13.7
+// ms from 610 to 530, 11.6 with the weights in integers, 10.4 with the indicators too;
+// MP5 on 125 elements 1.53 -> 0.41 ms.
 template <int RECON>
 __global__ void __launch_bounds__(64, 8) k_fd_flux(Dev d, const int* list, int ci, int w0) {
     const int n = chunk_n(d, ci, w0);
