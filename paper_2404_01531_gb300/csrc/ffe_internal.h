@@ -53,6 +53,8 @@ struct Tables {
     double Dabs;                   // largest row sum of |D|
     int fx_d;                      // D in units of 2^-fx_d (its rows sum to less than 2^59)
     Fx FxD[MAXNP][MAXNP];
+    int fx_pi;                     // Pi in units of 2^-56, for a field of fx_pi bits
+    Fx FxPi[MAXNP][MAXNP];
     double Pi[MAXNP][MAXNP];       // projection on Legendre modes p <= P - M
     double P2F[MAXNC][MAXNP];      // DG -> FD (Lagrange evaluation at subcell centres)
     double F2D[MAXNP][MAXNC];      // FD -> DG (6-point Lagrange, shifted inside)
@@ -60,9 +62,11 @@ struct Tables {
 };
 
 // Constants of the pointwise stiff solve with dta = dt a: c = eta dta, 1/(1 + kappa dta)
-// of the two cleaning fields, -c/(1+c) and eta/(1+c).
+// of the two cleaning fields, -c/(1+c) and eta/(1+c); and the factors of the explicit
+// parts (substep_explicit): dt, dt (1 - a), dt/4, dt b, dt h, dt z, dt/6, 2 dt/3.
 struct SolveK {
     double dta, c, ipsi, iphi, cm, eta1;
+    double dt, dt1a, dt4, dtb, dth, dtz, dt6, dt23;
 };
 inline SolveK solve_consts(double eta, double kpsi, double kphi, double dt) {
     SolveK k;
@@ -72,6 +76,14 @@ inline SolveK solve_consts(double eta, double kpsi, double kphi, double dt) {
     k.iphi = 1.0 / (1.0 + kphi * k.dta);
     k.cm = -k.c / (1.0 + k.c);
     k.eta1 = eta / (1.0 + k.c);
+    k.dt = dt;
+    k.dt1a = dt * (1.0 - IM_A);
+    k.dt4 = 0.25 * dt;
+    k.dtb = dt * IM_B;
+    k.dth = dt * IM_H;
+    k.dtz = dt * (0.5 - IM_B - IM_H - IM_A);
+    k.dt6 = dt / 6.0;
+    k.dt23 = 2.0 * dt / 3.0;
     return k;
 }
 

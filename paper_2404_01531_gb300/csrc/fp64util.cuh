@@ -14,6 +14,9 @@ __device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigne
 __device__ __forceinline__ double flip(double x, unsigned long long sign) {
     return __longlong_as_double((long long)(fbits(x) ^ sign));
 }
+__device__ __forceinline__ bool is_finite(double x) { return fmag(x) < 0x7ff0000000000000ULL; }
+// x > y for x >= 0 and y >= 0 (false where one is NaN, as the FP64 comparison)
+__device__ __forceinline__ bool above(double x, double y) { return fbits(x) > fbits(y) && fbits(x) <= 0x7ff0000000000000ULL; }
 __device__ __forceinline__ bool is_zero(double x) { return fmag(x) == 0; }
 
 // 1/d for a normal d whose reciprocal is normal: the hardware

@@ -217,6 +217,16 @@ void build_tables(int P, double fa, double fb, int M, Tables& T) {
     T.fx_d = 59 - (int)ceil(log2(T.Dabs));
     for (int i = 0; i < np1; ++i)
         for (int j = 0; j < np1; ++j) T.FxD[i][j] = fx_limbs_host(ldexpl((ld)T.D[i][j], T.fx_d));
+    double row = 1.0;
+    for (int i = 0; i < np1; ++i) {
+        double s = 0.0;
+        for (int j = 0; j < np1; ++j) {
+            s += fabs(T.Pi[i][j]);
+            T.FxPi[i][j] = fx_limbs_host(ldexpl((ld)T.Pi[i][j], 56));
+        }
+        row = std::max(row, s);
+    }
+    T.fx_pi = 58 - (int)ceil(3.0 * log2(row));
     fixed_filter(T);
     std::vector<ld> xc(nc);
     const ld dxi = 2.0L / nc;

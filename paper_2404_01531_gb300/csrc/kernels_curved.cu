@@ -9,6 +9,7 @@
 // filter, stiff solve, clamp, indicator).  The stiff solve, clamp and indicator
 // use the gamma inner product.
 #include "dgfilter.cuh"
+#include "dgtci.cuh"
 #include "ffe_internal.h"
 #include "physics.cuh"
 #include "physics_gen.cuh"
@@ -23,36 +24,15 @@ struct DGC {
     static constexpr int nn = np1 * np1 * np1;
     static constexpr int nf = np1 * np1;
     static constexpr int NT = ((nn + 31) / 32) * 32;
-    static constexpr int NW = NT / 32;
     static constexpr int FR = (6 * nf + NT - 1) / NT;   // face nodes per thread
     // CTAs per SM the registers are bounded for (see k_dg_curved)
     static constexpr int CTAS = NT <= 128 ? (KS ? 3 : 4) : 2;
-    // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn] | fixed point:
+    // shared doubles: U[9][nn] (later the filter's buffer) | J[3][nn] | fixed point:
     // U and J [12][nn], Kerr-Schild: F[27][nn] as doubles, then in fixed point (later the
-    // filter's fields) | dU/dt[9][nn] | red[2][NW] and the flag
+    // filter's and the indicator's fields) | dU/dt[9][nn] | red[2] and the flag
     static constexpr int NS = KS ? 30 : 15;
-    static constexpr int SMEM = ((18 + NS) * nn + 2 * NW + 1) * 8;
+    static constexpr int SMEM = ((18 + NS) * nn + 3) * 8;
 };
-
-template <int NW>
-__device__ __forceinline__ void block_sum2c(double& x, double& y, double* red) {
-    for (int o = 16; o > 0; o >>= 1) {
-        x += __shfl_down_sync(0xffffffffu, x, o);
-        y += __shfl_down_sync(0xffffffffu, y, o);
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) { red[w] = x; red[NW + w] = y; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sx = 0.0, sy = 0.0;
-        for (int i = 0; i < NW; ++i) { sx += red[i]; sy += red[NW + i]; }
-        red[0] = sx;
-        red[NW] = sy;
-    }
-    __syncthreads();
-    x = red[0];
-    y = red[NW];
-}
 
 // neighbour's node for my face node (ta, tb) of face f
 template <int P>
@@ -194,13 +174,13 @@ __device__ __forceinline__ void flux_normal_gen(const double* n, const PM& m, co
 }
 
 // One element of order P processed by a block of NT threads (NT >= (P+1)^3).
-// s_word, s_wordf [NV]: the largest words (fx_word) of the volume term's blocks, zero
-// on entry and on return, and of the filter's.
+// s_word [NV]: the largest words (fx_word) of the volume term's blocks, zero on entry
+// and on return; s_wordf [NV + 1]: of the filter's and of |B~|.
 template <int P, int NT, int SUB, bool KS>
 __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, int e, double* sm, unsigned* s_word,
                                                unsigned* s_wordf) {
     using K = DGC<P, KS>;
-    constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NW = NT / 32;
+    constexpr int np1 = K::np1, nn = K::nn, nf = K::nf;
     double* sU = sm;                 // [9][nn]
     double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
     double* sF = sJ + 3 * nn;        // fixed point [12][nn]; Kerr-Schild: [3][9][nn] F^j
@@ -250,7 +230,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
         if ((tid & 31) == 0) atomicMax(s_word + b, word[b]);
     }
     __syncthreads();
-    if (tid < NV) s_wordf[tid] = 0;
+    if (tid <= NV) s_wordf[tid] = 0;
     unsigned top = 0;
     for (int b = 0; b < NB; ++b) top = max(top, s_word[b]);
     const bool fixed = !d.fp64_lines && top < (unsigned)FX_EMAX << 20;
@@ -407,7 +387,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
     if (act) {
         if (SUB != SUB_C)
             for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
-        substep_explicit(d, SUB, du, eb + tid, false, a, dt, u);
+        substep_explicit(SUB, du, eb + tid, false, a, solve_k(d, e), u);
     }
     if (d.filter_on) {
         filter_element<P, NT>(T, act, sU, (long long*)sF, s_wordf, u);
@@ -433,28 +413,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
     }
     bool flagged = false;
     if (d.tci_on) {
-        if (act) sU[tid] = mag;
-        __syncthreads();
-        double low = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            const int stride = k == 0 ? 1 : (k == 1 ? np1 : np1 * np1);
-            if (act) {
-                const int base = tid - ci[k] * stride;
-                double acc = 0.0;
-                for (int mm = 0; mm < np1; ++mm) acc = fma(T.Pi[ci[k]][mm], sU[k * nn + base + mm * stride], acc);
-                if (k < 2) sU[(k + 1) * nn + tid] = acc;
-                else low = acc;
-            }
-            __syncthreads();
-        }
-        double num = 0.0, den = 0.0;
-        if (act) {
-            const double uh = mag - low;
-            num = uh * uh;
-            den = mag * mag;
-        }
-        block_sum2c<NW>(num, den, red);
-        const double ratio = den > 0.0 ? sqrt(num / den) : 0.0;
+        const double ratio = indicator_ratio<P, NT>(T, act, mag, (long long*)sF, s_wordf + NV, red);
         const double thr = d.thr_dgP[P];
         if (tid == 0) {
             int fl = ratio > thr;
@@ -465,10 +424,10 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
             } else {
                 fl = 0;
             }
-            red[2 * NW] = fl;
+            red[2] = fl;
         }
         __syncthreads();
-        flagged = red[2 * NW] != 0.0;
+        flagged = red[2] != 0.0;
     }
     if (!flagged && tid == 0) {
         atomicAdd(d.units, (unsigned long long)nn);
@@ -478,7 +437,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
         bool bad = false;
         for (int v = 0; v < NV; ++v) {
             a.Uout.dg(v)[eb + tid] = u[v];
-            bad |= !isfinite(u[v]);
+            bad |= !is_finite(u[v]);
         }
         if (bad) atomic_status(d, 1);
     }
@@ -502,7 +461,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
 template <int P, int SUB, bool KS>
 __global__ void __launch_bounds__(DGC<P, KS>::NT, DGC<P, KS>::CTAS) k_dg_curved(Dev d, SubArgs a, const int* list, int ci) {
     extern __shared__ double sm[];
-    __shared__ unsigned s_word[NV], s_wordf[NV];
+    __shared__ unsigned s_word[NV], s_wordf[NV + 1];
     if (threadIdx.x < NV) s_word[threadIdx.x] = 0;
     __syncthreads();
     const int nwork = d.counts[ci];

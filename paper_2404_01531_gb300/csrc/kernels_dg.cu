@@ -13,6 +13,7 @@
 #include <cstdio>
 
 #include "dgfilter.cuh"
+#include "dgtci.cuh"
 #include "fd_common.cuh"
 #include "ffe_internal.h"
 #include "physics.cuh"
@@ -29,14 +30,13 @@ struct DGK {
     static constexpr int nn = np1 * np1 * np1;
     static constexpr int nf = np1 * np1;
     static constexpr int NT = ((nn + 31) / 32) * 32;
-    static constexpr int NW = NT / 32;
     static constexpr int FR = (6 * nf + NT - 1) / NT;   // face nodes per thread
     // CTAs per SM the registers are bounded for
     static constexpr int CTAS = P == 6 ? 2 : 3;
-    // shared doubles: U[9][nn] (later the filter's and indicator's buffer) | J[3][nn] | dU/dt[9][nn] |
-    // fixed point: U and J [12][nn] (later the filter's fields) | red[2][NW] | D scaled by the
+    // shared doubles: U[9][nn] (later the filter's buffer) | J[3][nn] | dU/dt[9][nn] |
+    // fixed point: U and J [12][nn] (later the filter's and the indicator's fields) | red[2] | D scaled by the
     // element's d xi/d x, per axis [3][np1][np1]
-    static constexpr int SMEM = (33 * nn + 2 * NW + 3 * nf) * 8;
+    static constexpr int SMEM = (33 * nn + 2 + 3 * nf) * 8;
 };
 
 // ---------------------------------------------------------------------------
@@ -184,26 +184,6 @@ void launch_stage12(const Dev& d, Field un, Field Ua, Field G1, Field G2, Field 
     g_launch_counter += 1;
 }
 
-// Deterministic block sum of two values (warp shuffles, then warp 0 in order).
-template <int NW>
-__device__ __forceinline__ void block_sum2(double& x, double& y, double* red) {
-    for (int o = 16; o > 0; o >>= 1) {
-        x += __shfl_down_sync(0xffffffffu, x, o);
-        y += __shfl_down_sync(0xffffffffu, y, o);
-    }
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) { red[w] = x; red[NW + w] = y; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sx = 0.0, sy = 0.0;
-        for (int i = 0; i < NW; ++i) { sx += red[i]; sy += red[NW + i]; }
-        red[0] = sx; red[NW] = sy;
-    }
-    __syncthreads();
-    x = red[0];
-    y = red[NW];
-}
-
 // tangential node coordinates of face direction dd: t1 < t2 are the other two axes
 __device__ __forceinline__ void face_axes(int dd, int& t1, int& t2) {
     t1 = dd == 0 ? 1 : 0;
@@ -308,17 +288,17 @@ __device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* s
 template <int P, int SUB>
 __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, SubArgs a) {
     using K = DGK<P>;
-    constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NT = K::NT, NW = K::NW;
+    constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NT = K::NT;
     extern __shared__ double sm[];
     double* sU = sm;                 // [9][nn]
     double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
     double* sR = sJ + 3 * nn;        // [9][nn] dU/dt
     Fx* fU = (Fx*)(sR + 9 * nn);     // [12][nn] U and J~ in fixed point
     double* red = sR + 21 * nn;
-    double* sD = red + 2 * NW;       // [3][np1][np1]: (d xi^a/d x^a) D
+    double* sD = red + 2;            // [3][np1][np1]: (d xi^a/d x^a) D
     Fx* fD = (Fx*)sD;
     __shared__ int s_flag;
-    __shared__ unsigned s_word[3], s_wordf[NV];  // largest words (fx_word) of the volume term's blocks, of the filter's
+    __shared__ unsigned s_word[3], s_wordf[NV + 1];  // largest words (fx_word) of the volume term's blocks, of the filter's, of |B~|
     const Tables& T = *d.tab;
     const int tid = threadIdx.x;
     const bool act = tid < nn;
@@ -356,7 +336,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
         const double rows = T.Dabs * (fabs(sx) + fabs(sy) + fabs(sz));   // bounds the sums' |D| entries
         const int eD = (int)(fx_word(rows) >> 20);
         __syncthreads();
-        if (tid < NV) s_wordf[tid] = 0;
+        if (tid <= NV) s_wordf[tid] = 0;
         const int eE = fx_exp(s_word[0]), eB = fx_exp(s_word[1]), eJ = fx_exp(s_word[2]);
         const bool fixed = max(eE, max(eB, eJ)) < FX_EMAX && eD > 1023 - 60 && eD < 1023 + 60;
         for (int t = tid; t < 3 * nf; t += NT) {
@@ -489,7 +469,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
         if (act) {
             if (SUB != SUB_C)
                 for (int v = 0; v < NV; ++v) a.Fout.dg(v)[eb + tid] = du[v];
-            substep_explicit(d, SUB, du, eb + tid, false, a, d.dt, u);
+            substep_explicit(SUB, du, eb + tid, false, a, d.sk, u);
         }
         if (d.filter_on) {
             filter_element<P, NT>(T, act, sU, (long long*)fU, s_wordf, u);
@@ -498,35 +478,8 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
         if (act) substep_implicit<SUB>(d, d.sk, a, eb + tid, false, u);
         bool flagged = false;
         if (d.tci_on) {
-            // u = |B~| ; u^ = u - (Pi x Pi x Pi) u ; ratio = sqrt(sum u^2 / sum u^)
-            double mag = act ? sqrt(fma(u[5], u[5], fma(u[4], u[4], u[3] * u[3]))) : 0.0;
-            if (act) sU[tid] = mag;
-            __syncthreads();
-            if (act) {
-                const int ox = np1 * (j + np1 * k);
-                double acc = 0.0;
-                for (int m = 0; m < np1; ++m) acc = fma(T.Pi[i][m], sU[ox + m], acc);
-                sU[nn + tid] = acc;
-            }
-            __syncthreads();
-            if (act) {
-                const int oy = i + np1 * np1 * k;
-                double acc = 0.0;
-                for (int m = 0; m < np1; ++m) acc = fma(T.Pi[j][m], sU[nn + oy + np1 * m], acc);
-                sU[2 * nn + tid] = acc;
-            }
-            __syncthreads();
-            double num = 0.0, den = 0.0;
-            if (act) {
-                const int oz = i + np1 * j;
-                double acc = 0.0;
-                for (int m = 0; m < np1; ++m) acc = fma(T.Pi[k][m], sU[2 * nn + oz + np1 * np1 * m], acc);
-                const double uh = mag - acc;
-                num = uh * uh;
-                den = mag * mag;
-            }
-            block_sum2<NW>(num, den, red);
-            const double ratio = den > 0.0 ? sqrt(num / den) : 0.0;
+            const double mag = act ? sqrt(fma(u[5], u[5], fma(u[4], u[4], u[3] * u[3]))) : 0.0;
+            const double ratio = indicator_ratio<P, NT>(T, act, mag, (long long*)fU, &s_wordf[NV], red);
             if (tid == 0) {
                 int fl = ratio > d.thr_dg;
                 if (fabs(ratio - d.thr_dg) <= 1e-12 * d.thr_dg) d.near_list[atomicAdd(&d.counts[3], 1) & 4095] = e;
@@ -549,7 +502,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
             bool bad = false;
             for (int v = 0; v < NV; ++v) {
                 a.Uout.dg(v)[eb + tid] = u[v];
-                bad |= !isfinite(u[v]);
+                bad |= !is_finite(u[v]);
             }
             if (bad) atomic_status(d, 1);
         }

@@ -601,7 +601,7 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
         if (SUB != SUB_C)
             for (int v = 0; v < NV; ++v) a.Fout.fd(v)[p] = du[v];
         double u[NV];
-        substep_explicit(d, SUB, du, p, true, a, dt_of(d, e), u);
+        substep_explicit(SUB, du, p, true, a, solve_k(d, e), u);
         if (KS) {
             if (SUB != SUB_C && !stiff_solve_gen(u, m, d, dt_of(d, e) * IM_A)) atomic_status(d, 2);
             if (d.mode != FFE_RELAX) hard_clamp_gen(u, m);
@@ -616,7 +616,7 @@ __global__ void k_fd_update(Dev d, const int* list, int ci, int w0, SubArgs a) {
         bool bad = false;
         for (int v = 0; v < NV; ++v) {
             a.Uout.fd(v)[p] = u[v];
-            bad |= !isfinite(u[v]);
+            bad |= !is_finite(u[v]);
         }
         if (bad) atomic_status(d, 1);
     }

@@ -205,7 +205,7 @@ __device__ __forceinline__ bool implicit_stage_flat(double* U, const Dev& d, con
         if (d.eta != 0.0) {
             const double f = dot3(E, B) * ib2, r = f * k.cm;   // r = f (1/(1+c) - 1)
             const double e0[3] = {fma(r, B[0], E[0]), fma(r, B[1], E[1]), fma(r, B[2], E[2])};
-            if (!(dot3(e0, e0) > B2)) {
+            if (!above(dot3(e0, e0), B2)) {
                 E[0] = e0[0]; E[1] = e0[1]; E[2] = e0[2];
                 const double g = f * k.eta1;
                 jp[0] = g * B[0]; jp[1] = g * B[1]; jp[2] = g * B[2];

@@ -18,24 +18,22 @@ __device__ __forceinline__ void atomic_status(const Dev& d, int bits) { atomicOr
 // followed by the algebraic clamp when the constraint mode asks for it.  DG
 // kernels filter R between the explicit and the implicit part.
 // Explicit part R of the substep (DG elements filter R before the implicit part).
-__device__ __forceinline__ void substep_explicit(const Dev& d, int sub, const double* f, int64_t p, bool isfd,
-                                                 const SubArgs& a, double dt, double* u) {
+__device__ __forceinline__ void substep_explicit(int sub, const double* f, int64_t p, bool isfd, const SubArgs& a,
+                                                 const SolveK& k, double* u) {
     auto ld = [&](const Field& F, int v) { return isfd ? F.fd(v)[p] : F.dg(v)[p]; };
     const int gv[NG] = {0, 1, 2, 6, 7};
     for (int v = 0; v < NV; ++v) u[v] = ld(a.un, v);
     if (sub == SUB_A) {
-        for (int v = 0; v < NV; ++v) u[v] = fma(dt, f[v], u[v]);
-        for (int c = 0; c < NG; ++c) u[gv[c]] = fma(dt * (1.0 - IM_A), ld(a.G2, c), u[gv[c]]);
+        for (int v = 0; v < NV; ++v) u[v] = fma(k.dt, f[v], u[v]);
+        for (int c = 0; c < NG; ++c) u[gv[c]] = fma(k.dt1a, ld(a.G2, c), u[gv[c]]);
     } else if (sub == SUB_B) {
-        for (int v = 0; v < NV; ++v) u[v] = fma(0.25 * dt, ld(a.F2, v) + f[v], u[v]);
-        const double z = 0.5 - IM_B - IM_H - IM_A;
+        for (int v = 0; v < NV; ++v) u[v] = fma(k.dt4, ld(a.F2, v) + f[v], u[v]);
         for (int c = 0; c < NG; ++c)
-            u[gv[c]] = fma(dt, IM_B * ld(a.G1, c) + IM_H * ld(a.G2, c) + z * ld(a.G3, c), u[gv[c]]);
+            u[gv[c]] = fma(k.dtb, ld(a.G1, c), fma(k.dth, ld(a.G2, c), fma(k.dtz, ld(a.G3, c), u[gv[c]])));
     } else {
-        for (int v = 0; v < NV; ++v)
-            u[v] = fma(dt, (ld(a.F2, v) + ld(a.F3, v)) * (1.0 / 6.0) + f[v] * (2.0 / 3.0), u[v]);
+        for (int v = 0; v < NV; ++v) u[v] = fma(k.dt6, ld(a.F2, v) + ld(a.F3, v), fma(k.dt23, f[v], u[v]));
         for (int c = 0; c < NG; ++c)
-            u[gv[c]] = fma(dt, (ld(a.G2, c) + ld(a.G3, c)) * (1.0 / 6.0) + ld(a.G4, c) * (2.0 / 3.0), u[gv[c]]);
+            u[gv[c]] = fma(k.dt6, ld(a.G2, c) + ld(a.G3, c), fma(k.dt23, ld(a.G4, c), u[gv[c]]));
     }
 }
 
