@@ -134,13 +134,18 @@ Fx fx_limbs_host(ld v) {
     return {(int)((z - lo) / (1LL << 28)), (int)lo};
 }
 
-// The filter's vectors in fixed point.  Along the three axes a field grows by at most
-// the filter's row sum each, and a mode's coefficient is at most its row of W times
-// the field: both have to stay below 2^58.  Filters that would leave the fields fewer
-// than 55 bits keep the FP64 form (three more than FP64's 53 cover the cuts).
+// Bits for fields that grow by at most a factor g before they are taken apart into
+// limbs (below 2^59)
+int fx_bits_for(double g) { return std::min(58, (int)floor(59.0 - log2(g) - 1e-6)); }
+
+// The filter's vectors in fixed point.  Before the third axis a field has grown by the
+// filter's row sum twice at most, and a mode's coefficient is at most its row of W
+// times that.  Filters that would leave the fields fewer than 54 bits keep the FP64
+// form (whose own error is 2^-50 of the largest value at worst; at a = 36, b = 50
+// the fields have 55 bits for P = 4 and 5, 54 for P = 6).
 void fixed_filter(Tables& T) {
     const int np1 = T.np1;
-    double row = 1.0, w = 0.0;
+    double row = 1.0, w = 1.0;
     for (int i = 0; i < np1; ++i) {
         double s = 0.0;
         for (int j = 0; j < np1; ++j) s += fabs(T.Filt[i][j]);
@@ -151,9 +156,9 @@ void fixed_filter(Tables& T) {
         for (int j = 0; j < np1; ++j) s += fabs(T.FrW[r][j]);
         w = std::max(w, s);
     }
-    T.fx_bits = 58 - (int)ceil(log2(std::max(row * row * row, row * row * w)));
+    T.fx_bits = fx_bits_for(row * row * w);
     T.fx_k = w > 4.0 ? (int)ceil(log2(w)) - 2 : 0;
-    if (T.fx_bits < 55) T.fx_bits = 0;
+    if (T.fx_bits < 54) T.fx_bits = 0;
     for (int r = 0; r < T.nfr; ++r)
         for (int i = 0; i < np1; ++i) {
             T.FxV[r][i] = fx_limbs_host(ldexpl((ld)T.FrV[r][i], 56));
@@ -226,7 +231,7 @@ void build_tables(int P, double fa, double fb, int M, Tables& T) {
         }
         row = std::max(row, s);
     }
-    T.fx_pi = 58 - (int)ceil(3.0 * log2(row));
+    T.fx_pi = fx_bits_for(row * row);
     fixed_filter(T);
     std::vector<ld> xc(nc);
     const ld dxi = 2.0L / nc;

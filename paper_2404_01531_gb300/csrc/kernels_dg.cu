@@ -276,15 +276,17 @@ __device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* s
 }
 
 // What bounds it: the FP64 pipe (2 lanes a clock and SM; a warp instruction takes
-// 16 clocks of an SM).  So the line contractions of the volume term and of the filter,
-// 270 of 430 FP64 slots a thread, run on the integer pipes (fixed.cuh: a 32 x 32 -> 64
-// bit multiply-add takes one clock a warp, three of them replace an FMA); in the rest
+// 16 clocks of an SM).  So the line contractions of the volume term, the filter and the
+// indicator, 290 of 430 FP64 slots a thread, run on the integer pipes (fixed.cuh: a
+// 32 x 32 -> 64 bit multiply-add takes one clock a warp, three of them replace an FMA);
+// in the rest
 // the work per node is what counts: five lift values per face node instead of nine,
 // their sum into dU/dt axis by axis instead of node by node under divergence, no FP64
 // comparisons, and the stage's G and currents from its solve (substep_implicit).
 // Three CTAs an SM: their barriers hide each other's (two without spills: 3% slower).
-// 4096 elements at P = 5, average of the substeps: 0.757 -> 0.551 ms (0.870 with the
-// work per node as it was).
+// 4096 elements at P = 5, average of the substeps: 0.870 ms, 0.757 with less work per
+// node, 0.551 with the volume term in integers, 0.493 with the indicator, 0.444 with the
+// filter.
 template <int P, int SUB>
 __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, SubArgs a) {
     using K = DGK<P>;
