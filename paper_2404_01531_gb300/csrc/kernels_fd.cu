@@ -23,6 +23,16 @@
 namespace ffe {
 
 // ---------------------------------------------------------------------------
+// The 12 quantities of a cell, all loads before the first store that follows: the
+// compiler has to assume that a store to the extended block changes what the next
+// load reads, and a load waits some 700 clocks (125 elements of a box: fill 72 -> 64 us).
+__device__ __forceinline__ void load_cell(const Field& U, const Field& J, int64_t p, double* q) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) q[v] = U.fd(v)[p];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[NV + k] = J.fd(3 + k)[p];
+}
+
 // The element's own cells, to the middle of its extended block.
 __device__ __forceinline__ void fill_interior(const Dev& d, int wl, int e, const Field& U, const Field& J) {
     const ES s = esz(d, e);
@@ -31,8 +41,9 @@ __device__ __forceinline__ void fill_interior(const Dev& d, int wl, int e, const
     for (int c = threadIdx.x; c < s.ncell; c += blockDim.x) {
         const int x = c % nc, y = (c / nc) % nc, z = c / (nc * nc);
         const int o = (x + GH) + ne * ((y + GH) + ne * (z + GH));
-        for (int v = 0; v < NV; ++v) ext_at(d, v, wl)[o] = U.fd(v)[fb + c];
-        for (int k = 0; k < 3; ++k) ext_at(d, NV + k, wl)[o] = J.fd(3 + k)[fb + c];
+        double q[NQ];
+        load_cell(U, J, fb + c, q);
+        for (int v = 0; v < NQ; ++v) ext_at(d, v, wl)[o] = q[v];
     }
 }
 
@@ -200,8 +211,9 @@ __global__ void k_fd_fill(Dev d, const int* list, int ci, int w0, Field U, Field
                 c[u2] = b2;
                 const int64_t p = nbase + c[0] + nc * (c[1] + nc * c[2]);
                 const int64_t og = ghost_offset(g, ta, tb);
-                for (int v = 0; v < NV; ++v) ext_at(d, v, wl)[og] = U.fd(v)[p];
-                for (int k = 0; k < 3; ++k) ext_at(d, NV + k, wl)[og] = J.fd(3 + k)[p];
+                double q[NQ];
+                load_cell(U, J, p, q);
+                for (int v = 0; v < NQ; ++v) ext_at(d, v, wl)[og] = q[v];
             }
         } else if (nb >= 0) {
             // DG neighbour: its polynomial at its own subcell centres (DG -> FD), 3
