@@ -477,33 +477,32 @@ struct Weno5zLineVjp {
         const double s0 = q0 + t2, s1 = q1 + t2, s2 = q2 + t2;
         const double P0 = q1 * q2, P1 = q0 * q2, P2 = q0 * q1;
         const double S0 = s0 * P0, S1 = 10.0 * (s1 * P1), S2 = s2 * P2;
-        // right value: weights (1, 10, 5), g = h + e/2; left value: (5, 10, 1), h - e/2
+        // The candidates differ from the central one by u = h_1 - h_0 and w = h_2 - h_1 only:
+        // right (weights 1, 10, 5) -3 u and -w, left (5, 10, 1) u and 3 w; vr, vl: the values
+        // less the central candidate
         const double T2 = 5.0 * S2, T0 = 5.0 * S0;
         const double iR = recip_nr((S0 + S1) + T2), iL = recip_nr((T0 + S1) + S2);
-        const double r0 = fma(0.5, e0, hA), r1 = fma(0.5, e1, hB), r2 = fma(0.5, e2, hC);
-        const double l0 = fma(-0.5, e0, hA), l1 = fma(-0.5, e1, hB), l2 = fma(-0.5, e2, hC);
-        const double vr = fma(S0, r0, fma(S1, r1, T2 * r2)) * iR, vl = fma(T0, l0, fma(S1, l1, S2 * l2)) * iL;
+        const double u = hB - hA, w = hC - hB, x0 = S0 * u, x2 = S2 * w;
+        const double vr = fma(-3.0, x0, -5.0 * x2) * iR, vl = fma(5.0, x0, 3.0 * x2) * iL;
         const double y = yr * iR, z = yl * iL;
-        const double R0 = y * S0, R1 = y * S1, R2 = y * T2, L0 = z * T0, L1 = z * S1, L2 = z * S2;   // of r_k, l_k
+        const double ub = S0 * fma(5.0, z, -3.0 * y), wb = S2 * fma(3.0, z, -5.0 * y);   // of u and w
         const double y5 = 5.0 * y, z5 = 5.0 * z;
-        const double W0 = fma(y, r0 - vr, z5 * (l0 - vl));
-        const double W1 = 2.0 * fma(y5, r1 - vr, z5 * (l1 - vl));
-        const double W2 = fma(y5, r2 - vr, z * (l2 - vl));
+        const double W0 = fma(y, fma(-3.0, u, -vr), z5 * (u - vl));
+        const double W1 = -2.0 * fma(y5, vr, z5 * vl);
+        const double W2 = fma(-y5, w + vr, z * fma(3.0, w, -vl));
         const double W0P0 = W0 * P0, W0s0 = W0 * s0, W1s1 = W1 * s1, W2s2 = W2 * s2;
         const double T = fma(W1, P1, fma(W2, P2, W0P0));
         const double X0 = fma(W1s1, q2, fma(W2s2, q1, W0P0));
         const double X1 = fma(W0s0, q2, fma(W2s2, q0, W1 * P1));
         const double X2 = fma(W0s0, q1, fma(W1s1, q0, W2 * P2));
-        const double sc2 = 2.0 * sc;
-        const double B0 = sc2 * fma(t, T, b0 * X0), B1 = sc2 * (b1 * X1), B2 = sc2 * fma(-t, T, b2 * X2);
+        const double sc4 = 4.0 * sc;   // B_k: twice the adjoint of b_k
+        const double B0 = sc4 * fma(t, T, b0 * X0), B1 = sc4 * (b1 * X1), B2 = sc4 * fma(-t, T, b2 * X2);
         // b = e^2 + K h^2 + eps: to e (slopes) and h
-        const double E0 = fma(2.0 * e0, B0, 0.5 * (R0 - L0));
-        const double E1 = fma(2.0 * e1, B1, 0.5 * (R1 - L1));
-        const double E2 = fma(2.0 * e2, B2, 0.5 * (R2 - L2));
-        constexpr double K2 = 13.0 / 12.0 * 128.0;
-        hb0 += fma(K2 * hA, B0, fma(4.0, E0, R0 + L0));
-        hb1 += fma(K2 * hB, B1, fma(4.0, E1, R1 + L1));
-        hb2 += fma(K2 * hC, B2, fma(-4.0, E2, R2 + L2));
+        const double E0 = e0 * B0, E1 = fma(e1, B1, 0.5 * (yr - yl)), E2 = e2 * B2;
+        constexpr double K = 13.0 / 12.0 * 64.0;
+        hb0 += fma(K * hA, B0, fma(4.0, E0, -ub));
+        hb1 += fma(K * hB, B1, fma(4.0, E1, (yr + yl) + (ub - wb)));
+        hb2 += fma(K * hC, B2, fma(-4.0, E2, wb));
         dAb += E0 + E1;
         dBb += E2;
         dA = dB; dB = dC;
