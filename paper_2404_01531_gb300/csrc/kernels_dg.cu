@@ -32,11 +32,11 @@ struct DGK {
     static constexpr int NT = ((nn + 31) / 32) * 32;
     static constexpr int FR = (6 * nf + NT - 1) / NT;   // face nodes per thread
     // CTAs per SM the registers are bounded for
-    static constexpr int CTAS = P == 6 ? 2 : 3;
-    // shared doubles: U[9][nn] (later the filter's buffer) | J[3][nn] | dU/dt[9][nn] |
+    static constexpr int CTAS = P == 6 ? 2 : 4;
+    // shared doubles: U[9][nn] (later the filter's buffer) | dU/dt[9][nn] |
     // fixed point: U and J [12][nn] (later the filter's and the indicator's fields) | red[2] | D scaled by the
     // element's d xi/d x, per axis [3][np1][np1]
-    static constexpr int SMEM = (33 * nn + 2 + 3 * nf) * 8;
+    static constexpr int SMEM = (30 * nn + 2 + 3 * nf) * 8;
 };
 
 // ---------------------------------------------------------------------------
@@ -250,7 +250,7 @@ __device__ void dg_external_state(const Dev& d, const SubArgs& a, int e, int f, 
 
 // The volume term in FP64, for elements whose values fixed point does not hold.
 template <int P>
-__device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* sU, const double* sJ, const double* sD, double* r) {
+__device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* sU, const double* sD, double* r) {
     constexpr int np1 = P + 1, nf = np1 * np1, nn = nf * np1;
     const int tid = threadIdx.x, i = tid % np1, j = (tid / np1) % np1, k = tid / nf;
     const double *Dx = sD + np1 * i, *Dy = sD + nf + np1 * j, *Dz = sD + 2 * nf + np1 * k;
@@ -269,7 +269,7 @@ __device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* s
         bZ += Dy[m] * U(0, iy) - Dx[m] * U(1, ix) - Dz[m] * U(7, iz);
         ps -= Dx[m] * U(0, ix) + Dy[m] * U(1, iy) + Dz[m] * U(2, iz);
         ph -= Dx[m] * U(3, ix) + Dy[m] * U(4, iy) + Dz[m] * U(5, iz);
-        qq -= Dx[m] * sJ[ix] + Dy[m] * sJ[nn + iy] + Dz[m] * sJ[2 * nn + iz];
+        qq -= Dx[m] * J.dg(3)[eb + ix] + Dy[m] * J.dg(4)[eb + iy] + Dz[m] * J.dg(5)[eb + iz];
     }
     r[0] = eX; r[nn] = eY; r[2 * nn] = eZ; r[3 * nn] = bX; r[4 * nn] = bY; r[5 * nn] = bZ;
     r[6 * nn] = ps; r[7 * nn] = ph; r[8 * nn] = qq;
@@ -283,18 +283,19 @@ __device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* s
 // the work per node is what counts: five lift values per face node instead of nine,
 // their sum into dU/dt axis by axis instead of node by node under divergence, no FP64
 // comparisons, and the stage's G and currents from its solve (substep_implicit).
-// Three CTAs an SM: their barriers hide each other's (two without spills: 3% slower).
+// Four CTAs an SM, whose barriers hide each other's, at 72 registers: J~ is not kept in
+// shared memory but for its fixed-point form (three CTAs: 0.413 ms a substep of the
+// current sheet against 0.402; two without spills: 3% slower than three).
 // 4096 elements at P = 5, average of the substeps: 0.870 ms, 0.757 with less work per
 // node, 0.551 with the volume term in integers, 0.493 with the indicator, 0.444 with the
-// filter.
+// filter, 0.440 with four CTAs.
 template <int P, int SUB>
 __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, SubArgs a) {
     using K = DGK<P>;
     constexpr int np1 = K::np1, nn = K::nn, nf = K::nf, NT = K::NT;
     extern __shared__ double sm[];
     double* sU = sm;                 // [9][nn]
-    double* sJ = sU + 9 * nn;        // [3][nn] J~ (full)
-    double* sR = sJ + 3 * nn;        // [9][nn] dU/dt
+    double* sR = sU + 9 * nn;        // [9][nn] dU/dt
     Fx* fU = (Fx*)(sR + 9 * nn);     // [12][nn] U and J~ in fixed point
     double* red = sR + 21 * nn;
     double* sD = red + 2;            // [3][np1][np1]: (d xi^a/d x^a) D
@@ -315,11 +316,13 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
         const double sx = d.ijac[3 * e], sy = d.ijac[3 * e + 1], sz = d.ijac[3 * e + 2];
         double* r = sR + tid;
         unsigned wE = 0, wB = 0, wJ = 0;
+        double jx[3] = {0.0, 0.0, 0.0};
         if (act) {
 #pragma unroll
             for (int v = 0; v < 12; ++v) {
                 const double x = v < NV ? a.Uin.dg(v)[eb + tid] : a.J.dg(3 + v - NV)[eb + tid];
-                sU[v * nn + tid] = x;
+                if (v < NV) sU[v * nn + tid] = x;
+                else jx[v - NV] = x;
                 const unsigned w = fx_word(x);
                 if (v < 3 || v == 7) wE = max(wE, w);
                 else if (v < 7) wB = max(wB, w);
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
         if (act && fixed) {
 #pragma unroll
             for (int v = 0; v < 12; ++v)
-                fU[v * nn + tid] = fx_limbs(fx_from(sU[v * nn + tid], v < 3 || v == 7 ? eE : (v < 7 ? eB : eJ), FX_BITS));
+                fU[v * nn + tid] = fx_limbs(fx_from(v < NV ? sU[v * nn + tid] : jx[v < NV ? 0 : v - NV], v < 3 || v == 7 ? eE : (v < 7 ? eB : eJ), FX_BITS));
         }
         __syncthreads();
         if (tid < 3) s_word[tid] = 0;
@@ -400,7 +403,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
                 r[8 * nn] = out(X, eJ);
             }
         } else if (act) {
-            volume_fp64<P>(a.J, eb, sU, sJ, sD, r);
+            volume_fp64<P>(a.J, eb, sU, sD, r);
         }
         // Lift, one thread per face node.  The jump (dU, dJ) to the exterior state
         // enters through the pairs (a, b, s) of flux_pair: with t = s (outward sign)
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
             if (d.nbr[e * 6 + f] < 0 && d.bc[e * 6 + f] == FFE_BC_STAR)
                 for (int q = 0; q < 3; ++q) xn[q] = d.xyz_dg[(int64_t)q * d.ndg + eb + me[r]];
             dg_external_state<P>(d, a, e, f, ta, tb, Ui, xn, Ue, Je);
-            const double jump = (dd == 0 ? Je[0] : (dd == 1 ? Je[1] : Je[2])) - sJ[dd * nn + me[r]];
+            const double jump = (dd == 0 ? Je[0] : (dd == 1 ? Je[1] : Je[2])) - a.J.dg(3 + dd)[eb + me[r]];
             const unsigned long long sg = s ? 0ULL : 0x8000000000000000ULL;
             const double scale = 0.5 * (dd == 0 ? sx : (dd == 1 ? sy : sz)) * w0inv;   // |grad xi^d| / (2 w0)
             for (int v = 0; v < NV; ++v) Ue[v] -= Ui[v];
