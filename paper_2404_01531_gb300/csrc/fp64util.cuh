@@ -24,10 +24,9 @@ __device__ __forceinline__ bool is_zero(double x) { return fmag(x) == 0; }
 // f(y) = 1/y - d, y <- y + y (1 - d y) (each squares the relative error; the
 // residual 1 - d y is exact in one FMA when y is close to 1/d).  Within about
 // one ulp of the rounded quotient (ffe_eval_recip exposes it for tests); used
-// for the WENO5-Z weight denominators (positive sums bounded away from zero;
-// for sums above 2^1022 the flushed reciprocal is 0, where the quotient it
-// replaces would overflow for candidates above 4 in magnitude) and, through
-// recip_any, for the pointwise physics.
+// for the adjoint's WENO5-Z weight denominators (positive sums bounded away from
+// zero; for sums above 2^1022 the flushed reciprocal is 0) and, through recip_any,
+// for the pointwise physics.
 __device__ __forceinline__ double recip_nr(double d) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));

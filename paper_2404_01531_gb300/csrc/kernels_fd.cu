@@ -433,7 +433,8 @@ __global__ void __launch_bounds__(128, 4) k_fd_flux_faces(Dev d, const int* list
         if (!face_coords(fi, nc, m, ta, tb)) continue;
         double UL[NQ], UR[NQ], Um[NQ], Up[NQ];
         int64_t stride;
-        const int64_t base = line_start(k, ta, tb, nc, stride) + m * stride;
+        int64_t base = line_start(k, ta, tb, nc, stride);   // sets stride
+        base += m * stride;
         for (int qq = 0; qq < NQ; ++qq) {
             const double* src = ext_at(d, qq, wl) + base;
             const double v0 = src[0], v1 = src[stride], v2 = src[2 * stride];
@@ -471,7 +472,8 @@ template <int RECON>
 __device__ __forceinline__ void reconstruct(const Dev& d, int wl, int k, int m, int ta, int tb, int nc,
                                             double* UL, double* UR) {
     int64_t stride;
-    const int64_t base = line_start(k, ta, tb, nc, stride) + m * stride;
+    int64_t base = line_start(k, ta, tb, nc, stride);   // sets stride
+    base += m * stride;
     for (int qq = 0; qq < NQ; ++qq) {
         const double* src = ext_at(d, qq, wl) + base;
         typename LineOf<RECON>::type A;
