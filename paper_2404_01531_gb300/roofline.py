@@ -1,7 +1,9 @@
 """Algorithmic FP64 operation counts of the hot kernels (FMA = 2 flops,
 add/mul/div/sqrt = 1), counted from the operations the method defines, not
 from the instructions the kernels happen to issue.  Used for the roofline
-fraction: achieved = count x units per launch / launch time."""
+fraction: achieved = count x units per launch / launch time.  The kernels share
+work between neighbouring face values and run line contractions and WENO5-Z
+weights on the integer pipes, so the fraction of the FP64 peak can exceed 1."""
 import math
 
 
