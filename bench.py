@@ -428,7 +428,7 @@ def run_shell(args):
     ctx.set_profiling(False)
     prof = ctx.profile_read()
     n_fd = j1.fd_elem_updates - j0.fd_elem_updates
-    fl = n_fd * fd_faces_per_element(ctx.P) * fd_flux_flops(RECON[args.recon])
+    fl = n_fd * fd_faces_per_element(ctx.P) * fd_flux_flops(RECON[args.recon], 12)
     ach = fl / (prof["fd_flux"][1] / 1e3) / 1e12
     line = {"metric": METRIC, "value": (i1.node_updates - i0.node_updates) / (ms / 1e3), "unit": UNIT, "n_gpus": 1,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
