@@ -229,7 +229,8 @@ __device__ __forceinline__ double u64_double(unsigned long long a) {
 __device__ __forceinline__ ZWeights z_weights(Pos b0, Pos b1, Pos b2) {
     const int eM = max(b0.e, b2.e);
     const unsigned long long u = b0.m >> min(eM - b0.e, 63), v = b2.m >> min(eM - b2.e, 63), tt = u > v ? u - v : v - u;
-    const int lzt = __clzll((long long)(tt | 1ULL)), et = eM - lzt;
+    // T = 0: its terms lie below all others, else they would shift the first square away
+    const int lzt = __clzll((long long)(tt | 1ULL)), et = tt ? eM - lzt : -(1 << 20);
     const unsigned long long ft = tt << lzt;
     // half the right shifts of T's terms against the first square, none of them below the least
     const int s0 = b0.e - et, s1 = b1.e - et, s2 = b2.e - et, least = min(0, min(s0, min(s1, s2)));

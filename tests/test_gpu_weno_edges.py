@@ -1,0 +1,112 @@
+"""WENO5-Z face values where the indicators are equal, vanish or differ by many
+orders of magnitude: the line kernels (boxes, flat and Kerr-Schild shells, the
+allocation-free entry point) on data of few heights, where b_0 - b_2 is exactly
+zero beside a flat middle."""
+import numpy as np
+import pytest
+
+import ffe_workloads as W
+from oracle.fd import rhs_fd, weno5z
+from oracle.problem import Problem
+from test_gpu_parity import ffe  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+GH = 3
+
+
+def _plateaus(kind, shape, rng):
+    """Fields [..., z, y, x] of two or three heights, or of plateaus whose middle cell is one
+    rounding higher (along every axis every window of five cells is then symmetric or has a jump
+    on one side only)."""
+    if kind == "two":
+        return rng.integers(1, 3, size=shape).astype(float)
+    if kind == "three":
+        return rng.integers(0, 3, size=shape).astype(float)
+    z, y, x = np.meshgrid(*[np.arange(n) for n in shape[-3:]], indexing="ij")
+    row = np.array([2.0, 1.0, 1.0 + 2.0 ** -52, 1.0])
+    return np.broadcast_to(row[(x + y + 2 * z) % 4], shape).copy()
+
+
+def _flux(u, k):
+    """Flat flux along axis k of the first eight variables, J~ = 0."""
+    i, j = (k + 1) % 3, (k + 2) % 3
+    f = np.zeros_like(u)
+    f[k], f[3 + k], f[6], f[7] = u[6], u[7], u[k], u[3 + k]
+    f[i], f[j], f[3 + i], f[3 + j] = u[3 + j], -u[3 + i], -u[j], u[i]
+    return f
+
+
+def _block_rhs(ext, h, eps):
+    """Right-hand side of extended blocks [9][E][ne^3] with eta = q~ = 0 and no corrector, in
+    extended precision."""
+    u = ext.astype(np.longdouble)
+    n = ext.shape[-1] - 2 * GH
+    out = np.zeros(u.shape[:2] + (n,) * 3, np.longdouble)
+    for k in range(3):
+        ax = 4 - k
+        idx = [slice(None), slice(None)] + [slice(GH, GH + n)] * 3
+
+        def cells(o):
+            idx[ax] = slice(GH + o, GH + o + n + 1)
+            return u[tuple(idx)]
+        v = [cells(o) for o in range(-3, 3)]
+        L, R = weno5z(*v[:5], np.longdouble(eps)), weno5z(*v[:0:-1], np.longdouble(eps))
+        F = 0.5 * (_flux(L, k) + _flux(R, k)) - 0.5 * (R - L)
+        out -= np.diff(F, axis=ax) * (np.longdouble(n) / h[k])
+    return out
+
+
+def _noalloc(ffe, P, ext, h, eps):  # noqa: F811
+    out = torch.full(ext.shape[:2] + (2 * P + 1,) * 3, float("nan"), dtype=torch.float64, device="cuda")
+    ffe.fd_rhs_noalloc(P, torch.from_numpy(ext).cuda(), h, 0.0, eps, 0, out)
+    torch.cuda.synchronize()
+    return out.cpu().numpy()
+
+
+H = (0.25, 0.5, 1.0)
+
+
+@pytest.mark.parametrize("kind", ["two", "three", "ulp"])
+def test_blocks_plateaus(ffe, kind):  # noqa: F811
+    """Bound: 6 face fluxes of two values, each within 16 roundings of the largest cell."""
+    P = 4
+    rng = np.random.default_rng(3)
+    ext = _plateaus(kind, (9, 2) + (2 * P + 7,) * 3, rng)
+    ext[8] = 0.0
+    err = np.abs(_noalloc(ffe, P, ext, H, 1e-40) - _block_rhs(ext, H, 1e-40)).max()
+    assert err <= 2.0 ** -53 * 6 * 2 * 16 * 2.0 * (2 * P + 1) / min(H), err
+
+
+@pytest.mark.parametrize("mesh", ["box", "shell", "kerr-schild"])
+@pytest.mark.parametrize("kind", ["two", "three"])
+def test_plateaus(ffe, mesh, kind):  # noqa: F811
+    """Cells that reach only cells of their own element: the oracle's ghosts on a box carry an
+    interpolation's rounding, which decides the weights of a plateau."""
+    P = 5
+    if mesh == "box":
+        cfg = W.breakdown(nx=2, ny=2, nz=1, P=P, x_half=0.1)
+    elif mesh == "shell":
+        cfg = W.pulsar(r_lc=3.0, chi=0.4, n_ang=1, n_rad=2, P=P, r_out=4.0)
+    else:
+        cfg = W.wald(spin=0.7, n_ang=1, n_rad=2, P=P)
+    cfg["params"].update(eta=0.0, recon=0, fd_corrector=0, tci_on=1)
+    pr = Problem(cfg)
+    E, n = pr.disc.E, 2 * P + 1
+    u = _plateaus(kind, (9, E, n, n, n), np.random.default_rng(4))
+    u[8] = 0.0
+    u[3] += 3.0   # B~ does not vanish
+    st = dict(mask=np.ones(E, np.uint8), udg=np.ones((9, E) + (P + 1,) * 3), ufd=u)
+    ctx = ffe.Context(cfg)
+    ctx.set_initial()
+    U = torch.from_numpy(ctx.join(st["udg"], u)).cuda()
+    ctx.set_state(U, torch.ones(E, dtype=torch.uint8, device="cuda"))
+    out = torch.zeros_like(U)
+    ctx.rhs(U, out)
+    torch.cuda.synchronize()
+    got = ctx.split(out.cpu().numpy())[1]
+    ctx.close()
+    own = (slice(None), slice(None)) + (slice(3, n - 3),) * 3
+    ref = rhs_fd(st, pr.disc, pr.met, pr.prm)[own]
+    assert np.abs(got[own] - ref).max() <= 1e-11 * np.abs(ref).max()
