@@ -191,16 +191,19 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
 // square, and the weights are sums of two of them, (b_0 b_1 b_2)^2 + (T b_1 b_2)^2 and
 // its permutations.  A positive number is m 2^(e - 1022 - 64); products of 64-bit
 // fractions m keep the upper half (4 clocks of an SM where an FP64 product takes 16),
-// sums the bits that both terms have at the larger one's scale.  Cut at 2^-58 of the
-// largest term, where FP64 rounds each of 16 operations at 2^-53.  No range of
-// indicators overflows; arguments that are not finite give finite weights without
-// meaning (the third differences they multiply are not finite either).
+// sums the bits that both terms have at the larger one's scale: cut at 2^-57 of the
+// larger term, where FP64 rounds each of 16 operations at 2^-53.  Every S_k has a
+// scale of its own: a stencil across a jump gets the weight it has (1e-80 and less),
+// not one cut at the others' last bit.  No range of indicators overflows; arguments
+// that are not finite give finite weights without meaning (the differences they
+// multiply are not finite either).
 struct Pos {
     unsigned long long m;
     int e;
 };
 struct ZWeights {
-    double s0, s2, right, left;   // S_0, S_2, S_0 + 10 S_1 + 5 S_2 and 5 S_0 + 10 S_1 + S_2
+    double s0, s0x5, s1x10, s2, s2x5;   // S_0, 5 S_0, 10 S_1, S_2, 5 S_2
+    double right, left;                 // 2 (S_0 + 10 S_1 + 5 S_2) and 2 (5 S_0 + 10 S_1 + S_2)
 };
 __device__ __forceinline__ Pos pos_of(double x) {
     return {(fbits(x) << 11) | 0x8000000000000000ULL, (int)(fmag(x) >> 52)};
@@ -218,12 +221,13 @@ __device__ __forceinline__ Pos pos_norm(Pos x) {
     const int lz = __clz((int)(x.m >> 32));
     return {x.m << lz, x.e - lz};
 }
-// a positive integer (as 1 where it is 0), rounded to nearest
-__device__ __forceinline__ double u64_double(unsigned long long a) {
-    a |= 1ULL;
-    const int lz = __clzll((long long)a);
-    const unsigned long long m = a << lz;
-    return __longlong_as_double((long long)((m >> 11) + ((m >> 10) & 1ULL) + ((unsigned long long)(1085 - lz) << 52)));
+// m 2^e rounded to nearest, for 2^63 <= m and for any positive m
+__device__ __forceinline__ double norm_double(unsigned long long m, int e) {
+    return __longlong_as_double((long long)((m >> 11) + ((m >> 10) & 1ULL) + ((unsigned long long)(1085 + e) << 52)));
+}
+__device__ __forceinline__ double pos_double(unsigned long long m, int e) {
+    const int lz = __clzll((long long)m);
+    return norm_double(m << lz, e - lz);
 }
 // b_k of magnitude 2^63 <= m
 __device__ __forceinline__ ZWeights z_weights(Pos b0, Pos b1, Pos b2) {
@@ -239,27 +243,43 @@ __device__ __forceinline__ ZWeights z_weights(Pos b0, Pos b1, Pos b2) {
     const unsigned long long r0 = __umul64hi(ft, c0), r1 = __umul64hi(ft, c1), r2 = __umul64hi(ft, c2);
     const unsigned long long Y = __umul64hi(b1.m, c1);
     const unsigned long long q0 = __umul64hi(r0, r0), q1 = __umul64hi(r1, r1), q2 = __umul64hi(r2, r2), qX = __umul64hi(Y, Y);
-    // the largest term is 2^58 or more; five bits of room for the weighted sums
+    // a weight at its larger term's scale, to 2^63 <= m (the terms are 2^58 or more there; T = 0 leaves X alone)
+    auto sum = [&](unsigned long long q, int n) -> Pos {
+        const int k = min(n, nX);
+        const unsigned long long m = (qX >> min(nX - k + 1, 63)) + (q >> min(n - k + 1, 63));
+        const int lz = __clz((int)(m >> 32));
+        return {m << lz, 1 - lz - min(k, 1000)};
+    };
+    const Pos S0 = sum(q0, n0), S1 = sum(q1, n1), S2 = sum(q2, n2);
+    // the sums at the largest term's scale (2^58 or more there); five bits of room
     auto top = [](unsigned long long q, int n) { return (unsigned)(q >> 32) >> min(n, 31); };
     const int room = 5 - min(5, __clz((int)(top(q0, n0) | top(q1, n1) | top(q2, n2) | top(qX, nX))));
     auto down = [&](unsigned long long q, int n) { return q >> min(n + room, 63); };
-    const unsigned long long X = down(qX, nX), S0 = X + down(q0, n0), S1 = X + down(q1, n1), S2 = X + down(q2, n2);
-    return {u64_double(S0), u64_double(S2), u64_double(S0 + 5 * (2 * S1 + S2)), u64_double(S2 + 5 * (2 * S1 + S0))};
+    const unsigned long long X = 16 * down(qX, nX), t0 = down(q0, n0), t1 = X + 10 * down(q1, n1), t2 = down(q2, n2);
+    ZWeights w;
+    w.s0 = norm_double(S0.m, S0.e);
+    w.s0x5 = pos_double(5 * (S0.m >> 3), S0.e + 3);
+    w.s1x10 = pos_double(5 * (S1.m >> 3), S1.e + 4);
+    w.s2 = norm_double(S2.m, S2.e);
+    w.s2x5 = pos_double(5 * (S2.m >> 3), S2.e + 3);
+    w.right = pos_double(t0 + t1 + 5 * t2, room + 1);
+    w.left = pos_double(5 * t0 + t1 + t2, room + 1);
+    return w;
 }
 
 // WENO5-Z: with a_k the second difference of stencil k (left, centred, right) and
 // e_k its slope at the centre, the candidate at the face +-1/2 is
 // v_c + a_k / 8 +- e_k / 2, and beta_k = (13/12) a_k^2 + e_k^2 (the kept per-stencil
 // values are a and k = (13/12) a^2 + eps); ideal weights (1, 10, 5) towards the
-// right face and (5, 10, 1) towards the left one.  Neighbouring candidates differ by
-// third differences t_0 = a_1 - a_0, t_1 = a_2 - a_1 only, so that
-//   right = v_c + a_1/8 + e_1/2 - (3/8 S_0 t_0 + 5/8 S_2 t_1) / (S_0 + 10 S_1 + 5 S_2),
-//   left  = v_c + a_1/8 - e_1/2 + (5/8 S_0 t_0 + 3/8 S_2 t_1) / (5 S_0 + 10 S_1 + S_2).
-// 23 FP64 operations per cell and quantity, the pipe that bounds these kernels
-// (52 with the candidates formed one by one and the weights in FP64, 87 in a thread
-// per face).  eps is at least 1e-51.
+// right face and (5, 10, 1) towards the left one.  Twice the candidates' offsets from
+// v_c are one operation each from the differences.  25 FP64 operations per cell and
+// quantity, the pipe that bounds these kernels (87 in a thread per face).  Every
+// offset is formed from its own stencil's differences: beside a jump, the values of the
+// smooth side are as accurate as its cells (candidates by their differences from the
+// central one, 23 operations, and weights at one scale leave 2^-54 of the jump there;
+// two steps of the 64x8x8 current sheet 9.46 -> 9.60 ms, 19 blocks 88 -> 91 us).
 struct Weno5zLine {
-    double dA, dB, aA, aB, tA, vc, vn;
+    double dA, dB, aA, aB, vc, vn;
     Pos kA, kB, eps;
     __device__ __forceinline__ Pos curv(double a) const {
         const Pos q = pos_square(a);
@@ -272,7 +292,6 @@ struct Weno5zLine {
         dB = v3 - v2;
         aA = dA - d01;
         aB = dB - dA;
-        tA = aB - aA;
         kA = curv(aA);
         kB = curv(aB);
         vc = v2;
@@ -280,18 +299,20 @@ struct Weno5zLine {
     }
     template <bool LEFT, bool RIGHT>
     __device__ __forceinline__ void cell(double v4, double& left, double& right) {
-        const double dC = v4 - vn, aC = dC - dB, tB = aC - aB;
+        const double dC = v4 - vn, aC = dC - dB;
         const Pos kC = curv(aC);
         const double e0 = fma(0.5, aA, dA), e1 = fma(0.5, aB, dA), e2 = fma(-0.5, aC, dB);   // slopes at the centre
         const ZWeights S = z_weights(pos_norm(pos_add(pos_square(e0), kA)), pos_norm(pos_add(pos_square(e1), kB)),
                                      pos_norm(pos_add(pos_square(e2), kC)));
-        const double x = S.s0 * tA, y = S.s2 * tB, z = fma(0.125, aB, vc);
-        if (RIGHT) right = fma(fma(-0.375, x, -0.625 * y), recip_nr3(S.right), fma(0.5, e1, z));
-        if (LEFT) left = fma(fma(0.625, x, 0.375 * y), recip_nr3(S.left), fma(-0.5, e1, z));
+        if (RIGHT)
+            right = fma(fma(S.s0, fma(0.75, aA, dA), fma(S.s1x10, fma(0.75, aB, dA), S.s2x5 * fma(-0.25, aC, dB))),
+                        recip_nr3(S.right), vc);
+        if (LEFT)
+            left = fma(fma(-S.s0x5, fma(0.25, aA, dA), fma(-S.s1x10, fma(0.25, aB, dA), -S.s2 * fma(-0.75, aC, dB))),
+                       recip_nr3(S.left), vc);
         dA = dB; dB = dC;
         aA = aB; aB = aC;
         kA = kB; kB = kC;
-        tA = tB;
         vc = vn; vn = v4;
     }
 };

@@ -60,7 +60,7 @@ __global__ void k_na_current(NA a) {
 // context path does (fd_common.cuh).  Single-warp CTAs: a call holds at most 19
 // elements at P = 5, 1078 warps, and the FP64 pipe wants them spread evenly over
 // the SMs.  19 elements: 0.49 -> 0.16 ms for the three kernels, against a thread
-// per face with four divisions per value, and 0.088 ms with indicators and weights in
+// per face with four divisions per value, and 0.091 ms with indicators and weights in
 // integers.
 __global__ void __launch_bounds__(32) k_na_flux(NA a) {
     const int nc = a.nc, nl = nc * nc, per = 3 * FLUX_PAIRS * nl;

@@ -110,3 +110,21 @@ def test_plateaus(ffe, mesh, kind):  # noqa: F811
     own = (slice(None), slice(None)) + (slice(3, n - 3),) * 3
     ref = rhs_fd(st, pr.disc, pr.met, pr.prm)[own]
     assert np.abs(got[own] - ref).max() <= 1e-11 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("h", [1e-6, 1e-12])
+def test_blocks_beside_jump(ffe, h, axis):  # noqa: F811
+    """Cells of size h beside cells of order one: away from the jump's own face, errors are roundings
+    of h, not of the jump.  1e-12: a face value of random cells moves by up to 300 of its roundings
+    with those of the indicators, two of which are subtracted."""
+    P = 4
+    n = 2 * P + 1
+    rng = np.random.default_rng(8 + axis)
+    shape = (9, 2) + (2 * P + 7,) * 3
+    c = np.arange(2 * P + 7).reshape([-1 if a == 2 - axis else 1 for a in range(3)])
+    ext = np.where(c < GH + 5, h * (1.0 + 0.1 * rng.normal(size=shape)), 2.0 + rng.random(shape))
+    ext[8] = 0.0
+    err = np.abs(_noalloc(ffe, P, ext, H, 1e-60) - _block_rhs(ext, H, 1e-60))
+    low = np.moveaxis(err, 4 - axis, 0)[:4]   # the fifth cell's flux crosses the jump
+    assert low.max() <= 1e-12 * 1.5 * h * n / min(H), low.max()
