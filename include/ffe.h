@@ -107,7 +107,7 @@ typedef struct {
     double cfl, c_over_D, dt;
     int filter_on; double filter_a, filter_b;        /* exponential filter (Sec. III.A) */
     int tci_on, tci_M; double tci_alpha;             /* troubled-cell indicator          */
-    double weno_eps; int fd_corrector;               /* FD subcell scheme                */
+    double weno_eps; int fd_corrector;               /* FD subcell scheme; eps below 2^-1000 counts as 2^-1000 */
     int constraint_mode;                             /* FFE_RELAX | FFE_HARD | ...        */
     double omega_star;                               /* star rotation (FFE_BC_STAR)       */
     int recon;                                       /* FFE_RECON_WENO5Z | FFE_RECON_MP5  */
@@ -284,7 +284,7 @@ ffe_status ffe_profile_read(ffe_ctx* ctx, char* buf, size_t cap);
  * 27 (2P+2)(2P+1)^2 doubles, e.g. at most 19 elements at P = 5) are rejected
  * with FFE_EINVAL, as are P outside [3, 6], n_elem < 0, NULL buffers, widths that
  * are not positive and finite, eta < 0 or weno_eps <= 0 (non-finite values
- * included); these checks make no CUDA call, and n_elem = 0 returns FFE_OK
+ * included; weno_eps below 2^-1000 counts as 2^-1000); these checks make no CUDA call, and n_elem = 0 returns FFE_OK
  * without one.  Devices 0 to 63 are served (FFE_EINVAL on a higher index).
  * The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current and keeps it for the life

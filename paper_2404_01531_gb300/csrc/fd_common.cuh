@@ -134,7 +134,23 @@ __device__ __forceinline__ int chunk_n(const Dev& d, int ci, int w0) {
 // weno5z_combine: the Z-weighted combination of three candidates from their
 // indicators b_k (eps included); the ideal weights are taken as (1, 10, 5)
 // (scale-free).
+// The eps of every WENO5-Z form: weno_eps, zero and values below 2^-1000 as 2^-1000 (the
+// reverse mode divides by it; nothing else needs a least value).
+__device__ __forceinline__ double indicator_eps(double weno_eps) { return fmax(weno_eps, 9.332636185032189e-302); }
+
+// The weights are homogeneous of degree 0 in the indicators, which are first scaled by
+// one power of two, the largest to [1, 2) (exponents only: exact, and products of six
+// stay in range), none to less than 2^-250 (a weight that far out is 2^-500).
+// Arguments that are not finite stay so.
+__device__ __forceinline__ void scale_indicators(double& b0, double& b1, double& b2) {
+    const unsigned long long e = umax(fbits(b0), umax(fbits(b1), fbits(b2))) >> 52;   // positive: ordered as integers
+    const long long shift = e >= 2047 ? 0 : ((long long)e - 1023) << 52, least = (1023LL - 250) << 52;
+    b0 = __longlong_as_double(max(__double_as_longlong(b0) - shift, least));
+    b1 = __longlong_as_double(max(__double_as_longlong(b1) - shift, least));
+    b2 = __longlong_as_double(max(__double_as_longlong(b2) - shift, least));
+}
 __device__ __forceinline__ double weno5z_combine(double b0, double b1, double b2, double p0, double p1, double p2) {
+    scale_indicators(b0, b1, b2);
     // A_k = d_k (b_k^2 + t^2) P_k with P_k the product of the other two b_j^2
     // is d_k (X + t^2 P_k), X = b_0^2 b_1^2 b_2^2 shared by the three
     const double t = b0 - b2;
@@ -165,7 +181,7 @@ __device__ __forceinline__ void weno5z_pair(double v0, double v1, double v2, dou
     const double a012 = d12 - d01, a123 = d23 - d12, a234 = d34 - d23, a345 = d45 - d34;
     const double eL0 = fma(2.0, d12, a012), eL1 = d12 + d23, eL2 = fma(-2.0, d23, a234);
     const double eR0 = fma(-2.0, d34, a345), eR1 = d23 + d34, eR2 = fma(2.0, d23, a123);
-    const double c = 13.0 / 3.0, eps4 = 4.0 * eps;
+    const double c = 13.0 / 3.0, eps4 = 4.0 * indicator_eps(eps);
     const double c123 = c * a123, c234 = c * a234;
     const double bL0 = fma(c * a012, a012, fma(eL0, eL0, eps4));
     const double bL1 = fma(c123, a123, fma(eL1, eL1, eps4));
@@ -286,7 +302,7 @@ struct Weno5zLine {
         return pos_add({__umul64hi(q.m, 0x8aaaaaaaaaaaaaabULL), q.e + 1}, eps);   // 13/24 2^64
     }
     __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double weno_eps) {
-        eps = pos_of(fmax(weno_eps, 1e-51));
+        eps = pos_of(indicator_eps(weno_eps));
         const double d01 = v1 - v0;
         dA = v2 - v1;
         dB = v3 - v2;
@@ -476,7 +492,7 @@ struct Weno5zLineVjp {
     double dA, dB, hA, hB, kA, kB, vn, eps;
     __device__ __forceinline__ double curv(double h) const { return fma((13.0 / 12.0 * 64.0) * h, h, eps); }
     __device__ __forceinline__ void init(double v0, double v1, double v2, double v3, double weno_eps) {
-        eps = fmax(weno_eps, 1e-51);
+        eps = indicator_eps(weno_eps);
         const double d01 = v1 - v0;
         dA = v2 - v1;
         dB = v3 - v2;
@@ -493,7 +509,8 @@ struct Weno5zLineVjp {
         const double c0 = fma(e0, e0, kA), c1 = fma(e1, e1, kB), c2 = fma(e2, e2, kC);
         // positive: ordered as integers
         const double sc = pow2_inv_scale(__longlong_as_double((long long)umax(fbits(c0), umax(fbits(c1), fbits(c2)))));
-        const double b0 = c0 * sc, b1 = c1 * sc, b2 = c2 * sc;
+        double b0 = c0, b1 = c1, b2 = c2;
+        scale_indicators(b0, b1, b2);
         const double t = b0 - b2, t2 = t * t;
         const double q0 = b0 * b0, q1 = b1 * b1, q2 = b2 * b2;
         const double s0 = q0 + t2, s1 = q1 + t2, s2 = q2 + t2;

@@ -128,3 +128,60 @@ def test_blocks_beside_jump(ffe, h, axis):  # noqa: F811
     err = np.abs(_noalloc(ffe, P, ext, H, 1e-60) - _block_rhs(ext, H, 1e-60))
     low = np.moveaxis(err, 4 - axis, 0)[:4]   # the fifth cell's flux crosses the jump
     assert low.max() <= 1e-12 * 1.5 * h * n / min(H), low.max()
+
+
+@pytest.mark.parametrize("eps", [1e-100, 1e-290])
+def test_blocks_small_eps(ffe, eps):  # noqa: F811
+    """Cells of 1e-28, whose indicators lie far below 1e-51, with an eps below those: the bound of
+    test_blocks_plateaus, with 600 roundings for random cells as above."""
+    P = 4
+    ext = 1e-28 * (1.0 + 0.1 * np.random.default_rng(5).normal(size=(9, 2) + (2 * P + 7,) * 3))
+    ext[8] = 0.0
+    err = np.abs(_noalloc(ffe, P, ext, H, eps) - _block_rhs(ext, H, eps)).max()
+    assert err <= 2.0 ** -53 * 6 * 2 * 600 * 2e-28 * (2 * P + 1) / min(H), err
+
+
+def _fd_shell(ffe, weno_eps, scale):  # noqa: F811
+    """rhs, its VJP and an adjoint step of a shell of two heights, all on FD; scale: of the state."""
+    cfg = W.pulsar(r_lc=3.0, chi=0.4, n_ang=1, n_rad=2, P=4, r_out=4.0)
+    cfg["params"].update(eta=0.0, recon=0, tci_on=0, weno_eps=weno_eps)
+    ctx = ffe.Context(cfg)
+    ctx.set_initial()
+    rng = np.random.default_rng(6)
+    u = _plateaus("two", (9, ctx.n_elem) + (ctx.nc,) * 3, rng)
+    u[8] = 0.0
+    U = torch.from_numpy(ctx.join(np.zeros((9, ctx.n_elem) + (ctx.P + 1,) * 3), u)).cuda() * scale
+    nd = 9 * ctx.n_dg
+    lam = torch.from_numpy(rng.normal(size=U.numel())).cuda()
+    lam[:nd] = 0.0
+    ctx.set_state(U, torch.ones(ctx.n_elem, dtype=torch.uint8, device="cuda"))
+    out = [torch.zeros_like(U) for _ in range(3)]
+    ctx.rhs(U, out[0])
+    ctx.rhs_vjp(U, lam, out[1])
+    ctx.adjoint_step(U, lam, out[2])
+    torch.cuda.synchronize()
+    ctx.close()
+    return [x[nd:].cpu().numpy() for x in out]
+
+
+def _close(a, b, tol):
+    assert np.isfinite(a).all() and np.abs(a - b).max() <= tol * np.abs(b).max(), np.abs(a - b).max() / np.abs(b).max()
+
+
+def test_shell_eps_scales_with_state(ffe):  # noqa: F811
+    """With eta = q~ = 0 the right-hand side is of degree 1 in (state, sqrt(eps)) and its derivative of
+    degree 0; the VJPs add contributions in any order."""
+    s = 2.0 ** -93
+    a, b = _fd_shell(ffe, 1e-40, 1.0), _fd_shell(ffe, 1e-40 * s * s, s)
+    assert np.array_equal(a[0] * s, b[0])
+    _close(b[1], a[1], 1e-12)
+    _close(b[2], a[2], 1e-9)
+
+
+def test_shell_zero_eps(ffe):  # noqa: F811
+    """eps = 0 (allowed without the indicator): flat stencils take the ideal weights, in the step, its
+    recomputation and its reverse."""
+    a, b = _fd_shell(ffe, 1e-60, 1.0), _fd_shell(ffe, 0.0, 1.0)
+    _close(b[0], a[0], 1e-12)
+    _close(b[1], a[1], 1e-12)
+    _close(b[2], a[2], 1e-9)
