@@ -31,7 +31,7 @@ constexpr double IM_H = 0.12915286960590;
 // substep kinds of the device stage kernels
 enum Sub : int { SUB_A = 0, SUB_B = 1, SUB_C = 2, SUB_RHS = 3 };
 
-// two limbs of a fixed-point number, hi 2^28 + lo (fixed.cuh)
+// two limbs of a fixed-point number, hi 2^30 + lo (fixed.cuh)
 struct Fx {
     int hi, lo;
 };
@@ -46,14 +46,14 @@ struct Tables {
     // more than 1e-20 (FrV[r][i] = P_m(x_i), FrW[r][j] = (1 - sigma_m) (V^-1)[m][j])
     int nfr;
     double FrV[MAXNP][MAXNP], FrW[MAXNP][MAXNP];
-    // the same in units of 2^-56 and 2^(fx_k - 56) (filter_fixed), for fields of
+    // the same in units of 2^-60 and 2^(fx_k - 60) (filter_fixed), for fields of
     // fx_bits bits; fx_bits = 0: this filter takes the FP64 form
     int fx_bits, fx_k;
     Fx FxV[MAXNP][MAXNP], FxW[MAXNP][MAXNP];
     double Dabs;                   // largest row sum of |D|
-    int fx_d;                      // D in units of 2^-fx_d (its rows sum to less than 2^59)
+    int fx_d;                      // D in units of 2^-fx_d (its rows sum to less than 2^60)
     Fx FxD[MAXNP][MAXNP];
-    int fx_pi;                     // Pi in units of 2^-56, for a field of fx_pi bits
+    int fx_pi;                     // Pi in units of 2^-60, for a field of fx_pi bits
     Fx FxPi[MAXNP][MAXNP];
     double Pi[MAXNP][MAXNP];       // projection on Legendre modes p <= P - M
     double P2F[MAXNC][MAXNP];      // DG -> FD (Lagrange evaluation at subcell centres)

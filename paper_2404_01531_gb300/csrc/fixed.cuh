@@ -2,38 +2,59 @@
 //
 // A contraction sum_m D_m u_m along a line of an element is FP64 work of 6 slots a
 // value on a pipe with 2 lanes a clock and SM; the integer multiply-adds run 32
-// lanes or more.  The values of a block (a variable, or variables that meet in one
-// sum) are therefore scaled by one power of two per element and held as integers
-// of up to 58 bits in two limbs, z = hi 2^28 + lo with |lo| <= 2^27; the operator's
-// rows likewise.  A product is three 32 x 32 -> 64 bit multiply-adds into two
-// 64-bit sums (hi hi into a, hi lo + lo hi into b; lo lo stays below the quantum),
-// exact until the one rounding of the result to double.
+// lanes or more.  The values of a variable are therefore scaled by one power of two
+// per element and held as integers of up to 60 bits in two limbs, z = hi 2^30 + lo
+// with |lo| <= 2^29; the operator's rows likewise.  A product is three
+// 32 x 32 -> 64 bit multiply-adds into two 64-bit sums (hi hi into a, hi lo + lo hi
+// into b; lo lo stays below the quantum), exact until the one rounding of the result.
+// Sums of several variables or axes are formed at the scale of the largest of them.
 //
-// Error: the operands are cut at 2^-58 of the block's largest value and 2^-56 of
-// the operator's largest entry, where the FP64 sum rounds each product and partial
-// sum at 2^-53 of their size, so the sum's error is smaller by 2^3 or more wherever
-// the line holds values of the size of the block's largest.  Blocks with values of
-// 2^900 or more, infinities or NaN take the FP64 form (FX_EMAX); values below
-// 2^-958 count as zero.
+// Error: the operands are cut at 2^-59 of the variable's largest value in the element
+// and 2^-60 of the operator's largest row sum, where the FP64 sum rounds each product
+// and partial sum at 2^-53 of their size.  So the sum is the more accurate one on a
+// line that holds values of 2^-6 of the variable's largest in the element or more, and
+// the less accurate one on lines far below that (absolute error 2^-58 of the largest).
+// The sizes of other variables and, on boxes, the widths along other axes do not
+// enter.  Elements with a variable whose largest value is 2^900 or more, not finite,
+// or below 2^-800 but not zero take the FP64 form (fx_inside).
 #pragma once
 #include "ffe_internal.h"
 #include "fp64util.cuh"
 
 namespace ffe {
 
-constexpr int FX_BITS = 58;              // |z| < 2^FX_BITS
-constexpr int FX_EMIN = 1023 - 900;      // biased exponents of a block's largest value
+constexpr int FX_BITS = 60;              // |z| < 2^FX_BITS
+constexpr int FX_EMIN = 1023 - 800;      // biased exponents of a variable's largest value
 constexpr int FX_EMAX = 1023 + 900;
 
-// the biased exponent's word of a value (its maximum over a block is the block's)
-__device__ __forceinline__ unsigned fx_word(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-// exponent of a block from the largest word
+// the biased exponent's word of a value (its maximum over an element is the largest
+// value's); not zero where the value is not
+__device__ __forceinline__ unsigned fx_word(double x) {
+    const unsigned long long m = fbits(x);
+    return ((unsigned)(m >> 32) & 0x7fffffffu) | ((unsigned)m != 0u);
+}
+// exponent of a variable from its largest word, and whether fixed point holds it
 __device__ __forceinline__ int fx_exp(unsigned word) {
     const int e = (int)(word >> 20);
     return e < FX_EMIN ? FX_EMIN : e;
 }
+__device__ __forceinline__ bool fx_inside(unsigned word) {
+    return word == 0u || word - ((unsigned)FX_EMIN << 20) < (unsigned)(FX_EMAX - FX_EMIN) << 20;
+}
+// Largest words of N variables over a warp, added to top[N] (shared); every lane calls it
+template <int N>
+__device__ __forceinline__ void fx_largest(const unsigned* word, unsigned* top) {
+    static_assert(N <= 32, "a lane per variable");
+    unsigned mine = 0;
+#pragma unroll
+    for (int v = 0; v < N; ++v) {
+        const unsigned w = __reduce_max_sync(0xffffffffu, word[v]);
+        if ((int)(threadIdx.x & 31) == v) mine = w;
+    }
+    if ((threadIdx.x & 31) < N && mine) atomicMax(top + (threadIdx.x & 31), mine);
+}
 
-// x of a block with exponent e, in units of 2^(e - 1022 - bits): |z| < 2^bits, cut towards zero
+// x of a variable with exponent e, in units of 2^(e - 1022 - bits): |z| < 2^bits, cut towards zero
 __device__ __forceinline__ long long fx_from(double x, int e, int bits) {
     const unsigned long long b = fbits(x);
     const unsigned long long m = (b & 0x000fffffffffffffULL) | 0x0010000000000000ULL;
@@ -43,13 +64,12 @@ __device__ __forceinline__ long long fx_from(double x, int e, int bits) {
 }
 __device__ __forceinline__ Fx fx_limbs(long long z) {
     Fx r;
-    r.lo = ((int)(unsigned)z << 4) >> 4;
-    r.hi = (int)((z - r.lo) >> 28);
+    r.lo = ((int)((unsigned)z << 2)) >> 2;
+    r.hi = (int)((z - r.lo) >> 30);
     return r;
 }
-__device__ __forceinline__ Fx fx_neg(Fx a) { return {-a.hi, -a.lo}; }
 
-// sum of products, in units of 2^28: a 2^28 + b
+// sum of products, in units of 2^30: a 2^30 + b
 struct FxSum {
     long long a = 0, b = 0;
     __device__ __forceinline__ void add(Fx x, Fx y) {
@@ -57,8 +77,8 @@ struct FxSum {
         b += (long long)x.hi * y.lo;
         b += (long long)x.lo * y.hi;
     }
-    // in units of 2^56, rounded
-    __device__ __forceinline__ long long top() const { return a + ((b + (1LL << 27)) >> 28); }
+    // in units of 2^60, rounded
+    __device__ __forceinline__ long long top() const { return a + ((b + (1LL << 29)) >> 30); }
 };
 
 // h 2^e, rounded to nearest: integer operations only (the conversion instruction is

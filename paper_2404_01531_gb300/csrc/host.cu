@@ -130,19 +130,19 @@ ld lagrange(const std::vector<ld>& xs, int j, ld y) {
 }
 
 Fx fx_limbs_host(ld v) {
-    const long long z = llrintl(v), lo = ((z + (1LL << 27)) & ((1LL << 28) - 1)) - (1LL << 27);
-    return {(int)((z - lo) / (1LL << 28)), (int)lo};
+    const long long z = llrintl(v), lo = ((z + (1LL << 29)) & ((1LL << 30) - 1)) - (1LL << 29);
+    return {(int)((z - lo) / (1LL << 30)), (int)lo};
 }
 
 // Bits for fields that grow by at most a factor g before they are taken apart into
-// limbs (below 2^59)
-int fx_bits_for(double g) { return std::min(58, (int)floor(59.0 - log2(g) - 1e-6)); }
+// limbs (below 2^60)
+int fx_bits_for(double g) { return std::min(60, (int)floor(60.0 - log2(g) - 1e-6)); }
 
 // The filter's vectors in fixed point.  Before the third axis a field has grown by the
-// filter's row sum twice at most, and a mode's coefficient is at most its row of W
-// times that.  Filters that would leave the fields fewer than 54 bits keep the FP64
-// form (whose own error is 2^-50 of the largest value at worst; at a = 36, b = 50
-// the fields have 55 bits for P = 4 and 5, 54 for P = 6).
+// filter's row sum twice at most.  A mode's coefficient is at most its row of W times
+// that; it is held in units of 2^fx_k, below 2^61.  Filters that would leave fewer than
+// 55 bits keep the FP64 form (none of P = 2..6 at a = 36, b >= 2 does: 57 bits and
+// fx_k = 1 at P = 5 and b = 50, 56 at P = 6).
 void fixed_filter(Tables& T) {
     const int np1 = T.np1;
     double row = 1.0, w = 1.0;
@@ -156,13 +156,13 @@ void fixed_filter(Tables& T) {
         for (int j = 0; j < np1; ++j) s += fabs(T.FrW[r][j]);
         w = std::max(w, s);
     }
-    T.fx_bits = fx_bits_for(row * row * w);
-    T.fx_k = w > 4.0 ? (int)ceil(log2(w)) - 2 : 0;
-    if (T.fx_bits < 54) T.fx_bits = 0;
+    T.fx_bits = fx_bits_for(row * row);
+    T.fx_k = std::max(0, (int)ceil(log2(w)) - 1);
+    if (T.fx_bits - T.fx_k < 55) T.fx_bits = 0;
     for (int r = 0; r < T.nfr; ++r)
         for (int i = 0; i < np1; ++i) {
-            T.FxV[r][i] = fx_limbs_host(ldexpl((ld)T.FrV[r][i], 56));
-            T.FxW[r][i] = fx_limbs_host(ldexpl((ld)T.FrW[r][i], 56 - T.fx_k));
+            T.FxV[r][i] = fx_limbs_host(ldexpl((ld)T.FrV[r][i], 60));
+            T.FxW[r][i] = fx_limbs_host(ldexpl((ld)T.FrW[r][i], 60 - T.fx_k));
         }
 }
 
@@ -219,7 +219,7 @@ void build_tables(int P, double fa, double fb, int M, Tables& T) {
         for (int j = 0; j < np1; ++j) s += fabs(T.D[i][j]);
         T.Dabs = std::max(T.Dabs, s);
     }
-    T.fx_d = 59 - (int)ceil(log2(T.Dabs));
+    T.fx_d = 60 - (int)ceil(log2(T.Dabs));
     for (int i = 0; i < np1; ++i)
         for (int j = 0; j < np1; ++j) T.FxD[i][j] = fx_limbs_host(ldexpl((ld)T.D[i][j], T.fx_d));
     double row = 1.0;
@@ -227,7 +227,7 @@ void build_tables(int P, double fa, double fb, int M, Tables& T) {
         double s = 0.0;
         for (int j = 0; j < np1; ++j) {
             s += fabs(T.Pi[i][j]);
-            T.FxPi[i][j] = fx_limbs_host(ldexpl((ld)T.Pi[i][j], 56));
+            T.FxPi[i][j] = fx_limbs_host(ldexpl((ld)T.Pi[i][j], 60));
         }
         row = std::max(row, s);
     }

@@ -174,8 +174,8 @@ __device__ __forceinline__ void flux_normal_gen(const double* n, const PM& m, co
 }
 
 // One element of order P processed by a block of NT threads (NT >= (P+1)^3).
-// s_word [NV]: the largest words (fx_word) of the volume term's blocks, zero on entry
-// and on return; s_wordf [NV + 1]: of the filter's and of |B~|.
+// s_word [27, flat 12]: the largest words (fx_word) of the volume term's fields, zero on
+// entry and on return; s_wordf [NV + 1]: of the filter's and of |B~|.
 template <int P, int NT, int SUB, bool KS>
 __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, int e, double* sm, unsigned* s_word,
                                                unsigned* s_wordf) {
@@ -193,19 +193,18 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
     const int ci[3] = {tid % np1, (tid / np1) % np1, tid / (np1 * np1)};
     const int64_t eb = (int64_t)e * d.nn;
     const double dt = dt_of(d, e);
-    // Values of the volume term's contractions (fixed.cuh): 12 fields in three blocks --
-    // E~ and phi~ meet in the B~ equations, B~ and psi~ in those of E~, J~ alone --
-    // or on the Kerr-Schild background 27 fluxes in a block per variable.
-    constexpr int NB = KS ? NV : 3;
-    auto block = [](int v) { return KS ? v % NV : (v < 3 || v == 7 ? 0 : (v < NV ? 1 : 2)); };
+    // Fields of the volume term's contractions, each at its own scale (fixed.cuh): U and J~,
+    // or on the Kerr-Schild background the 27 fluxes.
+    constexpr int NB = KS ? 27 : 12;
     unsigned word[NB];
+#pragma unroll
     for (int b = 0; b < NB; ++b) word[b] = 0;
     if (act) {
 #pragma unroll
         for (int v = 0; v < (KS ? NV : 12); ++v) {
             const double x = v < NV ? a.Uin.dg(v)[eb + tid] : a.J.dg(3 + v - NV)[eb + tid];
             sU[v * nn + tid] = x;
-            if (!KS) word[block(v)] = max(word[block(v)], fx_word(x));
+            if (!KS && v != 8) word[v] = fx_word(x);   // q~ is not differentiated
         }
         if (KS) {
             PM m;
@@ -218,26 +217,22 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
             for (int j = 0; j < 3; ++j)
                 for (int v = 0; v < NV; ++v) {
                     sF[(j * NV + v) * nn + tid] = F[j][v];
-                    word[v % NB] = max(word[v % NB], fx_word(F[j][v]));
+                    word[(j * NV + v) % NB] = fx_word(F[j][v]);
                 }
             sources_gen(u, jd, m, d.met, d.ndg, eb + tid, S);
             for (int v = 0; v < NV; ++v) sR[v * nn + tid] = S[v];
         }
     }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        word[b] = __reduce_max_sync(0xffffffffu, word[b]);
-        if ((tid & 31) == 0) atomicMax(s_word + b, word[b]);
-    }
+    fx_largest<NB>(word, s_word);
     __syncthreads();
     if (tid <= NV) s_wordf[tid] = 0;
-    unsigned top = 0;
-    for (int b = 0; b < NB; ++b) top = max(top, s_word[b]);
-    const bool fixed = !d.fp64_lines && top < (unsigned)FX_EMAX << 20;
+    bool fixed = !d.fp64_lines;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) fixed = fixed && fx_inside(s_word[b]);
     if (act && fixed) {
 #pragma unroll
-        for (int v = 0; v < (KS ? 27 : 12); ++v)
-            fF[v * nn + tid] = fx_limbs(fx_from((KS ? sF : sU)[v * nn + tid], fx_exp(s_word[block(v)]), FX_BITS));
+        for (int v = 0; v < NB; ++v)
+            if (KS || v != 8) fF[v * nn + tid] = fx_limbs(fx_from((KS ? sF : sU)[v * nn + tid], fx_exp(s_word[v]), FX_BITS));
     }
     __syncthreads();
     if (act) {
@@ -294,8 +289,8 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
                     FxSum s;
 #pragma unroll
                     for (int mm = 0; mm < np1; ++mm) s.add(Dk[mm], fF[v * nn + base + mm * stride]);
-                    // units: 2^56 2^-fx_d 2^(e - 1022 - 58)
-                    return fx_double(s.top(), fx_exp(s_word[block(v)]) - 1024 - T.fx_d);
+                    // units: 2^60 2^-fx_d 2^(e - 1022 - 60)
+                    return fx_double(s.top(), fx_exp(s_word[v]) - 1022 - T.fx_d);
                 });
             }
         } else {
@@ -461,8 +456,8 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
 template <int P, int SUB, bool KS>
 __global__ void __launch_bounds__(DGC<P, KS>::NT, DGC<P, KS>::CTAS) k_dg_curved(Dev d, SubArgs a, const int* list, int ci) {
     extern __shared__ double sm[];
-    __shared__ unsigned s_word[NV], s_wordf[NV + 1];
-    if (threadIdx.x < NV) s_word[threadIdx.x] = 0;
+    __shared__ unsigned s_word[27], s_wordf[NV + 1];
+    if (threadIdx.x < 27) s_word[threadIdx.x] = 0;
     __syncthreads();
     const int nwork = d.counts[ci];
     for (int w = blockIdx.x; w < nwork; w += gridDim.x)

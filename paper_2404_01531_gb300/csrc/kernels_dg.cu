@@ -248,6 +248,15 @@ __device__ void dg_external_state(const Dev& d, const SubArgs& a, int e, int f, 
     current_flat(Ue, d.eta, jd, Je);
 }
 
+// The volume term of equation q (as numbered in U) takes D_k of variable term_var(q, k)
+// (9..11: J~) along axis k, with the sign term_neg(q, k).
+__host__ __device__ constexpr int term_var(int q, int k) {
+    return q < 3 ? (q == k ? 6 : 6 - q - k) : (q < 6 ? (q - 3 == k ? 7 : 6 - q - k) : (q == 6 ? k : (q == 7 ? 3 + k : 9 + k)));
+}
+__host__ __device__ constexpr bool term_neg(int q, int k) {
+    return q >= 6 || q % 3 == k || (q < 3) == ((q + 3 - k) % 3 == 1);
+}
+
 // The volume term in FP64, for elements whose values fixed point does not hold.
 template <int P>
 __device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* sU, const double* sD, double* r) {
@@ -301,106 +310,95 @@ __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, 
     double* sD = red + 2;            // [3][np1][np1]: (d xi^a/d x^a) D
     Fx* fD = (Fx*)sD;
     __shared__ int s_flag;
-    __shared__ unsigned s_word[3], s_wordf[NV + 1];  // largest words (fx_word) of the volume term's blocks, of the filter's, of |B~|
+    // largest words (fx_word) of U and J~, of the filter's variables, of |B~|
+    __shared__ unsigned s_word[12], s_wordf[NV + 1];
+    __shared__ int s_eq[NV], s_shift[3 * NV];   // exponents of the volume term's sums, shifts of their terms to them
     const Tables& T = *d.tab;
     const int tid = threadIdx.x;
     const bool act = tid < nn;
     const int i = tid % np1, j = (tid / np1) % np1, k = tid / (np1 * np1);
     const double w0inv = 1.0 / T.w0;
     const int nwork = d.counts[0];
-    if (tid < 3) s_word[tid] = 0;
+    if (tid < 12) s_word[tid] = 0;
     __syncthreads();
     for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
         const int e = d.dg_list[w];
         const int64_t eb = (int64_t)e * nn;
         const double sx = d.ijac[3 * e], sy = d.ijac[3 * e + 1], sz = d.ijac[3 * e + 2];
         double* r = sR + tid;
-        unsigned wE = 0, wB = 0, wJ = 0;
+        unsigned word[12];
         double jx[3] = {0.0, 0.0, 0.0};
-        if (act) {
 #pragma unroll
-            for (int v = 0; v < 12; ++v) {
-                const double x = v < NV ? a.Uin.dg(v)[eb + tid] : a.J.dg(3 + v - NV)[eb + tid];
-                if (v < NV) sU[v * nn + tid] = x;
-                else jx[v - NV] = x;
-                const unsigned w = fx_word(x);
-                if (v < 3 || v == 7) wE = max(wE, w);
-                else if (v < 7) wB = max(wB, w);
-                else if (v >= NV) wJ = max(wJ, w);
-            }
+        for (int v = 0; v < 12; ++v) {
+            word[v] = 0;
+            if (!act) continue;
+            const double x = v < NV ? a.Uin.dg(v)[eb + tid] : a.J.dg(3 + v - NV)[eb + tid];
+            if (v < NV) sU[v * nn + tid] = x;
+            else jx[v - NV] = x;
+            if (v != 8) word[v] = fx_word(x);   // q~ is not differentiated
         }
-        // blocks: E~ and phi~ meet in the B~ equations, B~ and psi~ in those of E~, J~ alone
-        wE = __reduce_max_sync(0xffffffffu, wE);
-        wB = __reduce_max_sync(0xffffffffu, wB);
-        wJ = __reduce_max_sync(0xffffffffu, wJ);
-        if ((tid & 31) == 0) {
-            atomicMax(&s_word[0], wE);
-            atomicMax(&s_word[1], wB);
-            atomicMax(&s_word[2], wJ);
+        fx_largest<12>(word, s_word);
+        const double rows[3] = {T.Dabs * fabs(sx), T.Dabs * fabs(sy), T.Dabs * fabs(sz)};   // bound the rows' |D| sums
+        int eD[3];
+        bool fixed = true;
+        for (int k = 0; k < 3; ++k) {
+            eD[k] = (int)(fx_word(rows[k]) >> 20);
+            fixed = fixed && eD[k] > 1023 - 60 && eD[k] < 1023 + 60;
         }
-        const double rows = T.Dabs * (fabs(sx) + fabs(sy) + fabs(sz));   // bounds the sums' |D| entries
-        const int eD = (int)(fx_word(rows) >> 20);
         __syncthreads();
         if (tid <= NV) s_wordf[tid] = 0;
-        const int eE = fx_exp(s_word[0]), eB = fx_exp(s_word[1]), eJ = fx_exp(s_word[2]);
-        const bool fixed = max(eE, max(eB, eJ)) < FX_EMAX && eD > 1023 - 60 && eD < 1023 + 60;
+#pragma unroll
+        for (int v = 0; v < 12; ++v) fixed = fixed && fx_inside(s_word[v]);
+        if (tid < NV) {
+            int e[3];
+            for (int k = 0; k < 3; ++k) e[k] = fx_exp(s_word[term_var(tid, k)]) + eD[k];
+            const int top = max(e[0], max(e[1], e[2]));
+            s_eq[tid] = top;
+            for (int k = 0; k < 3; ++k) s_shift[3 * tid + k] = min(top - e[k], 63);
+        }
         for (int t = tid; t < 3 * nf; t += NT) {
-            const double D = (t < nf ? sx : (t < 2 * nf ? sy : sz)) * T.D[(t % nf) / np1][t % np1];
-            if (fixed) fD[t] = fx_limbs(fx_from(D, eD, FX_BITS + 1));
+            const int k = t < nf ? 0 : (t < 2 * nf ? 1 : 2);
+            const double D = (k == 0 ? sx : (k == 1 ? sy : sz)) * T.D[(t % nf) / np1][t % np1];
+            if (fixed) fD[t] = fx_limbs(fx_from(D, k == 0 ? eD[0] : (k == 1 ? eD[1] : eD[2]), FX_BITS));
             else sD[t] = D;
         }
         if (act && fixed) {
 #pragma unroll
             for (int v = 0; v < 12; ++v)
-                fU[v * nn + tid] = fx_limbs(fx_from(v < NV ? sU[v * nn + tid] : jx[v < NV ? 0 : v - NV], v < 3 || v == 7 ? eE : (v < 7 ? eB : eJ), FX_BITS));
+                if (v != 8) fU[v * nn + tid] = fx_limbs(fx_from(v < NV ? sU[v * nn + tid] : jx[v < NV ? 0 : v - NV], fx_exp(s_word[v]), FX_BITS));
         }
         __syncthreads();
-        if (tid < 3) s_word[tid] = 0;
+        if (tid < 12) s_word[tid] = 0;
         if (act && fixed) {
-            const int ox = np1 * (j + np1 * k), oy = i + np1 * np1 * k, oz = i + np1 * j;
-            const Fx *Dx = fD + np1 * i, *Dy = fD + nf + np1 * j, *Dz = fD + 2 * nf + np1 * k;
-            auto ux = [&](int v, int m) { return fU[v * nn + ox + m]; };
-            auto uy = [&](int v, int m) { return fU[v * nn + oy + np1 * m]; };
-            auto uz = [&](int v, int m) { return fU[v * nn + oz + np1 * np1 * m]; };
-            // units: 2^56 2^(e - 1022 - 58) 2^(eD - 1022 - 59)
-            auto out = [&](const FxSum& X, int e) { return fx_double(X.top(), e + eD - 2105); };
-            {   // E: curl B - grad psi, phi: -div B
-                FxSum X, Y, Z, W;
+            // Nine sums of three lines each: E~: curl B~ - grad psi~ - J~, B~: -curl E~ - grad phi~,
+            // psi~: -div E~ + q~, phi~: -div B~, q~: -div J~; axis by axis, so that a row of D is
+            // loaded once, every line at its own scale and shifted to its sum's
+            long long acc[NV];
 #pragma unroll
-                for (int m = 0; m < np1; ++m) {
-                    const Fx p = Dx[m], q = Dy[m], t = Dz[m], np = fx_neg(p), nq = fx_neg(q), nt = fx_neg(t);
-                    X.add(uy(5, m), q); X.add(uz(4, m), nt); X.add(ux(6, m), np);
-                    Y.add(uz(3, m), t); Y.add(ux(5, m), np); Y.add(uy(6, m), nq);
-                    Z.add(ux(4, m), p); Z.add(uy(3, m), nq); Z.add(uz(6, m), nt);
-                    W.add(ux(3, m), np); W.add(uy(4, m), nq); W.add(uz(5, m), nt);
+            for (int q = 0; q < NV; ++q) acc[q] = 0;
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                const int stride = ax == 0 ? 1 : (ax == 1 ? np1 : nf), c = ax == 0 ? i : (ax == 1 ? j : k);
+                const Fx* line = fU + tid - c * stride;
+                Fx Dr[np1];
+#pragma unroll
+                for (int m = 0; m < np1; ++m) Dr[m] = fD[ax * nf + np1 * c + m];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    FxSum s;
+#pragma unroll
+                    for (int m = 0; m < np1; ++m) s.add(line[term_var(q, ax) * nn + m * stride], Dr[m]);
+                    const long long t = s.top() >> s_shift[3 * q + ax];
+                    acc[q] += term_neg(q, ax) ? -t : t;
                 }
-                r[0] = out(X, eB) - a.J.dg(0)[eb + tid];
-                r[nn] = out(Y, eB) - a.J.dg(1)[eb + tid];
-                r[2 * nn] = out(Z, eB) - a.J.dg(2)[eb + tid];
-                r[7 * nn] = out(W, eB);
             }
-            {   // B: -curl E - grad phi, psi: -div E + q
-                FxSum X, Y, Z, W;
+            // units: 2^60 2^(e - 1022 - 60) 2^(eD - 1022 - 60)
 #pragma unroll
-                for (int m = 0; m < np1; ++m) {
-                    const Fx p = Dx[m], q = Dy[m], t = Dz[m], np = fx_neg(p), nq = fx_neg(q), nt = fx_neg(t);
-                    X.add(uy(2, m), nq); X.add(uz(1, m), t); X.add(ux(7, m), np);
-                    Y.add(uz(0, m), nt); Y.add(ux(2, m), p); Y.add(uy(7, m), nq);
-                    Z.add(ux(1, m), np); Z.add(uy(0, m), q); Z.add(uz(7, m), nt);
-                    W.add(ux(0, m), np); W.add(uy(1, m), nq); W.add(uz(2, m), nt);
-                }
-                r[3 * nn] = out(X, eE);
-                r[4 * nn] = out(Y, eE);
-                r[5 * nn] = out(Z, eE);
-                r[6 * nn] = out(W, eE) + sU[8 * nn + tid];
-            }
-            {   // q: -div J
-                FxSum X;
-#pragma unroll
-                for (int m = 0; m < np1; ++m) {
-                    X.add(ux(9, m), fx_neg(Dx[m])); X.add(uy(10, m), fx_neg(Dy[m])); X.add(uz(11, m), fx_neg(Dz[m]));
-                }
-                r[8 * nn] = out(X, eJ);
+            for (int q = 0; q < NV; ++q) {
+                double x = fx_double(acc[q], s_eq[q] - 2104);
+                if (q < 3) x -= a.J.dg(q)[eb + tid];
+                if (q == 6) x += sU[8 * nn + tid];
+                r[q * nn] = x;
             }
         } else if (act) {
             volume_fp64<P>(a.J, eb, sU, sD, r);
