@@ -47,3 +47,28 @@ def test_concurrent_contexts_on_their_own_streams_equal_sequential_runs(ffe):
         assert np.array_equal(mc, m)
         assert np.array_equal(Uc, U)
         c.close()
+
+
+def test_step_captured_by_the_caller(ffe):
+    """A caller that captures the context's stream gets the step's launches themselves, also from a
+    context that has its own step graph: replays advance the state as steps do."""
+    cfg = W.pulsar(r_lc=5.0, chi=math.radians(60.0), n_ang=2, n_rad=4, P=5, r_out=20.0)
+    s = torch.cuda.Stream()
+    own, ref = ffe.Context(cfg, stream=s), ffe.Context(cfg, stream=s)
+    for c in (own, ref):
+        c.set_initial()
+        c.step(4)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="thread_local"):
+        own.step(1)
+    with torch.cuda.stream(s):
+        for _ in range(3):
+            g.replay()
+    ref.step(3)
+    torch.cuda.synchronize()
+    (Ua, ma), (Ub, mb) = own.download(), ref.download()
+    assert np.array_equal(ma, mb) and np.array_equal(Ua, Ub)
+    assert own.status() == 0
+    for c in (own, ref):
+        c.close()
