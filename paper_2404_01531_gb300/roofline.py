@@ -1,9 +1,13 @@
-"""Algorithmic FP64 operation counts of the hot kernels (FMA = 2 flops,
-add/mul/div/sqrt = 1), counted from the operations the method defines, not
-from the instructions the kernels happen to issue.  Used for the roofline
-fraction: achieved = count x units per launch / launch time.  The kernels share
-work between neighbouring face values and run line contractions and WENO5-Z
-weights on the integer pipes, so the fraction of the FP64 peak can exceed 1."""
+"""Operation counts of the hot kernels, two kinds.
+
+*_flops: the method's FP64 work (FMA = 2 flops, add/mul/div/sqrt = 1), counted
+from the operations the method defines.  The kernels share work between
+neighbouring face values and run line contractions and WENO5-Z weights on the
+integer pipes, so this divided by the launch time can exceed the FP64 peak.
+
+*_fp64_ops: FP64 operations the kernels issue.  Each takes one FMA slot of the
+FP64 pipe, the pipe with the highest use, so 2 x ops / time over the peak is
+the fraction of that bound (at most 1)."""
 import math
 
 
@@ -62,3 +66,28 @@ def fd_flux_flops(recon, quantities=10):
 def fd_faces_per_element(P):
     nc = 2 * P + 1
     return 3 * (nc + 1) * nc * nc
+
+
+def fd_flux_fp64_ops(recon, P, quantities=10, corrector=True):
+    """FP64 operations per face that k_fd_flux (a box: 10 quantities a direction) or
+    k_fd_states (a flat shell: 12) issues: a line of nc cells takes nc two-sided
+    reconstructions, two one-sided ones and 5 differences (MP5: its unlimited path),
+    a face the flux of 5 pairs of quantities, or the states of 6.  ncu counts
+    the same 308.3 for k_fd_flux at P = 5 with the corrector."""
+    nc = 2 * P + 1
+    both, one = (14, 8) if recon == 1 else (25, 15)
+    line = quantities * (nc * both + 2 * one + 5) / (nc + 1)
+    if quantities == 12:
+        return line + (66 if corrector else 42)
+    return line + (50 if corrector else 30)
+
+
+# FP64 operations a thread of k_dg_substep issues per node in substeps A, B and C at
+# P = 5, flat metric, filter (a = 36, b = 50) and indicator on: FP64-pipe instructions
+# (ncu sm__inst_executed_pipe_fp64) over 28672 warps of 4096 elements
+DG_FP64_OPS_P5 = (138.1, 157.1, 122.1)
+
+
+def dg_fp64_ops_per_element(P):
+    """Mean over the substeps, for the threads of an element's CTA; None at other orders."""
+    return sum(DG_FP64_OPS_P5) / 3.0 * 224 if P == 5 else None
