@@ -448,7 +448,7 @@ __device__ __forceinline__ void dg_curved_elem(const Dev& d, const SubArgs& a, i
 // contracted with the normal at once (27 FMAs; with the general metric's flux and a
 // constant flat metric it was 170 slots), and the face sums go axis by axis.  Two CTAs
 // an SM at P = 5 (P <= 4: three or four), also with the metric, which had one and idled
-// at its barriers.  7146 elements of orders 4 and 5: substep 0.97 -> 0.63 ms (1.42 before
+// at its barriers.  7146 elements of orders 4 and 5: substep 0.97 -> 0.64 ms (1.42 before
 // the work outside the contractions went down); Kerr-Schild, 1536 elements: 0.77 ->
 // 0.48 ms.  Batched contexts launch each order's elements separately, in
 // CTAs sized for that order (one kernel dispatching on the order would keep every

@@ -297,7 +297,7 @@ __device__ __forceinline__ void volume_fp64(Field J, int64_t eb, const double* s
 // current sheet against 0.402; two without spills: 3% slower than three).
 // 4096 elements at P = 5, average of the substeps: 0.870 ms, 0.757 with less work per
 // node, 0.551 with the volume term in integers, 0.493 with the indicator, 0.444 with the
-// filter, 0.440 with four CTAs, 0.432 axis by axis with a scale for every variable and
+// filter, 0.440 with four CTAs, 0.421 axis by axis with a scale for every variable and
 // axis (a row of D is loaded once, 588 bytes of spills instead of 952).
 template <int P, int SUB>
 __global__ void __launch_bounds__(DGK<P>::NT, DGK<P>::CTAS) k_dg_substep(Dev d, SubArgs a) {

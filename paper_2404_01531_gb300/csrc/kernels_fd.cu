@@ -335,10 +335,11 @@ __global__ void k_fd_fill(Dev d, const int* list, int ci, int w0, Field U, Field
 // from one set of smoothness indicators (Weno5zLine), for the two quantities
 // that a pair of flux components needs, so that the flux is formed in registers;
 // the two components of J~ across the direction are not reconstructed.  At P = 5
-// that is 320 FP64 operations per face, the indicators and weights hidden on the
+// that is 308 FP64 operations per face, the indicators and weights hidden on the
 // integer pipes (z_weights), against about 1100 of a thread per face: 384 elements
 // 3.44 -> 1.84 ms with 610 of them; two steps of the 64x8x8 current sheet 14.8 -> 13.7
-// ms from 610 to 530, 11.6 with the weights in integers, 10.4 with the indicators too;
+// ms from 610 to 530, 11.6 with the weights in integers, 10.4 with the indicators too
+// (9.6 with all of the step as it is);
 // MP5 on 125 elements 1.53 -> 0.41 ms.
 template <int RECON>
 __global__ void __launch_bounds__(64, 8) k_fd_flux(Dev d, const int* list, int ci, int w0) {
@@ -376,7 +377,8 @@ __global__ void __launch_bounds__(64, 8) k_fd_flux(Dev d, const int* list, int c
 // (2/3)(L + R) - (U_m + U_p)/6 -- and D = (U_R - U_L)/2 -- times 4/3 -- of the 9
 // variables: F^j = F^j(G) - n^_j D, formed once per cell by k_fd_update instead
 // of once per face (21 values a face instead of 27, no normals here): 300 elements
-// 2.74 -> 1.77 ms at P = 5, k_fd_update 0.28 -> 0.31 ms.
+// 2.74 -> 1.77 ms at P = 5 (0.92 with indicators and weights in integers),
+// k_fd_update 0.28 -> 0.25 ms.
 template <int RECON>
 __global__ void __launch_bounds__(64, 8) k_fd_states(Dev d, const int* list, int ci, int w0) {
     const int n = chunk_n(d, ci, w0);
